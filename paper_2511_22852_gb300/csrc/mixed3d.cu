@@ -1,11 +1,22 @@
 // mixed3d.cu -- the neighbour passes (rows a3, a5) of the 3+1D step in the mixed-precision
-// form: cell-tiled over the 27 neighbouring 2h-cells, positions relative to the origin of their
-// cell in single precision, separations (r_a - r_b) - o (2h) formed from numbers of size <= 2h,
-// a proven float error band around (2h)^2 inside which the FP64 test r^2 < (2h)^2 (separately
-// rounded products) decides -- the neighbour sets are those of the FP64 form -- and sums
-// accumulated in float in short runs folded into Neumaier-compensated sums, a particle's lanes
-// combined with error-free FP32 additions.  The EoS inversion, equations of motion and
-// reductions stay FP64 (step3d.cu).
+// form: positions relative to the origin of their cell in single precision, separations
+// (r_a - r_b) - o (2h) formed from numbers of size <= 2h, a proven float error band around (2h)^2
+// inside which the FP64 test r^2 < (2h)^2 (separately rounded products) decides -- the neighbour
+// sets are those of the FP64 form.  The EoS inversion, equations of motion and reductions stay
+// FP64 (step3d.cu).
+//
+// One warp takes two consecutive particles of a cell through the candidates of the 27 cells of
+// side 2h around it, 32 candidates at a time, both particles in one packed two-wide FP32
+// instruction.  The cells hold 216 h^3 of candidates for 33.5 h^3 of neighbours (6.4 to 1), so
+// rejecting has to be cheap and the pair arithmetic must not run on rejected candidates: cells
+// farther than 2h from both particles are left out (20.6 of 27 remain on average), accepted
+// candidates are compacted into a queue (with their separation), and 32 at a time the kernel and
+// the sums run on full warps.  Each lane sums at most kRun terms in plain FP32; the lanes' sums
+// are then combined by error-free additions, one lane per sum over a transposed copy in shared
+// memory, and converted to FP64 once.
+//
+// Bound: instruction issue (the rejection walk, about 1,500 warp instructions per particle and
+// pass, against 900 for the accepted pairs of the density and 1,400 of the gradient pass).
 #include <algorithm>
 
 #include "sph_internal.cuh"
@@ -24,414 +35,349 @@ __device__ __forceinline__ uint32_t key3m(const EvView &v, int cx, int cy, int c
     return v.spread[cx] | v.spread[1024 + cy] | v.spread[2048 + cz];
 }
 
-// cell-relative single-precision positions of the sorted particles
-__global__ void k_relpos3(EvView v, const double *__restrict__ y, float4 *__restrict__ rel)
+// cell-relative single-precision positions of the sorted particles, w: the cell's coordinates
+// (10 bits per axis), and the density pass's per-particle values (S, N_B, N_S, N_Q) in FP32
+__global__ void k_relpos3(EvView v, const double *__restrict__ y, const double *__restrict__ Nq,
+                          float4 *__restrict__ rel, float4 *__restrict__ fq)
 {
     int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= v.n) return;
+    const size_t n = (size_t)v.n;
     const double cs = 2.0 * v.h;
     float r[3];
+    int pk = 0;
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
         const double xm = dec_double(v.sc->xmin_enc[d]);
-        const double x = y[(size_t)d * v.n + j];
+        const double x = y[(size_t)d * n + j];
         const int c = cell_coord(x, xm, v.inv_cell);
         r[d] = __double2float_rn(__dsub_rn(__dsub_rn(x, xm), (double)c * cs));
+        pk |= min(max(c, 0), (1 << v.B3[d]) - 1) << (10 * d);  // as the sort clamps it
     }
-    rel[j] = make_float4(r[0], r[1], r[2], 0.0f);
+    rel[j] = make_float4(r[0], r[1], r[2], __int_as_float(pk));
+    fq[j] = make_float4((float)y[6 * n + j], (float)Nq[j], (float)Nq[n + j], (float)Nq[2 * n + j]);
 }
 
-// Cell-tiled passes (the 3+1D counterpart of the 2+1D ones): one block per occupied cell
-// (grid-stride over the cell grid) stages the candidates of the 3x3x3 block of 2h-cells -- 27
-// runs of the sorted order -- in shared memory, two candidates per float4 entry (packed
-// two-wide FP32 arithmetic), and the cell's particles scan them with L lanes each.  A candidate
-// carries its own-cell-relative position and its cell's offset separately, and r^2 is nested
-// as fmaf(dx, dx, fmaf(dy, dy, dz dz)), the rounding the 3+1D shell bound assumes.
-constexpr int kTT3 = 256;    // threads of a tiled block; all its warps share a cell's particles
-constexpr int kTile3 = 512;  // candidates staged at a time
-
-struct Runs27 {
-    int rs[27];
-    int cum[28];
-    float o[3][27];  // the run's cell offset times the float cell side, per axis
-};
-
-__device__ __forceinline__ void runs27_setup(const EvView &v, const uint32_t *__restrict__ start,
-                                             const uint32_t *__restrict__ cnt, const int c[3], Runs27 &R)
+// the gradient pass's inputs in FP32: rows 4 m .. 4 m + 3 of gin in fx[m n ..]
+__global__ void k_fx3(int n_, const double *__restrict__ gin, float4 *__restrict__ fx)
 {
-    const int t = threadIdx.x;
-    if (t < 27) {
-        const int d[3] = {t % 3 - 1, (t / 3) % 3 - 1, t / 9 - 1};
-        int nc[3];
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= n_) return;
+    const size_t n = (size_t)n_;
+#pragma unroll
+    for (int m = 0; m < 3; ++m)
+        fx[m * n + j] = make_float4((float)gin[(4 * m) * n + j], (float)gin[(4 * m + 1) * n + j],
+                                    (float)gin[(4 * m + 2) * n + j], (float)gin[(4 * m + 3) * n + j]);
+}
+
+constexpr int kWW = 8;                // warps per block, two particles each
+constexpr unsigned kFull = 0xFFFFFFFFu;
+
+struct WalkMem {
+    float4 q[2][64];  // queued pairs of the two particles: separation and candidate index
+};
+// one particle's lane sums, transposed: NV values of 33 floats (over the queues when they are empty)
+static_assert(sizeof(WalkMem) >= 15 * 33 * sizeof(float), "the sums fit over the queues");
+
+// NV per-lane sums of one particle combined into lane v < NV (its running hi + lo), error-free:
+// hi = TwoSum(hi, term) with the rounding errors in lo
+template <int NV>
+__device__ __forceinline__ void flush_sums(float *red, float (&s)[NV], int lane, bool mine, int slot, CSum &tot)
+{
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+        red[k * 33 + lane] = s[k];
+        s[k] = 0.0f;
+    }
+    __syncwarp();
+    if (mine) {
+        float hi = tot.hi, lo = tot.lo;
+#pragma unroll 8
+        for (int j = 0; j < 32; ++j) {
+            const float x = red[slot * 33 + j];
+            const float t = hi + x, bb = t - hi;
+            lo += (hi - (t - bb)) + (x - bb);
+            hi = t;
+        }
+        tot = CSum{hi, lo};
+    }
+    __syncwarp();
+}
+
+// The walk of one warp over the candidates of particles a0 and a1 = a0 + 1 (both in the cell of
+// ra0; two = false: a0 alone).  pair(which, entry) receives an accepted pair per lane; done(force)
+// is called after every kRun batches and at the end, with empty queues.
+// nacc: accepted candidates (self included); shell: candidates decided by the FP64 test.
+template <class Pair, class Flush>
+__device__ __forceinline__ void walk27_two(const EvView &v, const double *__restrict__ y,
+                                           const float4 *__restrict__ rel, const uint32_t *__restrict__ start,
+                                           const uint32_t *__restrict__ cnt, int a0, bool two, float4 ra0, float4 ra1,
+                                           WalkMem &M, int lane, int (&nacc)[2], unsigned &shell, Pair &&pair,
+                                           Flush &&flush)
+{
+    const size_t n = (size_t)v.n;
+    const unsigned lt = (1u << lane) - 1u;
+    const float slo = v.shell_lo, shi = v.shell_hi, cell = v.cell_f;
+    const int pk = __float_as_int(ra0.w);
+    if (!two) ra1 = make_float4(kFar, kFar, kFar, 0.0f);  // never accepted
+    // lane t < 27: the neighbour cell t, kept when it holds particles and its box lies within 2h
+    // (with a margin far above the positions' rounding) of either particle
+    int st = 0, len = 0;
+    if (lane < 27) {
+        const int o[3] = {lane % 3 - 1, (lane / 3) % 3 - 1, lane / 9 - 1};
+        int c[3];
         bool in = true;
+        float d0 = 0.0f, d1 = 0.0f;
+        const float p0[3] = {ra0.x, ra0.y, ra0.z}, p1[3] = {ra1.x, ra1.y, ra1.z};
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            nc[k] = c[k] + d[k];
-            in = in && nc[k] >= 0 && nc[k] < (1 << v.B3[k]);
+            c[k] = ((pk >> (10 * k)) & 1023) + o[k];
+            in = in && c[k] >= 0 && c[k] < (1 << v.B3[k]);
+            const float g0 = o[k] < 0 ? p0[k] : (o[k] > 0 ? cell - p0[k] : 0.0f);
+            const float g1 = o[k] < 0 ? p1[k] : (o[k] > 0 ? cell - p1[k] : 0.0f);
+            d0 = fmaf(fmaxf(g0, 0.0f), g0, d0);
+            d1 = fmaf(fmaxf(g1, 0.0f), g1, d1);
         }
-        int st = 0, len = 0;
-        if (in) {
-            const uint32_t k = key3m(v, nc[0], nc[1], nc[2]);
+        const float lim = shi * 1.0001f;
+        // written so that a NaN position keeps the cell
+        if (in && (!(d0 > lim) || (two && !(d1 > lim)))) {
+            const uint32_t k = key3m(v, c[0], c[1], c[2]);
             st = (int)start[k];
             len = (int)cnt[k];
         }
-        R.rs[t] = st;
-        R.cum[t + 1] = len;
+    }
+    unsigned cells = __ballot_sync(kFull, len > 0);
+    const float2 ax = make_float2(ra0.x, ra1.x), ay = make_float2(ra0.y, ra1.y), az = make_float2(ra0.z, ra1.z);
+    int qn[2] = {0, 0}, nb = 0;
+    while (cells) {
+        const int o = __ffs(cells) - 1;
+        cells &= cells - 1u;
+        const int b0 = __shfl_sync(kFull, st, o), ln = __shfl_sync(kFull, len, o);
+        const float ox = -(float)(o % 3 - 1) * cell, oy = -(float)((o / 3) % 3 - 1) * cell, oz = -(float)(o / 9 - 1) * cell;
+        for (int base = 0; base < ln; base += 32) {
+            const bool in = base + lane < ln;
+            const int b = b0 + base + lane;
+            float4 rb = make_float4(-kFar, -kFar, -kFar, 0.0f);
+            if (in) rb = rel[b];
+            // (r_a - r_b) - o (2h), rounded step by step as the shell bound assumes
+            const float2 dx = __fadd2_rn(__fadd2_rn(ax, make_float2(-rb.x, -rb.x)), make_float2(ox, ox));
+            const float2 dy = __fadd2_rn(__fadd2_rn(ay, make_float2(-rb.y, -rb.y)), make_float2(oy, oy));
+            const float2 dz = __fadd2_rn(__fadd2_rn(az, make_float2(-rb.z, -rb.z)), make_float2(oz, oz));
+            const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
+            bool acc0 = r2.x <= shi, acc1 = r2.y <= shi;
+            if ((acc0 && r2.x >= slo) || (acc1 && r2.y >= slo)) {  // thin shell: the exact FP64 decision
+                const double xb = y[b], yb = y[n + b], zb = y[2 * n + b];
+                if (acc0 && r2.x >= slo) {
+                    acc0 = dist2_3e(y[a0] - xb, y[n + a0] - yb, y[2 * n + a0] - zb) < v.supp2;
+                    ++shell;
+                }
+                if (acc1 && r2.y >= slo) {
+                    acc1 = dist2_3e(y[a0 + 1] - xb, y[n + a0 + 1] - yb, y[2 * n + a0 + 1] - zb) < v.supp2;
+                    ++shell;
+                }
+            }
+            const unsigned m0 = __ballot_sync(kFull, acc0), m1 = __ballot_sync(kFull, acc1);
+            if (m0) {
+                if (acc0) M.q[0][qn[0] + __popc(m0 & lt)] = make_float4(dx.x, dy.x, dz.x, __int_as_float(b));
+                qn[0] += __popc(m0);
+                nacc[0] += __popc(m0);
+            }
+            if (m1) {
+                if (acc1) M.q[1][qn[1] + __popc(m1 & lt)] = make_float4(dx.y, dy.y, dz.y, __int_as_float(b));
+                qn[1] += __popc(m1);
+                nacc[1] += __popc(m1);
+            }
 #pragma unroll
-        for (int k = 0; k < 3; ++k) R.o[k][t] = (float)d[k] * v.cell_f;
-    }
-    __syncthreads();
-    if (t == 0) {
-        R.cum[0] = 0;
-        for (int o = 0; o < 27; ++o) R.cum[o + 1] += R.cum[o];
-    }
-    __syncthreads();
-}
-
-__device__ __forceinline__ int run27_of(const Runs27 &R, int q)
-{
-    int lo = 0, hi = 26;  // the last run whose start is <= q
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (R.cum[mid] <= q) lo = mid;
-        else hi = mid - 1;
-    }
-    return lo;
-}
-
-// the candidate's staged geometry: (-x, -y) and (-z, -o_z) pairs, and the (-o_x, -o_y) offsets
-__device__ __forceinline__ void stage_geom(float4 *cP, float4 *cPz, float4 *cO, int i, float4 rb, const Runs27 &R,
-                                           int o)
-{
-    put_pair(cP, i, -rb.x, -rb.y);
-    put_pair(cPz, i, -rb.z, -R.o[2][o]);
-    put_pair(cO, i, -R.o[0][o], -R.o[1][o]);
-}
-__device__ __forceinline__ void stage_far(float4 *cP, float4 *cPz, float4 *cO, int i)
-{
-    put_pair(cP, i, kFar, kFar);
-    put_pair(cPz, i, kFar, 0.0f);
-    put_pair(cO, i, 0.0f, 0.0f);
-}
-
-// separations and r^2 of a candidate pair, (r_a - r_b) - o (2h) per axis
-__device__ __forceinline__ void sep2(float4 ra, float4 pk, float4 pz, float4 po, float2 &dx, float2 &dy, float2 &dz,
-                                     float2 &r2)
-{
-    dx = __fadd2_rn(__fadd2_rn(make_float2(ra.x, ra.x), lo2(pk)), lo2(po));
-    dy = __fadd2_rn(__fadd2_rn(make_float2(ra.y, ra.y), hi2(pk)), hi2(po));
-    dz = __fadd2_rn(__fadd2_rn(make_float2(ra.z, ra.z), lo2(pz)), hi2(pz));
-    r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
-}
-
-__global__ void __launch_bounds__(kTT3) k_tiled_density3m(EvView v, const double *__restrict__ y,
-                                                          const float4 *__restrict__ rel,
-                                                          const double *__restrict__ Nq,
-                                                          const uint32_t *__restrict__ start,
-                                                          const uint32_t *__restrict__ cnt,
-                                                          double *__restrict__ dens, int *__restrict__ nnb)
-{
-    __shared__ float4 cP[kTile3 / 2], cPz[kTile3 / 2], cO[kTile3 / 2];
-    __shared__ float4 cQa[kTile3 / 2];  // (S_0, S_1, N_B0, N_B1)
-    __shared__ float4 cQb[kTile3 / 2];  // (N_S0, N_S1, N_Q0, N_Q1)
-    __shared__ Runs27 R;
-    __shared__ unsigned long long s_acc[2];
-    const size_t n = (size_t)v.n;
-    const double *S = y + 6 * n;
-    const int l0 = 1 << v.B3[0], l1 = 1 << v.B3[1];
-    const long long ncell = (long long)l0 * l1 * (1 << v.B3[2]);
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    constexpr int NW = kTT3 / 32;
-    const float ih = (float)v.inv_h, slo = v.shell_lo, shi = v.shell_hi;
-    const double supp2 = v.supp2, sd = v.sigma_d;
-    if (tid == 0) s_acc[0] = s_acc[1] = 0ull;
-    for (long long ci = blockIdx.x; ci < ncell; ci += gridDim.x) {  // block-uniform
-        const int c[3] = {(int)(ci % l0), (int)((ci / l0) % l1), (int)(ci / ((long long)l0 * l1))};
-        const uint32_t kc = key3m(v, c[0], c[1], c[2]);
-        const int na = (int)cnt[kc];
-        if (na == 0) continue;
-        __syncthreads();
-        runs27_setup(v, start, cnt, c, R);
-        const int M = R.cum[27], first = (int)start[kc];
-        const int L = lanes_per_particle(na, NW), ppw = 32 / L;
-        const int pl = lane / L, l = lane - pl * L;
-        unsigned pairs = 0u, shell = 0u;
-        for (int g0 = 0; g0 < na; g0 += NW * ppw) {
-            const int my = g0 + warp * ppw + pl;
-            const bool valid = pl < ppw && my < na;
-            const int a = first + (valid ? my : 0);
-            const double xa[3] = {y[a], y[n + a], y[2 * n + a]};
-            const float4 ra = rel[a];
-            CSum sg = {0.f, 0.f}, ss = {0.f, 0.f}, sb = {0.f, 0.f}, sS = {0.f, 0.f}, sq = {0.f, 0.f};
-            int nacc = 0;
-            for (int t0 = 0; t0 < M; t0 += kTile3) {
-                const int mt = min(kTile3, M - t0);
-                if (g0 == 0 || M > kTile3) {
-                    if (t0 > 0 || g0 > 0) __syncthreads();
-                    for (int i = tid; i < mt; i += kTT3) {
-                        const int q = t0 + i, o = run27_of(R, q), b = R.rs[o] + (q - R.cum[o]);
-                        stage_geom(cP, cPz, cO, i, rel[b], R, o);
-                        put_pair(cQa, i, (float)S[b], (float)Nq[b]);
-                        put_pair(cQb, i, (float)Nq[n + b], (float)Nq[2 * n + b]);
-                    }
-                    if ((mt & 1) && tid == 0) {
-                        stage_far(cP, cPz, cO, mt);
-                        put_pair(cQa, mt, 0.0f, 0.0f);
-                        put_pair(cQb, mt, 0.0f, 0.0f);
-                    }
-                    __syncthreads();
+            for (int p = 0; p < 2; ++p)
+                if (qn[p] >= 32) {
+                    __syncwarp();
+                    pair(p, M.q[p][lane]);
+                    const float4 rest = M.q[p][32 + lane];
+                    __syncwarp();
+                    qn[p] -= 32;
+                    if (lane < qn[p]) M.q[p][lane] = rest;
+                    ++nb;
                 }
-                if (valid) {
-                    const float2 ih2 = make_float2(ih, ih);
-                    const int np = (mt + 1) >> 1;
-                    for (int kb = l; kb < np; kb += (kRun / 2) * L) {
-                        const int ke = min(np, kb + (kRun / 2) * L);
-                        float2 pg = make_float2(0.f, 0.f), ps = pg, pB = pg, pS = pg, pQ = pg;
-#pragma unroll 2
-                        for (int k = kb; k < ke; k += L) {
-                            float2 dx, dy, dz, r2;
-                            sep2(ra, cP[k], cPz[k], cO[k], dx, dy, dz, r2);
-                            bool a0 = r2.x < slo, a1 = r2.y < slo;
-                            if (r2.x >= slo && r2.x <= shi) {  // thin shell: the exact FP64 decision
-                                const int q = t0 + 2 * k, o = run27_of(R, q), b = R.rs[o] + (q - R.cum[o]);
-                                a0 = dist2_3e(xa[0] - y[b], xa[1] - y[n + b], xa[2] - y[2 * n + b]) < supp2;
-                                ++shell;
-                            }
-                            if (r2.y >= slo && r2.y <= shi) {
-                                const int q = t0 + 2 * k + 1, o = run27_of(R, q), b = R.rs[o] + (q - R.cum[o]);
-                                a1 = dist2_3e(xa[0] - y[b], xa[1] - y[n + b], xa[2] - y[2 * n + b]) < supp2;
-                                ++shell;
-                            }
-                            const float2 qq = __fmul2_rn(make_float2(sqrt_apx(r2.x), sqrt_apx(r2.y)), ih2);
-                            float2 t2, t, u2, u;
-                            spline_terms2(qq, t2, t, u2, u);
-                            float2 w = __ffma2_rn(__fmul2_rn(make_float2(0.25f, 0.25f), t2), t,
-                                                  __fmul2_rn(u2, make_float2(-u.x, -u.y)));
-                            w.x = a0 ? w.x : 0.0f;
-                            w.y = a1 ? w.y : 0.0f;
-                            const float4 qa = cQa[k], qb = cQb[k];
-                            pg = __fadd2_rn(pg, w);
-                            ps = __ffma2_rn(lo2(qa), w, ps);
-                            pB = __ffma2_rn(hi2(qa), w, pB);
-                            pS = __ffma2_rn(lo2(qb), w, pS);
-                            pQ = __ffma2_rn(hi2(qb), w, pQ);
-                            nacc += (int)a0 + (int)a1;
-                        }
-                        cadd(sg, pg.x + pg.y);
-                        cadd(ss, ps.x + ps.y);
-                        cadd(sb, pB.x + pB.y);
-                        cadd(sS, pS.x + pS.y);
-                        cadd(sq, pQ.x + pQ.y);
-                    }
-                }
-            }
-            sg = seg_csum(sg, l, L);
-            ss = seg_csum(ss, l, L);
-            sb = seg_csum(sb, l, L);
-            sS = seg_csum(sS, l, L);
-            sq = seg_csum(sq, l, L);
-            for (int o = 1; o < L; o <<= 1) {
-                const int t = __shfl_down_sync(0xFFFFFFFFu, nacc, o);
-                if ((l & (2 * o - 1)) == 0 && l + o < L) nacc += t;
-            }
-            if (valid && l == 0) {
-                dens[a] = sd * cval(sg);
-                dens[n + a] = sd * cval(ss);
-                dens[2 * n + a] = sd * cval(sb);
-                dens[3 * n + a] = sd * cval(sS);
-                dens[4 * n + a] = sd * cval(sq);
-                nnb[a] = nacc;
-                pairs += (unsigned)nacc;
+            if (nb >= kRun) {  // at most kRun plain terms per lane
+                __syncwarp();
+                if (lane < qn[0]) pair(0, M.q[0][lane]);
+                if (lane < qn[1]) pair(1, M.q[1][lane]);
+                qn[0] = qn[1] = nb = 0;
+                flush();
             }
         }
-        pairs = __reduce_add_sync(0xFFFFFFFFu, pairs);
-        shell = __reduce_add_sync(0xFFFFFFFFu, shell);
+    }
+    __syncwarp();
+    if (lane < qn[0]) pair(0, M.q[0][lane]);
+    if (lane < qn[1]) pair(1, M.q[1][lane]);
+    flush();
+}
+
+// Density pass (row a3).
+__global__ void __launch_bounds__(32 * kWW, 4) k_walk_density3m(EvView v, const double *__restrict__ y,
+                                                             const float4 *__restrict__ rel,
+                                                             const float4 *__restrict__ fq,
+                                                             const uint32_t *__restrict__ start,
+                                                             const uint32_t *__restrict__ cnt,
+                                                             double *__restrict__ dens, int *__restrict__ nnb)
+{
+    __shared__ WalkMem mem[kWW];
+    __shared__ unsigned s_pairs, s_shell;
+    if (threadIdx.x == 0) s_pairs = s_shell = 0u;
+    __syncthreads();
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const size_t n = (size_t)v.n;
+    WalkMem &M = mem[wid];
+    float *red = reinterpret_cast<float *>(&M);
+    const long long w = (long long)blockIdx.x * kWW + wid;
+    const float ih = (float)v.inv_h;
+    unsigned shell = 0u, pairs = 0u;
+    for (int a0 = (int)min(2 * w, (long long)v.n), end = min(a0 + 2, v.n); a0 < end;) {  // warp-uniform
+        const float4 ra0 = rel[a0], ra1 = rel[min(a0 + 1, end - 1)];
+        const bool two = a0 + 1 < end && __float_as_int(ra0.w) == __float_as_int(ra1.w);
+        float s0[5] = {0.f, 0.f, 0.f, 0.f, 0.f}, s1[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+        CSum tot = {0.f, 0.f};  // lanes 0-4: a0's sums, 16-20: a1's
+        int nacc[2] = {0, 0};
+        auto pair = [&](int which, float4 e) {
+            const int b = __float_as_int(e.w);
+            const float4 qb = fq[b];
+            const float r2 = fmaf(e.x, e.x, fmaf(e.y, e.y, e.z * e.z));
+            const float q = sqrt_apx(r2) * ih;
+            // w(q) = (2-q)^3/4 - max(1-q,0)^3 on 0 <= q <= 2
+            const float t = 2.0f - q, u = fmaxf(1.0f - q, 0.0f);
+            const float wv = fmaf(0.25f * (t * t), t, -(u * u) * u);
+            float(&s)[5] = which ? s1 : s0;
+            s[0] += wv;
+            s[1] = fmaf(qb.x, wv, s[1]);
+            s[2] = fmaf(qb.y, wv, s[2]);
+            s[3] = fmaf(qb.z, wv, s[3]);
+            s[4] = fmaf(qb.w, wv, s[4]);
+        };
+        auto flush = [&]() {
+            flush_sums<5>(red, s0, lane, lane < 5, lane, tot);
+            if (two) flush_sums<5>(red, s1, lane, lane >= 16 && lane < 21, lane - 16, tot);
+        };
+        walk27_two(v, y, rel, start, cnt, a0, two, ra0, ra1, M, lane, nacc, shell, pair, flush);
+        const int k = lane & 15;
+        if (k < 5 && (lane < 16 || two)) dens[(size_t)k * n + a0 + (lane >> 4)] = v.sigma_d * cval(tot);
         if (lane == 0) {
-            if (pairs) atomicAdd(&s_acc[0], (unsigned long long)pairs);
-            if (shell) atomicAdd(&s_acc[1], (unsigned long long)shell);
+            nnb[a0] = nacc[0];
+            pairs += (unsigned)nacc[0];
+            if (two) {
+                nnb[a0 + 1] = nacc[1];
+                pairs += (unsigned)nacc[1];
+            }
         }
+        a0 += two ? 2 : 1;
+    }
+    shell = __reduce_add_sync(kFull, shell);
+    if (lane == 0) {
+        atomicAdd(&s_pairs, pairs);
+        if (shell) atomicAdd(&s_shell, shell);
     }
     __syncthreads();
-    if (tid == 0) {
-        if (s_acc[0]) atomicAdd(&v.sc->pairs, s_acc[0]);
-        if (s_acc[1]) atomicAdd(&v.sc->shell_tests, s_acc[1]);
+    if (threadIdx.x == 0) {
+        if (s_pairs) atomicAdd(&v.sc->pairs, (unsigned long long)s_pairs);
+        if (s_shell) atomicAdd(&v.sc->shell_tests, (unsigned long long)s_shell);
     }
 }
 
-// gin rows: X^{ji}/sigma*^2 at 3 j + i, u^j/sigma* at 9 + j; gout rows: d_k u^j at 3 k + j, then
-// F^i at 9 + i (the layout of the FP64 3+1D gradient pass).  Candidate rows r = 0..11 are staged
-// as six pair arrays (row 2m in the low, 2m + 1 in the high half of entry m).
-__global__ void __launch_bounds__(kTT3) k_tiled_gradient3m(EvView v, int stage, const double *__restrict__ y,
-                                                           const float4 *__restrict__ rel,
-                                                           const double *__restrict__ gin,
-                                                           const uint32_t *__restrict__ start,
-                                                           const uint32_t *__restrict__ cnt, double *__restrict__ gout)
+// Gradient pass (row a5).  gin rows: X^{ji}/sigma*^2 at 3 j + i, u^j/sigma* at 9 + j; gout rows:
+// d_k u^j at 3 k + j, then F^i at 9 + i (the layout of the FP64 3+1D gradient pass).  The 15
+// sums: 0-2 sum grad W, 3-5 sum_b X_b^{j i} grad_j W, 6 + 3 k + j sum_b u_b^j grad_k W.
+__global__ void __launch_bounds__(32 * kWW, 3) k_walk_gradient3m(EvView v, int stage, const double *__restrict__ y,
+                                                              const float4 *__restrict__ rel,
+                                                              const double *__restrict__ gin,
+                                                              const float4 *__restrict__ fx,
+                                                              const uint32_t *__restrict__ start,
+                                                              const uint32_t *__restrict__ cnt,
+                                                              double *__restrict__ gout)
 {
-    __shared__ float4 cP[kTile3 / 2], cPz[kTile3 / 2], cO[kTile3 / 2];
-    __shared__ float4 cV[6][kTile3 / 2];
-    __shared__ Runs27 R;
+    __shared__ WalkMem mem[kWW];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const size_t n = (size_t)v.n;
-    const int l0 = 1 << v.B3[0], l1 = 1 << v.B3[1];
-    const long long ncell = (long long)l0 * l1 * (1 << v.B3[2]);
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    constexpr int NW = kTT3 / 32;
-    const float ih = (float)v.inv_h, slo = v.shell_lo, shi = v.shell_hi;
-    const double supp2 = v.supp2;
-    for (long long ci = blockIdx.x; ci < ncell; ci += gridDim.x) {  // block-uniform
-        const int c[3] = {(int)(ci % l0), (int)((ci / l0) % l1), (int)(ci / ((long long)l0 * l1))};
-        const uint32_t kc = key3m(v, c[0], c[1], c[2]);
-        const int na = (int)cnt[kc];
-        if (na == 0) continue;
-        __syncthreads();
-        runs27_setup(v, start, cnt, c, R);
-        const int M = R.cum[27], first = (int)start[kc];
-        const int L = lanes_per_particle(na, NW), ppw = 32 / L;
-        const int pl = lane / L, l = lane - pl * L;
-        for (int g0 = 0; g0 < na; g0 += NW * ppw) {
-            const int my = g0 + warp * ppw + pl;
-            const bool valid = pl < ppw && my < na;
-            const int a = first + (valid ? my : 0);
-            const double xa[3] = {y[a], y[n + a], y[2 * n + a]};
-            const float4 ra = rel[a];
-            CSum G[3], H[3], du[3][3];
+    WalkMem &M = mem[wid];
+    float *red = reinterpret_cast<float *>(&M);
+    const long long w = (long long)blockIdx.x * kWW + wid;
+    const float ih = (float)v.inv_h;
+    for (int a0 = (int)min(2 * w, (long long)v.n), end = min(a0 + 2, v.n); a0 < end;) {  // warp-uniform
+        const float4 ra0 = rel[a0], ra1 = rel[min(a0 + 1, end - 1)];
+        const bool two = a0 + 1 < end && __float_as_int(ra0.w) == __float_as_int(ra1.w);
+        float s0[15], s1[15];
+#pragma unroll
+        for (int k = 0; k < 15; ++k) s0[k] = s1[k] = 0.0f;
+        CSum tot = {0.f, 0.f};  // lanes 0-14: a0's sums, 16-30: a1's
+        int nacc[2] = {0, 0};
+        unsigned shell = 0u;
+        auto pair = [&](int which, float4 e) {
+            const int b = __float_as_int(e.w);
+            const float4 f0 = fx[b], f1 = fx[n + b], f2 = fx[2 * n + b];
+            const float row[12] = {f0.x, f0.y, f0.z, f0.w, f1.x, f1.y, f1.z, f1.w, f2.x, f2.y, f2.z, f2.w};
+            const float r2 = fmaf(e.x, e.x, fmaf(e.y, e.y, e.z * e.z));
+            // r = 0 (the particle itself) gives dw/dq = 0: a zero term
+            const float ir = rsqrt_apx(fmaxf(r2, 1e-30f));
+            const float q = (r2 * ir) * ih;
+            const float t = 2.0f - q, u = fmaxf(1.0f - q, 0.0f);
+            const float fac = fmaf(-0.75f, t * t, 3.0f * (u * u)) * ir;
+            const float g[3] = {fac * e.x, fac * e.y, fac * e.z};
+            float(&s)[15] = which ? s1 : s0;
 #pragma unroll
             for (int i = 0; i < 3; ++i) {
-                G[i] = H[i] = CSum{0.f, 0.f};
-#pragma unroll
-                for (int j = 0; j < 3; ++j) du[i][j] = CSum{0.f, 0.f};
-            }
-            for (int t0 = 0; t0 < M; t0 += kTile3) {
-                const int mt = min(kTile3, M - t0);
-                if (g0 == 0 || M > kTile3) {
-                    if (t0 > 0 || g0 > 0) __syncthreads();
-                    for (int i = tid; i < mt; i += kTT3) {
-                        const int q = t0 + i, o = run27_of(R, q), b = R.rs[o] + (q - R.cum[o]);
-                        stage_geom(cP, cPz, cO, i, rel[b], R, o);
-#pragma unroll
-                        for (int m = 0; m < 6; ++m)
-                            put_pair(cV[m], i, (float)gin[(size_t)(2 * m) * n + b], (float)gin[(size_t)(2 * m + 1) * n + b]);
-                    }
-                    if ((mt & 1) && tid == 0) {
-                        stage_far(cP, cPz, cO, mt);
-#pragma unroll
-                        for (int m = 0; m < 6; ++m) put_pair(cV[m], mt, 0.0f, 0.0f);
-                    }
-                    __syncthreads();
-                }
-                if (valid) {
-                    const float2 ih2 = make_float2(ih, ih);
-                    const int np = (mt + 1) >> 1;
-                    for (int kb = l; kb < np; kb += (kRun / 2) * L) {
-                        const int ke = min(np, kb + (kRun / 2) * L);
-                        float2 pG[3], pH[3], pdu[3][3];
-#pragma unroll
-                        for (int i = 0; i < 3; ++i) {
-                            pG[i] = pH[i] = make_float2(0.f, 0.f);
-#pragma unroll
-                            for (int j = 0; j < 3; ++j) pdu[i][j] = make_float2(0.f, 0.f);
-                        }
-                        for (int k = kb; k < ke; k += L) {
-                            float2 dx, dy, dz, r2;
-                            sep2(ra, cP[k], cPz[k], cO[k], dx, dy, dz, r2);
-                            bool a0 = r2.x < slo, a1 = r2.y < slo;
-                            if (r2.x >= slo && r2.x <= shi) {  // thin shell: the exact FP64 decision
-                                const int q = t0 + 2 * k, o = run27_of(R, q), b = R.rs[o] + (q - R.cum[o]);
-                                a0 = dist2_3e(xa[0] - y[b], xa[1] - y[n + b], xa[2] - y[2 * n + b]) < supp2;
-                            }
-                            if (r2.y >= slo && r2.y <= shi) {
-                                const int q = t0 + 2 * k + 1, o = run27_of(R, q), b = R.rs[o] + (q - R.cum[o]);
-                                a1 = dist2_3e(xa[0] - y[b], xa[1] - y[n + b], xa[2] - y[2 * n + b]) < supp2;
-                            }
-                            // r = 0 (the particle itself) gives dw/dq = 0: a zero term
-                            const float2 ir = make_float2(rsqrt_apx(fmaxf(r2.x, 1e-30f)), rsqrt_apx(fmaxf(r2.y, 1e-30f)));
-                            float2 t2, t, u2, u;
-                            spline_terms2(__fmul2_rn(__fmul2_rn(r2, ir), ih2), t2, t, u2, u);
-                            float2 fac = __fmul2_rn(__ffma2_rn(make_float2(-0.75f, -0.75f), t2,
-                                                               __fmul2_rn(make_float2(3.0f, 3.0f), u2)), ir);
-                            fac.x = a0 ? fac.x : 0.0f;
-                            fac.y = a1 ? fac.y : 0.0f;
-                            const float2 g[3] = {__fmul2_rn(fac, dx), __fmul2_rn(fac, dy), __fmul2_rn(fac, dz)};
-                            float2 row[12];
-#pragma unroll
-                            for (int m = 0; m < 6; ++m) {
-                                const float4 e = cV[m][k];
-                                row[2 * m] = lo2(e);
-                                row[2 * m + 1] = hi2(e);
-                            }
-#pragma unroll
-                            for (int i = 0; i < 3; ++i) {
-                                pG[i] = __fadd2_rn(pG[i], g[i]);
-                                // sum_j X^{ji} g_j, j = 0, 1, 2 in turn
-                                pH[i] = __ffma2_rn(row[6 + i], g[2],
-                                                   __ffma2_rn(row[3 + i], g[1], __ffma2_rn(row[i], g[0], pH[i])));
-                            }
-#pragma unroll
-                            for (int j = 0; j < 3; ++j)
-#pragma unroll
-                                for (int kk = 0; kk < 3; ++kk) pdu[kk][j] = __ffma2_rn(row[9 + j], g[kk], pdu[kk][j]);
-                        }
-#pragma unroll
-                        for (int i = 0; i < 3; ++i) {
-                            cadd(G[i], pG[i].x + pG[i].y);
-                            cadd(H[i], pH[i].x + pH[i].y);
-#pragma unroll
-                            for (int j = 0; j < 3; ++j) cadd(du[i][j], pdu[i][j].x + pdu[i][j].y);
-                        }
-                    }
-                }
+                s[i] += g[i];
+                s[3 + i] = fmaf(row[6 + i], g[2], fmaf(row[3 + i], g[1], fmaf(row[i], g[0], s[3 + i])));
             }
 #pragma unroll
-            for (int i = 0; i < 3; ++i) {
-                G[i] = seg_csum(G[i], l, L);
-                H[i] = seg_csum(H[i], l, L);
+            for (int j = 0; j < 3; ++j)
 #pragma unroll
-                for (int j = 0; j < 3; ++j) du[i][j] = seg_csum(du[i][j], l, L);
-            }
-            if (valid && l == 0) {
+                for (int k = 0; k < 3; ++k) s[6 + 3 * k + j] = fmaf(row[9 + j], g[k], s[6 + 3 * k + j]);
+        };
+        auto flush = [&]() {
+            flush_sums<15>(red, s0, lane, lane < 15, lane, tot);
+            if (two) flush_sums<15>(red, s1, lane, lane >= 16 && lane < 31, lane - 16, tot);
+        };
+        walk27_two(v, y, rel, start, cnt, a0, two, ra0, ra1, M, lane, nacc, shell, pair, flush);
+        const double d = cval(tot);
+        const int k = lane & 15, first = lane & 16;
+        const size_t a = (size_t)a0 + (lane >> 4);
+        const double G0 = __shfl_sync(kFull, d, first), G1 = __shfl_sync(kFull, d, first + 1),
+                     G2 = __shfl_sync(kFull, d, first + 2);
+        if (k >= 3 && k < 15 && (lane < 16 || two)) {
+            const double cf = v.sigma_d * v.inv_h;
+            if (k >= 6) {
+                gout[(size_t)(k - 6) * n + a] = cf * d;
+            } else {
+                // minus the stress divergence: sum X_b grad W + X_a . sum grad W, times sqrt(-g)
                 const double tau = v.sc->tau + (stage == 2 ? v.dtau : 0.0);
                 const double sqrtg = v.milne ? tau : 1.0;
-                const double cf = v.sigma_d * v.inv_h;
-                double tG[3];
-#pragma unroll
-                for (int i = 0; i < 3; ++i) tG[i] = cval(G[i]);
-#pragma unroll
-                for (int kk = 0; kk < 3; ++kk)
-#pragma unroll
-                    for (int j = 0; j < 3; ++j) gout[(size_t)(3 * kk + j) * n + a] = cf * cval(du[kk][j]);
-#pragma unroll
-                for (int i = 0; i < 3; ++i) {
-                    double F = cval(H[i]);
-#pragma unroll
-                    for (int j = 0; j < 3; ++j) F = fma(gin[(size_t)(3 * j + i) * n + a], tG[j], F);
-                    gout[(size_t)(9 + i) * n + a] = -sqrtg * cf * F;
-                }
+                const int i = k - 3;
+                double F = fma(gin[(size_t)i * n + a], G0, d);
+                F = fma(gin[(size_t)(3 + i) * n + a], G1, F);
+                F = fma(gin[(size_t)(6 + i) * n + a], G2, F);
+                gout[(size_t)(9 + i) * n + a] = -sqrtg * cf * F;
             }
         }
+        a0 += two ? 2 : 1;
     }
 }
 
 inline int nblk(int n, int t) { return (n + t - 1) / t; }
-
-// blocks of the tiled passes: one per cell of the grid, at most 8 per SM (the rest grid-stride)
-inline int tiled_grid3(const EvView &v)
-{
-    const long long ncell = 1ll << (v.B3[0] + v.B3[1] + v.B3[2]);
-    return (int)std::min<long long>(ncell, 8ll * device_sm_count());
-}
 
 }  // namespace
 
 void launch_density3m(const EvView &v, const double *y, const double *Nq, CellBufs cb, double *dens, int *nnb,
                       cudaStream_t st)
 {
-    k_relpos3<<<nblk(v.n, 256), 256, 0, st>>>(v, y, cb.fpos3);
-    k_tiled_density3m<<<tiled_grid3(v), kTT3, 0, st>>>(v, y, cb.fpos3, Nq, cb.start, cb.cnt, dens, nnb);
+    k_relpos3<<<nblk(v.n, 256), 256, 0, st>>>(v, y, Nq, cb.fpos3, cb.fq);
+    k_walk_density3m<<<nblk(v.n, 2 * kWW), 32 * kWW, 0, st>>>(v, y, cb.fpos3, cb.fq, cb.start, cb.cnt, dens, nnb);
 }
 
 void launch_gradient3m(const EvView &v, int stage, const double *y, const double *gin, CellBufs cb, double *gout,
                        cudaStream_t st)
 {
-    k_tiled_gradient3m<<<tiled_grid3(v), kTT3, 0, st>>>(v, stage, y, cb.fpos3, gin, cb.start, cb.cnt, gout);
+    k_fx3<<<nblk(v.n, 256), 256, 0, st>>>(v.n, gin, cb.fx);
+    k_walk_gradient3m<<<nblk(v.n, 2 * kWW), 32 * kWW, 0, st>>>(v, stage, y, cb.fpos3, gin, cb.fx, cb.start, cb.cnt,
+                                                               gout);
 }
 
 }  // namespace sphg
