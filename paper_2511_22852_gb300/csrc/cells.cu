@@ -10,7 +10,8 @@
 //   scatter   particle -> provisional slot inside its bucket (atomic cursor)
 //   rank      final slot = bucket start + number of bucket members with a smaller
 //             original id: the order is (key, id), deterministic and stable
-//   permute   gather of every per-particle array into the new order
+//   permute   gather of every per-particle array into the new order, with the single-precision
+//             positions of the neighbour passes
 #include "sph_internal.cuh"
 
 namespace sphg {
@@ -234,15 +235,41 @@ struct PermArgs {
     int ngroups;
 };
 
-__global__ void k_permute(int n, const uint32_t *__restrict__ perm, PermArgs a, const int *__restrict__ id_in,
-                          int *id_out)
+__global__ void k_permute(EvView v, const uint32_t *__restrict__ perm, PermArgs a, const int *__restrict__ id_in,
+                          int *id_out, float2 *__restrict__ fpos, float4 *__restrict__ fpos3, double *__restrict__ dens)
 {
+    const int n = v.n;
     int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= n) return;
     uint32_t s = perm[j];
     for (int g = 0; g < a.ngroups; ++g)
         for (int r = 0; r < a.rows[g]; ++r) a.dst[g][(size_t)r * n + j] = a.src[g][(size_t)r * n + s];
     id_out[j] = id_in[s];
+    // what the neighbour passes read per particle in single precision, from the state just gathered
+    // (the rows from dst[0] on)
+    const double *y = a.dst[0] + j;
+    if (v.dim == 3) {
+        if (v.mixed) return;  // k_relpos3
+        float f[3];
+#pragma unroll
+        for (int d = 0; d < 3; ++d)
+            f[d] = __double2float_rn(__dsub_rn(y[(size_t)d * n], dec_double(v.sc->xmin_enc[d])));
+        fpos3[j] = make_float4(f[0], f[1], f[2], 0.0f);
+        return;
+    }
+    float f[2];
+#pragma unroll
+    for (int d = 0; d < 2; ++d) {
+        const double xm = dec_double(v.sc->xmin_enc[d]), x = y[(size_t)d * n];
+        double r = __dsub_rn(x, xm);  // plain form: relative to the bounding-box minimum
+        if (v.mixed) r = __dsub_rn(r, (double)cell_coord(x, xm, v.inv_cell) * (2.0 * v.h));  // to the cell's origin
+        f[d] = __double2float_rn(r);
+    }
+    fpos[j] = make_float2(f[0], f[1]);
+    if (!v.mixed) {  // u0 = sqrt(1 + u.u) (density row 5)
+        const double ux = y[2 * (size_t)n], uy = y[3 * (size_t)n];
+        dens[5 * (size_t)n + j] = sqrt(fma(ux, ux, fma(uy, uy, 1.0)));
+    }
 }
 
 // neighbour pairs for the test interface: pass 1 counts (offs == nullptr), pass 2 writes
@@ -365,8 +392,8 @@ void launch_cells(const EvView &v, const double *y, const int *id, CellBufs cb, 
     k_rank<<<nblk(v.n, 128), 128, 0, st>>>(v.n, cb.key, cb.start, cb.cnt, cb.tmp, id, cb.perm);
 }
 
-void launch_permute(const EvView &v, const uint32_t *perm, const double *const *src, double *const *dst,
-                    const int *nrows, int ngroups, const int *id_in, int *id_out, cudaStream_t st)
+void launch_permute(const EvView &v, const CellBufs &cb, const double *const *src, double *const *dst,
+                    const int *nrows, int ngroups, const int *id_in, int *id_out, double *dens, cudaStream_t st)
 {
     PermArgs a;
     a.ngroups = ngroups;
@@ -375,7 +402,7 @@ void launch_permute(const EvView &v, const uint32_t *perm, const double *const *
         a.dst[g] = dst[g];
         a.rows[g] = nrows[g];
     }
-    k_permute<<<nblk(v.n, 256), 256, 0, st>>>(v.n, perm, a, id_in, id_out);
+    k_permute<<<nblk(v.n, 256), 256, 0, st>>>(v, cb.perm, a, id_in, id_out, cb.fpos, cb.fpos3, dens);
 }
 
 void launch_neighbors_list(const EvView &v, const double *y, const int *id, CellBufs cb, const long long *offs,

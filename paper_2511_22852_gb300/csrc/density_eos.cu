@@ -28,19 +28,6 @@ namespace sphg {
 
 namespace {
 
-// single-precision positions relative to the bounding-box minimum (prefilter input), and
-// u0 = sqrt(1 + u.u) (density row 5), one thread per particle
-__global__ void k_fpos(EvView v, const double *__restrict__ y, float2 *__restrict__ fpos, double *__restrict__ dens)
-{
-    int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= v.n) return;
-    double xmin0 = dec_double(v.sc->xmin_enc[0]), xmin1 = dec_double(v.sc->xmin_enc[1]);
-    fpos[j] = make_float2(__double2float_rn(__dsub_rn(y[j], xmin0)), __double2float_rn(__dsub_rn(y[v.n + j], xmin1)));
-    const size_t N = (size_t)v.n;
-    const double ux = y[2 * N + j], uy = y[3 * N + j];
-    dens[5 * N + j] = sqrt(fma(ux, ux, fma(uy, uy, 1.0)));
-}
-
 constexpr int kWarps = 4;  // warps (particles in flight) per block of the neighbour passes
 
 // Density pass, one warp per particle.  For each of the 3x3 cells the lanes take 32
@@ -253,78 +240,115 @@ __device__ __forceinline__ double eos2_store(const EvView &v, int stage, size_t 
     return wcontrib;
 }
 
-// Plain and mixed single-event forms: persistent blocks of kEosWarps warps run the lane-refill
-// pass (eos_lanes) over the event's particles; the work rate goes to wpart[a] (summed in a fixed
-// order by the work kernel), the work counters and the status bits are warp-aggregated.
+// The two halves of the EoS pass (eos_device.cuh).  First half: persistent blocks of kEosWarps
+// warps run the lane-refill search over the event's particles; second half: a thread per particle.
 constexpr int kEosWarps = 4;
 #ifndef SPH_EOS_BLOCKS_PER_SM
 #define SPH_EOS_BLOCKS_PER_SM 3
 #endif
 constexpr int kEosBlocksPerSM = SPH_EOS_BLOCKS_PER_SM;  // resident blocks per SM (the register budget)
 
-struct Eos2Ctx {
+__device__ __forceinline__ void put_point(double *__restrict__ guess_out, uint32_t *__restrict__ status, size_t n,
+                                          size_t a, const double x[4], uint32_t st)
+{
+#pragma unroll
+    for (int k = 0; k < 4; ++k) guess_out[k * n + a] = x[k];
+    status[a] = st;
+}
+
+struct Find2Ctx {
     const EvView &v;
     int stage;
     size_t n;
     const double *__restrict__ y;
-    double *__restrict__ dens, *__restrict__ eos, *__restrict__ gin, *__restrict__ wpart, *__restrict__ guess_out;
+    double *__restrict__ dens, *__restrict__ guess_out;
     uint32_t *__restrict__ status;
     const double *__restrict__ guess_in;
-    unsigned st_or;
-    __device__ bool load(int a, double &s, double nq[3], double g[4], double &cap)
+    __device__ bool load(int a, double &s, double nq[3], double g[4])
     {
         double keep[4];
-        cap = v.tr.cs2_cap;
         eos2_load(v, v.eos, stage, n, (size_t)a, dens, guess_in, nullptr, s, nq, g, keep, y);
         return true;
     }
-    __device__ void store(int a, const EosOut &o, bool used)
-    {
-        wpart[a] = eos2_store(v, stage, n, (size_t)a, y, dens, eos, gin, status, guess_out, o, used);
-        st_or |= o.st;
-    }
+    __device__ void put(int a, const double x[4], uint32_t st) { put_point(guess_out, status, n, (size_t)a, x, st); }
 };
 
-__global__ void __launch_bounds__(32 * kEosWarps, kEosBlocksPerSM) k_eos2(EvView v, int stage, const double *__restrict__ y,
-                                                         double *__restrict__ dens, double *__restrict__ eos,
-                                                         double *__restrict__ gin, uint32_t *__restrict__ status,
-                                                         double *__restrict__ wpart,
-                                                         const double *__restrict__ guess_in,
-                                                         double *__restrict__ guess_out)
+__device__ __forceinline__ void add_eos_work(DevScalars *sc, const EosWork &w, unsigned st_or)
 {
-    Eos2Ctx ctx{v, stage, (size_t)v.n, y, dens, eos, gin, wpart, guess_out, status, guess_in, 0u};
-    EosWork w = {0u, 0u, 0u};
-    eos_lanes(v.eos, &v.sc->eos_claim, v.n, ctx, w);
     const unsigned wres = __reduce_add_sync(0xFFFFFFFFu, w.resid);
     const unsigned wsol = __reduce_add_sync(0xFFFFFFFFu, w.solve);
     const unsigned wg = __reduce_add_sync(0xFFFFFFFFu, w.g);
-    const unsigned sor = __reduce_or_sync(0xFFFFFFFFu, ctx.st_or);
+    const unsigned sor = __reduce_or_sync(0xFFFFFFFFu, st_or);
     if ((threadIdx.x & 31) == 0) {
-        atomicAdd(&v.sc->eos_resid, (unsigned long long)wres);
-        atomicAdd(&v.sc->eos_solve, (unsigned long long)wsol);
-        atomicAdd(&v.sc->eos_g, (unsigned long long)wg);
-        if (sor) atomicOr(&v.sc->status_or, sor);
+        if (wres) atomicAdd(&sc->eos_resid, (unsigned long long)wres);
+        if (wsol) atomicAdd(&sc->eos_solve, (unsigned long long)wsol);
+        if (wg) atomicAdd(&sc->eos_g, (unsigned long long)wg);
+        if (sor) atomicOr(&sc->status_or, sor);
     }
 }
 
-// Serving form: the same pass over the segmented arena (particles of every event active in this
-// stage; padding and inactive slots are skipped).  A lane's particles may belong to different
-// events: the per-event work counters and status bits are gathered per block in shared memory
-// and flushed once.  Stage 2 starts from the stage-1 solutions of this and the previous step,
+__global__ void __launch_bounds__(32 * kEosWarps, kEosBlocksPerSM)
+    k_eos2_find(EvView v, int stage, const double *__restrict__ y, double *__restrict__ dens,
+                uint32_t *__restrict__ status, const double *__restrict__ guess_in, double *__restrict__ guess_out)
+{
+    Find2Ctx ctx{v, stage, (size_t)v.n, y, dens, guess_out, status, guess_in};
+    EosWork w = {0u, 0u, 0u};
+    eos_find(v.eos, &v.sc->eos_claim, v.n, ctx, w);
+    add_eos_work(v.sc, w, 0u);
+}
+
+// wpart[block]: the block's work rate, summed in a fixed order (the work kernel adds the blocks)
+constexpr int kFinish = 64;
+__global__ void __launch_bounds__(kFinish, 5) k_eos2_finish(EvView v, int stage, const double *__restrict__ y,
+                                                         const double *__restrict__ dens, double *__restrict__ eos,
+                                                         double *__restrict__ gin, uint32_t *__restrict__ status,
+                                                         double *__restrict__ wpart, double *__restrict__ guess_out)
+{
+    __shared__ double red[kFinish / 32];
+    const int a = blockIdx.x * kFinish + threadIdx.x;
+    const size_t n = (size_t)v.n;
+    EosWork w = {0u, 0u, 0u};
+    double wc = 0.0;
+    unsigned st = 0u;
+    if (a < v.n) {
+        const double s = dens[n + a], nq[3] = {dens[2 * n + a], dens[3 * n + a], dens[4 * n + a]};
+        const double g[4] = {guess_out[a], guess_out[n + a], guess_out[2 * n + a], guess_out[3 * n + a]};
+        bool used = false;
+        const EosOut o = eos_finish(v.eos, v.tr.cs2_cap, s, nq, g, status[a], used, w);
+        wc = eos2_store(v, stage, n, (size_t)a, y, dens, eos, gin, status, guess_out, o, used);
+        st = o.st;
+    }
+    add_eos_work(v.sc, w, st);
+    if (v.milne) {
+        for (int o = 16; o > 0; o >>= 1) wc += __shfl_xor_sync(0xFFFFFFFFu, wc, o);
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = wc;
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+        if (v.milne)
+            for (int k = 0; k < kFinish / 32; ++k) t += red[k];
+        wpart[blockIdx.x] = t;
+    }
+}
+
+// Serving form: the same halves over the segmented arena (particles of every event active in this
+// stage; padding and inactive slots are skipped).  A lane's particles of the first half may belong to
+// different events: the per-event work counters are gathered per block in shared memory and
+// flushed once.  Stage 2 starts from the stage-1 solutions of this and the previous step,
 // extrapolated to the later time, and keeps this step's for the next.
-struct SegEosCtx {
+struct SegFindCtx {
     const Arena &A;
     const BatchTable *T;
     int stage;
     int grp;  // event group (-1: every event)
     size_t P;
     const double *__restrict__ y;
-    unsigned int *sh;  // [kMaxSlots][4]: table evaluations, solves, closed-form evaluations, status bits
+    unsigned int *sh;  // [kMaxSlots][4]: table evaluations, solves, closed-form evaluations
     EosWork *w;
     EosWork w0;
     int slot;
-    double keep[4];
-    __device__ bool load(int a, double &s, double nq[3], double g[4], double &cap)
+    __device__ bool load(int a, double &s, double nq[3], double g[4])
     {
         const int sl = A.segid[a];
         if (sl < 0 || !seg_active(T, sl, stage, false) || !in_group(T, sl, grp)) return false;
@@ -332,42 +356,35 @@ struct SegEosCtx {
         if (a - q.off >= q.n) return false;
         slot = sl;
         w0 = *w;
-        cap = A.segv[sl].tr.cs2_cap;
+        double keep[4];
         eos2_load(A.segv[sl], A.segv[sl].eos, stage, P, (size_t)a, A.dens, A.guess_in,
                   stage == 2 ? A.xs1[0] : nullptr, s, nq, g, keep, y);
-        return true;
-    }
-    __device__ void store(int a, const EosOut &o, bool used)
-    {
-        A.wpart[a] = eos2_store(A.segv[slot], stage, P, (size_t)a, y, A.dens, A.eosf, A.gin, A.status, A.wguess, o,
-                                used);
         if (stage == 2)
 #pragma unroll
             for (int k = 0; k < 4; ++k) A.xs1[0][k * P + a] = keep[k];
-        if (T->slots[slot].mode == SLOT_STEP) {  // float copies of the gradient-pass inputs
-            const double *g = A.gin;
-            A.fX[a] = make_float4((float)g[a], (float)g[P + a], (float)g[2 * P + a], (float)g[3 * P + a]);
-            A.fU[a] = make_float2((float)g[4 * P + a], (float)g[5 * P + a]);
-        }
+        return true;
+    }
+    __device__ void put(int a, const double x[4], uint32_t st)
+    {
+        put_point(A.wguess, A.status, P, (size_t)a, x, st);
         unsigned int *c = sh + 4 * slot;
-        atomicAdd_block(c, w->resid - w0.resid);
-        atomicAdd_block(c + 1, w->solve - w0.solve);
-        atomicAdd_block(c + 2, w->g - w0.g);
-        if (o.st) atomicOr_block(c + 3, o.st);
+        if (w->resid != w0.resid) atomicAdd_block(c, w->resid - w0.resid);
+        if (w->solve != w0.solve) atomicAdd_block(c + 1, w->solve - w0.solve);
+        if (w->g != w0.g) atomicAdd_block(c + 2, w->g - w0.g);
     }
 };
 
-__global__ void __launch_bounds__(32 * kEosWarps, kEosBlocksPerSM) k_eos2_seg(Arena A, EosDev E, int stage, const double *__restrict__ y,
-                                                                             int grp)
+__global__ void __launch_bounds__(32 * kEosWarps, kEosBlocksPerSM)
+    k_eos2_seg_find(Arena A, EosDev E, int stage, const double *__restrict__ y, int grp)
 {
     __shared__ unsigned int sh[kMaxSlots * 4];
     for (int i = threadIdx.x; i < kMaxSlots * 4; i += blockDim.x) sh[i] = 0u;
     __syncthreads();
     const BatchTable *T = A.tab;
     EosWork w = {0u, 0u, 0u};
-    SegEosCtx ctx{A, T, stage, grp, (size_t)A.P, y, sh, &w, w, -1, {0.0, 0.0, 0.0, 0.0}};
+    SegFindCtx ctx{A, T, stage, grp, (size_t)A.P, y, sh, &w, w, -1};
     // E is the server's EoS (every event's view carries the same)
-    eos_lanes(E, &A.claim[claim_of(CLAIM_EOS, grp)], T->hi, ctx, w);
+    eos_find(E, &A.claim[claim_of(CLAIM_EOS, grp)], T->hi, ctx, w);
     __syncthreads();
     const int ns = T->nslots;
     for (int s = threadIdx.x; s < ns; s += blockDim.x) {
@@ -375,7 +392,36 @@ __global__ void __launch_bounds__(32 * kEosWarps, kEosBlocksPerSM) k_eos2_seg(Ar
         if (c[0]) atomicAdd(&A.sc[s].eos_resid, (unsigned long long)c[0]);
         if (c[1]) atomicAdd(&A.sc[s].eos_solve, (unsigned long long)c[1]);
         if (c[2]) atomicAdd(&A.sc[s].eos_g, (unsigned long long)c[2]);
-        if (c[3]) atomicOr(&A.sc[s].status_or, c[3]);
+    }
+}
+
+// a warp's 32 positions lie in one event's range (ranges are multiples of kSegAlign)
+__global__ void __launch_bounds__(128, 3) k_eos2_seg_finish(Arena A, EosDev E, int stage, const double *__restrict__ y, int grp)
+{
+    const BatchTable *T = A.tab;
+    const int hi = T->hi;
+    const size_t P = (size_t)A.P;
+    for (int a0 = (blockIdx.x * blockDim.x + threadIdx.x) & ~31; a0 < hi; a0 += gridDim.x * blockDim.x) {  // warp-uniform
+        const int sl = A.segid[a0];
+        if (sl < 0 || !seg_active(T, sl, stage, false) || !in_group(T, sl, grp)) continue;
+        const int a = a0 + (threadIdx.x & 31);
+        EosWork w = {0u, 0u, 0u};
+        unsigned st = 0u;
+        if (a - T->slots[sl].off < T->slots[sl].n) {
+            const double *D = A.dens;
+            const double s = D[P + a], nq[3] = {D[2 * P + a], D[3 * P + a], D[4 * P + a]};
+            const double g[4] = {A.wguess[a], A.wguess[P + a], A.wguess[2 * P + a], A.wguess[3 * P + a]};
+            bool used = false;
+            const EosOut o = eos_finish(E, A.segv[sl].tr.cs2_cap, s, nq, g, A.status[a], used, w);
+            A.wpart[a] = eos2_store(A.segv[sl], stage, P, (size_t)a, y, A.dens, A.eosf, A.gin, A.status, A.wguess, o, used);
+            st = o.st;
+            if (T->slots[sl].mode == SLOT_STEP) {  // float copies of the gradient-pass inputs
+                const double *q = A.gin;
+                A.fX[a] = make_float4((float)q[a], (float)q[P + a], (float)q[2 * P + a], (float)q[3 * P + a]);
+                A.fU[a] = make_float2((float)q[4 * P + a], (float)q[5 * P + a]);
+            }
+        }
+        add_eos_work(&A.sc[sl], w, st);
     }
 }
 
@@ -394,7 +440,6 @@ void launch_density(const EvView &v, const double *y, const double *Nq, CellBufs
         launch_density2m(v, y, Nq, cb, dens, nnb, st);
         return;
     }
-    k_fpos<<<nblk(v.n, 256), 256, 0, st>>>(v, y, cb.fpos, dens);
     const int lists = cb.pl.total > 0;
     if (lists) launch_pairs_density(v, y, Nq, cb, dens, nnb, st);
     // as the fallback of the pair-list passes it usually exits at once: a few blocks per SM
@@ -415,13 +460,12 @@ void launch_eos(const EvView &v, int stage, const double *y, const double *dens,
     // more than another), or a lane per particle when it is smaller than one block per SM
     const int sms = device_sm_count(), need = nblk(v.n, 32 * kEosWarps);
     const int grid = need >= kEosBlocksPerSM * sms ? kEosBlocksPerSM * sms : (need >= sms ? (need / sms) * sms : std::max(1, need));
-    k_eos2<<<grid, 32 * kEosWarps, 0, st>>>(v, stage, y, const_cast<double *>(dens), eos, gin, status, wpart,
-                                              guess_in, guess_out);
+    k_eos2_find<<<grid, 32 * kEosWarps, 0, st>>>(v, stage, y, const_cast<double *>(dens), status, guess_in, guess_out);
+    k_eos2_finish<<<nblk(v.n, kFinish), kFinish, 0, st>>>(v, stage, y, dens, eos, gin, status, wpart, guess_out);
 }
 
-// entries of the work-rate partials: one per particle in 2D (the lane-refill pass), one per
-// 64-particle block in 3D
-int eos_block_count(int n, int dim) { return dim == 2 ? n : nblk(n, 64); }
+// entries of the work-rate partials: one per block of the second half
+int eos_block_count(int n, int dim) { return dim == 2 ? nblk(n, kFinish) : nblk(n, 64); }
 
 int device_sm_count()
 {
@@ -476,7 +520,8 @@ void launch_inverse_build(const EosDev &E, double *inv, long long nnodes, cudaSt
 
 void launch_eos2_seg(const Arena &A, const EosDev &E, int stage, const double *y, int grid, cudaStream_t st, int grp)
 {
-    k_eos2_seg<<<grid, 32 * kEosWarps, 0, st>>>(A, E, stage, y, grp);
+    k_eos2_seg_find<<<grid, 32 * kEosWarps, 0, st>>>(A, E, stage, y, grp);
+    k_eos2_seg_finish<<<8 * device_sm_count(), 128, 0, st>>>(A, E, stage, y, grp);
 }
 
 int eos_seg_grid(int sms) { return kEosBlocksPerSM * sms; }

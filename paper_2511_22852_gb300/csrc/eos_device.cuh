@@ -10,6 +10,11 @@ namespace {
 // closed-form EoS
 __device__ __forceinline__ void an_shape(const EosDev &E, double T, double &f, double &fp, double &fpp)
 {
+    if (E.a1 == 0.0) {  // conformal: no crossover term
+        f = E.a0;
+        fp = fpp = 0.0;
+        return;
+    }
     double k = kHbarc / E.w_GeV;
     double th = tanh((T * kHbarc - E.Tc_GeV) / E.w_GeV);
     double sech2 = fma(-th, th, 1.0);
@@ -46,9 +51,58 @@ __device__ __forceinline__ void an_g(const EosDev &E, double T, double s, double
 {
     double f, fp, fpp;
     an_shape(E, T, f, fp, fpp);
+    const double iT = 1.0 / T, cT3 = c * (iT * iT * iT);  // one reciprocal for both quotients
     double T2 = T * T, T3 = T2 * T, T4 = T2 * T2;
-    g = 4.0 * T3 * f + T4 * fp + c / T3 - s;
-    gp = 12.0 * T2 * f + 8.0 * T3 * fp + T4 * fpp - 3.0 * c / T4;
+    g = 4.0 * T3 * f + T4 * fp + cT3 - s;
+    gp = 12.0 * T2 * f + 8.0 * T3 * fp + T4 * fpp - 3.0 * cT3 * iT;
+}
+
+// The closed form's root in single precision by the same bracketing and safeguarded Newton
+// iteration as an_invert's (0: not found), as the start of the FP64 iteration: an FP64 evaluation
+// of g is a chain of about 50 operations at 64 cycles each, a single-precision one costs 1/15 of it.
+__device__ __forceinline__ void an_gf(float a0, float a1, float Tc, float iw, float k, float T, float s, float c,
+                                      float &g, float &gp)
+{
+    const float th = tanhf((T * (float)kHbarc - Tc) * iw), sech2 = fmaf(-th, th, 1.0f);
+    const float f = fmaf(0.5f * a1, 1.0f + th, a0), fp = 0.5f * a1 * sech2 * k, fpp = -a1 * sech2 * th * k * k;
+    const float iT = 1.0f / T, cT3 = c * (iT * iT * iT), T2 = T * T, T3 = T2 * T;
+    g = 4.0f * T3 * f + T2 * T2 * fp + cT3 - s;
+    gp = 12.0f * T2 * f + 8.0f * T3 * fp + T2 * T2 * fpp - 3.0f * cT3 * iT;
+}
+__device__ __noinline__ float an_seed(const EosDev &E, double sd, double cd, double Tguess)
+{
+    const float a0 = (float)E.a0, a1 = (float)E.a1, Tc = (float)E.Tc_GeV, iw = 1.0f / (float)E.w_GeV,
+                k = (float)kHbarc * iw, s = (float)sd, c = (float)cd, Tg = (float)Tguess;
+    float Thi = cbrtf(s / (4.0f * a0));
+    const bool warm = Tg > 0.0f && Tg < Thi;
+    const float t0 = warm ? Tg : Thi, step = warm ? 0.99f : 0.8f;
+    float g, gp, Tlo = t0, t = t0;
+    an_gf(a0, a1, Tc, iw, k, t0, s, c, g, gp);
+    if (g > 0.0f) {
+        Thi = t0;
+        float gprev = g;
+        int j = 0;
+        for (; j < 400; ++j) {
+            Tlo *= step;
+            float gl, gpl;
+            an_gf(a0, a1, Tc, iw, k, Tlo, s, c, gl, gpl);
+            if (gl <= 0.0f) break;
+            if (!(gl <= gprev)) return 0.0f;
+            gprev = gl;
+        }
+        if (j == 400) return 0.0f;
+    }
+    for (int it = 0; it < 40; ++it) {
+        an_gf(a0, a1, Tc, iw, k, t, s, c, g, gp);
+        if (g > 0.0f) Thi = t;
+        else Tlo = t;
+        float tn = t - g / gp;
+        if (!(gp > 0.0f) || !(tn > Tlo && tn < Thi)) tn = 0.5f * (Tlo + Thi);
+        const bool done = fabsf(tn - t) <= 4e-7f * t;
+        t = tn;
+        if (done) break;
+    }
+    return t;
 }
 
 // Tguess > 0: the particle's closed-form T of its previous stage (warm start of the bracket and of
@@ -62,6 +116,28 @@ __device__ uint32_t an_invert(const EosDev &E, double s, const double *n, double
     for (int q = 0; q < 3; ++q) {
         if (E.chi[q] > 0.0) c += n[q] * n[q] / E.chi[q];
         else if (n[q] != 0.0) return PST_NOCONV;
+    }
+    {
+        // FP64 Newton from the single-precision root (about 1e-7 of T off): a step below 1e-9 of T
+        // leaves an error of its square, so two evaluations reach the root (measured on the ideal
+        // Gubser event: 3 instead of 12 evaluations, EoS pass 303 -> 30 us a stage); anything
+        // unexpected leaves the root to the bracketed iteration below
+        const double t0 = (double)an_seed(E, s, c, Tguess);
+        double t = t0;
+        for (int it = 0; it < 5 && t > 0.0; ++it) {
+            double g, gp;
+            an_g(E, t, s, c, g, gp);
+            ++w.g;
+            const double d = g / gp, ad = fabs(d);
+            if (!(gp > 0.0) || !(ad <= 1e-5 * t)) break;
+            t -= d;
+            if (ad <= 1e-9 * t) {
+                T = t;
+                const double it2 = 1.0 / (t * t);
+                for (int q = 0; q < 3; ++q) mu[q] = E.chi[q] > 0.0 ? n[q] / E.chi[q] * it2 : 0.0;
+                return 0u;
+            }
+        }
     }
     double Thi = cbrt(s / (4.0 * E.a0));
     // start: the bound cbrt(s / 4 a0) >= T, or a warm start below it
@@ -113,14 +189,28 @@ __device__ uint32_t an_invert(const EosDev &E, double s, const double *n, double
 // ---------------------------------------------------------------------------
 // table: the quadrilinear interpolant reduced one axis at a time (mu_Q, mu_S inside each of the
 // four (T, mu_B) corner patches, then mu_B, then T), carrying the partial derivatives along
+// the cell of grid coordinate r and the position in it: the integer part of r >= 1 from its
+// mantissa bits and back into a double by bits (a conversion between int and double costs as much
+// as an FP64 operation), clamped to [0, nx - 2]; r < 1 (negative too) lies in cell 0
+__device__ __forceinline__ void locate_steps(double r, int nx, int &i, double &t)
+{
+    const int hi = __double2hiint(r);
+    int k = 0;
+    if (hi >= 0x3FF00000) {
+        if (nx <= (1 << 20)) k = ((hi & 0xFFFFF) | 0x100000) >> max(0, 20 - ((hi >> 20) - 1023));
+        else k = __double2int_rz(r);
+    }
+    k = min(k, nx - 2);
+    i = k;
+    const int e = 31 - __clz(k | 1);
+    const double kd = k == 0 ? 0.0
+                      : nx <= (1 << 20) ? __hiloint2double(((e + 1023) << 20) | ((k << (20 - e)) & 0xFFFFF), 0)
+                                        : (double)k;
+    t = r - kd;
+}
 __device__ __forceinline__ void locate(double x, double x0, double inv, int nx, int &i, double &t)
 {
-    const double r = (x - x0) * inv;
-    // the cell below r: truncation toward zero is the floor for r >= 0, and the clamp to
-    // [0, nx - 2] takes every r < 0 to cell 0 as the floor would (no rounding instruction)
-    const int k = max(0, min(__double2int_rz(r), nx - 2));
-    i = k;
-    t = r - (double)k;
+    locate_steps((x - x0) * inv, nx, i, t);
 }
 
 // sn: interpolated (s, nB, nS, nQ); J[f][k] = d sn_f / d x_k per grid step of axis k (times
@@ -580,25 +670,332 @@ __device__ EosOut eos_invert(const EosDev &E, double cs2_cap, double s, const do
 }
 
 // ---------------------------------------------------------------------------
-// Lane-refill EoS pass.  The table Newton's work varies from particle to particle (iterations,
-// line-search trials, the polishing step), so a warp that inverts 32 particles together leaves
-// its finished lanes idle until the slowest is done, and every FP64 instruction of the 1:64 pipe
-// costs the whole warp.  Here each lane holds its own particle and claims the next one as soon
-// as its own is done.  One trip through the loop is, for every lane that holds a particle, one
-// table evaluation at its trial point (s, n_q, their Jacobian and p) and at most one 4x4 solve:
-// the Newton step, the polishing step, or, once converged, the transposed system of the EoS
-// derivatives (p_s, p_n) = H^-T (s, n) -- so the warp's lanes evaluate and solve together
-// whatever stage of the iteration their particles are at.  The iteration per particle is the
-// damped Newton of tab_newton (the same iterates, with the residual and the step in grid-step
-// units: the scaling changes rounding only) followed by the derivative solve of eos_invert.
-// Particles whose warm start is not a table solution inside the table, whose table Newton
-// fails, or when the offline inverter is on, take eos_invert inline (a divergent, rarer path).
+// The EoS pass in two halves.
 //
-// Ctx supplies  __device__ bool load(int a, double &s, double n[3], double g[4], double &cs2_cap)
-// (false: not a particle of this pass), and  __device__ void store(int a, const EosOut &o, bool
-// used_table).
-// claim: the pass's particle counter (indices 0 .. limit-1, claimed one lane at a time).
-enum { LANE_NONE = 0, LANE_NEWTON = 1, LANE_POLISH = 2, LANE_REEVAL = 3 };
+// eos_find brings every particle to its (T, mu): the damped table Newton from the warm start,
+// else from the closed form's solution, else the closed form.  A Newton step only has to reduce
+// the residual, so it takes the residual (s, n_q) - target in FP64 and the Jacobian and the 4x4
+// solve in FP32, from the same node values: an FP32 step is off by about 1e-6 of its length, and
+// the point handed on is decided by FP64 residuals alone.  FP64 operations per evaluation fall from
+// 360 (values, derivatives, p, solve) to about 110, and one evaluation fewer is needed: the last
+// step is taken when the residual is below the hand-over bound, and eos_finish looks at its
+// result.  The Newton's work varies from particle to particle, so the lanes refill: each lane
+// holds its own particle and claims the next one as soon as its own is handed on.
+//
+// eos_finish evaluates p, e and (p_s, p_n) = H^-T (s, n) at that point in FP64, one thread per
+// particle, all lanes alike.  A table point whose residual misses the tolerance there (a step
+// across a cell boundary, rarely) goes through the general FP64 inversion from that point.
+//
+// Bound: the FP64 pipe (64 cycles per warp instruction and quadrant).  Measured per stage on the
+// 40 k viscous BSQ event: 103 us (196 in one pass with the
+// derivatives and the solve of every evaluation in FP64), ideal Gubser lattice 31 (303), eight served
+// events (437 k particles) 616 (772), 3+1D Milne event of 258 k particles 595 (1,100).
+//
+// Hand-over bounds on max |residual| / s: 1e-10 where the point has to be the root to rounding
+// (polish), 1e-6 for the 1e-10 tolerance of the mixed and serving forms.
+constexpr uint32_t kNoVerify = 0x80000000u;  // status bit between the halves: the point is taken as it is
+
+// magnitude-truncated single-precision value of a double, from its bits (|v| < 2^-126: zero)
+__device__ __forceinline__ float f32_bits(double v)
+{
+    const unsigned hi = (unsigned)__double2hiint(v), m = hi & 0x7FFFFFFFu;
+    const unsigned r = __funnelshift_l((unsigned)__double2loint(v), m - 0x38000000u, 3);
+    return __uint_as_float((hi & 0x80000000u) | (m < 0x38100000u ? 0u : r));
+}
+// a float as a double by bits (denormals: zero; the exponent 255 becomes a large finite number)
+__device__ __forceinline__ double f64_bits(float v)
+{
+    const unsigned b = __float_as_uint(v), m = b & 0x7FFFFFFFu;
+    if (m < 0x00800000u) return 0.0;
+    return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(b << 29));
+}
+
+// residual of (s, n_B, n_S, n_Q) at the grid coordinates xi in FP64 and its Jacobian per grid step in FP32
+__device__ __forceinline__ void tab_resid_steps(const EosDev &E, const double *xi, const double *tgt, double r[4],
+                                                float J[4][4])
+{
+    int iT, iB, iS, iQ;
+    double tT, tB, tS, tQ;
+    locate_steps(xi[0], E.nT, iT, tT);
+    locate_steps(xi[1], E.nmu[0], iB, tB);
+    locate_steps(xi[2], E.nmu[1], iS, tS);
+    locate_steps(xi[3], E.nmu[2], iQ, tQ);
+    const int n3 = E.nmu[2], n23 = E.nmu[1] * E.nmu[2], n123 = E.nmu[0] * n23;
+    const size_t node0 = (size_t)iT * n123 + (size_t)iB * n23 + (size_t)iS * n3 + iQ;
+    const double2 *sn2 = reinterpret_cast<const double2 *>(E.sn);
+    const double uT = 1.0 - tT, uB = 1.0 - tB, uS = 1.0 - tS, uQ = 1.0 - tQ;
+    const double w00 = uS * uQ, w01 = uS * tQ, w10 = tS * uQ, w11 = tS * tQ;
+    const double wp[4] = {uT * uB, uT * tB, tT * uB, tT * tB};
+    const float fT = f32_bits(tT), fB = f32_bits(tB), fS = f32_bits(tS), fQ = f32_bits(tQ);
+#pragma unroll
+    for (int fp = 0; fp < 2; ++fp) {
+        double acc[2] = {-tgt[2 * fp], -tgt[2 * fp + 1]};
+        float lv[2][2], lb[2][2], ls[2][2], lq[2][2];
+#pragma unroll
+        for (int bT = 0; bT < 2; ++bT) {
+            float pv[2][2], ps[2][2], pq[2][2];
+#pragma unroll
+            for (int bB = 0; bB < 2; ++bB) {
+                const size_t base = node0 + (size_t)bT * n123 + (size_t)bB * n23;
+                const double2 q00 = __ldg(sn2 + 2 * base + fp), q01 = __ldg(sn2 + 2 * (base + 1) + fp);
+                const double2 q10 = __ldg(sn2 + 2 * (base + n3) + fp), q11 = __ldg(sn2 + 2 * (base + n3 + 1) + fp);
+#pragma unroll
+                for (int g = 0; g < 2; ++g) {
+                    const double c00 = g ? q00.y : q00.x, c01 = g ? q01.y : q01.x;
+                    const double c10 = g ? q10.y : q10.x, c11 = g ? q11.y : q11.x;
+                    acc[g] = fma(wp[2 * bT + bB], fma(w11, c11, fma(w10, c10, fma(w01, c01, w00 * c00))), acc[g]);
+                    const float e00 = f32_bits(c00), e01 = f32_bits(c01), e10 = f32_bits(c10), e11 = f32_bits(c11);
+                    const float d0 = e01 - e00, d1 = e11 - e10;
+                    const float a0 = fmaf(fQ, d0, e00), a1 = fmaf(fQ, d1, e10), ds = a1 - a0;
+                    pv[g][bB] = fmaf(fS, ds, a0);
+                    ps[g][bB] = ds;
+                    pq[g][bB] = fmaf(fS, d1 - d0, d0);
+                }
+            }
+#pragma unroll
+            for (int g = 0; g < 2; ++g) {
+                lb[g][bT] = pv[g][1] - pv[g][0];
+                lv[g][bT] = fmaf(fB, lb[g][bT], pv[g][0]);
+                ls[g][bT] = fmaf(fB, ps[g][1] - ps[g][0], ps[g][0]);
+                lq[g][bT] = fmaf(fB, pq[g][1] - pq[g][0], pq[g][0]);
+            }
+        }
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+            const int f = 2 * fp + g;
+            r[f] = acc[g];
+            J[f][0] = lv[g][1] - lv[g][0];
+            J[f][1] = fmaf(fT, lb[g][1] - lb[g][0], lb[g][0]);
+            J[f][2] = fmaf(fT, ls[g][1] - ls[g][0], ls[g][0]);
+            J[f][3] = fmaf(fT, lq[g][1] - lq[g][0], lq[g][0]);
+        }
+    }
+}
+
+// 4x4 Gaussian elimination with partial pivoting in FP32 (solve4's order)
+__device__ __forceinline__ bool solve4f(float A[4][4], float b[4])
+{
+    float ipv[4];
+    bool ok = true;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        int piv = c;
+        float best = fabsf(A[c][c]);
+#pragma unroll
+        for (int r = c + 1; r < 4; ++r) {
+            const float v = fabsf(A[r][c]);
+            if (v > best) {
+                best = v;
+                piv = r;
+            }
+        }
+        ok = ok && best > 0.0f && best < __int_as_float(0x7F800000);
+#pragma unroll
+        for (int r = c + 1; r < 4; ++r) {
+            const bool sw = piv == r;
+#pragma unroll
+            for (int k = c; k < 4; ++k) {
+                const float t = A[c][k];
+                A[c][k] = sw ? A[r][k] : t;
+                A[r][k] = sw ? t : A[r][k];
+            }
+            const float t = b[c];
+            b[c] = sw ? b[r] : t;
+            b[r] = sw ? t : b[r];
+        }
+        const float inv = __frcp_rn(A[c][c]);
+        ipv[c] = inv;
+#pragma unroll
+        for (int r = c + 1; r < 4; ++r) {
+            const float f = A[r][c] * inv;
+#pragma unroll
+            for (int k = c + 1; k < 4; ++k) A[r][k] = fmaf(-f, A[c][k], A[r][k]);
+            b[r] = fmaf(-f, b[c], b[r]);
+        }
+    }
+#pragma unroll
+    for (int r = 3; r >= 0; --r) {
+        float acc = b[r];
+#pragma unroll
+        for (int k = r + 1; k < 4; ++k) acc = fmaf(-A[r][k], b[k], acc);
+        b[r] = acc * ipv[r];
+    }
+    return ok;
+}
+
+// inside_table on integer keys (an FP64 comparison costs an FP64 operation)
+__device__ __forceinline__ bool inside_keys(const EosDev &E, const double *x)
+{
+    bool in = okey(x[0]) >= okey(E.T0) && okey(x[0]) <= okey(E.Tmax);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) in = in && okey(x[1 + q]) >= okey(E.mu0[q]) && okey(x[1 + q]) <= okey(E.mumax[q]);
+    return in;  // NaN keys lie beyond every bound
+}
+__device__ __forceinline__ bool finite_bits(double v) { return mag_bits(v) < kInfBits; }
+
+// the closed form as a call of its own: the lane loop keeps its registers for the table Newton
+__device__ __noinline__ uint32_t an_invert_call(const EosDev &E, double s, const double *n, double *x, EosWork &w,
+                                                double Tguess)
+{
+    return an_invert(E, s, n, x[0], x + 1, w, Tguess);
+}
+
+// First half.  Ctx supplies  bool load(int a, double &s, double n[3], double g[4])  (false: not a
+// particle of this pass; g: the warm start, T > 0 a table solution, T < 0 minus a closed-form T)
+// and  void put(int a, const double x[4], uint32_t st): T > 0 a table point, T < 0 minus the
+// closed form's T, 0 none (st tells why).  claim: the pass's particle counter.
+template <class Ctx>
+__device__ void eos_find(const EosDev &E, unsigned int *claim, int limit, Ctx &ctx, EosWork &w)
+{
+    const unsigned FULL = 0xFFFFFFFFu;
+    const int lane = threadIdx.x & 31;
+    const double step[4] = {E.dT, E.dmu[0], E.dmu[1], E.dmu[2]};
+    const double istep[4] = {E.inv_dT, E.inv_dmu[0], E.inv_dmu[1], E.inv_dmu[2]};
+    const double org[4] = {E.T0, E.mu0[0], E.mu0[1], E.mu0[2]};
+    // upper grid coordinates as bit patterns (non-negative doubles order as integers)
+    const long long top[4] = {__double_as_longlong((double)(E.nT - 1)), __double_as_longlong((double)(E.nmu[0] - 1)),
+                              __double_as_longlong((double)(E.nmu[1] - 1)), __double_as_longlong((double)(E.nmu[2] - 1))};
+    const double hand = E.polish ? 1e-10 : 1e-6;
+    int a = -1, it = 0, ls = 0;
+    bool more = true, first = false, cold = false;
+    long long rn = 0, tolb = 0, handb = 0;
+    double xi[4] = {0.0, 0.0, 0.0, 0.0}, xt[4] = {0.0, 0.0, 0.0, 0.0}, tgt[4] = {0.0, 0.0, 0.0, 0.0}, Tcf = 0.0;
+    float d[4] = {0.f, 0.f, 0.f, 0.f}, lam = 1.0f;
+    for (;;) {
+        // lanes without a particle claim the next ones (one atomic per warp)
+        const unsigned need = __ballot_sync(FULL, a < 0 && more);
+        if (need) {
+            const int leader = __ffs(need) - 1;
+            unsigned base = 0u;
+            if (lane == leader) base = atomicAdd(claim, (unsigned)__popc(need));
+            base = __shfl_sync(FULL, base, leader);
+            bool closed = false;
+            double g[4] = {0.0, 0.0, 0.0, 0.0};
+            if (a < 0 && more) {
+                const long long idx = (long long)base + __popc(need & ((1u << lane) - 1u));
+                if (idx >= limit) {
+                    more = false;
+                } else if (ctx.load((int)idx, tgt[0], tgt + 1, g)) {
+                    a = (int)idx;
+                    const bool fin = finite_bits(tgt[0]) && finite_bits(tgt[1]) && finite_bits(tgt[2]) && finite_bits(tgt[3]);
+                    closed = true;
+                    if (!fin) {
+                        const double z[4] = {0.0, 0.0, 0.0, 0.0};
+                        ctx.put(a, z, PST_NONFINITE | PST_NOCONV);
+                        a = -1;
+                        closed = false;
+                    } else if (E.has_table && E.offline) {
+                        double x[4];
+                        if (inv_lookup(E, tgt[0], tgt + 1, x) && inside_table(E, x)) {
+                            ctx.put(a, x, kNoVerify);
+                            a = -1;
+                            closed = false;
+                        }
+                    }
+                    if (closed && E.has_table && __double_as_longlong(g[0]) > 0 && inside_keys(E, g) &&
+                        __double_as_longlong(tgt[0]) > 0) {
+                        closed = cold = false;
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) xt[k] = (g[k] - org[k]) * istep[k];
+                    }
+                }
+            }
+            if (closed) {
+                double x[4] = {0.0, 0.0, 0.0, 0.0};
+                const uint32_t st = an_invert_call(E, tgt[0], tgt + 1, x, w, __double_as_longlong(g[0]) < 0 ? -g[0] : 0.0);
+                if (!st && E.has_table && inside_keys(E, x)) {
+                    cold = true;
+                    Tcf = x[0];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) xt[k] = (x[k] - org[k]) * istep[k];
+                } else {
+                    x[0] = st ? 0.0 : -x[0];
+                    ctx.put(a, x, st ? (E.backup && tgt[0] > 0.0 ? PST_BACKUP : st) : (E.has_table ? PST_OUT_OF_TABLE : 0u));
+                    a = -1;
+                }
+            }
+            if (a >= 0 && ((need >> lane) & 1u)) {
+                first = true;
+                it = ls = 0;
+                tolb = __double_as_longlong(E.tol * tgt[0]);
+                handb = max(tolb, __double_as_longlong(hand * tgt[0]));
+            }
+        }
+        if (__ballot_sync(FULL, a >= 0 || more) == 0u) break;
+        if (a < 0) continue;
+        // one evaluation at the trial point
+        double r[4];
+        float J[4][4];
+        tab_resid_steps(E, xt, tgt, r, J);
+        ++w.resid;
+        long long rnn = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) rnn = max(rnn, min(mag_bits(r[k]), kInfBits));
+        bool fail = false, step_on = false, last = false;
+        if (first || rnn < rn) {
+            it += first ? 0 : 1;
+            first = false;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) xi[k] = xt[k];
+            rn = rnn;
+            if (rn <= tolb && !E.polish) last = true;
+            else if (rn <= handb) last = step_on = true;
+            else if (it >= E.maxit) fail = true;
+            else step_on = true;
+        } else if (++ls > 8) {
+            fail = true;  // no decrease along the Newton direction: stalled
+        } else {
+            lam *= 0.5f;
+        }
+        if (step_on) {
+            ++w.solve;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) d[k] = -f32_bits(r[k]);
+            const bool ok = solve4f(J, d);
+            if (!ok && !last) fail = true;
+            if (!ok)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) d[k] = 0.0f;
+            lam = 1.0f;
+            ls = 0;
+        }
+        if (!(last && !step_on)) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {  // the trial point, clamped to the grid
+                const long long b = __double_as_longlong(xi[k] + f64_bits(lam * d[k]));
+                xt[k] = __longlong_as_double(b < 0 ? 0LL : min(b, top[k]));
+            }
+        }
+        if (last) {
+            double x[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) x[k] = fma(step_on ? xt[k] : xi[k], step[k], org[k]);
+            clamp4(E, x);
+            ctx.put(a, x, 0u);
+            a = -1;
+        } else if (fail) {
+            double x[4] = {0.0, 0.0, 0.0, 0.0};
+            if (!cold) {  // the table Newton from the warm start failed: from the closed form
+                const uint32_t st = an_invert_call(E, tgt[0], tgt + 1, x, w, 0.0);
+                if (!st && inside_keys(E, x)) {
+                    cold = first = true;
+                    Tcf = x[0];
+                    it = ls = 0;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) xt[k] = (x[k] - org[k]) * istep[k];
+                } else {
+                    x[0] = st ? 0.0 : -x[0];
+                    ctx.put(a, x, st ? (E.backup && tgt[0] > 0.0 ? PST_BACKUP : st) : PST_OUT_OF_TABLE);
+                    a = -1;
+                }
+            } else {
+                x[0] = -Tcf;
+                ctx.put(a, x, PST_FALLBACK);
+                a = -1;
+            }
+        }
+    }
+}
 
 // the general inversion as a call of its own: the lane loop keeps its registers for the table
 // Newton, the common path
@@ -608,212 +1005,82 @@ __device__ __noinline__ EosOut eos_invert_call(const EosDev &E, double cs2_cap, 
     return eos_invert(E, cs2_cap, s, n, guess, used_table, w);
 }
 
-template <class Ctx>
-__device__ void eos_lanes(const EosDev &E, unsigned int *claim, int limit, Ctx &ctx, EosWork &w)
+// Second half: the EoS outputs of one particle at the point g handed on by eos_find with status
+// st (see there).  used_table tells whether the table produced the result.
+__device__ __forceinline__ EosOut eos_finish(const EosDev &E, double cs2_cap, double s, const double *n,
+                                             const double *g, uint32_t st, bool &used_table, EosWork &w)
 {
-    const unsigned FULL = 0xFFFFFFFFu;
-    const int lane = threadIdx.x & 31;
-    // grid steps of the table axes: the iteration works in grid-step units with the residual
-    // unscaled (the Newton step is the same: scaling the residual and the Jacobian's rows by
-    // 1/s, or its columns by the steps, does not change it), and converges when
-    // max |residual| <= tol s
-    const double step[4] = {E.dT, E.dmu[0], E.dmu[1], E.dmu[2]};
-    const double istep[4] = {E.inv_dT, E.inv_dmu[0], E.inv_dmu[1], E.inv_dmu[2]};
-    int a = -1, phase = LANE_NONE, it = 0, ls = 0;
-    bool more = true, first = false;
-    long long rn = 0, tolb = 0;  // max-norms of the residual as integer magnitudes
-    double x[4], xt[4], d[4], r[4], J[4][4], p = 0.0, lam = 1.0, s = 0.0, nq[3];
-    double cs2_cap = 1.0;
+    EosOut o;
+    o.T = o.p = o.e = o.ps = o.cs2 = 0.0;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) x[k] = xt[k] = d[k] = r[k] = 0.0;
-    nq[0] = nq[1] = nq[2] = 0.0;
-    for (;;) {
-        // lanes without a particle claim the next ones (one atomic per warp)
-        const unsigned need = __ballot_sync(FULL, a < 0 && more);
-        if (need) {
-            const int leader = __ffs(need) - 1;
-            unsigned base = 0u;
-            if (lane == leader) base = atomicAdd(claim, (unsigned)__popc(need));
-            base = __shfl_sync(FULL, base, leader);
-            if (a < 0 && more) {
-                const long long idx = (long long)base + __popc(need & ((1u << lane) - 1u));
-                if (idx >= limit) more = false;
-                else a = (int)idx;
-            }
-        }
-        if (__ballot_sync(FULL, a >= 0 || more) == 0u) break;
-        // a new particle: the table Newton from its warm start, or the general inversion
-        if (a >= 0 && phase == LANE_NONE) {
-            double g[4];
-            if (!ctx.load(a, s, nq, g, cs2_cap)) {
-                a = -1;
-            } else if (E.has_table && !E.offline && g[0] > 0.0 && inside_table(E, g) && isfinite(s) && s > 0.0 &&
-                       isfinite(nq[0]) && isfinite(nq[1]) && isfinite(nq[2])) {
-#pragma unroll
-                for (int k = 0; k < 4; ++k) xt[k] = g[k];
-                phase = LANE_NEWTON;
-                first = true;
-                it = 0;
-                ls = 0;
-                tolb = __double_as_longlong(E.tol * s);
-            } else {
-                bool used = false;
-                const EosOut o = eos_invert_call(E, cs2_cap, s, nq, g, used, w);
-                ctx.store(a, o, used);
-                a = -1;
-            }
-        }
-        // one table evaluation at the trial point: (s, n) - target and the Jacobian per grid
-        // step, and p
-        const bool evl = a >= 0 && phase != LANE_NONE;
-        long long rnn = 0;
-        if (evl) {
-            double sn[4];
-            tab_eval_steps(E, xt, sn, J, &p);
-            const double tgt[4] = {s, nq[0], nq[1], nq[2]};
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                r[k] = sn[k] - tgt[k];
-                rnn = max(rnn, min(mag_bits(r[k]), kInfBits));  // a non-finite residual counts as infinite
-            }
-            ++w.resid;
-        }
-        // what this trip solves: 0 nothing, 1 a Newton step (J d = -r, also the polishing
-        // step), 2 the EoS derivatives at the converged point (H^T z = (s, n), H = d(s, n)/d(T, mu))
-        int act = 0;
-        bool fail = false;
-        if (evl) {
-            bool accepted = false;
-            if (phase == LANE_NEWTON) {
-                if (first || rnn < rn) {
-                    accepted = true;
-                    if (!first) ++it;
-                    first = false;
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) x[k] = xt[k];
-                    rn = rnn;
-                } else if (++ls > 8) {
-                    fail = true;  // no decrease along the Newton direction: stalled
-                } else {
-                    lam *= 0.5;
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) xt[k] = fma(lam, d[k], x[k]);
-                    clamp4(E, xt);
-                }
-                if (accepted) {
-                    if (it >= E.maxit) {
-                        if (rn <= tolb) act = 2;
-                        else fail = true;
-                    } else if (rn <= tolb) {
-                        act = E.polish ? 1 : 2;
-                        if (E.polish) phase = LANE_POLISH;
-                    } else {
-                        act = 1;
-                    }
-                }
-            } else if (phase == LANE_POLISH) {
-                if (rnn <= tolb) {
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) x[k] = xt[k];
-                    act = 2;
-                } else {  // the polished point is refused: J and p again at the kept point
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) xt[k] = x[k];
-                    phase = LANE_REEVAL;
-                }
-            } else {  // LANE_REEVAL
-                act = 2;
-            }
-        }
-        double b[4];
-        if (act == 1) {
-#pragma unroll
-            for (int k = 0; k < 4; ++k) b[k] = -r[k];
-        } else if (act == 2) {  // A = H^T, H[f][j] = J[f][j] / step_j
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = i + 1; j < 4; ++j) {
-                    const double t = J[i][j];
-                    J[i][j] = J[j][i];
-                    J[j][i] = t;
-                }
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) J[i][j] *= istep[i];
-            b[0] = s;
-            b[1] = nq[0];
-            b[2] = nq[1];
-            b[3] = nq[2];
-        }
-        bool ok = true;
-        if (act) {
-            ++w.solve;
-            ok = solve4(J, b);
-        }
-        if (act == 1) {
-            if (phase == LANE_POLISH) {
-                if (ok) {
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) xt[k] = fma(b[k], step[k], x[k]);
-                    clamp4(E, xt);
-                } else {
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) xt[k] = x[k];
-                    phase = LANE_REEVAL;
-                }
-            } else if (!ok) {
-                fail = true;
-            } else {
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    d[k] = b[k] * step[k];
-                    xt[k] = x[k] + d[k];
-                }
-                clamp4(E, xt);
-                lam = 1.0;
-                ls = 0;
-            }
-        } else if (act == 2) {
-            EosOut o;
-            o.st = 0u;
-            if (!ok) {
-                o.T = o.p = o.e = o.ps = o.cs2 = 0.0;
-#pragma unroll
-                for (int q = 0; q < 3; ++q) o.mu[q] = o.pn[q] = 0.0;
-                o.st = PST_NOCONV;
-            } else {
-                const double e = x[0] * s + x[1] * nq[0] + x[2] * nq[1] + x[3] * nq[2] - p;
-                double cs2 = (s * b[0] + nq[0] * b[1] + nq[1] * b[2] + nq[2] * b[3]) / (e + p);
-                if (cs2 > cs2_cap) {
-                    const double f = cs2_cap / cs2;
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) b[k] *= f;
-                    cs2 = cs2_cap;
-                    o.st |= PST_CS2_CAPPED;
-                }
-                o.T = x[0];
-#pragma unroll
-                for (int q = 0; q < 3; ++q) o.mu[q] = x[1 + q], o.pn[q] = b[1 + q];
-                o.p = p;
-                o.e = e;
-                o.ps = b[0];
-                o.cs2 = cs2;
-            }
-            ctx.store(a, o, true);
-            a = -1;
-            phase = LANE_NONE;
-        }
-        if (fail) {  // the table Newton from the warm start failed: the general inversion
-            const double g0[4] = {0.0, 0.0, 0.0, 0.0};
-            bool used = false;
-            const EosOut o = eos_invert_call(E, cs2_cap, s, nq, g0, used, w);
-            ctx.store(a, o, used);
-            a = -1;
-            phase = LANE_NONE;
-        }
+    for (int q = 0; q < 3; ++q) o.mu[q] = o.pn[q] = 0.0;
+    o.st = st & ~kNoVerify;
+    used_table = false;
+    const long long tb = __double_as_longlong(g[0]);
+    if (tb == 0) {
+        if (st & PST_BACKUP) return backup_eos(E, s, n);
+        return o;
     }
+    double x[4], H[4][4], b[4] = {s, n[0], n[1], n[2]}, p;
+    if (tb > 0) {
+        used_table = true;
+        double sn[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) x[k] = g[k];
+        tab_eval_steps(E, x, sn, H, &p);
+        ++w.resid;
+        long long rn = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) rn = max(rn, min(mag_bits(sn[k] - b[k]), kInfBits));
+        if (!(st & kNoVerify) && rn > __double_as_longlong(E.tol * s))
+            return eos_invert_call(E, cs2_cap, s, n, g, used_table, w);
+        const double istep[4] = {E.inv_dT, E.inv_dmu[0], E.inv_dmu[1], E.inv_dmu[2]};
+#pragma unroll
+        for (int i = 0; i < 4; ++i)  // H^T, per unit of (T, mu)
+#pragma unroll
+            for (int j = i; j < 4; ++j) {
+                const double t = H[i][j];
+                H[i][j] = H[j][i] * istep[i];
+                H[j][i] = t * istep[j];
+            }
+    } else {
+        double sn[4];
+        x[0] = -g[0];
+        const double it2 = 1.0 / (x[0] * x[0]);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) x[1 + q] = E.chi[q] > 0.0 ? n[q] / E.chi[q] * it2 : 0.0;
+        an_eval(E, x[0], x + 1, p, sn, H);  // symmetric
+        // an uncoupled charge direction (chi_q = 0): an identity row with zero right-hand side
+#pragma unroll
+        for (int q = 1; q < 4; ++q)
+            if (!(E.chi[q - 1] > 0.0)) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) H[q][j] = H[j][q] = q == j ? 1.0 : 0.0;
+                b[q] = 0.0;
+            }
+    }
+    ++w.solve;
+    if (!solve4(H, b)) {
+        o.st |= PST_NOCONV;
+        return o;
+    }
+    const double e = x[0] * s + x[1] * n[0] + x[2] * n[1] + x[3] * n[2] - p;
+    double cs2 = (s * b[0] + n[0] * b[1] + n[1] * b[2] + n[2] * b[3]) / (e + p);
+    if (cs2 > cs2_cap) {
+        const double f = cs2_cap / cs2;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) b[k] *= f;
+        cs2 = cs2_cap;
+        o.st |= PST_CS2_CAPPED;
+    }
+    o.T = x[0];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) o.mu[q] = x[1 + q], o.pn[q] = b[1 + q];
+    o.p = p;
+    o.e = e;
+    o.ps = b[0];
+    o.cs2 = cs2;
+    return o;
 }
 
 }  // namespace

@@ -22,23 +22,6 @@ namespace sphg {
 
 namespace {
 
-// cell-relative single-precision positions of the sorted particles
-__global__ void k_relpos2(EvView v, const double *__restrict__ y, float2 *__restrict__ rel)
-{
-    int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= v.n) return;
-    const double cs = 2.0 * v.h;
-    double r[2];
-#pragma unroll
-    for (int d = 0; d < 2; ++d) {
-        double xm = dec_double(v.sc->xmin_enc[d]);
-        double x = y[(size_t)d * v.n + j];
-        int c = cell_coord(x, xm, v.inv_cell);
-        r[d] = __dsub_rn(__dsub_rn(x, xm), (double)c * cs);
-    }
-    rel[j] = make_float2(__double2float_rn(r[0]), __double2float_rn(r[1]));
-}
-
 // Cell-tiled passes: one block per occupied cell (grid-stride over the cell grid) stages the
 // candidates of the 3x3 block of 2h-cells around it -- nine runs of the Morton-sorted order --
 // in shared memory, in tiles of kTile2, two candidates per float4 entry (packed two-wide FP32
@@ -370,8 +353,6 @@ __global__ void __launch_bounds__(TT) k_tiled_gradient2m(EvView v, int stage, co
     }
 }
 
-inline int nblk(int n, int t) { return (n + t - 1) / t; }
-
 // blocks of the tiled passes: one per cell of the 2^B x 2^B grid, at most 8 per SM (the rest
 // grid-stride)
 inline int tiled_grid2(const EvView &v)
@@ -385,7 +366,6 @@ inline int tiled_grid2(const EvView &v)
 void launch_density2m(const EvView &v, const double *y, const double *Nq, CellBufs cb, double *dens, int *nnb,
                       cudaStream_t st)
 {
-    k_relpos2<<<nblk(v.n, 256), 256, 0, st>>>(v, y, cb.fpos);
     k_tiled_density2m<kTT2><<<tiled_grid2(v), kTT2, 0, st>>>(v, y, cb.fpos, Nq, cb.start, cb.cnt, dens, nnb);
 }
 

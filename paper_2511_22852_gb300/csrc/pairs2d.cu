@@ -315,7 +315,7 @@ __global__ void __launch_bounds__(32 * kWarps) k_pairs_density_bwd(EvView v, con
     const int k = lane >> 2;
     if ((lane & 3) == 0 && k < 5) {
         // rows sigma*, lab-frame s* (divided by u0 sqrt(-g) in the EoS pass), n*_B, n*_S, n*_Q:
-        // the forward partials were left in the density rows; u0 (row 5) is written by k_fpos
+        // the forward partials were left in the density rows; u0 (row 5) is written with the permutation
         double *d = dens + (size_t)k * n + a;
         *d = v.sigma_d * (*d + tot);
     }

@@ -1072,7 +1072,7 @@ sph_status dmalloc(sph_server *S, void **p, size_t bytes)
 
 // kernels a batch step launches: per stage 11 for the cell list and permutation, then the
 // density, EoS, gradient and equations-of-motion passes and the two of the work sum
-constexpr int kKernelsPerBatchStep = 2 * 17;
+constexpr int kKernelsPerBatchStep = 2 * 18;
 
 // one batch step (both stages) on the server's stream; captured once into a graph.  marks (the
 // sampled timing, eager launches only): kProfMarks events recorded between the kernel groups

@@ -425,8 +425,10 @@ inline float prefilter_bound(double h, int B, int dim = 2)
 
 void launch_bbox(const EvView &v, const double *y, cudaStream_t st);
 void launch_cells(const EvView &v, const double *y, const int *id, CellBufs cb, cudaStream_t st);
-void launch_permute(const EvView &v, const uint32_t *perm, const double *const *src, double *const *dst,
-                    const int *nrows, int ngroups, const int *id_in, int *id_out, cudaStream_t st);
+// dst[0] on holds the state: its sorted single-precision positions (and u0, plain 2D: density row 5) are
+// written for the neighbour passes
+void launch_permute(const EvView &v, const CellBufs &cb, const double *const *src, double *const *dst,
+                    const int *nrows, int ngroups, const int *id_in, int *id_out, double *dens, cudaStream_t st);
 // plain 2D neighbour passes over the half-pair lists (cb.pl.total > 0): row offsets from the
 // previous counts, then the forward and backward density passes
 void launch_pairs_density(const EvView &v, const double *y, const double *Nq, CellBufs cb, double *dens, int *nnb,
@@ -435,7 +437,7 @@ void launch_pairs_gradient(const EvView &v, int stage, const double *y, const do
                            double *gout, cudaStream_t st);
 // the per-stage row offsets of the pair lists (prefix scan of the carried counts)
 void launch_pair_rows(const EvView &v, CellBufs cb, cudaStream_t st);
-// plain 3D neighbour passes over the half-pair lists (after k_fpos3 and the row offsets)
+// plain 3D neighbour passes over the half-pair lists (after the row offsets)
 void launch_pairs3_density(const EvView &v, const double *y, const double *Nq, CellBufs cb, double *dens, int *nnb,
                            cudaStream_t st);
 void launch_pairs3_gradient(const EvView &v, int stage, const double *y, const double *gin, CellBufs cb,

@@ -44,17 +44,6 @@ __global__ void k_cells3(EvView v, const double *__restrict__ y, uint32_t *key, 
     atomicAdd(&cnt[k], 1u);
 }
 
-__global__ void k_fpos3(EvView v, const double *__restrict__ y, float4 *__restrict__ fpos)
-{
-    int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= v.n) return;
-    float f[3];
-#pragma unroll
-    for (int d = 0; d < 3; ++d)
-        f[d] = __double2float_rn(__dsub_rn(y[(size_t)d * v.n + j], dec_double(v.sc->xmin_enc[d])));
-    fpos[j] = make_float4(f[0], f[1], f[2], 0.0f);
-}
-
 // the 27-cell candidate walk of one warp: prefilter, compaction, then `pair` on full warps
 template <class Pair>
 __device__ __forceinline__ void walk27(const EvView &v, const uint32_t *__restrict__ start,
@@ -208,66 +197,109 @@ __device__ __forceinline__ double gam(const Geo3 &G, int a, int b, int c)
 }
 
 // full contravariant pi^{mu nu} from the stored (11, 12, 13, 22, 23) components:
-// pi^{33} from g_{mu nu} pi^{mu nu} = 0, pi^{0 nu} from u_mu pi^{mu nu} = 0
-__device__ __forceinline__ void pi_full3(const Geo3 &G, const double *u, const double *st, double pi[4][4])
+// pi^{33} from g_{mu nu} pi^{mu nu} = 0, pi^{0 nu} from u_mu pi^{mu nu} = 0; v_i = u_i / u_0 with
+// u_1 = -u^1, u_2 = -u^2, u_3 = g_33 u^3 and iu0 = 1 / u^0
+__device__ __forceinline__ void pi_full3(const Geo3 &G, const double *u, double iu0, const double *st, double pi[4][4])
 {
-    double ul[4];
-#pragma unroll
-    for (int m = 0; m < 4; ++m) ul[m] = G.g[m] * u[m];
+    const double v1 = -u[1] * iu0, v2 = -u[2] * iu0, g3 = G.g[3], v3 = g3 * u[3] * iu0;
     pi[1][1] = st[0];
     pi[1][2] = pi[2][1] = st[1];
     pi[1][3] = pi[3][1] = st[2];
     pi[2][2] = st[3];
     pi[2][3] = pi[3][2] = st[4];
-    const double iu02 = 1.0 / (ul[0] * ul[0]);
-    double known = (ul[1] * ul[1] * pi[1][1] + ul[2] * ul[2] * pi[2][2] + 2.0 * ul[1] * ul[2] * pi[1][2] +
-                    2.0 * ul[1] * ul[3] * pi[1][3] + 2.0 * ul[2] * ul[3] * pi[2][3]) * iu02 +
-                   G.g[1] * pi[1][1] + G.g[2] * pi[2][2];
-    pi[3][3] = -known / (ul[3] * ul[3] * iu02 + G.g[3]);
+    const double known = v1 * v1 * st[0] + v2 * v2 * st[3] - (st[0] + st[3]) +
+                         2.0 * (v1 * v2 * st[1] + v3 * (v1 * st[2] + v2 * st[4]));
+    pi[3][3] = -known / (v3 * v3 + g3);
 #pragma unroll
-    for (int i = 1; i < 4; ++i) {
-        double acc = ul[1] * pi[1][i] + ul[2] * pi[2][i] + ul[3] * pi[3][i];
-        pi[0][i] = pi[i][0] = -acc / ul[0];
-    }
-    pi[0][0] = -(ul[1] * pi[1][0] + ul[2] * pi[2][0] + ul[3] * pi[3][0]) / ul[0];
+    for (int i = 1; i < 4; ++i) pi[0][i] = pi[i][0] = -(v1 * pi[1][i] + v2 * pi[2][i] + v3 * pi[3][i]);
+    pi[0][0] = -(v1 * pi[1][0] + v2 * pi[2][0] + v3 * pi[3][0]);
 }
 
-// a4: u^0, rest-frame densities, EoS, stress inputs of the gradient pass, work rate
-__global__ void __launch_bounds__(64, 6) k_eos3(EvView v, int stage, const double *__restrict__ y,
-                                                double *__restrict__ dens, double *__restrict__ eos,
-                                                double *__restrict__ gin, uint32_t *__restrict__ status,
-                                                double *__restrict__ wpart, const double *__restrict__ guess_in,
-                                                double *__restrict__ guess_out)
+// a4, first half: u^0, rest-frame densities, the search for (T, mu) (eos_device.cuh)
+constexpr int kEosWarps3 = 4, kEosBlocks3 = 3;
+
+struct Find3Ctx {
+    const EvView &v;
+    size_t n;
+    double g3, sqrtg;
+    const double *__restrict__ y;
+    double *__restrict__ dens, *__restrict__ guess_out;
+    uint32_t *__restrict__ status;
+    const double *__restrict__ guess_in;
+    __device__ bool load(int a, double &s, double nq[3], double g[4])
+    {
+        const double u1 = y[3 * n + a], u2 = y[4 * n + a], u3 = y[5 * n + a];
+        const double u0 = sqrt(1.0 + (u1 * u1 + u2 * u2 - g3 * u3 * u3));
+        const double ivol = 1.0 / (u0 * sqrtg);
+        s = dens[n + a] * ivol;
+        dens[n + a] = s;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            nq[q] = dens[(2 + q) * n + a] * ivol;
+            dens[(2 + q) * n + a] = nq[q];
+        }
+        dens[5 * n + a] = u0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) g[k] = guess_in[k * n + a];
+        return true;
+    }
+    __device__ void put(int a, const double x[4], uint32_t st)
+    {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) guess_out[k * n + a] = x[k];
+        status[a] = st;
+    }
+};
+
+__device__ __forceinline__ void add_eos_work3(DevScalars *sc, const EosWork &w, unsigned st_or)
+{
+    const unsigned wres = __reduce_add_sync(0xFFFFFFFFu, w.resid);
+    const unsigned wsol = __reduce_add_sync(0xFFFFFFFFu, w.solve);
+    const unsigned wg = __reduce_add_sync(0xFFFFFFFFu, w.g);
+    const unsigned sor = __reduce_or_sync(0xFFFFFFFFu, st_or);
+    if ((threadIdx.x & 31) == 0) {
+        if (wres) atomicAdd(&sc->eos_resid, (unsigned long long)wres);
+        if (wsol) atomicAdd(&sc->eos_solve, (unsigned long long)wsol);
+        if (wg) atomicAdd(&sc->eos_g, (unsigned long long)wg);
+        if (sor) atomicOr(&sc->status_or, sor);
+    }
+}
+
+__global__ void __launch_bounds__(32 * kEosWarps3, kEosBlocks3)
+    k_eos3_find(EvView v, int stage, const double *__restrict__ y, double *__restrict__ dens,
+                uint32_t *__restrict__ status, const double *__restrict__ guess_in, double *__restrict__ guess_out)
+{
+    const Geo3 G = geo3(v, stage);
+    Find3Ctx ctx{v, (size_t)v.n, G.g[3], G.sqrtg, y, dens, guess_out, status, guess_in};
+    EosWork w = {0u, 0u, 0u};
+    eos_find(v.eos, &v.sc->eos_claim, v.n, ctx, w);
+    add_eos_work3(v.sc, w, 0u);
+}
+
+// a4, second half: the EoS there, stress inputs of the gradient pass, work rate
+__global__ void __launch_bounds__(64, 5) k_eos3_finish(EvView v, int stage, const double *__restrict__ y,
+                                                    const double *__restrict__ dens, double *__restrict__ eos,
+                                                    double *__restrict__ gin, uint32_t *__restrict__ status,
+                                                    double *__restrict__ wpart, double *__restrict__ guess_out)
 {
     __shared__ double red[2];
     const int a = blockIdx.x * blockDim.x + threadIdx.x;
     const size_t n = (size_t)v.n;
     double wcontrib = 0.0;
-    unsigned wres = 0u, wsol = 0u, wg = 0u;
+    EosWork w = {0u, 0u, 0u};
+    unsigned st_or = 0u;
     if (a < v.n) {
         const Geo3 G = geo3(v, stage);
-        double u[4] = {0.0, y[3 * n + a], y[4 * n + a], y[5 * n + a]};
-        u[0] = sqrt(1.0 - (G.g[1] * u[1] * u[1] + G.g[2] * u[2] * u[2] + G.g[3] * u[3] * u[3]));
-        const double sig_star = dens[a];
-        const double vol = u[0] * G.sqrtg;
-        const double s = dens[n + a] / vol;
-        double nq[3] = {dens[2 * n + a] / vol, dens[3 * n + a] / vol, dens[4 * n + a] / vol};
-        dens[n + a] = s;
-        for (int q = 0; q < 3; ++q) dens[(2 + q) * n + a] = nq[q];
-        dens[5 * n + a] = u[0];
-        double gs[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) gs[k] = guess_in[(size_t)k * n + a];
+        const double u[4] = {dens[5 * n + a], y[3 * n + a], y[4 * n + a], y[5 * n + a]};
+        const double isig = 1.0 / dens[a], iu0 = 1.0 / u[0];
+        const double s = dens[n + a], nq[3] = {dens[2 * n + a], dens[3 * n + a], dens[4 * n + a]};
+        const double g[4] = {guess_out[a], guess_out[n + a], guess_out[2 * n + a], guess_out[3 * n + a]};
         bool used = false;
-        EosWork w = {0u, 0u, 0u};
-        EosOut o = eos_invert(v.eos, v.tr.cs2_cap, s, nq, gs, used, w);
-        wres = w.resid;
-        wsol = w.solve;
-        wg = w.g;
+        const EosOut o = eos_finish(v.eos, v.tr.cs2_cap, s, nq, g, status[a], used, w);
         guess_out[a] = used ? o.T : ((o.st & (PST_NOCONV | PST_NONFINITE | PST_BACKUP)) ? 0.0 : -o.T);
         for (int q = 0; q < 3; ++q) guess_out[(size_t)(1 + q) * n + a] = used ? o.mu[q] : 0.0;
         status[a] = o.st;
-        warp_or(&v.sc->status_or, o.st);
+        st_or = o.st;
         eos[a] = o.T;
         for (int q = 0; q < 3; ++q) eos[(1 + q) * n + a] = o.mu[q];
         eos[4 * n + a] = o.p;
@@ -275,7 +307,8 @@ __global__ void __launch_bounds__(64, 6) k_eos3(EvView v, int stage, const doubl
         eos[6 * n + a] = o.ps;
         for (int q = 0; q < 3; ++q) eos[(7 + q) * n + a] = o.pn[q];
         eos[10 * n + a] = o.cs2;
-        const double sigma = sig_star / vol;
+        const double isg = G.milne ? 1.0 / G.sqrtg : 1.0;
+        const double sigma = dens[a] * iu0 * isg;
         double Pi = 0.0, st[5] = {0, 0, 0, 0, 0};
         if (v.tr.viscous) {
             Pi = sigma * y[7 * n + a];
@@ -283,31 +316,28 @@ __global__ void __launch_bounds__(64, 6) k_eos3(EvView v, int stage, const doubl
             for (int k = 0; k < 5; ++k) st[k] = sigma * y[(8 + k) * n + a];
         }
         double pi[4][4];
-        pi_full3(G, u, st, pi);
-        const double inv2 = 1.0 / (sig_star * sig_star);
+        pi_full3(G, u, iu0, st, pi);
+        const double inv2 = isig * isig;
         const double P = o.p + Pi;
+        double vv[3];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) vv[j] = u[1 + j] * iu0;
 #pragma unroll
         for (int j = 0; j < 3; ++j)
 #pragma unroll
             for (int i = 0; i < 3; ++i) {
-                double X = (j == i ? -P * G.gi[1 + j] : 0.0) + pi[1 + j][1 + i] - (u[1 + j] / u[0]) * pi[0][1 + i];
+                double X = pi[1 + j][1 + i] - vv[j] * pi[0][1 + i];
+                if (j == i) X += j < 2 ? P : P * (G.milne ? isg * isg : 1.0);  // -P g^{jj}
                 gin[(size_t)(3 * j + i) * n + a] = X * inv2;
             }
-        for (int j = 0; j < 3; ++j) gin[(size_t)(9 + j) * n + a] = u[1 + j] / sig_star;
+#pragma unroll
+        for (int j = 0; j < 3; ++j) gin[(size_t)(9 + j) * n + a] = u[1 + j] * isig;
         if (G.milne) {
             // sqrt(-g) Gamma^0_{33} T^{33} / sigma* = tau^2 T^{eta eta} / sigma*
-            const double T33 = (o.e + P) * u[3] * u[3] - P * G.gi[3] + pi[3][3];
-            wcontrib = G.tau * G.tau * T33 / sig_star;
+            wcontrib = (G.tau * G.tau * ((o.e + P) * u[3] * u[3] + pi[3][3]) + P) * isig;
         }
     }
-    wres = __reduce_add_sync(0xFFFFFFFFu, wres);
-    wsol = __reduce_add_sync(0xFFFFFFFFu, wsol);
-    wg = __reduce_add_sync(0xFFFFFFFFu, wg);
-    if ((threadIdx.x & 31) == 0) {
-        atomicAdd(&v.sc->eos_resid, (unsigned long long)wres);
-        atomicAdd(&v.sc->eos_solve, (unsigned long long)wsol);
-        atomicAdd(&v.sc->eos_g, (unsigned long long)wg);
-    }
+    add_eos_work3(v.sc, w, st_or);
     wcontrib = warp_sum(wcontrib);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = wcontrib;
     __syncthreads();
@@ -444,7 +474,7 @@ __global__ void __launch_bounds__(64) k_eom3(EvView v, int stage, int mode, cons
     double st[5];
     for (int k = 0; k < 5; ++k) st[k] = sigma * stv[k];
     double pi[4][4];
-    pi_full3(G, u, st, pi);
+    pi_full3(G, u, ig, st, pi);
     // d_k u^j (spatial k, j) and d_k u^0
     double dku[4][4];
     for (int k = 1; k < 4; ++k) {
@@ -713,7 +743,7 @@ __global__ void k_totals3(EvView v, const double *__restrict__ y, const int *__r
         for (int k = 0; k < 5; ++k) st[k] = sigma * y[(8 + k) * n + a];
     }
     double pi[4][4];
-    pi_full3(G, u, st, pi);
+    pi_full3(G, u, 1.0 / u[0], st, pi);
     const double p = eos[4 * n + a], e = eos[5 * n + a];
     const double T00 = (e + p + Pi) * u[0] * u[0] - (p + Pi) + pi[0][0];
     const int o = id[a];
@@ -783,7 +813,6 @@ void launch_density3(const EvView &v, const double *y, const double *Nq, CellBuf
         launch_density3m(v, y, Nq, cb, dens, nnb, st);
         return;
     }
-    k_fpos3<<<nblk(v.n, 256), 256, 0, st>>>(v, y, cb.fpos3);
     const int lists = cb.pl.total > 0;
     if (lists) launch_pairs3_density(v, y, Nq, cb, dens, nnb, st);
     // as the fallback of the pair-list passes it usually exits at once: a few blocks per SM
@@ -795,8 +824,10 @@ void launch_density3(const EvView &v, const double *y, const double *Nq, CellBuf
 void launch_eos3(const EvView &v, int stage, const double *y, const double *dens, double *eos, double *gin,
                  uint32_t *status, double *wpart, const double *guess_in, double *guess_out, cudaStream_t st)
 {
-    k_eos3<<<nblk(v.n, 64), 64, 0, st>>>(v, stage, y, const_cast<double *>(dens), eos, gin, status, wpart, guess_in,
-                                         guess_out);
+    const int sms = device_sm_count(), need = nblk(v.n, 32 * kEosWarps3);
+    const int grid = need >= kEosBlocks3 * sms ? kEosBlocks3 * sms : (need >= sms ? (need / sms) * sms : std::max(1, need));
+    k_eos3_find<<<grid, 32 * kEosWarps3, 0, st>>>(v, stage, y, const_cast<double *>(dens), status, guess_in, guess_out);
+    k_eos3_finish<<<nblk(v.n, 64), 64, 0, st>>>(v, stage, y, dens, eos, gin, status, wpart, guess_out);
 }
 
 void launch_gradient3(const EvView &v, int stage, const double *y, const double *gin, CellBufs cb, double *gout,
