@@ -139,7 +139,189 @@ __global__ void __launch_bounds__(32 * kWarps) k_gradient2(EvView v, int stage, 
     }
 }
 
-// equations of motion of one particle (rows n apart): mode 0 writes y1 = y + dt f(y),
+// Heun's use of the rates f[0 .. nv): mode 0 writes y1 = y + dt f(y), mode 1 closes the step in
+// place, mode 2 writes the rates
+__device__ __forceinline__ void heun_store(double dt, int mode, int nv, size_t n, size_t a, const double *f,
+                                           const double *__restrict__ ys, double *__restrict__ yout,
+                                           double *__restrict__ rates)
+{
+    if (mode == 0) {
+#pragma unroll
+        for (int k = 0; k < nv; ++k) yout[k * n + a] = ys[k * n + a] + dt * f[k];
+    } else if (mode == 1) {
+#pragma unroll
+        for (int k = 0; k < nv; ++k) yout[k * n + a] = 0.5 * ((yout[k * n + a] + ys[k * n + a]) + dt * f[k]);
+    } else {
+#pragma unroll
+        for (int k = 0; k < nv; ++k) rates[k * n + a] = f[k];
+    }
+}
+
+// Equations of motion of one particle, minimal Israel-Stewart without diffusion (the general form
+// with DNMR and diffusion is eom2_particle).  Every rate is {c, x, y} = c + x a^x + y a^y, written
+// out with the terms that vanish left out (the compiler has to keep 0 * x and x + 0) and in the
+// per-sigma variables B = Pi/sigma, P = pi/sigma that the state carries, where the volume rate
+// d sigma = -(sigma/u0) theta cancels from most terms:
+//   theta = th0 + v.a,  dS = (P:sigma - B theta)/(u0 T),  dB = -(zeta theta + Pi)/(tau_Pi u0 sigma),
+//   dP^{ij} = ((2 eta/sigma sigma^{ij} - P^{ij})/tau_pi - P^{ij} theta/3)/u0 - u^i C^j - u^j C^i,
+//   C^j = P^{0j} v.a - P^{jk} a^k,
+//   dP_lab^i = u^i D + (w/sigma) a^i + d(P^{0i}/u0),
+//   D = (T + p_s) dS + dB + (e + p - (T + p_s) s - sum (mu + p_n) n) theta / (u0 sigma).
+// Bound: the FP64 pipe; about 250 FP64 operations a particle instead of 585 (437 k particles of
+// eight served events: 406 -> 256 us a stage; the 40 k event: 63 -> 36).
+__device__ __forceinline__ void eom2_min_is(const EvView &v, int stage, int mode, size_t n, size_t a,
+                                            const double *__restrict__ ys, const double *__restrict__ dens,
+                                            const double *__restrict__ eos, const double *__restrict__ gout,
+                                            double *__restrict__ yout, double *__restrict__ rates,
+                                            uint32_t *__restrict__ status)
+{
+    const double tau = v.sc->tau + (stage == 2 ? v.dtau : 0.0);
+    const double hub = v.milne ? 1.0 / tau : 0.0;  // Gamma^eta_{eta tau}
+    const double sqrtg = v.milne ? tau : 1.0, isqg = v.milne ? hub : 1.0;
+    const double ux = ys[2 * n + a], uy = ys[3 * n + a];
+    const double g = dens[5 * n + a], T = eos[a];
+    const double ig = 1.0 / g, vx = ux * ig, vy = uy * ig;
+    const uint32_t st_in = status[a];
+    double f[kJRow];
+    if ((st_in & (PST_NOCONV | PST_NONFINITE)) || (v.tr.T_stop_GeV > 0.0 && T * kHbarc < v.tr.T_stop_GeV)) {
+        // no EoS solution, or below the stop temperature: ballistic motion only
+        f[0] = vx;
+        f[1] = vy;
+#pragma unroll
+        for (int k = 2; k < kJRow; ++k) f[k] = 0.0;
+        heun_store(v.dtau, mode, kJRow, n, a, f, ys, yout, rates);
+        const double dN0[3] = {0.0, 0.0, 0.0};  // frozen: the charges stay as they are
+        heun_charges(v, mode, n, a, dN0);
+        return;
+    }
+    const double sig_star = dens[a], s = dens[n + a];
+    const double p = eos[4 * n + a], e = eos[5 * n + a], ps = eos[6 * n + a];
+    const double m0 = eos[n + a] + eos[7 * n + a], m1 = eos[2 * n + a] + eos[8 * n + a], m2 = eos[3 * n + a] + eos[9 * n + a];
+    const double Q = m0 * dens[2 * n + a] + m1 * dens[3 * n + a] + m2 * dens[4 * n + a];
+    const double dxux = gout[a], dxuy = gout[n + a], dyux = gout[2 * n + a], dyuy = gout[3 * n + a];
+    double Fx = gout[4 * n + a], Fy = gout[5 * n + a];
+    const double isig = 1.0 / sig_star, sigma = sig_star * ig * isqg, isg = g * sqrtg * isig;
+    const double ep = e + p, iT = 1.0 / T;
+    // theta: d_k u^0 = v_j d_k u^j
+    const double th0 = dxux + dyuy + g * hub - (vx * (vx * dxux + vy * dxuy) + vy * (vx * dyux + vy * dyuy));
+    double w = ep;
+    double dSc = 0.0, dSx = 0.0, dSy = 0.0, dBc = 0.0, dBx = 0.0, dBy = 0.0;
+    double xxc = 0.0, xxx = 0.0, xxy = 0.0, xyc = 0.0, xyx = 0.0, xyy = 0.0, yyc = 0.0, yyx = 0.0, yyy = 0.0;
+    double Pxx = 0.0, Pxy = 0.0, Pyy = 0.0, Pvx = 0.0, Pvy = 0.0;
+    if (v.tr.viscous) {
+        const double B = ys[5 * n + a];
+        Pxx = ys[6 * n + a];
+        Pxy = ys[7 * n + a];
+        Pyy = ys[8 * n + a];
+        const double Pi = sigma * B;
+        w += Pi;
+        const double third = 1.0 / 3.0;
+        const double cxx = fma(third * ux, ux, third), cxy = third * ux * uy, cyy = fma(third * uy, uy, third);
+        // sigma^{ij} = -(d_i u^j + d_j u^i)/2 - u^0 (u^i a^j + u^j a^i)/2 + (delta^{ij} + u^i u^j) theta/3
+        const double gux = g * ux, guy = g * uy;
+        const double sxxc = fma(cxx, th0, -dxux), sxxx = fma(cxx, vx, -gux), sxxy = cxx * vy;
+        const double sxyc = fma(cxy, th0, -0.5 * (dxuy + dyux)), sxyx = fma(cxy, vx, -0.5 * guy), sxyy = fma(cxy, vy, -0.5 * gux);
+        const double syyc = fma(cyy, th0, -dyuy), syyx = cyy * vx, syyy = fma(cyy, vy, -guy);
+        const double seec = fma(third, th0, -g * hub);  // tau^2 sigma^{eta eta} (z z if Cartesian); {., vx/3, vy/3}
+        Pvx = vx * Pxx + vy * Pxy;  // P^{0i}
+        Pvy = vx * Pxy + vy * Pyy;
+        const double Pvv = vx * Pvx + vy * Pvy;
+        const double Pee = Pvv - Pxx - Pyy;  // tau^2 P^{eta eta}
+        // P:sigma with the 0-components of both tensors written by their spatial ones
+        const double Mxx = fma(vx, fma(vx, Pvv, -2.0 * Pvx), Pxx), Myy = fma(vy, fma(vy, Pvv, -2.0 * Pvy), Pyy);
+        const double Mxy = 2.0 * (fma(vx, fma(vy, Pvv, -Pvy), Pxy) - vy * Pvx);
+        const double kS = ig * iT, Pe3 = third * Pee - B;
+        dSc = kS * (Mxx * sxxc + Mxy * sxyc + Myy * syyc + Pee * seec - B * th0);
+        dSx = kS * (Mxx * sxxx + Mxy * sxyx + Myy * syyx + Pe3 * vx);
+        dSy = kS * (Mxx * sxxy + Mxy * sxyy + Myy * syyy + Pe3 * vy);
+        const double eta = v.tr.eta_over_s * s;
+        const double dTg = T * kHbarc - v.tr.zeta_T_GeV;
+        const double zeta = v.tr.zeta_peak * exp(-dTg * dTg / (2.0 * v.tr.zeta_w_GeV * v.tr.zeta_w_GeV)) * s;
+        // 1/tau_pi = (e + p) / (c eta), tau_pi = c eta / (e + p); tau_Pi = ratio tau_pi
+        const double itp = ep / (v.tr.tau_pi_coef * eta);
+        const double kB = -(ig * isg) * (itp / v.tr.tau_Pi_ratio), kz = kB * zeta;
+        dBc = fma(kz, th0, kB * Pi);
+        dBx = kz * vx;
+        dBy = kz * vy;
+        const double q2 = ig * itp, q1 = 2.0 * eta * q2 * isg, q3 = third * ig;
+        const double ec = fma(q3, th0, q2), ex = q3 * vx, ey = q3 * vy;
+        const double Cxx = Pvx * vx - Pxx, Cxy = Pvx * vy - Pxy, Cyx = Pvy * vx - Pxy, Cyy = Pvy * vy - Pyy;
+        xxc = q1 * sxxc - Pxx * ec;
+        xxx = q1 * sxxx - Pxx * ex - 2.0 * ux * Cxx;
+        xxy = q1 * sxxy - Pxx * ey - 2.0 * ux * Cxy;
+        xyc = q1 * sxyc - Pxy * ec;
+        xyx = q1 * sxyx - Pxy * ex - ux * Cyx - uy * Cxx;
+        xyy = q1 * sxyy - Pxy * ey - ux * Cyy - uy * Cxy;
+        yyc = q1 * syyc - Pyy * ec;
+        yyx = q1 * syyx - Pyy * ex - 2.0 * uy * Cyx;
+        yyy = q1 * syyy - Pyy * ey - 2.0 * uy * Cyy;
+    }
+    double dN[3] = {0.0, 0.0, 0.0}, Dsrc = 0.0;
+    if (v.ntrack > 0 || v.nparton > 0) {
+        // jet tracks (Cartesian) and partons: dP^i/dx0 gains sqrt(-g) I^i/sigma*, dS/dx0 gains
+        // u_nu I^nu/(u^0 sigma T); parton charges: dN_q/dx0 = sqrt(-g) I_q/sigma*, and dS/dx0
+        // gains -mu_q/T dN_q/dx0 (eq. dsdnrewr, R^S_q = -mu_q/T)
+        double I[4] = {0.0, 0.0, 0.0, 0.0}, Ik[4], Iq[3] = {0.0, 0.0, 0.0};
+        if (v.ntrack > 0) {
+            jet_deposit(v, tau, ys[a], ys[n + a], 0.0, Ik);
+            for (int k = 0; k < 4; ++k) I[k] += Ik[k];
+        }
+        if (v.nparton > 0) {
+            const double xa[3] = {ys[a], ys[n + a], 0.0};
+            parton_deposit(v, tau, sqrtg, xa, Ik, Iq);
+            for (int k = 0; k < 4; ++k) I[k] += Ik[k];
+        }
+        Fx += sqrtg * I[1] * isig;
+        Fy += sqrtg * I[2] * isig;
+        // no eta component in 2+1D
+        const double uI = g * I[0] - ux * I[1] - uy * I[2] -
+                          (eos[n + a] * Iq[0] + eos[2 * n + a] * Iq[1] + eos[3 * n + a] * Iq[2]);
+        dSc += (ig * isg * iT) * uI;
+        for (int c = 0; c < 3; ++c) dN[c] = sqrtg * Iq[c] * isig;
+        Dsrc = m0 * dN[0] + m1 * dN[1] + m2 * dN[2];
+    }
+    const double Tps = T + ps, k3 = (isg * ig) * (ep - Tps * s - Q);
+    const double Dc = fma(Tps, dSc, fma(k3, th0, dBc + Dsrc)), Dx = fma(Tps, dSx, fma(k3, vx, dBx)),
+                 Dy = fma(Tps, dSy, fma(k3, vy, dBy));
+    const double W = w * isg, ig2 = ig * ig, hx = 2.0 * Pvx * ig2, hy = 2.0 * Pvy * ig2;
+    const double Axx = W + fma(ux, Dx, ig2 * (Pxx + ux * xxx + uy * xyx)) - hx * vx;
+    const double Axy = fma(ux, Dy, ig2 * (Pxy + ux * xxy + uy * xyy)) - hx * vy;
+    const double Ayx = fma(uy, Dx, ig2 * (Pxy + ux * xyx + uy * yyx)) - hy * vx;
+    const double Ayy = W + fma(uy, Dy, ig2 * (Pyy + ux * xyy + uy * yyy)) - hy * vy;
+    const double r0 = Fx - fma(ux, Dc, ig2 * (ux * xxc + uy * xyc));
+    const double r1 = Fy - fma(uy, Dc, ig2 * (ux * xyc + uy * yyc));
+    const double det = Axx * Ayy - Axy * Ayx;
+    uint32_t st = 0;
+    double acx = 0.0, acy = 0.0;
+    if (isfinite(det) && det != 0.0) {
+        const double idet = 1.0 / det;
+        acx = (r0 * Ayy - Axy * r1) * idet;
+        acy = (Axx * r1 - Ayx * r0) * idet;
+    } else {
+        st |= PST_SOLVE_FAIL;
+    }
+    f[0] = vx;
+    f[1] = vy;
+    f[2] = acx;
+    f[3] = acy;
+    f[4] = fma(dSx, acx, fma(dSy, acy, dSc));
+    f[5] = fma(dBx, acx, fma(dBy, acy, dBc));
+    f[6] = fma(xxx, acx, fma(xxy, acy, xxc));
+    f[7] = fma(xyx, acx, fma(xyy, acy, xyc));
+    f[8] = fma(yyx, acx, fma(yyy, acy, yyc));
+    bool fin = true;
+#pragma unroll
+    for (int k = 0; k < kJRow; ++k) fin = fin && isfinite(f[k]);
+    if (!fin) st |= PST_NONFINITE;
+    if (st) {
+        status[a] = st_in | st;
+        atomicOr(&v.sc->status_or, st);
+    }
+    heun_store(v.dtau, mode, kJRow, n, a, f, ys, yout, rates);
+    heun_charges(v, mode, n, a, dN);
+}
+
+// equations of motion of one particle with DNMR or diffusion (rows n apart): mode 0 writes y1 = y + dt f(y),
 // mode 1 closes Heun in place, mode 2 writes the rates
 __device__ __forceinline__ void eom2_particle(const EvView &v, int stage, int mode, size_t n, size_t a,
                                               const double *__restrict__ ys, const double *__restrict__ dens,
@@ -433,14 +615,17 @@ __device__ __forceinline__ void eom2_particle(const EvView &v, int stage, int mo
     heun_charges(v, mode, n, a, dN);
 }
 
-__global__ void __launch_bounds__(128) k_eom2(EvView v, int stage, int mode, const double *__restrict__ ys,
+// GEN: the general form (DNMR, diffusion), else minimal Israel-Stewart
+template <bool GEN>
+__global__ void __launch_bounds__(GEN ? 128 : 64) k_eom2(EvView v, int stage, int mode, const double *__restrict__ ys,
                                               const double *__restrict__ dens, const double *__restrict__ eos,
                                               const double *__restrict__ gout, double *__restrict__ yout,
                                               double *__restrict__ rates, uint32_t *__restrict__ status)
 {
     int a = blockIdx.x * blockDim.x + threadIdx.x;
     if (a >= v.n) return;
-    eom2_particle(v, stage, mode, (size_t)v.n, (size_t)a, ys, dens, eos, gout, yout, rates, status);
+    if (GEN) eom2_particle(v, stage, mode, (size_t)v.n, (size_t)a, ys, dens, eos, gout, yout, rates, status);
+    else eom2_min_is(v, stage, mode, (size_t)v.n, (size_t)a, ys, dens, eos, gout, yout, rates, status);
 }
 
 // Serving form: the equations of motion over the segmented arena (persistent grid)
@@ -453,8 +638,8 @@ __global__ void __launch_bounds__(128) k_eom2_seg(Arena A, int stage, int mode, 
         const int s = A.segid[a];
         if (s < 0 || !seg_active(T, s, stage, true) || !in_group(T, s, grp)) continue;
         if (a - T->slots[s].off >= T->slots[s].n) continue;
-        eom2_particle(A.segv[s], stage, mode, (size_t)A.P, (size_t)a, ys, A.dens, A.eosf, A.gout, yout, nullptr,
-                      A.status);
+        eom2_min_is(A.segv[s], stage, mode, (size_t)A.P, (size_t)a, ys, A.dens, A.eosf, A.gout, yout, nullptr,
+                    A.status);
     }
 }
 
@@ -566,7 +751,10 @@ void launch_eom(const EvView &v, int stage, int mode, const double *ys, const do
         launch_eom3(v, stage, mode, ys, dens, eos, gout, yout, rates, status, st);
         return;
     }
-    k_eom2<<<nblk(v.n, 128), 128, 0, st>>>(v, stage, mode, ys, dens, eos, gout, yout, rates, status);
+    if (v.diff || v.tr.model != 0)
+        k_eom2<true><<<nblk(v.n, 128), 128, 0, st>>>(v, stage, mode, ys, dens, eos, gout, yout, rates, status);
+    else
+        k_eom2<false><<<nblk(v.n, 64), 64, 0, st>>>(v, stage, mode, ys, dens, eos, gout, yout, rates, status);
 }
 
 void launch_eom2_seg(const Arena &A, int stage, int mode, const double *ys, double *yout, int grid,

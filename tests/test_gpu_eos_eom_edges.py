@@ -1,5 +1,6 @@
 """The EoS search and finish kernels over the whole range of densities (below, inside, at the edges of
-and above the table; cold and warm starts; block remainders), against the oracle."""
+and above the table; cold and warm starts; block remainders), and the minimal Israel-Stewart equations
+of motion at random viscous states, against the oracle."""
 import numpy as np
 import pytest
 
@@ -49,4 +50,27 @@ def test_eos_over_the_density_range(form, n):
             assert np.max(np.abs(f[k] - v)) <= TOL * np.max(np.abs(v)), k
         mu = aux[A["muB"]:A["muQ"] + 1]
         assert np.max(np.abs(f["MU"] - mu)) <= TOL * max(np.max(np.abs(mu)), 1e-300)
+    g.free()
+
+
+@pytest.mark.parametrize("dim,milne", [(2, True), (2, False), (3, True), (3, False)])
+@pytest.mark.parametrize("n", [1, 64, 321])
+def test_rates_of_random_viscous_states(dim, milne, n):
+    if dim == 2:
+        ev = I.smooth_blob_2p1(half_width=0.1, with_table=False, eos=I.CAUSAL_EOS)
+        ev.milne = milne
+    else:
+        ev = I.smooth_blob_3d(milne=milne, half_widths=(0.16, 0.16, 0.12), with_table=False, eos=I.CAUSAL_EOS)
+    npi = 3 if dim == 2 else 5
+    ev.x = I.random_points(n, dim, 0.5, 41)
+    ev.u = I.random_points(n, dim, 0.8, 42)
+    ev.S = 0.05 + 0.1 * I.uniform01(43, n)
+    ev.Nq = 0.02 * (2.0 * I.uniform01(44, 3 * n).reshape(3, n) - 1.0) * ev.S
+    ev.Bv = 0.02 * (2.0 * I.uniform01(45, n) - 1.0)
+    ev.Pv = 0.02 * (2.0 * I.uniform01(46, npi * n).reshape(npi, n) - 1.0)
+    g = Bd.GpuEvent(ev)
+    rates, _ = g.rates()
+    want = O.OracleRun.start(ev).stage()[0]
+    for k in range(want.shape[0]):
+        assert np.max(np.abs(rates[k] - want[k])) <= TOL * max(np.max(np.abs(want[k])), 1e-300), k
     g.free()
