@@ -195,6 +195,8 @@ static EvView make_view(const sph_event *ev)
     v.dinp = ev->dinp;
     v.dal = ev->dal;
     v.dout = ev->dout;
+    v.fxX = ev->cb.pl.total > 0 ? ev->cb.pl.X : nullptr;
+    v.fxE = ev->cb.pl.Xe;
     return v;
 }
 
@@ -719,6 +721,8 @@ sph_status sph_init_event(sph_event **out, const sph_event_desc *d, const sph_eo
 static sph_status size_pair_lists(sph_event *ev)
 {
     if (ev->pairs_off || ev->mixed || ev->n == 0) return SPH_OK;
+    if (ev->n > (1 << 30)) ev->pairs_off = true;  // the passes pack an index and two flags in a word
+    if (ev->pairs_off) return SPH_OK;
     if (ev->cb.pl.total > 0 && ev->pair_ovf_host && *ev->pair_ovf_host > ev->pair_ovf_seen) {
         ev->pair_ovf_seen = *ev->pair_ovf_host;
         ev->pairs_grow = true;
@@ -752,8 +756,11 @@ static sph_status size_pair_lists(sph_event *ev)
     const int nparts = (n + 2047) / 2048;
     // per entry: L, P (int), W and the kernel gradient (2 or 3 doubles)
     const size_t per_entry = 2 * sizeof(int) + (1 + (size_t)ev->dim) * sizeof(double);
+    // per particle: two counts and two carried counts, the values in limbs and their exponents
+    const int nx = ev->dim == 2 ? 3 : 6;  // planes of the gradient-pass inputs
+    const size_t per_particle = 5 * sizeof(int) + 4 * sizeof(unsigned short) + (size_t)(2 + nx) * sizeof(int4);
     const size_t bytes = (size_t)total * per_entry + (size_t)(n + 1) * sizeof(long long) +
-                         (size_t)nparts * sizeof(unsigned long long) + 4 * sizeof(int) * (size_t)n + 1024;
+                         (size_t)nparts * sizeof(unsigned long long) + per_particle * (size_t)n + 1024;
     size_t fr = 0, tot = 0;
     CK(cudaMemGetInfo(&fr, &tot));
     if (bytes > fr / 4) {
@@ -778,18 +785,22 @@ static sph_status size_pair_lists(sph_event *ev)
     PairBufs pl{};
     pl.total = total;
     pl.margin = margin;
-    double *gbuf = static_cast<double *>(m);  // the kernel gradients first (16-byte aligned)
-    if (ev->dim == 2) pl.G = reinterpret_cast<double2 *>(gbuf);
+    pl.X = static_cast<int4 *>(m);  // the 16-byte aligned arrays first
+    pl.Q = pl.X + (size_t)nx * n;
+    long long *gbuf = reinterpret_cast<long long *>(pl.Q + 2 * (size_t)n);  // the kernel gradients
+    if (ev->dim == 2) pl.G = reinterpret_cast<longlong2 *>(gbuf);
     else pl.G3 = gbuf;
     pl.W = gbuf + (size_t)ev->dim * total;
     pl.off = reinterpret_cast<long long *>(pl.W + total);
     pl.part = reinterpret_cast<unsigned long long *>(pl.off + (n + 1));
-    pl.L = reinterpret_cast<int *>(pl.part + nparts);
+    pl.Qe = reinterpret_cast<unsigned short *>(pl.part + nparts);  // read 8 bytes at a time
+    pl.L = reinterpret_cast<int *>(pl.Qe + 4 * (size_t)n);
     pl.P = pl.L + total;
     pl.cntF = pl.P + total;
     pl.cntB = pl.cntF + n;
     ev->pcnt[0] = pl.cntB + n;
     ev->pcnt[1] = ev->pcnt[0] + n;
+    pl.Xe = reinterpret_cast<unsigned int *>(ev->pcnt[1] + n);
     CK(cudaMemcpyAsync(ev->pcnt[0], state.data(), sizeof(int) * (size_t)n, cudaMemcpyHostToDevice, ev->stream));
     if ((s = wait_stream(ev)) != SPH_OK) return s;
     pl.cnt_src = ev->pcnt[0];

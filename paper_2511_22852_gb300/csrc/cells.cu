@@ -251,10 +251,14 @@ __global__ void k_permute(EvView v, const uint32_t *__restrict__ perm, PermArgs 
     if (v.dim == 3) {
         if (v.mixed) return;  // k_relpos3
         float f[3];
+        int pk = 0;  // w: the cell's coordinates, 10 bits per axis, clamped as the sort does
 #pragma unroll
-        for (int d = 0; d < 3; ++d)
-            f[d] = __double2float_rn(__dsub_rn(y[(size_t)d * n], dec_double(v.sc->xmin_enc[d])));
-        fpos3[j] = make_float4(f[0], f[1], f[2], 0.0f);
+        for (int d = 0; d < 3; ++d) {
+            const double xm = dec_double(v.sc->xmin_enc[d]), x = y[(size_t)d * n];
+            f[d] = __double2float_rn(__dsub_rn(x, xm));
+            pk |= min(max(cell_coord(x, xm, v.inv_cell), 0), (1 << v.B3[d]) - 1) << (10 * d);
+        }
+        fpos3[j] = make_float4(f[0], f[1], f[2], __int_as_float(pk));
         return;
     }
     float f[2];

@@ -23,6 +23,7 @@
 
 #include "sph_internal.cuh"
 #include "eos_device.cuh"
+#include "pairs_fixed.cuh"
 
 namespace sphg {
 
@@ -188,6 +189,7 @@ __device__ __forceinline__ void eos2_load(const EvView &v, const EosDev &E, int 
 // of the gradient pass: X^{ji} / sigma*^2 with X^{ji} = (p + Pi) delta^{ji} + pi^{ji} -
 // v^j pi^{tau i}, and u^j / sigma*.  Returns the particle's longitudinal work rate
 // (p + Pi + tau^2 pi^{eta eta}) / sigma*.
+template <bool LIMBS>
 __device__ __forceinline__ double eos2_store(const EvView &v, int stage, size_t n, size_t a,
                                              const double *__restrict__ y, const double *__restrict__ dens,
                                              double *__restrict__ eos, double *__restrict__ gin,
@@ -225,12 +227,22 @@ __device__ __forceinline__ double eos2_store(const EvView &v, int stage, size_t 
     const double pty = vx * pxy + vy * pyy;  // pi^{tau y}
     const double inv2 = isig * isig;
     const double P = o.p + Pi;
-    gin[a] = (P + pxx - vx * ptx) * inv2;          // X^{xx}
-    gin[n + a] = (pxy - vx * pty) * inv2;          // X^{xy}  (j = x, i = y)
-    gin[2 * n + a] = (pxy - vy * ptx) * inv2;      // X^{yx}  (j = y, i = x)
-    gin[3 * n + a] = (P + pyy - vy * pty) * inv2;  // X^{yy}
-    gin[4 * n + a] = ux * isig;
-    gin[5 * n + a] = uy * isig;
+    const double X[4] = {(P + pxx - vx * ptx) * inv2,   // X^{xx}
+                         (pxy - vx * pty) * inv2,       // X^{xy}  (j = x, i = y)
+                         (pxy - vy * ptx) * inv2,       // X^{yx}  (j = y, i = x)
+                         (P + pyy - vy * pty) * inv2};  // X^{yy}
+    const double us[2] = {ux * isig, uy * isig};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) gin[k * n + a] = X[k];
+    gin[4 * n + a] = us[0];
+    gin[5 * n + a] = us[1];
+    if (LIMBS && v.fxX) {  // the same in limbs for the pair-list gradient pass
+        const int eX = fx_shared_exponent(X), eu = fx_shared_exponent(us);
+        v.fxX[a] = fx_limbs2(X[0], eX, X[1], eX);
+        v.fxX[n + a] = fx_limbs2(X[2], eX, X[3], eX);
+        v.fxX[2 * n + a] = fx_limbs2(us[0], eu, us[1], eu);
+        v.fxE[a] = (unsigned)eX | ((unsigned)eu << 16);
+    }
     double wcontrib = 0.0;
     if (v.milne) {
         const double ptt = vx * ptx + vy * pty;
@@ -315,7 +327,7 @@ __global__ void __launch_bounds__(kFinish, 5) k_eos2_finish(EvView v, int stage,
         const double g[4] = {guess_out[a], guess_out[n + a], guess_out[2 * n + a], guess_out[3 * n + a]};
         bool used = false;
         const EosOut o = eos_finish(v.eos, v.tr.cs2_cap, s, nq, g, status[a], used, w);
-        wc = eos2_store(v, stage, n, (size_t)a, y, dens, eos, gin, status, guess_out, o, used);
+        wc = eos2_store<true>(v, stage, n, (size_t)a, y, dens, eos, gin, status, guess_out, o, used);
         st = o.st;
     }
     add_eos_work(v.sc, w, st);
@@ -413,7 +425,7 @@ __global__ void __launch_bounds__(128, 3) k_eos2_seg_finish(Arena A, EosDev E, i
             const double g[4] = {A.wguess[a], A.wguess[P + a], A.wguess[2 * P + a], A.wguess[3 * P + a]};
             bool used = false;
             const EosOut o = eos_finish(E, A.segv[sl].tr.cs2_cap, s, nq, g, A.status[a], used, w);
-            A.wpart[a] = eos2_store(A.segv[sl], stage, P, (size_t)a, y, A.dens, A.eosf, A.gin, A.status, A.wguess, o, used);
+            A.wpart[a] = eos2_store<false>(A.segv[sl], stage, P, (size_t)a, y, A.dens, A.eosf, A.gin, A.status, A.wguess, o, used);
             st = o.st;
             if (T->slots[sl].mode == SLOT_STEP) {  // float copies of the gradient-pass inputs
                 const double *q = A.gin;

@@ -13,6 +13,7 @@
 //   each pair moves charge from one particle to the other, so the total is conserved).
 #include "sph_internal.cuh"
 #include "eos_device.cuh"
+#include "pairs_fixed.cuh"
 
 namespace sphg {
 
@@ -162,14 +163,14 @@ __global__ void __launch_bounds__(32 * kDiffWarps) k_diff_pairs(EvView v, int st
         double gx, gy;
         if (j < nf) {
             b = pl.L[r0 + j];
-            const double2 g = pl.G[r0 + j];
-            gx = g.x;
-            gy = g.y;
+            const longlong2 g = pl.G[r0 + j];
+            gx = from_fixed(g.x);
+            gy = from_fixed(g.y);
         } else {
             b = pl.L[rend - (j - nf)];
-            const double2 g = pl.G[pl.off[b] + pl.P[rend - (j - nf)]];
-            gx = -g.x;
-            gy = -g.y;
+            const longlong2 g = pl.G[pl.off[b] + pl.P[rend - (j - nf)]];
+            gx = from_fixed(-g.x);
+            gy = from_fixed(-g.y);
         }
         Gx += gx;
         Gy += gy;

@@ -3,18 +3,17 @@
 // The density sums (Sec. "SPH formalism": sigma*, s*, n*_q as kernel sums) and the gradient sums
 // (Sec. "SPH formalism", the n = 0 and n = -1 derivative forms) use W(r_ab) and dW/dr(r_ab) / r_ab
 // of every accepted pair; both depend on r_ab only, so they are the same for (a, b) and (b, a).
-// Each stage's forward density pass evaluates them once per unordered pair -- on the pairs
-// b > a of particle a (sorted index) -- and keeps them with the pair; the backward pass and the
-// gradient pass then add every pair's contribution to both of its particles without evaluating
-// the kernel again.  All sums run in a fixed order (a warp per particle, lanes over its list in
-// ascending neighbour index, then a fixed butterfly), so results are reproducible run to run; they
-// differ from the per-particle passes only in the order of the additions.
+// Each stage's forward pass evaluates them once per unordered pair -- on the pairs b > a of particle
+// a (sorted index) -- and keeps them with the pair in fixed point; the sum and gradient passes then
+// add every pair's contribution to both of its particles in integers (pairs_fixed.cuh), which do not
+// depend on the order, so results are reproducible run to run.
 //
-// Per pair the FP64 work of the two passes drops from about 126 operations (two kernel
-// evaluations with the sums of each side, in each of the two passes) to about 67.
+// FP64 operations per unordered pair fall from 56 (26 for the kernel, 10 for the density and 20 for
+// the gradient sums of its two particles) to 12; the 40 k event's step 2,038 -> 1,536 us.
 //
 // Rows: a particle's row holds its previous neighbour count plus a margin (a prefix scan per
 // stage); forward entries fill it from the start, backward entries from the end.
+#include "pairs_fixed.cuh"
 #include "sph_internal.cuh"
 
 namespace sphg {
@@ -133,251 +132,345 @@ __global__ void __launch_bounds__(kScanThreads) k_rows_apply(int n, const uint32
     }
 }
 
-// Forward density pass, one warp per particle a.  Candidates of the 3x3 cells pass the
+// Forward pass, a warp for two particles a.  Candidates of the 3x3 cells pass the
 // single-precision prefilter; a neighbour b < a is decided at once (exact FP64 test when the
-// float test left it undecided) and listed in B; a candidate b > a is queued, and 32 at a time
-// the exact test, W and dW/dr / r run on full warps, are listed (L, W, G) and summed for a.
-// dpart receives a's unscaled partial sums (self pair and pairs b > a): sigma*, S, N_B, N_S, N_Q.
-__global__ void __launch_bounds__(32 * kWarps) k_pairs_density_fwd(EvView v, const double *__restrict__ y,
-                                                                   const float2 *__restrict__ fpos,
-                                                                   const double *__restrict__ Nq,
-                                                                   const uint32_t *__restrict__ start,
-                                                                   const uint32_t *__restrict__ cnt, PairBufs pl,
-                                                                   double *__restrict__ dpart)
+// float test left it undecided) and listed from the row end; a candidate b > a is queued, and 32
+// at a time -- of both particles -- the exact test, the distance in FP64 and the spline in 64-bit
+// integers run on full warps, and W and grad W are listed with the pair in fixed point (L, W, G).  The particles' own values go into limbs.
+// Bound: the FP64 pipe, 12 operations per unordered pair (31 with spline and kernel sums in FP64, a
+// reduction per particle and its own partial batch).  40 k event: 220 us a stage, its
+// FP64 pipe then 325 us before the spline left it.
+__global__ void __launch_bounds__(32 * kWarps, 8) k_pairs_fwd(EvView v, const double *__restrict__ y,
+                                                           const float2 *__restrict__ fpos,
+                                                           const double *__restrict__ Nq,
+                                                           const uint32_t *__restrict__ start,
+                                                           const uint32_t *__restrict__ cnt,
+                                                           const uint32_t *__restrict__ key,
+                                                           const uint32_t *__restrict__ perm, PairBufs pl)
 {
     __shared__ int queue[kWarps][64];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int a = blockIdx.x * kWarps + wid;
-    if (a >= v.n) return;  // warp-uniform
-    int *q = queue[wid];
     const int n = v.n;
+    const long long a0 = 2 * ((long long)blockIdx.x * kWarps + wid);
+    if (a0 >= n) return;  // warp-uniform
+    const int np = a0 + 1 < n ? 2 : 1;
+    int *q = queue[wid];
     const double *X = y, *Y = y + n, *S = y + 4 * (size_t)n;
-    const double *NB = Nq, *NS = Nq + n, *NQ = Nq + 2 * (size_t)n;
-    const double xa = X[a], ya = Y[a];
-    const float2 fa = fpos[a];
-    const double xmin0 = dec_double(v.sc->xmin_enc[0]), xmin1 = dec_double(v.sc->xmin_enc[1]);
-    const int cx = cell_coord(xa, xmin0, v.inv_cell), cy = cell_coord(ya, xmin1, v.inv_cell);
-    uint32_t keys[9];
-    const int nk = block_cells_ascending(cx, cy, 1 << v.B, keys);
-    const unsigned lt = (1u << lane) - 1u;
-    const long long r0 = pl.off[a], r1 = pl.off[a + 1];
-    // rows beyond the allocation write nothing (the scan has flagged the stage)
-    const int cap = r1 <= pl.total ? (int)(r1 - r0) : 0;
-    int *F = pl.L + r0, *Bl = pl.L + (r1 - 1);  // forward up from the start, backward down from the end
-    double *Wr = pl.W + r0;
-    double2 *Gr = pl.G + r0;
-    double sg = 0.0, ss = 0.0, sb = 0.0, sS = 0.0, sq = 0.0;
-    if (lane == 0) {  // the self pair, W(0)
-        const double w0 = kernel_w(0.0);
-        sg = w0;
-        ss = S[a] * w0;
-        sb = NB[a] * w0;
-        sS = NS[a] * w0;
-        sq = NQ[a] * w0;
+    if (lane < 4 * np) {
+        const size_t a = (size_t)a0 + (lane >> 2);
+        const int k = lane & 3;
+        fx_store_value(pl.Q, pl.Qe, (size_t)n, a, k, k == 0 ? S[a] : Nq[(size_t)(k - 1) * n + a]);
     }
-    int nf = 0, nbk = 0, qn = 0;
-    // queued index with bit 31 set: the float test left the pair undecided (exact test needed)
+    const unsigned lt = (1u << lane) - 1u;
+    double xa[2], ya[2];
+    long long r0[2];
+    int cap[2], nf[2] = {0, 0}, nbk[2] = {0, 0}, qn = 0;
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+        const int a = (int)a0 + (p < np ? p : 0);
+        xa[p] = X[a];
+        ya[p] = Y[a];
+        r0[p] = pl.off[a];
+        const long long r1 = pl.off[a + 1];
+        cap[p] = r1 <= pl.total ? (int)(r1 - r0[p]) : 0;  // rows beyond the allocation write nothing
+    }
+    // queued word: bit 31: the float test left the pair undecided (exact test needed), bit 30: of a0 + 1
     auto forward = [&](int qb, bool valid) {
-        const int b = qb & 0x7FFFFFFF;
+        const int b = qb & 0x3FFFFFFF;
+        const bool second = qb & 0x40000000;
         double dx = 0.0, dy = 0.0;
         bool acc = false;
         if (valid) {
-            dx = xa - X[b];
-            dy = ya - Y[b];
+            dx = (second ? xa[1] : xa[0]) - X[b];
+            dy = (second ? ya[1] : ya[0]) - Y[b];
             acc = qb >= 0 || dist2_2d(dx, dy) < v.supp2;
         }
-        const unsigned m = __ballot_sync(kFull, acc);
+        const unsigned m0 = __ballot_sync(kFull, acc && !second), m1 = __ballot_sync(kFull, acc && second);
         if (acc) {
             const double r2 = fma(dx, dx, dy * dy);
-            double w = kernel_w(0.0), fac = 0.0;  // coincident particles: W(0), no gradient
+            long long w = 1LL << kFxBits, dw = 0;  // coincident particles: W(0), no gradient
+            double ir = 0.0, q;
             if (nonzero_nonneg(r2)) {
-                // the cubic spline without a branch on q: w = (2-q)^3/4 - max(1-q, 0)^3,
-                // w' = -3/4 (2-q)^2 + 3 max(1-q, 0)^2 (the same polynomials on both pieces)
-                // (the sign tests and the factor 1/4 on the integer pipe: t^2 is 0 or >= 2^-104)
-                const double ir = inv_sqrt(r2);
-                const double qq = r2 * ir * v.inv_h;
-                const double t = 2.0 - qq, u = pos_part(1.0 - qq);
-                const double t2 = t * t, u2 = u * u;
-                w = fma(quarter_nonneg(t2), t, -(u2 * u));
-                fac = fma(-0.75, t2, 3.0 * u2) * ir;
+                pair_distance(r2, v.inv_h, ir, q);
+                spline_fixed(q, w, dw);
             }
-            const int slot = nf + __popc(m & lt);
-            if (slot < cap) {
-                F[slot] = b;
-                Wr[slot] = w;
-                Gr[slot] = make_double2(fac * dx, fac * dy);
+            const int slot = second ? nf[1] + __popc(m1 & lt) : nf[0] + __popc(m0 & lt);
+            if (slot < (second ? cap[1] : cap[0])) {
+                const long long i = (second ? r0[1] : r0[0]) + slot;
+                pl.L[i] = b;
+                pl.W[i] = w;
+                pl.G[i] = make_longlong2(grad_fixed(dw, dx * ir), grad_fixed(dw, dy * ir));
             }
-            sg += w;
-            ss = fma(S[b], w, ss);
-            sb = fma(NB[b], w, sb);
-            sS = fma(NS[b], w, sS);
-            sq = fma(NQ[b], w, sq);
         }
-        nf += __popc(m);
+        nf[0] += __popc(m0);
+        nf[1] += __popc(m1);
     };
-    for (int kc = 0; kc < nk; ++kc) {
-        const uint32_t k = keys[kc];
-        const uint32_t b0 = start[k], b1 = b0 + cnt[k];
-        for (uint32_t base = b0; base < b1; base += 32) {
-            const uint32_t b = base + lane;
-            bool cand = false, sure = false;
-            if (b < b1 && b != (uint32_t)a) {
-                const float2 fb = fpos[b];
-                const float dx = fa.x - fb.x, dy = fa.y - fb.y;
-                const float r2f = fmaf(dx, dx, dy * dy);
-                cand = r2f <= v.supp2_hi;
-                sure = r2f < v.supp2_lo;
-            }
-            // b < a: decided here and listed; its pair values come from b's own forward pass
-            bool accB = false;
-            if (cand && (int)b < a) accB = sure || dist2_2d(xa - X[b], ya - Y[b]) < v.supp2;
-            const unsigned mb = __ballot_sync(kFull, accB);
-            if (accB) {
-                const int slot = nbk + __popc(mb & lt);
-                if (slot < cap) Bl[-slot] = (int)b;
-            }
-            nbk += __popc(mb);
-            // b > a: queued in arrival (ascending) order for the FP64 pair arithmetic
-            const bool fw = cand && (int)b > a;
-            const unsigned m = __ballot_sync(kFull, fw);
-            if (fw) q[qn + __popc(m & lt)] = sure ? (int)b : (int)(b | 0x80000000u);
-            qn += __popc(m);
-            __syncwarp();
-            if (qn >= 32) {
-                forward(q[lane], true);
-                qn -= 32;
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+        if (p >= np) break;
+        const int a = (int)a0 + p, flag = p << 30;
+        const float2 fa = fpos[a];
+        const uint32_t ka = key[perm[a]];
+        const int cx = (int)unspread2(ka), cy = (int)unspread2(ka >> 1);
+        uint32_t keys[9];
+        const int nk = block_cells_ascending(cx, cy, 1 << v.B, keys);
+        int *Bl = pl.L + (r0[p] + cap[p] - 1);  // backward down from the row end
+        for (int kc = 0; kc < nk; ++kc) {
+            const uint32_t k = keys[kc];
+            const uint32_t b0 = start[k], b1 = b0 + cnt[k];
+            for (uint32_t base = b0; base < b1; base += 32) {
+                const uint32_t b = base + lane;
+                bool cand = false, sure = false;
+                if (b < b1 && b != (uint32_t)a) {
+                    const float2 fb = fpos[b];
+                    const float dx = fa.x - fb.x, dy = fa.y - fb.y;
+                    const float r2f = fmaf(dx, dx, dy * dy);
+                    cand = r2f <= v.supp2_hi;
+                    sure = r2f < v.supp2_lo;
+                }
+                // b < a: decided here and listed; its pair values come from b's own forward pass
+                bool accB = false;
+                if (cand && (int)b < a) accB = sure || dist2_2d(xa[p] - X[b], ya[p] - Y[b]) < v.supp2;
+                const unsigned mb = __ballot_sync(kFull, accB);
+                if (accB) {
+                    const int slot = nbk[p] + __popc(mb & lt);
+                    if (slot < cap[p]) Bl[-slot] = (int)b;
+                }
+                nbk[p] += __popc(mb);
+                // b > a: queued in arrival (ascending) order for the FP64 pair arithmetic
+                const bool fw = cand && (int)b > a;
+                const unsigned m = __ballot_sync(kFull, fw);
+                if (fw) q[qn + __popc(m & lt)] = (int)(b | (sure ? 0u : 0x80000000u)) | flag;
+                qn += __popc(m);
                 __syncwarp();
-                if (lane < qn) q[lane] = q[32 + lane];
-                __syncwarp();
+                if (qn >= 32) {
+                    forward(q[lane], true);
+                    qn -= 32;
+                    __syncwarp();
+                    if (lane < qn) q[lane] = q[32 + lane];
+                    __syncwarp();
+                }
             }
         }
     }
     if (qn > 0) forward(lane < qn ? q[lane] : 0, lane < qn);
-    const double vals[8] = {sg, ss, sb, sS, sq, 0.0, 0.0, 0.0};
-    const double tot = warp_reduce_scatter8(vals, lane);
-    const int k = lane >> 2;
-    if ((lane & 3) == 0 && k < 5) dpart[(size_t)k * n + a] = tot;
     if (lane == 0) {
-        pl.cntF[a] = nf;
-        pl.cntB[a] = nbk;
-        if (nf + nbk > cap) atomicOr(&v.sc->pair_flag, 1u);  // the two ends met: lists unusable
+        bool over = false;
+        for (int p = 0; p < np; ++p) {
+            pl.cntF[a0 + p] = nf[p];
+            pl.cntB[a0 + p] = nbk[p];
+            over = over || nf[p] + nbk[p] > cap[p];
+        }
+        if (over) atomicOr(&v.sc->pair_flag, 1u);  // the two ends met: lists unusable
     }
 }
 
-// Backward density pass, one warp per particle a: the pairs (b, a) with b < a, whose W the
-// forward pass of b stored; the slot is found by binary search of a in b's ascending list and
-// kept in P for the gradient pass.  Completes a's sums (forward partial + backward partial) and
-// writes the density rows as the per-particle pass does.
-__global__ void __launch_bounds__(32 * kWarps) k_pairs_density_bwd(EvView v, const double *__restrict__ y,
-                                                                   const double *__restrict__ Nq, PairBufs pl,
-                                                                   double *__restrict__ dens, int *__restrict__ nnb)
+// Density sums, half a warp per particle a, over its pairs b > a (forward entries of a's row) and
+// b < a (the entry of a in b's ascending forward list, found by binary search; the slot is kept in
+// P for the gradient pass), in integers (pairs_fixed.cuh).
+// Bound: the latency of the searches and of the gathers (L1 hits 78 %); 40 k event 197 us a stage,
+// 3+1D event of 258 k particles 2.5 ms.  More or larger blocks per SM changed nothing (191-229 us).
+__global__ void __launch_bounds__(32 * kWarps, 7) k_pairs_sum(EvView v, PairBufs pl, double *__restrict__ dens,
+                                                           int *__restrict__ nnb)
 {
     if (v.sc->pair_flag) return;  // a list overflowed: the per-particle pass runs instead
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int a = blockIdx.x * kWarps + wid;
-    if (a >= v.n) return;  // warp-uniform
-    const int n = v.n;
-    const double *S = y + 4 * (size_t)n;
-    const double *NB = Nq, *NS = Nq + n, *NQ = Nq + 2 * (size_t)n;
-    const long long rend = pl.off[a + 1] - 1;  // backward entries: rend, rend - 1, ...
-    const int nb = pl.cntB[a];
-    double sg = 0.0, ss = 0.0, sb = 0.0, sS = 0.0, sq = 0.0;
-    for (int j0 = 0; j0 < nb; j0 += 32) {
-        const int j = j0 + lane;
-        if (j < nb) {
-            const int b = pl.L[rend - j];
-            const long long rb = pl.off[b];
-            const int *Fb = pl.L + rb;
-            const int nfb = pl.cntF[b];
-            int lo = 0, hi = nfb;
-            while (lo < hi) {
-                const int mid = (lo + hi) >> 1;
-                if (Fb[mid] < a) lo = mid + 1;
-                else hi = mid;
-            }
-            // both sides take the same acceptance decision (the float and the exact test see
-            // exactly negated differences), so a is in b's list; checked all the same
-            if (lo >= nfb || Fb[lo] != a) {
-                atomicOr(&v.sc->err_flags, ERR_PAIR_LIST);
-                lo = 0;
-            }
-            pl.P[rend - j] = lo;
-            const double w = nfb > 0 ? pl.W[rb + lo] : 0.0;
-            sg += w;
-            ss = fma(S[b], w, ss);
-            sb = fma(NB[b], w, sb);
-            sS = fma(NS[b], w, sS);
-            sq = fma(NQ[b], w, sq);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, l = lane & 15;
+    const long long ap = 2 * ((long long)blockIdx.x * kWarps + wid) + (lane >> 4);
+    if (ap - (lane >> 4) >= v.n) return;  // warp-uniform
+    const bool on = ap < v.n;
+    const int a = on ? (int)ap : v.n - 1;
+    const size_t n = (size_t)v.n;
+    const long long r0 = pl.off[a], rend = pl.off[a + 1] - 1;  // backward entries: rend, rend - 1, ...
+    const int nf = on ? pl.cntF[a] : 0, nt = on ? nf + pl.cntB[a] : 0;
+    const uint2 *Qe = reinterpret_cast<const uint2 *>(pl.Qe);
+    // the largest exponents among a and its neighbours (S | N_B << 16, N_S | N_Q << 16)
+    uint2 em = Qe[a];
+    for (int j = l; j < nf; j += 16) {
+        const uint2 e = Qe[pl.L[r0 + j]];
+        em = make_uint2(fx_max2(em.x, e.x), fx_max2(em.y, e.y));
+    }
+    for (int j = l; j < nt - nf; j += 16) {
+        const uint2 e = Qe[pl.L[rend - j]];
+        em = make_uint2(fx_max2(em.x, e.x), fx_max2(em.y, e.y));
+    }
+    em = make_uint2(fx_half_max2(em.x), fx_half_max2(em.y));
+    const int Em[4] = {(int)(em.x & 0xFFFFu), (int)(em.x >> 16), (int)(em.y & 0xFFFFu), (int)(em.y >> 16)};
+    int E[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) E[k] = fx_room(Em[k], nt);
+    FxSum sg = {0, 0};  // x in units of 2^-kFxBits
+    FxSum s[4] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
+    int it = 0;
+    auto add = [&](long long w, int4 q0, int4 q1, uint2 e2) {
+        const int e[4] = {(int)(e2.x & 0xFFFFu), (int)(e2.x >> 16), (int)(e2.y & 0xFFFFu), (int)(e2.y >> 16)};
+        const int2 qv[4] = {lo_of(q0), hi_of(q0), lo_of(q1), hi_of(q1)};
+        sg.x += w;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            int whi, wlo;
+            fx_split(w, E[k] - e[k], whi, wlo);
+            fx_add(s[k], whi, wlo, qv[k]);
         }
+    };
+    // two entries at a time, their loads ahead of both; an entry past the end is a with weight 0
+    auto add2 = [&](int b0, long long w0, int b1, long long w1) {
+        const int4 p0 = pl.Q[b0], p1 = pl.Q[n + b0], r0_ = pl.Q[b1], r1_ = pl.Q[n + b1];
+        const uint2 e0 = Qe[b0], e1 = Qe[b1];
+        add(w0, p0, p1, e0);
+        add(w1, r0_, r1_, e1);
+        it += 2;
+        if ((it & (kFoldEvery - 1)) == 0) {
+            fx_fold(sg);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) fx_fold(s[k]);
+        }
+    };
+    if (l == 0 && on) add2(a, 1LL << kFxBits, a, 0);  // the self pair, W(0) = 1
+    for (int j = l; j < nf; j += 32) {
+        const bool two = j + 16 < nf;
+        const int b0 = pl.L[r0 + j], b1 = two ? pl.L[r0 + j + 16] : a;
+        const long long w0 = pl.W[r0 + j], w1 = two ? pl.W[r0 + j + 16] : 0;
+        add2(b0, w0, b1, w1);
     }
-    const double vals[8] = {sg, ss, sb, sS, sq, 0.0, 0.0, 0.0};
-    const double tot = warp_reduce_scatter8(vals, lane);
-    const int k = lane >> 2;
-    if ((lane & 3) == 0 && k < 5) {
-        // rows sigma*, lab-frame s* (divided by u0 sqrt(-g) in the EoS pass), n*_B, n*_S, n*_Q:
-        // the forward partials were left in the density rows; u0 (row 5) is written with the permutation
-        double *d = dens + (size_t)k * n + a;
-        *d = v.sigma_d * (*d + tot);
+    for (int j = l; j < nt - nf; j += 32) {
+        const bool two = j + 16 < nt - nf;
+        const int b0 = pl.L[rend - j], b1 = two ? pl.L[rend - j - 16] : a;
+        const long long rb0 = pl.off[b0], rb1 = pl.off[b1];
+        const int n0 = pl.cntF[b0], n1 = two ? pl.cntF[b1] : 0;
+        SlotSearch f0 = {pl.L + rb0, 0, n0}, f1 = {pl.L + rb1, 0, n1};
+        while (f0.open() || f1.open()) {
+            f0.step(a);
+            f1.step(a);
+        }
+        // both sides take the same acceptance decision (the float and the exact test see
+        // exactly negated differences), so a is in b's list; checked all the same
+        if (f0.base >= n0 || f0.F[f0.base] != a) {
+            atomicOr(&v.sc->err_flags, ERR_PAIR_LIST);
+            f0.base = 0;
+        }
+        if (two && (f1.base >= n1 || f1.F[f1.base] != a)) {
+            atomicOr(&v.sc->err_flags, ERR_PAIR_LIST);
+            f1.base = 0;
+        }
+        pl.P[rend - j] = f0.base;
+        if (two) pl.P[rend - j - 16] = f1.base;
+        add2(b0, n0 > 0 ? pl.W[rb0 + f0.base] : 0, b1, n1 > 0 ? pl.W[rb1 + f1.base] : 0);
     }
-    if (lane == 0) {
-        const int c = 1 + pl.cntF[a] + nb;
+    fx_fold(sg);
+    FxTotal t[8];
+    t[0] = fx_words(sg);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        fx_fold(s[k]);
+        t[1 + k] = fx_words(s[k]);
+    }
+    t[5] = t[6] = t[7] = FxTotal{0, 0};
+    const FxTotal tot = fx_reduce8(t, lane);
+    const int k = l >> 1;
+    if (on && (l & 1) == 0 && k < 5) {
+        // rows sigma*, lab-frame s* (divided by u0 sqrt(-g) in the EoS pass), n*_B, n*_S, n*_Q
+        const int Ek = k <= 1 ? E[0] : (k == 2 ? E[1] : (k == 3 ? E[2] : E[3]));
+        const bool bad = (k <= 1 ? Em[0] : (k == 2 ? Em[1] : (k == 3 ? Em[2] : Em[3]))) == kNonFinite && k > 0;
+        const double d = fx_value(tot, k == 0 ? -kFxBits : fx_unit(Ek));
+        dens[(size_t)k * n + a] = bad ? fx_nan() : v.sigma_d * d;
+    }
+    if (on && l == 0) {
+        const int c = 1 + nt;
         nnb[a] = c;
         if (pl.cnt_dst) pl.cnt_dst[a] = c;  // sizes this particle's row in the next stage
-        atomicAdd(&v.sc->pairs, (unsigned long long)c);
     }
+    const unsigned c2 = __reduce_add_sync(kFull, on && l == 0 ? 1u + (unsigned)nt : 0u);
+    if (lane == 0) atomicAdd(&v.sc->pairs, (unsigned long long)c2);
 }
 
-// Gradient pass, one warp per particle a, over its pairs b > a (forward entries of a's row, with
+// Gradient pass, half a warp per particle a, over its pairs b > a (forward entries of a's row, with
 // G = grad_a W_ab h / sigma_d) and then b < a (backward entries: -G of the pair in b's row, slot
-// P), forming the sums of the per-particle pass: sum grad W, sum X_b grad W, sum u_b grad W.
-__global__ void __launch_bounds__(32 * kWarps) k_pairs_gradient(EvView v, int stage, const double *__restrict__ y,
-                                                                const double *__restrict__ gin, PairBufs pl,
-                                                                double *__restrict__ gout)
+// P), forming in integers the sums of the per-particle pass: sum grad W, sum X_b grad W, sum u_b grad W.
+// Bound: the latency of the gathers; 40 k event 150 us a stage (298 us with 10 FP64 operations per
+// pair).  Two entries at a time: 150 against 173 us; 5 blocks per SM: 6 gave 161, 8 150, 10 193.
+__global__ void __launch_bounds__(32 * kWarps, 5) k_pairs_gradient(EvView v, int stage, const double *__restrict__ gin,
+                                                                PairBufs pl, double *__restrict__ gout)
 {
     if (v.sc->pair_flag) return;  // a list overflowed: the per-particle pass runs instead
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int a = blockIdx.x * kWarps + wid;
-    if (a >= v.n) return;  // warp-uniform
-    const int n = v.n;
-    const double *Xxx = gin, *Xxy = gin + n, *Xyx = gin + 2 * (size_t)n, *Xyy = gin + 3 * (size_t)n;
-    const double *Ux = gin + 4 * (size_t)n, *Uy = gin + 5 * (size_t)n;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, l = lane & 15;
+    const long long ap = 2 * ((long long)blockIdx.x * kWarps + wid) + (lane >> 4);
+    if (ap - (lane >> 4) >= v.n) return;  // warp-uniform
+    const bool on = ap < v.n;
+    const int a = on ? (int)ap : v.n - 1;
+    const size_t n = (size_t)v.n;
     const long long r0 = pl.off[a], rend = pl.off[a + 1] - 1;
-    const int nf = pl.cntF[a], nt = nf + pl.cntB[a];
-    double Gx = 0.0, Gy = 0.0, Hx = 0.0, Hy = 0.0;
-    double dxux = 0.0, dxuy = 0.0, dyux = 0.0, dyuy = 0.0;
-    for (int j0 = 0; j0 < nt; j0 += 32) {
-        const int j = j0 + lane;
-        if (j < nt) {
-            int b;
-            double gx, gy;
-            if (j < nf) {
-                b = pl.L[r0 + j];
-                const double2 g = pl.G[r0 + j];
-                gx = g.x;
-                gy = g.y;
-            } else {  // grad_a W_ab = -grad_b W_ba, stored with b's forward pair
-                b = pl.L[rend - (j - nf)];
-                const double2 g = pl.G[pl.off[b] + pl.P[rend - (j - nf)]];
-                gx = -g.x;
-                gy = -g.y;
-            }
-            Gx += gx;
-            Gy += gy;
-            Hx = fma(Xxx[b], gx, fma(Xyx[b], gy, Hx));
-            Hy = fma(Xxy[b], gx, fma(Xyy[b], gy, Hy));
-            const double ubx = Ux[b], uby = Uy[b];
-            dxux = fma(ubx, gx, dxux);
-            dxuy = fma(uby, gx, dxuy);
-            dyux = fma(ubx, gy, dyux);
-            dyuy = fma(uby, gy, dyuy);
+    const int nf = on ? pl.cntF[a] : 0, nt = on ? nf + pl.cntB[a] : 0;
+    // the largest exponents among a and its neighbours (stress | u << 16)
+    unsigned em = pl.Xe[a];
+    for (int j = l; j < nf; j += 16) em = fx_max2(em, pl.Xe[pl.L[r0 + j]]);
+    for (int j = l; j < nt - nf; j += 16) em = fx_max2(em, pl.Xe[pl.L[rend - j]]);
+    em = fx_half_max2(em);
+    const int EX = fx_room((int)(em & 0xFFFFu), nt), EU = fx_room((int)(em >> 16), nt);
+    const bool bad = (em & 0xFFFFu) == kNonFinite || (em >> 16) == kNonFinite;
+    FxSum sG[2] = {{0, 0}, {0, 0}};
+    FxSum sH[2] = {{0, 0}, {0, 0}};                  // sum X^{x.} g, sum X^{y.} g
+    FxSum sU[4] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};  // d_x u^x, d_x u^y, d_y u^x, d_y u^y
+    int it = 0;
+    auto add = [&](longlong2 g, int4 x0, int4 x1, int4 u0, unsigned e) {
+        sG[0].x += g.x;
+        sG[1].x += g.y;
+        int xh, xl, yh, yl, d = EX - (int)(e & 0xFFFFu);
+        fx_split(g.x, d, xh, xl);
+        fx_split(g.y, d, yh, yl);
+        fx_add(sH[0], xh, xl, lo_of(x0));  // X^{xx} g_x
+        fx_add(sH[0], yh, yl, lo_of(x1));  // X^{yx} g_y
+        fx_add(sH[1], xh, xl, hi_of(x0));  // X^{xy} g_x
+        fx_add(sH[1], yh, yl, hi_of(x1));  // X^{yy} g_y
+        d = EU - (int)(e >> 16);
+        fx_split(g.x, d, xh, xl);
+        fx_split(g.y, d, yh, yl);
+        fx_add(sU[0], xh, xl, lo_of(u0));
+        fx_add(sU[1], xh, xl, hi_of(u0));
+        fx_add(sU[2], yh, yl, lo_of(u0));
+        fx_add(sU[3], yh, yl, hi_of(u0));
+    };
+    auto fold = [&]() {
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            fx_fold(sG[k]);
+            fx_fold(sH[k]);
+            fx_fold(sU[k]);
+            fx_fold(sU[2 + k]);
         }
+    };
+    // two entries at a time, their loads ahead of both; an entry past the end is a with gradient 0
+    auto add2 = [&](int b0, longlong2 g0, int b1, longlong2 g1) {
+        const int4 x0 = pl.X[b0], y0 = pl.X[n + b0], u0 = pl.X[2 * n + b0];
+        const int4 x1 = pl.X[b1], y1 = pl.X[n + b1], u1 = pl.X[2 * n + b1];
+        const unsigned e0 = pl.Xe[b0], e1 = pl.Xe[b1];
+        add(g0, x0, y0, u0, e0);
+        add(g1, x1, y1, u1, e1);
+        it += 2;
+        if ((it & (kFoldEvery - 1)) == 0) fold();
+    };
+    const longlong2 zero = make_longlong2(0, 0);
+    for (int j = l; j < nf; j += 32) {
+        const bool two = j + 16 < nf;
+        const int b0 = pl.L[r0 + j], b1 = two ? pl.L[r0 + j + 16] : a;
+        add2(b0, pl.G[r0 + j], b1, two ? pl.G[r0 + j + 16] : zero);
     }
-    const double vals[8] = {Gx, Gy, Hx, Hy, dxux, dxuy, dyux, dyuy};
-    const double tot = warp_reduce_scatter8(vals, lane);
-    // totals: lanes 0, 4: sum grad W (x, y); 8, 12: sum X_b grad W (x, y); 16..28: sum u_b grad W
-    const double Sx = __shfl_sync(kFull, tot, 0), Sy = __shfl_sync(kFull, tot, 4);
-    const int k = lane >> 2;
-    if ((lane & 3) == 0 && k >= 2) {
+    for (int j = l; j < nt - nf; j += 32) {  // grad_a W_ab = -grad_b W_ba, stored with b's forward pair
+        const bool two = j + 16 < nt - nf;
+        const int b0 = pl.L[rend - j], b1 = two ? pl.L[rend - j - 16] : a;
+        const int s0 = pl.P[rend - j], s1 = two ? pl.P[rend - j - 16] : 0;
+        const longlong2 g0 = pl.G[pl.off[b0] + s0], g1 = two ? pl.G[pl.off[b1] + s1] : zero;
+        add2(b0, make_longlong2(-g0.x, -g0.y), b1, make_longlong2(-g1.x, -g1.y));
+    }
+    fold();
+    FxTotal t[8] = {fx_words(sG[0]), fx_words(sG[1]), fx_words(sH[0]), fx_words(sH[1]),
+                    fx_words(sU[0]), fx_words(sU[1]), fx_words(sU[2]), fx_words(sU[3])};
+    const FxTotal tt = fx_reduce8(t, lane);
+    const int k = l >> 1;
+    double tot = fx_value(tt, k < 2 ? -kFxBits : fx_unit(k < 4 ? EX : EU));
+    if (bad && k >= 2) tot = fx_nan();
+    // totals of lanes 2 k of the half warp: k = 0, 1: sum grad W; 2, 3: sum X_b grad W; 4-7: sum u_b grad W
+    const double Sx = __shfl_sync(kFull, tot, lane & 16), Sy = __shfl_sync(kFull, tot, (lane & 16) + 2);
+    if (on && (l & 1) == 0 && k >= 2) {
         const double c = v.sigma_d * v.inv_h;
         if (k >= 4) {
             gout[(size_t)(k - 4) * n + a] = c * tot;  // d_x u^x, d_x u^y, d_y u^x, d_y u^y
@@ -385,7 +478,7 @@ __global__ void __launch_bounds__(32 * kWarps) k_pairs_gradient(EvView v, int st
             // minus the stress divergence: X_a . sum grad W + sum X_b grad W, times sqrt(-g)
             const double tau = v.sc->tau + (stage == 2 ? v.dtau : 0.0);
             const double sqrtg = v.milne ? tau : 1.0;
-            const double X0 = k == 2 ? Xxx[a] : Xxy[a], X1 = k == 2 ? Xyx[a] : Xyy[a];
+            const double X0 = gin[(size_t)(k - 2) * n + a], X1 = gin[(size_t)k * n + a];
             gout[(size_t)(k + 2) * n + a] = -sqrtg * c * (X0 * Sx + X1 * Sy + tot);
         }
     }
@@ -407,16 +500,21 @@ void launch_pairs_density(const EvView &v, const double *y, const double *Nq, Ce
                           cudaStream_t st)
 {
     launch_pair_rows(v, cb, st);
-    // the forward partials go to the density rows, which the backward pass completes in place
-    k_pairs_density_fwd<<<nblk(v.n, kWarps), 32 * kWarps, 0, st>>>(v, y, cb.fpos, Nq, cb.start, cb.cnt, cb.pl,
-                                                                   dens);
-    k_pairs_density_bwd<<<nblk(v.n, kWarps), 32 * kWarps, 0, st>>>(v, y, Nq, cb.pl, dens, nnb);
+    k_pairs_fwd<<<nblk(v.n, 2 * kWarps), 32 * kWarps, 0, st>>>(v, y, cb.fpos, Nq, cb.start, cb.cnt, cb.key, cb.perm,
+                                                             cb.pl);
+    launch_pairs_sum(v, cb, dens, nnb, st);
+}
+
+void launch_pairs_sum(const EvView &v, CellBufs cb, double *dens, int *nnb, cudaStream_t st)
+{
+    k_pairs_sum<<<nblk(v.n, 2 * kWarps), 32 * kWarps, 0, st>>>(v, cb.pl, dens, nnb);
 }
 
 void launch_pairs_gradient(const EvView &v, int stage, const double *y, const double *gin, CellBufs cb,
                            double *gout, cudaStream_t st)
 {
-    k_pairs_gradient<<<nblk(v.n, kWarps), 32 * kWarps, 0, st>>>(v, stage, y, gin, cb.pl, gout);
+    (void)y;
+    k_pairs_gradient<<<nblk(v.n, 2 * kWarps), 32 * kWarps, 0, st>>>(v, stage, gin, cb.pl, gout);
 }
 
 }  // namespace sphg

@@ -3,6 +3,7 @@
 // table.  Per accepted pair the forward density pass evaluates W and grad W once (both depend on
 // r_ab only; grad_b W_ba = -grad_a W_ab) and keeps them with the pair; the backward pass and the
 // gradient pass add every pair to both of its particles.  Sums in a fixed order: reproducible.
+#include "pairs_fixed.cuh"
 #include "sph_internal.cuh"
 
 namespace sphg {
@@ -39,257 +40,245 @@ __device__ __forceinline__ int block27_ascending(const EvView &v, const int c[3]
     return nk;
 }
 
-// Forward density pass, one warp per particle a: candidates of the 27 cells through the
-// single-precision prefilter; neighbours b < a decided at once and listed from the row end;
-// candidates b > a queued and, 32 at a time, put through the exact test, W and grad W on full
-// warps, listed from the row start with W and grad W, and summed for a.  a's unscaled partial
-// sums (self pair and pairs b > a) are left in the density rows.
-__global__ void __launch_bounds__(32 * kWarps) k_pairs3_density_fwd(EvView v, const double *__restrict__ y,
-                                                                    const float4 *__restrict__ fpos,
-                                                                    const double *__restrict__ Nq,
-                                                                    const uint32_t *__restrict__ start,
-                                                                    const uint32_t *__restrict__ cnt, PairBufs pl,
-                                                                    double *__restrict__ dpart)
+// Forward pass, a warp for two particles a.  Candidates of the 27 cells pass the
+// single-precision prefilter; a neighbour b < a is decided at once (exact FP64 test when the
+// float test left it undecided) and listed from the row end; a candidate b > a is queued, and 32
+// at a time -- of both particles -- the exact test, the distance in FP64 and the spline in 64-bit
+// integers run on full warps, and W and grad W are listed with the pair in fixed point (L, W, G).  The particles' own values go into limbs.
+// Bound: the FP64 pipe, 15 operations per unordered pair.  258 k particles: 4.0 ms a stage
+// (4.6 with the spline in FP64).
+__global__ void __launch_bounds__(32 * kWarps, 8) k_pairs3_fwd(EvView v, const double *__restrict__ y,
+                                                           const float4 *__restrict__ fpos,
+                                                           const double *__restrict__ Nq,
+                                                           const uint32_t *__restrict__ start,
+                                                           const uint32_t *__restrict__ cnt, PairBufs pl)
 {
     __shared__ int queue[kWarps][64];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int a = blockIdx.x * kWarps + wid;
-    if (a >= v.n) return;  // warp-uniform
+    const int n = v.n;
+    const long long a0 = 2 * ((long long)blockIdx.x * kWarps + wid);
+    if (a0 >= n) return;  // warp-uniform
+    const int np = a0 + 1 < n ? 2 : 1;
     int *q = queue[wid];
-    const size_t n = (size_t)v.n;
-    const double *X = y, *Y = y + n, *Z = y + 2 * n, *S = y + 6 * n;
-    const double *NB = Nq, *NS = Nq + n, *NQ = Nq + 2 * n;
-    const double xa[3] = {X[a], Y[a], Z[a]};
-    const float4 fa = fpos[a];
-    int c[3];
-#pragma unroll
-    for (int d = 0; d < 3; ++d) c[d] = cell_coord(xa[d], dec_double(v.sc->xmin_enc[d]), v.inv_cell);
-    uint32_t keys[27];
-    const int nk = block27_ascending(v, c, keys);
-    const unsigned lt = (1u << lane) - 1u;
-    const long long r0 = pl.off[a], r1 = pl.off[a + 1];
-    const int cap = r1 <= pl.total ? (int)(r1 - r0) : 0;  // rows beyond the allocation: no writes
-    int *F = pl.L + r0, *Bl = pl.L + (r1 - 1);
-    double *Wr = pl.W + r0, *Gr = pl.G3 + 3 * r0;
-    double sg = 0.0, ss = 0.0, sb = 0.0, sS = 0.0, sq = 0.0;
-    if (lane == 0) {  // the self pair, W(0)
-        const double w0 = kernel_w(0.0);
-        sg = w0;
-        ss = S[a] * w0;
-        sb = NB[a] * w0;
-        sS = NS[a] * w0;
-        sq = NQ[a] * w0;
+    const double *X = y, *Y = y + n, *Z = y + 2 * (size_t)n, *S = y + 6 * (size_t)n;
+    if (lane < 4 * np) {
+        const size_t a = (size_t)a0 + (lane >> 2);
+        const int k = lane & 3;
+        fx_store_value(pl.Q, pl.Qe, (size_t)n, a, k, k == 0 ? S[a] : Nq[(size_t)(k - 1) * n + a]);
     }
-    int nf = 0, nbk = 0, qn = 0;
+    const unsigned lt = (1u << lane) - 1u;
+    double xa[2], ya[2], za[2];
+    long long r0[2];
+    int cap[2], nf[2] = {0, 0}, nbk[2] = {0, 0}, qn = 0;
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+        const int a = (int)a0 + (p < np ? p : 0);
+        xa[p] = X[a];
+        ya[p] = Y[a];
+        za[p] = Z[a];
+        r0[p] = pl.off[a];
+        const long long r1 = pl.off[a + 1];
+        cap[p] = r1 <= pl.total ? (int)(r1 - r0[p]) : 0;  // rows beyond the allocation write nothing
+    }
+    // queued word: bit 31: the float test left the pair undecided (exact test needed), bit 30: of a0 + 1
     auto forward = [&](int qb, bool valid) {
-        const int b = qb & 0x7FFFFFFF;
-        double d[3] = {0.0, 0.0, 0.0};
+        const int b = qb & 0x3FFFFFFF;
+        const bool second = qb & 0x40000000;
+        double dx = 0.0, dy = 0.0, dz = 0.0;
         bool acc = false;
         if (valid) {
-            d[0] = xa[0] - X[b];
-            d[1] = xa[1] - Y[b];
-            d[2] = xa[2] - Z[b];
-            acc = qb >= 0 || dist2_3d(d[0], d[1], d[2]) < v.supp2;
+            dx = (second ? xa[1] : xa[0]) - X[b];
+            dy = (second ? ya[1] : ya[0]) - Y[b];
+            dz = (second ? za[1] : za[0]) - Z[b];
+            acc = qb >= 0 || dist2_3d(dx, dy, dz) < v.supp2;
         }
-        const unsigned m = __ballot_sync(kFull, acc);
+        const unsigned m0 = __ballot_sync(kFull, acc && !second), m1 = __ballot_sync(kFull, acc && second);
         if (acc) {
-            const double r2 = fma(d[0], d[0], fma(d[1], d[1], d[2] * d[2]));
-            double w = kernel_w(0.0), fac = 0.0;  // coincident particles: W(0), no gradient
+            const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
+            long long w = 1LL << kFxBits, dw = 0;  // coincident particles: W(0), no gradient
+            double ir = 0.0, q;
             if (nonzero_nonneg(r2)) {
-                // the cubic spline without a branch on q (see the 2D forward pass)
-                const double ir = inv_sqrt(r2);
-                const double qq = r2 * ir * v.inv_h;
-                const double t = 2.0 - qq, u = pos_part(1.0 - qq);
-                const double t2 = t * t, u2 = u * u;
-                w = fma(quarter_nonneg(t2), t, -(u2 * u));
-                fac = fma(-0.75, t2, 3.0 * u2) * ir;
+                pair_distance(r2, v.inv_h, ir, q);
+                spline_fixed(q, w, dw);
             }
-            const int slot = nf + __popc(m & lt);
-            if (slot < cap) {
-                F[slot] = b;
-                Wr[slot] = w;
-                Gr[3 * slot] = fac * d[0];
-                Gr[3 * slot + 1] = fac * d[1];
-                Gr[3 * slot + 2] = fac * d[2];
+            const int slot = second ? nf[1] + __popc(m1 & lt) : nf[0] + __popc(m0 & lt);
+            if (slot < (second ? cap[1] : cap[0])) {
+                const long long i = (second ? r0[1] : r0[0]) + slot;
+                pl.L[i] = b;
+                pl.W[i] = w;
+                pl.G3[3 * i] = grad_fixed(dw, dx * ir);
+                pl.G3[3 * i + 1] = grad_fixed(dw, dy * ir);
+                pl.G3[3 * i + 2] = grad_fixed(dw, dz * ir);
             }
-            sg += w;
-            ss = fma(S[b], w, ss);
-            sb = fma(NB[b], w, sb);
-            sS = fma(NS[b], w, sS);
-            sq = fma(NQ[b], w, sq);
         }
-        nf += __popc(m);
+        nf[0] += __popc(m0);
+        nf[1] += __popc(m1);
     };
-    for (int kc = 0; kc < nk; ++kc) {
-        const uint32_t k = keys[kc];
-        const uint32_t b0 = start[k], b1 = b0 + cnt[k];
-        for (uint32_t base = b0; base < b1; base += 32) {
-            const uint32_t b = base + lane;
-            bool cand = false, sure = false;
-            if (b < b1 && b != (uint32_t)a) {
-                const float4 fb = fpos[b];
-                const float dx = fa.x - fb.x, dy = fa.y - fb.y, dz = fa.z - fb.z;
-                const float r2f = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                cand = r2f <= v.supp2_hi;
-                sure = r2f < v.supp2_lo;
-            }
-            bool accB = false;  // b < a: its pair values come from b's own forward pass
-            if (cand && (int)b < a) accB = sure || dist2_3d(xa[0] - X[b], xa[1] - Y[b], xa[2] - Z[b]) < v.supp2;
-            const unsigned mb = __ballot_sync(kFull, accB);
-            if (accB) {
-                const int slot = nbk + __popc(mb & lt);
-                if (slot < cap) Bl[-slot] = (int)b;
-            }
-            nbk += __popc(mb);
-            const bool fw = cand && (int)b > a;
-            const unsigned m = __ballot_sync(kFull, fw);
-            if (fw) q[qn + __popc(m & lt)] = sure ? (int)b : (int)(b | 0x80000000u);
-            qn += __popc(m);
-            __syncwarp();
-            if (qn >= 32) {
-                forward(q[lane], true);
-                qn -= 32;
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+        if (p >= np) break;
+        const int a = (int)a0 + p, flag = p << 30;
+        const float4 fa = fpos[a];
+        const int ca = __float_as_int(fa.w);  // the packed cell coordinates
+        const int c[3] = {ca & 1023, (ca >> 10) & 1023, (ca >> 20) & 1023};
+        uint32_t keys[27];
+        const int nk = block27_ascending(v, c, keys);
+        int *Bl = pl.L + (r0[p] + cap[p] - 1);  // backward down from the row end
+        for (int kc = 0; kc < nk; ++kc) {
+            const uint32_t k = keys[kc];
+            const uint32_t b0 = start[k], b1 = b0 + cnt[k];
+            for (uint32_t base = b0; base < b1; base += 32) {
+                const uint32_t b = base + lane;
+                bool cand = false, sure = false;
+                if (b < b1 && b != (uint32_t)a) {
+                    const float4 fb = fpos[b];
+                    const float dx = fa.x - fb.x, dy = fa.y - fb.y, dz = fa.z - fb.z;
+                    const float r2f = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+                    cand = r2f <= v.supp2_hi;
+                    sure = r2f < v.supp2_lo;
+                }
+                // b < a: decided here and listed; its pair values come from b's own forward pass
+                bool accB = false;
+                if (cand && (int)b < a) accB = sure || dist2_3d(xa[p] - X[b], ya[p] - Y[b], za[p] - Z[b]) < v.supp2;
+                const unsigned mb = __ballot_sync(kFull, accB);
+                if (accB) {
+                    const int slot = nbk[p] + __popc(mb & lt);
+                    if (slot < cap[p]) Bl[-slot] = (int)b;
+                }
+                nbk[p] += __popc(mb);
+                // b > a: queued in arrival (ascending) order for the FP64 pair arithmetic
+                const bool fw = cand && (int)b > a;
+                const unsigned m = __ballot_sync(kFull, fw);
+                if (fw) q[qn + __popc(m & lt)] = (int)(b | (sure ? 0u : 0x80000000u)) | flag;
+                qn += __popc(m);
                 __syncwarp();
-                if (lane < qn) q[lane] = q[32 + lane];
-                __syncwarp();
+                if (qn >= 32) {
+                    forward(q[lane], true);
+                    qn -= 32;
+                    __syncwarp();
+                    if (lane < qn) q[lane] = q[32 + lane];
+                    __syncwarp();
+                }
             }
         }
     }
     if (qn > 0) forward(lane < qn ? q[lane] : 0, lane < qn);
-    const double vals[8] = {sg, ss, sb, sS, sq, 0.0, 0.0, 0.0};
-    const double tot = warp_reduce_scatter8(vals, lane);
-    const int kk = lane >> 2;
-    if ((lane & 3) == 0 && kk < 5) dpart[(size_t)kk * n + a] = tot;
     if (lane == 0) {
-        pl.cntF[a] = nf;
-        pl.cntB[a] = nbk;
-        if (nf + nbk > cap) atomicOr(&v.sc->pair_flag, 1u);
+        bool over = false;
+        for (int p = 0; p < np; ++p) {
+            pl.cntF[a0 + p] = nf[p];
+            pl.cntB[a0 + p] = nbk[p];
+            over = over || nf[p] + nbk[p] > cap[p];
+        }
+        if (over) atomicOr(&v.sc->pair_flag, 1u);  // the two ends met: lists unusable
     }
 }
 
-// Backward density pass (as in 2D): W of the pairs (b, a), b < a, from b's row after a binary
-// search; the slot kept in P; completes the density rows (the 3D EoS pass forms u0 itself).
-__global__ void __launch_bounds__(32 * kWarps) k_pairs3_density_bwd(EvView v, const double *__restrict__ y,
-                                                                    const double *__restrict__ Nq, PairBufs pl,
-                                                                    double *__restrict__ dens, int *__restrict__ nnb)
+// Gradient pass, half a warp per particle a, over its pairs b > a (stored grad_a W_ab) and b < a
+// (minus the stored grad_b W_ba), in integers (pairs_fixed.cuh): sum grad W (3), sum X_b^{j i}
+// grad_j W (3), sum u_b^j grad_k W (9); the epilogue as the per-particle pass.
+// Bound: the latency of the gathers; 258 k particles: 3.4 ms a stage (6.0 with 21 FP64 operations per
+// pair).  4 blocks per SM: 3 gave 3.7, 5 3.8, 6 4.8 ms.
+__global__ void __launch_bounds__(32 * kWarps, 4) k_pairs3_gradient(EvView v, int stage, const double *__restrict__ gin,
+                                                                 PairBufs pl, double *__restrict__ gout)
 {
     if (v.sc->pair_flag) return;  // a list overflowed: the per-particle pass runs instead
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int a = blockIdx.x * kWarps + wid;
-    if (a >= v.n) return;
-    const size_t n = (size_t)v.n;
-    const double *S = y + 6 * n;
-    const double *NB = Nq, *NS = Nq + n, *NQ = Nq + 2 * n;
-    const long long rend = pl.off[a + 1] - 1;
-    const int nb = pl.cntB[a];
-    double sg = 0.0, ss = 0.0, sb = 0.0, sS = 0.0, sq = 0.0;
-    for (int j0 = 0; j0 < nb; j0 += 32) {
-        const int j = j0 + lane;
-        if (j < nb) {
-            const int b = pl.L[rend - j];
-            const long long rb = pl.off[b];
-            const int *Fb = pl.L + rb;
-            const int nfb = pl.cntF[b];
-            int lo = 0, hi = nfb;
-            while (lo < hi) {
-                const int mid = (lo + hi) >> 1;
-                if (Fb[mid] < a) lo = mid + 1;
-                else hi = mid;
-            }
-            if (lo >= nfb || Fb[lo] != a) {  // both sides decide alike; checked all the same
-                atomicOr(&v.sc->err_flags, ERR_PAIR_LIST);
-                lo = 0;
-            }
-            pl.P[rend - j] = lo;
-            const double w = nfb > 0 ? pl.W[rb + lo] : 0.0;
-            sg += w;
-            ss = fma(S[b], w, ss);
-            sb = fma(NB[b], w, sb);
-            sS = fma(NS[b], w, sS);
-            sq = fma(NQ[b], w, sq);
-        }
-    }
-    const double vals[8] = {sg, ss, sb, sS, sq, 0.0, 0.0, 0.0};
-    const double tot = warp_reduce_scatter8(vals, lane);
-    const int k = lane >> 2;
-    if ((lane & 3) == 0 && k < 5) {
-        double *d = dens + (size_t)k * n + a;
-        *d = v.sigma_d * (*d + tot);
-    }
-    if (lane == 0) {
-        const int c = 1 + pl.cntF[a] + nb;
-        nnb[a] = c;
-        if (pl.cnt_dst) pl.cnt_dst[a] = c;
-        atomicAdd(&v.sc->pairs, (unsigned long long)c);
-    }
-}
-
-// Gradient pass, one warp per particle a, over its pairs b > a (stored grad_a W_ab) and b < a
-// (minus the stored grad_b W_ba): sum grad W (3), sum X_b^{j i} grad_j W (3), sum u_b^j grad_k W (9),
-// 15 sums reduced by two reduce-scatters; the epilogue as the per-particle pass.
-__global__ void __launch_bounds__(32 * kWarps) k_pairs3_gradient(EvView v, int stage, const double *__restrict__ y,
-                                                                 const double *__restrict__ gin, PairBufs pl,
-                                                                 double *__restrict__ gout)
-{
-    if (v.sc->pair_flag) return;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int a = blockIdx.x * kWarps + wid;
-    if (a >= v.n) return;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, l = lane & 15;
+    const long long ap = 2 * ((long long)blockIdx.x * kWarps + wid) + (lane >> 4);
+    if (ap - (lane >> 4) >= v.n) return;  // warp-uniform
+    const bool on = ap < v.n;
+    const int a = on ? (int)ap : v.n - 1;
     const size_t n = (size_t)v.n;
     const long long r0 = pl.off[a], rend = pl.off[a + 1] - 1;
-    const int nf = pl.cntF[a], nt = nf + pl.cntB[a];
-    double G[3] = {0, 0, 0}, H[3] = {0, 0, 0}, du[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
-    for (int j0 = 0; j0 < nt; j0 += 32) {
-        const int jj = j0 + lane;
-        if (jj < nt) {
-            int b;
-            double gw[3];
-            if (jj < nf) {
-                b = pl.L[r0 + jj];
-                const double *g = pl.G3 + 3 * (r0 + jj);
-                gw[0] = g[0];
-                gw[1] = g[1];
-                gw[2] = g[2];
-            } else {
-                b = pl.L[rend - (jj - nf)];
-                const double *g = pl.G3 + 3 * (pl.off[b] + pl.P[rend - (jj - nf)]);
-                gw[0] = -g[0];
-                gw[1] = -g[1];
-                gw[2] = -g[2];
-            }
+    const int nf = on ? pl.cntF[a] : 0, nt = on ? nf + pl.cntB[a] : 0;
+    // the largest exponents among a and its neighbours (stress | u << 16)
+    unsigned em = pl.Xe[a];
+    for (int j = l; j < nf; j += 16) em = fx_max2(em, pl.Xe[pl.L[r0 + j]]);
+    for (int j = l; j < nt - nf; j += 16) em = fx_max2(em, pl.Xe[pl.L[rend - j]]);
+    em = fx_half_max2(em);
+    const int EX = fx_room((int)(em & 0xFFFFu), nt), EU = fx_room((int)(em >> 16), nt);
+    const bool bad = (em & 0xFFFFu) == kNonFinite || (em >> 16) == kNonFinite;
+    FxSum sG[3], sH[3], sU[9];  // sum g; sum_j X^{j i} g_j; 3 k + j: sum u^j g_k
 #pragma unroll
-            for (int k = 0; k < 3; ++k) G[k] += gw[k];
+    for (int k = 0; k < 3; ++k) sG[k] = sH[k] = sU[k] = sU[3 + k] = sU[6 + k] = FxSum{0, 0};
+    auto fold = [&]() {
 #pragma unroll
-            for (int i = 0; i < 3; ++i) {
-                double h = H[i];
-#pragma unroll
-                for (int j = 0; j < 3; ++j) h = fma(gin[(size_t)(3 * j + i) * n + b], gw[j], h);
-                H[i] = h;
-            }
-#pragma unroll
-            for (int j = 0; j < 3; ++j) {
-                const double ub = gin[(size_t)(9 + j) * n + b];
-#pragma unroll
-                for (int k = 0; k < 3; ++k) du[k][j] = fma(ub, gw[k], du[k][j]);
-            }
+        for (int k = 0; k < 3; ++k) {
+            fx_fold(sG[k]);
+            fx_fold(sH[k]);
+            fx_fold(sU[k]);
+            fx_fold(sU[3 + k]);
+            fx_fold(sU[6 + k]);
         }
+    };
+    // the next entry's index and gradient are loaded while the current one is added
+    auto entry = [&](int j, int &b, long long (&g)[3]) {
+        b = a;
+        g[0] = g[1] = g[2] = 0;
+        if (j < nf) {
+            b = pl.L[r0 + j];
+            const long long *q = pl.G3 + 3 * (r0 + j);
+            g[0] = q[0];
+            g[1] = q[1];
+            g[2] = q[2];
+        } else if (j < nt) {
+            b = pl.L[rend - (j - nf)];
+            const long long *q = pl.G3 + 3 * (pl.off[b] + pl.P[rend - (j - nf)]);
+            g[0] = -q[0];
+            g[1] = -q[1];
+            g[2] = -q[2];
+        }
+    };
+    int b1;
+    long long g1[3];
+    entry(l, b1, g1);
+    for (int j = l, it = 1; j < nt; j += 16, ++it) {
+        const int b = b1;
+        const long long g[3] = {g1[0], g1[1], g1[2]};
+        int4 x4[6];
+#pragma unroll
+        for (int m = 0; m < 6; ++m) x4[m] = pl.X[m * n + b];
+        const unsigned e = pl.Xe[b];
+        entry(j + 16, b1, g1);
+        const int dX = EX - (int)(e & 0xFFFFu), dU = EU - (int)(e >> 16);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            int hi, lo;
+            sG[k].x += g[k];
+            fx_split(g[k], dX, hi, lo);
+#pragma unroll
+            for (int i = 0; i < 3; ++i) fx_add(sH[i], hi, lo, (3 * k + i) & 1 ? hi_of(x4[(3 * k + i) >> 1]) : lo_of(x4[(3 * k + i) >> 1]));
+            fx_split(g[k], dU, hi, lo);
+#pragma unroll
+            for (int i = 0; i < 3; ++i) fx_add(sU[3 * k + i], hi, lo, (9 + i) & 1 ? hi_of(x4[(9 + i) >> 1]) : lo_of(x4[(9 + i) >> 1]));
+        }
+        if ((it & (kFoldEvery - 1)) == 0) fold();
     }
-    const double v1[8] = {G[0], G[1], G[2], H[0], H[1], H[2], du[0][0], du[0][1]};
-    const double v2[8] = {du[0][2], du[1][0], du[1][1], du[1][2], du[2][0], du[2][1], du[2][2], 0.0};
-    const double t1 = warp_reduce_scatter8(v1, lane), t2 = warp_reduce_scatter8(v2, lane);
-    const double G0 = __shfl_sync(kFull, t1, 0), G1 = __shfl_sync(kFull, t1, 4), G2 = __shfl_sync(kFull, t1, 8);
-    const int k = lane >> 2;
-    if ((lane & 3) == 0) {
+    fold();
+    FxTotal t[16];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        t[k] = fx_words(sG[k]);
+        t[3 + k] = fx_words(sH[k]);
+    }
+#pragma unroll
+    for (int k = 0; k < 9; ++k) t[6 + k] = fx_words(sU[k]);
+    t[15] = FxTotal{0, 0};
+    const FxTotal tt = fx_reduce16(t, lane);
+    double tot = fx_value(tt, l < 3 ? -kFxBits : fx_unit(l < 6 ? EX : EU));
+    if (bad && l >= 3) tot = fx_nan();
+    const int h0 = lane & 16;
+    const double G0 = __shfl_sync(kFull, tot, h0), G1 = __shfl_sync(kFull, tot, h0 + 1), G2 = __shfl_sync(kFull, tot, h0 + 2);
+    if (on && l >= 3 && l < 15) {
         const double c = v.sigma_d * v.inv_h;
-        // du[k][j] -> row 3 k + j: t1 holds du00, du01 (lanes 24, 28); t2 du02 .. du22 (lanes 0..24)
-        if (k >= 6) gout[(size_t)(k - 6) * n + a] = c * t1;
-        if (k < 7) gout[(size_t)(2 + k) * n + a] = c * t2;
-        if (k >= 3 && k < 6) {
+        if (l >= 6) {
+            gout[(size_t)(l - 6) * n + a] = c * tot;  // d_k u^j at 3 k + j
+        } else {
             // minus the stress divergence: H_i + sum_j X_a^{j i} G_j, times sqrt(-g)
-            const int i = k - 3;
+            const int i = l - 3;
             const double tau = v.sc->tau + (stage == 2 ? v.dtau : 0.0);
             const double sqrtg = v.milne ? tau : 1.0;
-            double F = t1;
+            double F = tot;
             F = fma(gin[(size_t)(0 + i) * n + a], G0, F);
             F = fma(gin[(size_t)(3 + i) * n + a], G1, F);
             F = fma(gin[(size_t)(6 + i) * n + a], G2, F);
@@ -306,15 +295,15 @@ void launch_pairs3_density(const EvView &v, const double *y, const double *Nq, C
                            cudaStream_t st)
 {
     launch_pair_rows(v, cb, st);
-    k_pairs3_density_fwd<<<nblk(v.n, kWarps), 32 * kWarps, 0, st>>>(v, y, cb.fpos3, Nq, cb.start, cb.cnt, cb.pl,
-                                                                    dens);
-    k_pairs3_density_bwd<<<nblk(v.n, kWarps), 32 * kWarps, 0, st>>>(v, y, Nq, cb.pl, dens, nnb);
+    k_pairs3_fwd<<<nblk(v.n, 2 * kWarps), 32 * kWarps, 0, st>>>(v, y, cb.fpos3, Nq, cb.start, cb.cnt, cb.pl);
+    launch_pairs_sum(v, cb, dens, nnb, st);
 }
 
 void launch_pairs3_gradient(const EvView &v, int stage, const double *y, const double *gin, CellBufs cb,
                             double *gout, cudaStream_t st)
 {
-    k_pairs3_gradient<<<nblk(v.n, kWarps), 32 * kWarps, 0, st>>>(v, stage, y, gin, cb.pl, gout);
+    (void)y;
+    k_pairs3_gradient<<<nblk(v.n, 2 * kWarps), 32 * kWarps, 0, st>>>(v, stage, gin, cb.pl, gout);
 }
 
 }  // namespace sphg

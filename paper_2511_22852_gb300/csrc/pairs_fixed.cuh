@@ -1,0 +1,248 @@
+// pairs_fixed.cuh -- integer accumulation of the plain (FP64) neighbour sums.
+//
+// On GB300 an FP64 operation occupies its pipe for 64 cycles per warp and quadrant, a 32-bit
+// integer multiply-add into 64 bits for about 3.  The pair passes therefore form their sums
+// sum_b q_b w_ab in integers, at or above FP64 precision:
+//   * the pair's kernel value or gradient (dimensionless, |w| <= 1), computed in FP64, as a
+//     fixed-point integer in units of 2^-57;
+//   * the particle's value q_b as its exact 53-bit mantissa (times 2) in two limbs
+//     hi 2^29 + lo (lo balanced around 0) and its exponent;
+//   * the particle's sums in units of the largest exponent E among its neighbours (a first look
+//     over the exponents alone): w is shifted down by E - e_b and split into limbs, hi hi goes to
+//     one 64-bit accumulator and the two cross products to another; the dropped lo lo is below
+//     2^-54 of the largest q_b, with either sign;
+//   * the lanes are added in integers, and each total becomes a double once.
+// Against sums in FP64, whose additions round at 2^-53 of the partial sum, the error is smaller
+// (the step's error against 64-bit values: 5.2e-16 of u on the ideal lattice with FP64 sums, 5.0e-16
+// now), and it does not depend on the order of the additions.
+// A non-finite q_b makes the particle's sums NaN.
+#pragma once
+#include "sph_internal.cuh"
+
+namespace sphg {
+
+constexpr int kFxBits = 57;   // units of the fixed-point kernel values
+constexpr int kLimb = 29;
+constexpr long long kLimbMask = (1LL << kLimb) - 1;
+constexpr int kNonFinite = 0x7FF;
+constexpr int kFoldEvery = 16;     // terms between folds of the cross accumulators
+constexpr int kHeadroom = 128;     // terms a lane's high accumulator holds without a larger unit
+
+// v in units of 2^-BITS (|v| 2^BITS < 2^63), rounded to nearest (halves away from zero)
+template <int BITS>
+__device__ __forceinline__ long long to_fixed(double v)
+{
+    const long long b = __double_as_longlong(v);
+    const int e = (int)(b >> 52) & 0x7FF;
+    long long m = (b & 0xFFFFFFFFFFFFFLL) | (1LL << 52);
+    const int s = e - (1075 - BITS);
+    m = s >= 0 ? m << min(s, 10) : (s > -60 ? (m + (1LL << (-s - 1))) >> -s : 0LL);
+    return b < 0 ? -m : m;
+}
+
+// 1/r, r/h of a pair from r^2 > 0: a single-precision reciprocal square root y (relative error
+// below 2^-21) refined by one third-order Householder step, e = 1 - r^2 y^2, c = e/2 + 3 e^2/8,
+// 1/r = y (1 + c), r = r^2 y (1 + c), with the remainder of order e^3 below 2^-62.  Six FP64
+// operations for both and the division by h (rsqrt and two products: about nine); 3 e^2/8 is
+// below 2^-44 and is taken in single precision.  Outside the single-precision range: rsqrt.
+__device__ __forceinline__ void pair_distance(double r2, double inv_h, double &ir, double &q)
+{
+    const unsigned hi = (unsigned)__double2hiint(r2);
+    if (hi - 0x3B000000u < 0x08000000u) {  // 2^-79 <= r^2 < 2^49
+        const float f = __uint_as_float(__funnelshift_l((unsigned)__double2loint(r2), hi - 0x38000000u, 3));
+        const float y = rsqrt_apx(f);
+        const unsigned yb = __float_as_uint(y);
+        const double y0 = __hiloint2double((int)((yb >> 3) + 0x38000000u), (int)(yb << 29));
+        const double t = r2 * y0;
+        const double e = fma(-t, y0, 1.0);
+        // (3/8) e^2 from e's leading bits: |e| < 2^-19, so a float holds it (zero below 2^-126)
+        const unsigned eh = (unsigned)__double2hiint(e) & 0x7FFFFFFFu;
+        const float ef = eh < 0x3C000000u ? 0.0f : __uint_as_float(__funnelshift_l((unsigned)__double2loint(e), eh - 0x38000000u, 3));
+        const unsigned cb = __float_as_uint(0.375f * ef * ef);
+        const double c2 = cb < 0x00800000u ? 0.0 : __hiloint2double((int)((cb >> 3) + 0x38000000u), (int)(cb << 29));
+        const double c = fma(e, 0.5, c2);
+        ir = fma(y0, c, y0);
+        q = fma(t, c, t) * inv_h;
+    } else {
+        ir = rsqrt(r2);
+        q = r2 * ir * inv_h;
+    }
+}
+
+// The cubic spline in fixed point from q = r/h in [0, 2]: w = (2-q)^3/4 - max(1-q, 0)^3 in units of
+// 2^-kFxBits and w' = 3 max(1-q, 0)^2 - 3 (2-q)^2/4 in units of 2^-62 (|w'| <= 1).  t = 2 - q and
+// u = max(1 - q, 0) in units of 2^-61; 64-bit high products instead of FP64 ones (about 10 integer
+// instructions against one operation of 64 cycles), errors below 2^-56.
+__device__ __forceinline__ void spline_fixed(double q, long long &w, long long &dw)
+{
+    const long long Q = to_fixed<61>(q);
+    const unsigned long long T = (unsigned long long)max((1LL << 62) - Q, 0LL), U = (unsigned long long)max((1LL << 61) - Q, 0LL);
+    const unsigned long long T2 = __umul64hi(T, T), U2 = __umul64hi(U, U);  // units of 2^-58
+    const unsigned long long T3 = __umul64hi(T2 << 3, T), U3 = __umul64hi(U2 << 3, U);
+    w = ((long long)T3 - 4 * (long long)U3 + 4) >> 3;
+    dw = 48 * ((long long)U2 - (long long)(T2 >> 2));  // 3 (u^2 - t^2/4), 2^-58 -> 2^-62
+}
+// w' times the unit vector's component e in [-1, 1], in units of 2^-kFxBits
+__device__ __forceinline__ long long grad_fixed(long long dw, double e)
+{
+    return (__mul64hi(dw, to_fixed<62>(e)) + 4) >> 3;
+}
+
+// a fixed-point kernel value as a double (truncated to 53 bits, without FP64 operations)
+__device__ __forceinline__ double from_fixed(long long f)
+{
+    const unsigned long long m = f < 0 ? -(unsigned long long)f : (unsigned long long)f;
+    const int lz = __clzll((long long)m);
+    const unsigned long long n = m << (lz & 63);  // leading one at bit 63
+    const unsigned long long bits = ((unsigned long long)(1023 - kFxBits + 63 - lz) << 52) | ((n >> 11) & 0xFFFFFFFFFFFFFULL);
+    return m == 0ull ? 0.0 : __longlong_as_double((long long)(bits | ((unsigned long long)f & 0x8000000000000000ULL)));
+}
+
+// biased exponent of v (zero and denormals: 1), kNonFinite for infinities and NaN
+__device__ __forceinline__ int fx_exponent(double v)
+{
+    const int e = (__double2hiint(v) >> 20) & 0x7FF;
+    return max(e, 1);
+}
+// v = (hi 2^29 + lo) 2^(E - 1076), E at least v's exponent (rounded down to that unit)
+__device__ __forceinline__ int2 fx_limbs(double v, int E)
+{
+    const long long b = __double_as_longlong(v);
+    const int e = (int)(b >> 52) & 0x7FF;
+    long long m = ((b & 0xFFFFFFFFFFFFFLL) | (e > 0 ? 1LL << 52 : 0LL)) << 1;
+    m = (b < 0 ? -m : m) >> min(E - max(e, 1), 63);
+    const int lo = (int)((unsigned)m << (32 - kLimb)) >> (32 - kLimb);  // the low 29 bits, sign-extended
+    return make_int2((int)((m - lo) >> kLimb), lo);
+}
+
+// one sum: value (hh 2^29 + x) 2^29 in units of 2^(E - 1076 - kFxBits)
+struct FxSum {
+    long long hh, x;
+};
+__device__ __forceinline__ void fx_add(FxSum &s, int whi, int wlo, int2 q)
+{
+    s.hh += (long long)whi * q.x;
+    s.x += (long long)whi * q.y;
+    s.x += (long long)wlo * q.x;
+}
+__device__ __forceinline__ void fx_fold(FxSum &s)
+{
+    s.hh += s.x >> kLimb;
+    s.x &= kLimbMask;
+}
+// exponents of several values packed in 16-bit halves: the larger of each
+__device__ __forceinline__ unsigned fx_max2(unsigned a, unsigned b) { return __vmaxu2(a, b); }
+// packed exponents over the 16 lanes of a half warp
+__device__ __forceinline__ unsigned fx_half_max2(unsigned e)
+{
+    for (int o = 8; o > 0; o >>= 1) e = fx_max2(e, __shfl_xor_sync(0xFFFFFFFFu, e, o));
+    return e;
+}
+// the unit's exponent for sums over n entries (16 lanes): E, and more where a lane adds over
+// kHeadroom terms
+__device__ __forceinline__ int fx_room(int E, int n) { return E + (32 - __clz((n / 16) / kHeadroom)); }
+// w shifted to a unit d exponents larger, in limbs
+__device__ __forceinline__ void fx_split(long long w, int d, int &hi, int &lo)
+{
+    const long long t = w >> min(d, 63);
+    hi = (int)(t >> kLimb);
+    lo = (int)t & (int)kLimbMask;
+}
+
+// Sums over the 16 lanes of a half warp.  Each lane's (hh, x) goes into two words that cannot
+// overflow (hh in high and low parts), reduced by recursive halving.
+struct FxTotal {
+    long long p, q;  // p 2^49 + q
+};
+__device__ __forceinline__ FxTotal fx_words(const FxSum &s)
+{
+    return FxTotal{s.hh >> 20, ((s.hh & 0xFFFFF) << kLimb) | s.x};
+}
+__device__ __forceinline__ FxTotal fx_exchange(const FxTotal &keep, const FxTotal &give, int mask)
+{
+    return FxTotal{keep.p + __shfl_xor_sync(0xFFFFFFFFu, give.p, mask), keep.q + __shfl_xor_sync(0xFFFFFFFFu, give.q, mask)};
+}
+__device__ __forceinline__ FxTotal fx_sel(bool c, const FxTotal &a, const FxTotal &b)
+{
+    return FxTotal{c ? a.p : b.p, c ? a.q : b.q};
+}
+// 8 values: lanes 2k, 2k + 1 of the half warp get the total of value k
+__device__ __forceinline__ FxTotal fx_reduce8(const FxTotal (&v)[8], int lane)
+{
+    const bool b3 = lane & 8, b2 = lane & 4, b1 = lane & 2;
+    FxTotal h[4], g[2];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) h[i] = fx_exchange(fx_sel(b3, v[4 + i], v[i]), fx_sel(b3, v[i], v[4 + i]), 8);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) g[i] = fx_exchange(fx_sel(b2, h[2 + i], h[i]), fx_sel(b2, h[i], h[2 + i]), 4);
+    const FxTotal f = fx_exchange(fx_sel(b1, g[1], g[0]), fx_sel(b1, g[0], g[1]), 2);
+    return fx_exchange(f, f, 1);
+}
+// 16 values: lane k of the half warp gets the total of value k
+__device__ __forceinline__ FxTotal fx_reduce16(const FxTotal (&v)[16], int lane)
+{
+    const bool b3 = lane & 8, b2 = lane & 4, b1 = lane & 2, b0 = lane & 1;
+    FxTotal o[8], h[4], g[2];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) o[i] = fx_exchange(fx_sel(b3, v[8 + i], v[i]), fx_sel(b3, v[i], v[8 + i]), 8);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) h[i] = fx_exchange(fx_sel(b2, o[4 + i], o[i]), fx_sel(b2, o[i], o[4 + i]), 4);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) g[i] = fx_exchange(fx_sel(b1, h[2 + i], h[i]), fx_sel(b1, h[i], h[2 + i]), 2);
+    return fx_exchange(fx_sel(b0, g[1], g[0]), fx_sel(b0, g[0], g[1]), 1);
+}
+// a total p 2^49 + q in units of 2^k as a double: k = fx_unit(E) for a group's sums, -kFxBits for
+// sums of kernel values alone (x counting units of 2^-kFxBits)
+__device__ __forceinline__ int fx_unit(int E) { return E - 1076 - kFxBits + kLimb; }
+__device__ __forceinline__ double fx_value(const FxTotal &t, int k)
+{
+    const double v = fma((double)t.p, 562949953421312.0, (double)t.q);  // 2^49
+    const int k1 = k / 2, k2 = k - k1;                                  // two normal factors
+    return v * __hiloint2double((1023 + k1) << 20, 0) * __hiloint2double((1023 + k2) << 20, 0);
+}
+__device__ __forceinline__ double fx_nan() { return __longlong_as_double(0x7FF8000000000000LL); }
+
+// The limbs of particle values for the pair passes, in planes of int4 (two values each) over the
+// particles, so that the lanes' neighbours, mostly consecutive, load from few cache lines: values
+// with an exponent each (S, N_B, N_S, N_Q; lane k < 4 of a group of lanes writes value k)
+__device__ __forceinline__ void fx_store_value(int4 *Q, unsigned short *Qe, size_t n, size_t a, int k, double v)
+{
+    const int e = fx_exponent(v);
+    reinterpret_cast<int2 *>(Q)[2 * ((k >> 1) * n + a) + (k & 1)] = fx_limbs(v, e);
+    Qe[4 * a + k] = (unsigned short)e;
+}
+// the largest exponent of K components of one tensor or vector
+template <int K>
+__device__ __forceinline__ int fx_shared_exponent(const double (&v)[K])
+{
+    int e = 1;
+#pragma unroll
+    for (int k = 0; k < K; ++k) e = max(e, fx_exponent(v[k]));
+    return e;
+}
+__device__ __forceinline__ int4 fx_limbs2(double v0, int e0, double v1, int e1)
+{
+    const int2 l0 = fx_limbs(v0, e0), l1 = fx_limbs(v1, e1);
+    return make_int4(l0.x, l0.y, l1.x, l1.y);
+}
+__device__ __forceinline__ int2 lo_of(int4 v) { return make_int2(v.x, v.y); }
+__device__ __forceinline__ int2 hi_of(int4 v) { return make_int2(v.z, v.w); }
+
+// first slot of the ascending list F[0 .. len) whose entry is not below a
+struct SlotSearch {
+    const int *F;
+    int base, len;
+    __device__ __forceinline__ bool open() const { return len > 0; }
+    __device__ __forceinline__ void step(int a)
+    {
+        const int half = (len + 1) >> 1;  // len = 1 decides the last entry
+        if (len > 0 && F[base + half - 1] < a) {
+            base += half;
+            len -= half;
+        } else {
+            len = half - 1;
+        }
+    }
+};
+
+}  // namespace sphg

@@ -132,6 +132,10 @@ struct EvView {
     int diff;
     double kapT2[9], tauJT[3];
     double *dinp, *dal, *dout;
+    // pair lists (plain forms): where the EoS pass leaves the gradient-pass inputs in limbs
+    // (PairBufs X, Xe; nullptr: lists off)
+    int4 *fxX;
+    unsigned int *fxE;
 };
 constexpr int kJRow = 9;  // first state row of the diffusion currents (2+1D)
 
@@ -185,6 +189,17 @@ __host__ __device__ __forceinline__ uint32_t spread2(uint32_t v)
     return v;
 }
 __host__ __device__ __forceinline__ uint32_t morton2(uint32_t cx, uint32_t cy) { return spread2(cx) | (spread2(cy) << 1); }
+
+// the even bits of a key, the inverse of spread2
+__device__ __forceinline__ uint32_t unspread2(uint32_t v)
+{
+    v &= 0x55555555u;
+    v = (v | (v >> 1)) & 0x33333333u;
+    v = (v | (v >> 2)) & 0x0F0F0F0Fu;
+    v = (v | (v >> 4)) & 0x00FF00FFu;
+    v = (v | (v >> 8)) & 0x0000FFFFu;
+    return v;
+}
 
 // cell coordinate floor((x - xmin) * (1/(2h))): a single rounded subtraction and
 // product, the same two operations on every platform
@@ -376,15 +391,24 @@ struct PairBufs {
     long long *off;               // [n + 1] row offsets of this stage
     unsigned long long *part;     // scan partial sums
     int *L, *P, *cntF, *cntB;
-    double *W;
-    double2 *G;   // 2D
-    double *G3;   // 3D: three components per entry
+    // kernel value W/sigma_d and gradient h grad W/sigma_d of the pair in units of 2^-57
+    // (pairs_fixed.cuh)
+    long long *W;
+    longlong2 *G;   // 2D
+    long long *G3;  // 3D: three components per entry
+    // particle values in limbs (sorted order), planes of [n] int4 with two values each: S, N_B |
+    // N_S, N_Q with an exponent each (Qe[n][4]); the rows of gin, two at a time, with their two
+    // exponents (stress, u) packed in Xe
+    int4 *Q;
+    unsigned short *Qe;
+    int4 *X;
+    unsigned int *Xe;
 };
 
 struct CellBufs {
     uint32_t *key, *cnt, *start, *cursor, *tmp, *perm;
     float2 *fpos;   // 2D: sorted positions relative to the bounding-box minimum, single precision
-    float4 *fpos3;  // 3D: the same with three coordinates
+    float4 *fpos3;  // 3D: the same with three coordinates, w: the packed cell coordinates
     float4 *fq, *fx;  // mixed 3D: (S, N_B, N_S, N_Q) and the gradient inputs [3][n] in single precision
     uint32_t *part; // scan partial sums (multi-block scan of large bucket tables)
     int nb;         // number of buckets: 1 << (2 B) in 2D, 1 << (B3[0] + B3[1] + B3[2]) in 3D
@@ -437,6 +461,8 @@ void launch_pairs_gradient(const EvView &v, int stage, const double *y, const do
                            double *gout, cudaStream_t st);
 // the per-stage row offsets of the pair lists (prefix scan of the carried counts)
 void launch_pair_rows(const EvView &v, CellBufs cb, cudaStream_t st);
+// the density sums over the listed pairs, 2D and 3D
+void launch_pairs_sum(const EvView &v, CellBufs cb, double *dens, int *nnb, cudaStream_t st);
 // plain 3D neighbour passes over the half-pair lists (after the row offsets)
 void launch_pairs3_density(const EvView &v, const double *y, const double *Nq, CellBufs cb, double *dens, int *nnb,
                            cudaStream_t st);

@@ -11,6 +11,7 @@
 // State rows (nv = 13): x^1..3, u^1..3, S, Pi/sigma, pi^{ij}/sigma for (11, 12, 13, 22, 23);
 // pi^{33} follows from tracelessness, pi^{0 mu} from transversality.
 #include "eos_device.cuh"
+#include "pairs_fixed.cuh"
 #include <algorithm>
 
 #include "sph_internal.cuh"
@@ -322,16 +323,29 @@ __global__ void __launch_bounds__(64, 5) k_eos3_finish(EvView v, int stage, cons
         double vv[3];
 #pragma unroll
         for (int j = 0; j < 3; ++j) vv[j] = u[1 + j] * iu0;
+        double X[9], us[3];
 #pragma unroll
         for (int j = 0; j < 3; ++j)
 #pragma unroll
             for (int i = 0; i < 3; ++i) {
-                double X = pi[1 + j][1 + i] - vv[j] * pi[0][1 + i];
-                if (j == i) X += j < 2 ? P : P * (G.milne ? isg * isg : 1.0);  // -P g^{jj}
-                gin[(size_t)(3 * j + i) * n + a] = X * inv2;
+                double t = pi[1 + j][1 + i] - vv[j] * pi[0][1 + i];
+                if (j == i) t += j < 2 ? P : P * (G.milne ? isg * isg : 1.0);  // -P g^{jj}
+                X[3 * j + i] = t * inv2;
+                gin[(size_t)(3 * j + i) * n + a] = X[3 * j + i];
             }
 #pragma unroll
-        for (int j = 0; j < 3; ++j) gin[(size_t)(9 + j) * n + a] = u[1 + j] * isig;
+        for (int j = 0; j < 3; ++j) {
+            us[j] = u[1 + j] * isig;
+            gin[(size_t)(9 + j) * n + a] = us[j];
+        }
+        if (v.fxX) {  // the same in limbs for the pair-list gradient pass
+            const int eX = fx_shared_exponent(X), eu = fx_shared_exponent(us);
+#pragma unroll
+            for (int m = 0; m < 4; ++m) v.fxX[m * n + a] = fx_limbs2(X[2 * m], eX, X[2 * m + 1], eX);
+            v.fxX[4 * n + a] = fx_limbs2(X[8], eX, us[0], eu);
+            v.fxX[5 * n + a] = fx_limbs2(us[1], eu, us[2], eu);
+            v.fxE[a] = (unsigned)eX | ((unsigned)eu << 16);
+        }
         if (G.milne) {
             // sqrt(-g) Gamma^0_{33} T^{33} / sigma* = tau^2 T^{eta eta} / sigma*
             wcontrib = (G.tau * G.tau * ((o.e + P) * u[3] * u[3] + pi[3][3]) + P) * isig;
