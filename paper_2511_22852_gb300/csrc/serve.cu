@@ -1165,7 +1165,9 @@ sph_status wait_event(sph_server *S, cudaEvent_t ev)
         if (e != cudaErrorNotReady) return sfail(SPH_ERR_CUDA, std::string("event: ") + cudaGetErrorString(e));
         const double el = now_s() - t0;
         if (el > S->timeout_s) return sfail(SPH_ERR_TIMEOUT, "device did not finish within the wait limit");
-        std::this_thread::sleep_for(std::chrono::microseconds(el < 0.01 ? 20 : 200));
+        // polls at first, then sleeps about 1 % of the time waited (as the single events' wait)
+        if (el < 0.001) std::this_thread::yield();
+        else std::this_thread::sleep_for(std::chrono::microseconds((long long)std::min(200.0, std::max(20.0, 1e4 * el))));
     }
 }
 
