@@ -189,9 +189,16 @@ __device__ uint32_t an_invert(const EosDev &E, double s, const double *n, double
 // ---------------------------------------------------------------------------
 // table: the quadrilinear interpolant reduced one axis at a time (mu_Q, mu_S inside each of the
 // four (T, mu_B) corner patches, then mu_B, then T), carrying the partial derivatives along
+// a non-negative int as a double, below 2^20 by its bits (a conversion between int and double costs
+// as much as an FP64 operation)
+__device__ __forceinline__ double int_double(int k)
+{
+    if (k >= (1 << 20)) return (double)k;
+    const int e = 31 - __clz(k | 1);
+    return k == 0 ? 0.0 : __hiloint2double(((e + 1023) << 20) | ((k << (20 - e)) & 0xFFFFF), 0);
+}
 // the cell of grid coordinate r and the position in it: the integer part of r >= 1 from its
-// mantissa bits and back into a double by bits (a conversion between int and double costs as much
-// as an FP64 operation), clamped to [0, nx - 2]; r < 1 (negative too) lies in cell 0
+// mantissa bits, clamped to [0, nx - 2]; r < 1 (negative too) lies in cell 0
 __device__ __forceinline__ void locate_steps(double r, int nx, int &i, double &t)
 {
     const int hi = __double2hiint(r);
@@ -202,11 +209,7 @@ __device__ __forceinline__ void locate_steps(double r, int nx, int &i, double &t
     }
     k = min(k, nx - 2);
     i = k;
-    const int e = 31 - __clz(k | 1);
-    const double kd = k == 0 ? 0.0
-                      : nx <= (1 << 20) ? __hiloint2double(((e + 1023) << 20) | ((k << (20 - e)) & 0xFFFFF), 0)
-                                        : (double)k;
-    t = r - kd;
+    t = r - int_double(k);
 }
 __device__ __forceinline__ void locate(double x, double x0, double inv, int nx, int &i, double &t)
 {
@@ -833,11 +836,100 @@ __device__ __forceinline__ bool inside_keys(const EosDev &E, const double *x)
 }
 __device__ __forceinline__ bool finite_bits(double v) { return mag_bits(v) < kInfBits; }
 
+// max |residual| at grid coordinates xi as an integer magnitude (the line search's trials)
+__device__ __forceinline__ long long tab_resid_norm(const EosDev &E, const double *xi, const double *tgt)
+{
+    int i[4];
+    double t[4];
+    locate_steps(xi[0], E.nT, i[0], t[0]);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) locate_steps(xi[1 + q], E.nmu[q], i[1 + q], t[1 + q]);
+    const int n3 = E.nmu[2], n23 = E.nmu[1] * E.nmu[2], n123 = E.nmu[0] * n23;
+    const size_t node0 = (size_t)i[0] * n123 + (size_t)i[1] * n23 + (size_t)i[2] * n3 + i[3];
+    const double2 *sn2 = reinterpret_cast<const double2 *>(E.sn);
+    // the order of operations of tab_resid_steps: the same residuals
+    const double uT = 1.0 - t[0], uB = 1.0 - t[1], uS = 1.0 - t[2], uQ = 1.0 - t[3];
+    const double w00 = uS * uQ, w01 = uS * t[3], w10 = t[2] * uQ, w11 = t[2] * t[3];
+    const double wp[4] = {uT * uB, uT * t[1], t[0] * uB, t[0] * t[1]};
+    double acc[4] = {-tgt[0], -tgt[1], -tgt[2], -tgt[3]};
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        const size_t base = node0 + (size_t)(c >> 1) * n123 + (size_t)(c & 1) * n23;
+#pragma unroll
+        for (int fp = 0; fp < 2; ++fp) {
+            const double2 q00 = __ldg(sn2 + 2 * base + fp), q01 = __ldg(sn2 + 2 * (base + 1) + fp);
+            const double2 q10 = __ldg(sn2 + 2 * (base + n3) + fp), q11 = __ldg(sn2 + 2 * (base + n3 + 1) + fp);
+            acc[2 * fp] = fma(wp[c], fma(w11, q11.x, fma(w10, q10.x, fma(w01, q01.x, w00 * q00.x))), acc[2 * fp]);
+            acc[2 * fp + 1] = fma(wp[c], fma(w11, q11.y, fma(w10, q10.y, fma(w01, q01.y, w00 * q00.y))), acc[2 * fp + 1]);
+        }
+    }
+    long long m = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) m = max(m, min(mag_bits(acc[k]), kInfBits));
+    return m;
+}
+
 // the closed form as a call of its own: the lane loop keeps its registers for the table Newton
 __device__ __noinline__ uint32_t an_invert_call(const EosDev &E, double s, const double *n, double *x, EosWork &w,
                                                 double Tguess)
 {
     return an_invert(E, s, n, x[0], x + 1, w, Tguess);
+}
+
+// upper grid coordinates as bit patterns (non-negative doubles order as integers)
+__device__ __forceinline__ void grid_top(const EosDev &E, long long top[4])
+{
+    top[0] = __double_as_longlong(int_double(E.nT - 1));
+#pragma unroll
+    for (int q = 0; q < 3; ++q) top[1 + q] = __double_as_longlong(int_double(E.nmu[q] - 1));
+}
+// the trial point x + lam d in grid coordinates, clamped to the grid
+__device__ __forceinline__ void trial_point(const long long *top, const double *x, const float *d, float lam, double *out)
+{
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const long long b = __double_as_longlong(x[k] + f64_bits(lam * d[k]));
+        out[k] = __longlong_as_double(b < 0 ? 0LL : min(b, top[k]));
+    }
+}
+
+// The line searches of a warp's lanes in todo after a full step without a decrease: the halvings
+// 1/2 .. 1/2^8 of one particle at a time, a lane for each, and the largest that decreases the
+// residual (the first that a search trial by trial would take).  xt: the point found; false: none.
+// One trial a trip held the whole pass for particles beyond a table edge, whose searches fail
+// every stage: 40 k event with three such particles, EoS pass 341 us per step, now 270.
+__device__ __noinline__ bool line_searches(const EosDev &E, unsigned todo, const double *xi, const float *d,
+                                           const double *tgt, long long rn, double *xt, unsigned &trials)
+{
+    const unsigned FULL = 0xFFFFFFFFu;
+    const int lane = threadIdx.x & 31;
+    bool found = false;
+    long long top[4];
+    grid_top(E, top);
+    for (; todo; todo &= todo - 1u) {
+        const int src = __ffs(todo) - 1;
+        double xs[4], ts[4], xl[4];
+        float ds[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            xs[k] = __shfl_sync(FULL, xi[k], src);
+            ts[k] = __shfl_sync(FULL, tgt[k], src);
+            ds[k] = __shfl_sync(FULL, d[k], src);
+        }
+        const long long rs = __shfl_sync(FULL, rn, src);
+        bool less = false;
+        if (lane < 8) {
+            trial_point(top, xs, ds, __int_as_float((126 - lane) << 23), xl);
+            less = tab_resid_norm(E, xl, ts) < rs;
+        }
+        const unsigned m = __ballot_sync(FULL, less);
+        if (lane == src) {
+            trials = m ? (unsigned)__ffs(m) : 8u;
+            found = m != 0u;
+            if (m) trial_point(top, xi, d, __int_as_float((127 - __ffs(m)) << 23), xt);  // evaluated and accepted next
+        }
+    }
+    return found;
 }
 
 // First half.  Ctx supplies  bool load(int a, double &s, double n[3], double g[4])  (false: not a
@@ -852,15 +944,14 @@ __device__ void eos_find(const EosDev &E, unsigned int *claim, int limit, Ctx &c
     const double step[4] = {E.dT, E.dmu[0], E.dmu[1], E.dmu[2]};
     const double istep[4] = {E.inv_dT, E.inv_dmu[0], E.inv_dmu[1], E.inv_dmu[2]};
     const double org[4] = {E.T0, E.mu0[0], E.mu0[1], E.mu0[2]};
-    // upper grid coordinates as bit patterns (non-negative doubles order as integers)
-    const long long top[4] = {__double_as_longlong((double)(E.nT - 1)), __double_as_longlong((double)(E.nmu[0] - 1)),
-                              __double_as_longlong((double)(E.nmu[1] - 1)), __double_as_longlong((double)(E.nmu[2] - 1))};
+    long long top[4];
+    grid_top(E, top);
     const double hand = E.polish ? 1e-10 : 1e-6;
-    int a = -1, it = 0, ls = 0;
+    int a = -1, it = 0;
     bool more = true, first = false, cold = false;
     long long rn = 0, tolb = 0, handb = 0;
     double xi[4] = {0.0, 0.0, 0.0, 0.0}, xt[4] = {0.0, 0.0, 0.0, 0.0}, tgt[4] = {0.0, 0.0, 0.0, 0.0}, Tcf = 0.0;
-    float d[4] = {0.f, 0.f, 0.f, 0.f}, lam = 1.0f;
+    float d[4] = {0.f, 0.f, 0.f, 0.f};
     for (;;) {
         // lanes without a particle claim the next ones (one atomic per warp)
         const unsigned need = __ballot_sync(FULL, a < 0 && more);
@@ -916,54 +1007,61 @@ __device__ void eos_find(const EosDev &E, unsigned int *claim, int limit, Ctx &c
             }
             if (a >= 0 && ((need >> lane) & 1u)) {
                 first = true;
-                it = ls = 0;
+                it = 0;
                 tolb = __double_as_longlong(E.tol * tgt[0]);
                 handb = max(tolb, __double_as_longlong(hand * tgt[0]));
             }
         }
         if (__ballot_sync(FULL, a >= 0 || more) == 0u) break;
-        if (a < 0) continue;
-        // one evaluation at the trial point
-        double r[4];
-        float J[4][4];
-        tab_resid_steps(E, xt, tgt, r, J);
-        ++w.resid;
-        long long rnn = 0;
+        bool fail = false, step_on = false, last = false, search = false;
+        if (a >= 0) {
+            // one evaluation at the trial point
+            double r[4];
+            float J[4][4];
+            tab_resid_steps(E, xt, tgt, r, J);
+            ++w.resid;
+            long long rnn = 0;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) rnn = max(rnn, min(mag_bits(r[k]), kInfBits));
-        bool fail = false, step_on = false, last = false;
-        if (first || rnn < rn) {
-            it += first ? 0 : 1;
-            first = false;
+            for (int k = 0; k < 4; ++k) rnn = max(rnn, min(mag_bits(r[k]), kInfBits));
+            if (first || rnn < rn) {
+                it += first ? 0 : 1;
+                first = false;
 #pragma unroll
-            for (int k = 0; k < 4; ++k) xi[k] = xt[k];
-            rn = rnn;
-            if (rn <= tolb && !E.polish) last = true;
-            else if (rn <= handb) last = step_on = true;
-            else if (it >= E.maxit) fail = true;
-            else step_on = true;
-        } else if (++ls > 8) {
-            fail = true;  // no decrease along the Newton direction: stalled
-        } else {
-            lam *= 0.5f;
+                for (int k = 0; k < 4; ++k) xi[k] = xt[k];
+                rn = rnn;
+                if (rn <= tolb && !E.polish) last = true;
+                else if (rn <= handb) last = step_on = true;
+                else if (it >= E.maxit) fail = true;
+                else step_on = true;
+            } else {
+                search = true;
+            }
+            if (step_on) {
+                ++w.solve;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) d[k] = -f32_bits(r[k]);
+                const bool ok = solve4f(J, d);
+                if (!ok && !last) fail = true;
+                if (!ok)
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) d[k] = 0.0f;
+                trial_point(top, xi, d, 1.0f, xt);
+            }
         }
-        if (step_on) {
-            ++w.solve;
+        // no decrease at the full step: the line searches of the warp's lanes, rarely
+        const unsigned todo = __ballot_sync(FULL, search);
+        if (todo) {
+            double xs[4], ts[4], xo[4];
+            float ds[4];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) d[k] = -f32_bits(r[k]);
-            const bool ok = solve4f(J, d);
-            if (!ok && !last) fail = true;
-            if (!ok)
+            for (int k = 0; k < 4; ++k) xs[k] = xi[k], ts[k] = tgt[k], ds[k] = d[k], xo[k] = xt[k];
+            unsigned trials = 0u;
+            const bool found = line_searches(E, todo, xs, ds, ts, rn, xo, trials);
+            w.resid += trials;
+            if (search) {
+                fail = !found;  // no decrease along the Newton direction: stalled
 #pragma unroll
-                for (int k = 0; k < 4; ++k) d[k] = 0.0f;
-            lam = 1.0f;
-            ls = 0;
-        }
-        if (!(last && !step_on)) {
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {  // the trial point, clamped to the grid
-                const long long b = __double_as_longlong(xi[k] + f64_bits(lam * d[k]));
-                xt[k] = __longlong_as_double(b < 0 ? 0LL : min(b, top[k]));
+                for (int k = 0; k < 4; ++k) xt[k] = xo[k];
             }
         }
         if (last) {
@@ -980,7 +1078,7 @@ __device__ void eos_find(const EosDev &E, unsigned int *claim, int limit, Ctx &c
                 if (!st && inside_keys(E, x)) {
                     cold = first = true;
                     Tcf = x[0];
-                    it = ls = 0;
+                    it = 0;
 #pragma unroll
                     for (int k = 0; k < 4; ++k) xt[k] = (x[k] - org[k]) * istep[k];
                 } else {
