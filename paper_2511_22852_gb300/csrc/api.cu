@@ -197,6 +197,7 @@ static EvView make_view(const sph_event *ev)
     v.dout = ev->dout;
     v.fxX = ev->cb.pl.total > 0 ? ev->cb.pl.X : nullptr;
     v.fxE = ev->cb.pl.Xe;
+    v.fX = ev->cb.fx;
     return v;
 }
 
@@ -643,9 +644,9 @@ sph_status sph_init_event(sph_event **out, const sph_event_desc *d, const sph_eo
     AL(ev->cb.perm, sizeof(uint32_t) * N);
     if (ev->dim == 2) AL(ev->cb.fpos, sizeof(float2) * N);
     else AL(ev->cb.fpos3, sizeof(float4) * N);
-    if (ev->dim == 3 && ev->mixed) {
+    if (ev->mixed) {
         AL(ev->cb.fq, sizeof(float4) * N);
-        AL(ev->cb.fx, sizeof(float4) * 3 * N);
+        AL(ev->cb.fx, (ev->dim == 3 ? 3 * sizeof(float4) : sizeof(float4) + sizeof(float2)) * N);
     }
     AL(ev->cb.part, sizeof(uint32_t) * (size_t)(ev->cb.nb / 4096 + 2));
     if (ev->dim == 3) AL(ev->spread, sizeof(uint32_t) * 3 * 1024);

@@ -236,6 +236,10 @@ __device__ __forceinline__ double eos2_store(const EvView &v, int stage, size_t 
     for (int k = 0; k < 4; ++k) gin[k * n + a] = X[k];
     gin[4 * n + a] = us[0];
     gin[5 * n + a] = us[1];
+    if (LIMBS && v.fX) {  // in single precision for the mixed form's
+        v.fX[a] = make_float4((float)X[0], (float)X[1], (float)X[2], (float)X[3]);
+        reinterpret_cast<float2 *>(v.fX + n)[a] = make_float2((float)us[0], (float)us[1]);
+    }
     if (LIMBS && v.fxX) {  // the same in limbs for the pair-list gradient pass
         const int eX = fx_shared_exponent(X), eu = fx_shared_exponent(us);
         v.fxX[a] = fx_limbs2(X[0], eX, X[1], eX);

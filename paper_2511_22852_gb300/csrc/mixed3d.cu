@@ -58,18 +58,6 @@ __global__ void k_relpos3(EvView v, const double *__restrict__ y, const double *
     fq[j] = make_float4((float)y[6 * n + j], (float)Nq[j], (float)Nq[n + j], (float)Nq[2 * n + j]);
 }
 
-// the gradient pass's inputs in FP32: rows 4 m .. 4 m + 3 of gin in fx[m n ..]
-__global__ void k_fx3(int n_, const double *__restrict__ gin, float4 *__restrict__ fx)
-{
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= n_) return;
-    const size_t n = (size_t)n_;
-#pragma unroll
-    for (int m = 0; m < 3; ++m)
-        fx[m * n + j] = make_float4((float)gin[(4 * m) * n + j], (float)gin[(4 * m + 1) * n + j],
-                                    (float)gin[(4 * m + 2) * n + j], (float)gin[(4 * m + 3) * n + j]);
-}
-
 constexpr int kWW = 8;                // warps per block, two particles each
 constexpr unsigned kFull = 0xFFFFFFFFu;
 
@@ -375,7 +363,6 @@ void launch_density3m(const EvView &v, const double *y, const double *Nq, CellBu
 void launch_gradient3m(const EvView &v, int stage, const double *y, const double *gin, CellBufs cb, double *gout,
                        cudaStream_t st)
 {
-    k_fx3<<<nblk(v.n, 256), 256, 0, st>>>(v.n, gin, cb.fx);
     k_walk_gradient3m<<<nblk(v.n, 2 * kWW), 32 * kWW, 0, st>>>(v, stage, y, cb.fpos3, gin, cb.fx, cb.start, cb.cnt,
                                                                gout);
 }

@@ -136,6 +136,10 @@ struct EvView {
     // (PairBufs X, Xe; nullptr: lists off)
     int4 *fxX;
     unsigned int *fxE;
+    // mixed forms: where the EoS pass leaves the gradient-pass inputs in single precision: 2D
+    // [n] float4 (X^{xx}, X^{xy}, X^{yx}, X^{yy}) and [n] float2 (u^x, u^y) behind it, 3D
+    // planes [3][n] of four rows each
+    float4 *fX;
 };
 constexpr int kJRow = 9;  // first state row of the diffusion currents (2+1D)
 
@@ -409,7 +413,7 @@ struct CellBufs {
     uint32_t *key, *cnt, *start, *cursor, *tmp, *perm;
     float2 *fpos;   // 2D: sorted positions relative to the bounding-box minimum, single precision
     float4 *fpos3;  // 3D: the same with three coordinates, w: the packed cell coordinates
-    float4 *fq, *fx;  // mixed 3D: (S, N_B, N_S, N_Q) and the gradient inputs [3][n] in single precision
+    float4 *fq, *fx;  // mixed: (S, N_B, N_S, N_Q) and the gradient inputs in single precision
     uint32_t *part; // scan partial sums (multi-block scan of large bucket tables)
     int nb;         // number of buckets: 1 << (2 B) in 2D, 1 << (B3[0] + B3[1] + B3[2]) in 3D
     PairBufs pl;    // plain 2D: half-pair lists (pl.total = 0: off)

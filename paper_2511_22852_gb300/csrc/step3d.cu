@@ -338,6 +338,11 @@ __global__ void __launch_bounds__(64, 5) k_eos3_finish(EvView v, int stage, cons
             us[j] = u[1 + j] * isig;
             gin[(size_t)(9 + j) * n + a] = us[j];
         }
+        if (v.fX) {  // in single precision for the mixed form's
+            v.fX[a] = make_float4((float)X[0], (float)X[1], (float)X[2], (float)X[3]);
+            v.fX[n + a] = make_float4((float)X[4], (float)X[5], (float)X[6], (float)X[7]);
+            v.fX[2 * n + a] = make_float4((float)X[8], (float)us[0], (float)us[1], (float)us[2]);
+        }
         if (v.fxX) {  // the same in limbs for the pair-list gradient pass
             const int eX = fx_shared_exponent(X), eu = fx_shared_exponent(us);
 #pragma unroll
