@@ -78,6 +78,8 @@ struct sph_event {
     int diff = 0;
     double kapT2[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0}, tauJT[3] = {0, 0, 0};
     double *dinp = nullptr, *dal = nullptr, *dout = nullptr;
+    int4 *dfx = nullptr;
+    uint4 *dfe = nullptr;
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     DevScalars *sc = nullptr;
@@ -195,6 +197,8 @@ static EvView make_view(const sph_event *ev)
     v.dinp = ev->dinp;
     v.dal = ev->dal;
     v.dout = ev->dout;
+    v.dfx = ev->dfx;
+    v.dfe = ev->dfe;
     v.fxX = ev->cb.pl.total > 0 ? ev->cb.pl.X : nullptr;
     v.fxE = ev->cb.pl.Xe;
     v.fX = ev->cb.fx;
@@ -370,7 +374,6 @@ static sph_status check_device_flags(sph_event *ev, DevScalars *hs)
         ev->pair_ovf_seen = hs->pair_ovf;
         ev->pairs_grow = true;
     }
-    if (hs->err_flags & ERR_PAIR_LIST) return fail(SPH_ERR_STATE, "inconsistent neighbour pair lists");
     if (hs->err_flags & ERR_CELL_OVERFLOW)
         return fail(SPH_ERR_STATE, "particles spread beyond the cell table fixed at sph_init_event");
     uint32_t bad = hs->status_or & ev->fatal_mask;
@@ -670,6 +673,10 @@ sph_status sph_init_event(sph_event **out, const sph_event_desc *d, const sph_eo
         AL(ev->dinp, dv * 9);
         AL(ev->dal, dv * 12);
         AL(ev->dout, dv * 9);
+        if (!ev->mixed) {
+            AL(ev->dfx, sizeof(int4) * 5 * N);
+            AL(ev->dfe, sizeof(uint4) * N);
+        }
         ev->charges = true;
     }
     AL(ev->ntot, sizeof(double) * (8 + 3 * 256));
@@ -758,8 +765,8 @@ static sph_status size_pair_lists(sph_event *ev)
     if (ev->pairs_grow) total = std::max<long long>(total, ev->cb.pl.total * 3 / 2);
     else if (const char *t = getenv("SPH_PAIR_TOTAL")) total = std::max<long long>(1, atoll(t));
     const int nparts = (n + 2047) / 2048;
-    // per entry: L, P (int), W and the kernel gradient (2 or 3 doubles)
-    const size_t per_entry = 2 * sizeof(int) + (1 + (size_t)ev->dim) * sizeof(double);
+    // per entry: L (int), W and the kernel gradient (2 or 3 64-bit integers)
+    const size_t per_entry = sizeof(int) + (1 + (size_t)ev->dim) * sizeof(double);
     // per particle: two counts and two carried counts, the values in limbs and their exponents
     const int nx = ev->dim == 2 ? 3 : 6;  // planes of the gradient-pass inputs
     const size_t per_particle = 5 * sizeof(int) + 4 * sizeof(unsigned short) + (size_t)(2 + nx) * sizeof(int4);
@@ -799,8 +806,7 @@ static sph_status size_pair_lists(sph_event *ev)
     pl.part = reinterpret_cast<unsigned long long *>(pl.off + (n + 1));
     pl.Qe = reinterpret_cast<unsigned short *>(pl.part + nparts);  // read 8 bytes at a time
     pl.L = reinterpret_cast<int *>(pl.Qe + 4 * (size_t)n);
-    pl.P = pl.L + total;
-    pl.cntF = pl.P + total;
+    pl.cntF = pl.L + total;
     pl.cntB = pl.cntF + n;
     ev->pcnt[0] = pl.cntB + n;
     ev->pcnt[1] = ev->pcnt[0] + n;

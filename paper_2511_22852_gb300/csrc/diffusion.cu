@@ -20,6 +20,7 @@ namespace sphg {
 namespace {
 
 constexpr int kDiffWarps = 4;
+constexpr unsigned kFull = 0xFFFFFFFFu;
 
 __global__ void __launch_bounds__(128) k_diff_prep(EvView v, int stage, const double *__restrict__ y,
                                                    const double *__restrict__ dens, const double *__restrict__ eos,
@@ -39,14 +40,30 @@ __global__ void __launch_bounds__(128) k_diff_prep(EvView v, int stage, const do
     const bool ok = !(st & (PST_NOCONV | PST_NONFINITE)) && T > 0.0;
     const double i2 = 1.0 / (sig_star * sig_star);
     double al[3];
+    double Fq[3][2];
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
         const double Jx = sigma * y[(kJRow + 2 * q) * n + a], Jy = sigma * y[(kJRow + 2 * q + 1) * n + a];
         const double J0 = (ux * Jx + uy * Jy) / u0;
         al[q] = ok ? eos[(1 + q) * n + a] / T : 0.0;
         v.dinp[q * n + a] = al[q];
-        v.dinp[(3 + 2 * q) * n + a] = (Jx - vx * J0) * i2;
-        v.dinp[(4 + 2 * q) * n + a] = (Jy - vy * J0) * i2;
+        Fq[q][0] = (Jx - vx * J0) * i2;
+        Fq[q][1] = (Jy - vy * J0) * i2;
+        v.dinp[(3 + 2 * q) * n + a] = Fq[q][0];
+        v.dinp[(4 + 2 * q) * n + a] = Fq[q][1];
+    }
+    if (v.dfx) {  // the same in limbs for the pair-list pass
+        int ea[3], ef[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            ea[q] = fx_exponent(al[q]);
+            ef[q] = fx_shared_exponent(Fq[q]);
+            v.dfx[(2 + q) * n + a] = fx_limbs2(Fq[q][0], ef[q], Fq[q][1], ef[q]);
+        }
+        v.dfx[a] = fx_limbs2(al[0], ea[0], al[1], ea[1]);
+        v.dfx[n + a] = fx_limbs2(al[2], ea[2], 0.0, ea[2]);
+        v.dfe[a] = make_uint4((unsigned)ea[0] | ((unsigned)ea[1] << 16), (unsigned)ea[2] | ((unsigned)ef[0] << 16),
+                              (unsigned)ef[1] | ((unsigned)ef[2] << 16), 0u);
     }
     double dal[3][4];
 #pragma unroll
@@ -142,47 +159,124 @@ __device__ __forceinline__ void diff_finish(const EvView &v, int stage, const do
     }
 }
 
-// pair-list form (plain 2D events): one warp per particle over its accepted pairs, with the
-// kernel gradient the density pass stored per pair (grad_a W_ab h / sigma_d: b > a forward in
-// a's row, b < a as minus the entry in b's row), so no distance or kernel is evaluated again
-__global__ void __launch_bounds__(32 * kDiffWarps) k_diff_pairs(EvView v, int stage, const double *__restrict__ dens,
-                                                                PairBufs pl)
+// pair-list form (plain 2D events): half a warp per particle over the entries of its row with the
+// kernel gradient stored there (grad_a W_ab h / sigma_d), in integers (pairs_fixed.cuh): alpha_b -
+// alpha_a is formed in units of the neighbours' largest alpha (zero for a uniform alpha), the fluxes
+// are summed as the gradient pass sums the stresses.
+// Bound: the latency of the gathers; 40 k event, diffusion and EoS passes per step 1,561 -> 860 us
+// (17 FP64 operations per pair before).
+__global__ void __launch_bounds__(32 * kDiffWarps, 4) k_diff_pairs(EvView v, int stage, const double *__restrict__ dens,
+                                                                   PairBufs pl)
 {
     if (v.sc->pair_flag) return;  // a list overflowed: the cell pass runs instead
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int a = blockIdx.x * kDiffWarps + wid;
-    if (a >= v.n) return;  // warp-uniform
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, l = lane & 15;
+    const long long ap = 2 * ((long long)blockIdx.x * kDiffWarps + wid) + (lane >> 4);
+    if (ap - (lane >> 4) >= v.n) return;  // warp-uniform
+    const bool on = ap < v.n;
+    const int a = on ? (int)ap : v.n - 1;
     const size_t n = (size_t)v.n;
-    const double *al = v.dinp, *F = v.dinp + 3 * n;
-    const double aa[3] = {al[a], al[n + a], al[2 * n + a]};
-    const long long r0 = pl.off[a], rend = pl.off[a + 1] - 1;
-    const int nf = pl.cntF[a], nt = nf + pl.cntB[a];
-    double ga[3][2] = {{0.0, 0.0}, {0.0, 0.0}, {0.0, 0.0}}, dv[3] = {0.0, 0.0, 0.0}, Gx = 0.0, Gy = 0.0;
-    for (int j = lane; j < nt; j += 32) {
-        int b;
-        double gx, gy;
-        if (j < nf) {
-            b = pl.L[r0 + j];
-            const longlong2 g = pl.G[r0 + j];
-            gx = from_fixed(g.x);
-            gy = from_fixed(g.y);
-        } else {
-            b = pl.L[rend - (j - nf)];
-            const longlong2 g = pl.G[pl.off[b] + pl.P[rend - (j - nf)]];
-            gx = from_fixed(-g.x);
-            gy = from_fixed(-g.y);
-        }
-        Gx += gx;
-        Gy += gy;
+    const long long r0 = pl.off[a], r1 = pl.off[a + 1];
+    const int nf = on ? pl.cntF[a] : 0, nt = on ? nf + pl.cntB[a] : 0;
+    auto at = [&](int j) { return j < nf ? r0 + j : r1 - nt + j; };  // entry j of a's row
+    uint4 em = v.dfe[a];
+    for (int j = l; j < nt; j += 16) {
+        const uint4 e = v.dfe[pl.L[at(j)]];
+        em = make_uint4(fx_max2(em.x, e.x), fx_max2(em.y, e.y), fx_max2(em.z, e.z), 0u);
+    }
+    em = make_uint4(fx_half_max2(em.x), fx_half_max2(em.y), fx_half_max2(em.z), 0u);
+    const int m[6] = {(int)(em.x & 0xFFFFu), (int)(em.x >> 16), (int)(em.y & 0xFFFFu),
+                      (int)(em.y >> 16), (int)(em.z & 0xFFFFu), (int)(em.z >> 16)};
+    int E[6];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        E[q] = fx_room(m[q] + 1, nt);  // the difference of two values
+        E[3 + q] = fx_room(m[3 + q], nt);
+    }
+    // a value's mantissa in units of 2^(E - 1076)
+    auto mantissa = [](int2 q, int d) { return ((long long)q.x * (1LL << kLimb) + q.y) >> min(d, 63); };
+    long long ma[3];
+    {
+        const int4 x0 = v.dfx[a], x1 = v.dfx[n + a];
+        const uint4 e = v.dfe[a];
+        ma[0] = mantissa(lo_of(x0), E[0] - (int)(e.x & 0xFFFFu));
+        ma[1] = mantissa(hi_of(x0), E[1] - (int)(e.x >> 16));
+        ma[2] = mantissa(lo_of(x1), E[2] - (int)(e.y & 0xFFFFu));
+    }
+    FxSum sG[2] = {{0, 0}, {0, 0}}, sA[3][2], sF[3];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) sA[q][0] = sA[q][1] = sF[q] = FxSum{0, 0};
+    auto fold = [&]() {
+        fx_fold(sG[0]);
+        fx_fold(sG[1]);
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
-            const double da = al[q * n + b] - aa[q];
-            ga[q][0] = fma(da, gx, ga[q][0]);
-            ga[q][1] = fma(da, gy, ga[q][1]);
-            dv[q] = fma(F[(2 * q) * n + b], gx, fma(F[(2 * q + 1) * n + b], gy, dv[q]));
+            fx_fold(sA[q][0]);
+            fx_fold(sA[q][1]);
+            fx_fold(sF[q]);
+        }
+    };
+    for (int j = l, it = 1; j < nt; j += 16, ++it) {
+        const long long i = at(j);
+        const int b = pl.L[i];
+        const longlong2 g = pl.G[i];
+        const int4 x0 = v.dfx[b], x1 = v.dfx[n + b];
+        const uint4 e = v.dfe[b];
+        const int eb[6] = {(int)(e.x & 0xFFFFu), (int)(e.x >> 16), (int)(e.y & 0xFFFFu),
+                           (int)(e.y >> 16), (int)(e.z & 0xFFFFu), (int)(e.z >> 16)};
+        const int2 al[3] = {lo_of(x0), hi_of(x0), lo_of(x1)};
+        sG[0].x += g.x;
+        sG[1].x += g.y;
+        int gxh, gxl, gyh, gyl;
+        fx_split(g.x, 0, gxh, gxl);
+        fx_split(g.y, 0, gyh, gyl);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const long long d = mantissa(al[q], E[q] - eb[q]) - ma[q];
+            const int lo = (int)((unsigned)d << (32 - kLimb)) >> (32 - kLimb);
+            const int2 da = make_int2((int)((d - lo) >> kLimb), lo);
+            fx_add(sA[q][0], gxh, gxl, da);
+            fx_add(sA[q][1], gyh, gyl, da);
+            const int4 F = v.dfx[(2 + q) * n + b];
+            int hi, lo2;
+            fx_split(g.x, E[3 + q] - eb[3 + q], hi, lo2);
+            fx_add(sF[q], hi, lo2, lo_of(F));
+            fx_split(g.y, E[3 + q] - eb[3 + q], hi, lo2);
+            fx_add(sF[q], hi, lo2, hi_of(F));
+        }
+        if ((it & (kFoldEvery - 1)) == 0) fold();
+    }
+    fold();
+    FxTotal t[16];
+    t[0] = fx_words(sG[0]);
+    t[1] = fx_words(sG[1]);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        t[2 + 2 * q] = fx_words(sA[q][0]);
+        t[3 + 2 * q] = fx_words(sA[q][1]);
+        t[8 + q] = fx_words(sF[q]);
+    }
+#pragma unroll
+    for (int k = 11; k < 16; ++k) t[k] = FxTotal{0, 0};
+    const FxTotal tt = fx_reduce16(t, lane);
+    // lane l: 0, 1 sum grad W; 2 + 2 q + i sum (alpha_b - alpha_a) grad_i W; 8 + q sum F_b . grad W
+    const int q = l < 8 ? (l - 2) >> 1 : l - 8;
+    const int Eq = l < 8 ? (q <= 0 ? E[0] : (q == 1 ? E[1] : E[2])) : (q == 0 ? E[3] : (q == 1 ? E[4] : E[5]));
+    const int mq = l < 8 ? (q <= 0 ? m[0] : (q == 1 ? m[1] : m[2])) : (q == 0 ? m[3] : (q == 1 ? m[4] : m[5]));
+    double tot = fx_value(tt, l < 2 ? -kFxBits : fx_unit(Eq));
+    if (l >= 2 && mq == kNonFinite) tot = fx_nan();
+    const double Gx = __shfl_sync(kFull, tot, lane & 16), Gy = __shfl_sync(kFull, tot, (lane & 16) + 1);
+    if (on && l >= 2 && l < 11) {
+        const double c = v.sigma_d * v.inv_h;
+        if (l < 8) {
+            v.dout[(size_t)(l - 2) * n + a] = c * tot * (1.0 / dens[a]);
+        } else {
+            const double tau = v.sc->tau + (stage == 2 ? v.dtau : 0.0);
+            const double sqrtg = v.milne ? tau : 1.0;
+            const double *F = v.dinp + 3 * n;
+            const double div = F[(2 * q) * n + a] * Gx + F[(2 * q + 1) * n + a] * Gy + tot;
+            v.dout[(6 + q) * n + a] = -sqrtg * c * div;
         }
     }
-    diff_finish(v, stage, dens, a, lane, Gx, Gy, ga, dv);
 }
 
 // one warp per particle: the 3x3 cells of side 2h around its own, the exact FP64 test r < 2h on
@@ -248,7 +342,7 @@ void launch_diffusion(const EvView &v, int stage, const double *y, const double 
     // the plain form keeps pair lists: the pass over them, with the cell pass standing by (at a
     // few blocks per SM) for a stage whose lists overflowed
     const int lists = !v.mixed && cb.pl.total > 0;
-    if (lists) k_diff_pairs<<<nblk(v.n, kDiffWarps), 32 * kDiffWarps, 0, st>>>(v, stage, dens, cb.pl);
+    if (lists) k_diff_pairs<<<nblk(v.n, 2 * kDiffWarps), 32 * kDiffWarps, 0, st>>>(v, stage, dens, cb.pl);
     const int grid = lists ? std::min(nblk(v.n, kDiffWarps), 8 * device_sm_count()) : nblk(v.n, kDiffWarps);
     k_diff2<<<grid, 32 * kDiffWarps, 0, st>>>(v, stage, y, dens, cb.start, cb.cnt, lists);
 }

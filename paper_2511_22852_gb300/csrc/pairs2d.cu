@@ -9,7 +9,7 @@
 // depend on the order, so results are reproducible run to run.
 //
 // FP64 operations per unordered pair fall from 56 (26 for the kernel, 10 for the density and 20 for
-// the gradient sums of its two particles) to 12; the 40 k event's step 2,038 -> 1,536 us.
+// the gradient sums of its two particles) to 12; the 40 k event's step 2,038 -> 1,310 us.
 //
 // Rows: a particle's row holds its previous neighbour count plus a margin (a prefix scan per
 // stage); forward entries fill it from the start, backward entries from the end.
@@ -22,29 +22,6 @@ namespace {
 
 constexpr int kWarps = 4;  // particles (warps) per block
 constexpr unsigned kFull = 0xFFFFFFFFu;
-
-// cells of the 3x3 block around (cx, cy) inside the grid, in ascending Morton key, so that their
-// particles come in ascending sorted index
-__device__ __forceinline__ int block_cells_ascending(int cx, int cy, int lim, uint32_t keys[9])
-{
-    int nk = 0;
-    for (int oy = -1; oy <= 1; ++oy) {
-        const int ny = cy + oy;
-        if (ny < 0 || ny >= lim) continue;
-        for (int ox = -1; ox <= 1; ++ox) {
-            const int nx = cx + ox;
-            if (nx < 0 || nx >= lim) continue;
-            const uint32_t k = morton2((uint32_t)nx, (uint32_t)ny);
-            int j = nk++;
-            while (j > 0 && keys[j - 1] > k) {
-                keys[j] = keys[j - 1];
-                --j;
-            }
-            keys[j] = k;
-        }
-    }
-    return nk;
-}
 
 // ---------------------------------------------------------------------------
 // Row offsets: row j (sorted order) holds cnt_src[perm[j]] - 1 + margin entries (the previous
@@ -127,19 +104,25 @@ __global__ void __launch_bounds__(kScanThreads) k_rows_apply(int n, const uint32
     long long run = (long long)pl.part[blockIdx.x] + wbase + incl - t;
 #pragma unroll
     for (int k = 0; k < kScanPer; ++k) {
-        if (base + k < n) pl.off[base + k] = run;
+        if (base + k < n) {
+            pl.off[base + k] = run;
+            pl.cntB[base + k] = 0;  // counted up by the forward pass
+        }
         run += v[k];
     }
 }
 
-// Forward pass, a warp for two particles a.  Candidates of the 3x3 cells pass the
-// single-precision prefilter; a neighbour b < a is decided at once (exact FP64 test when the
-// float test left it undecided) and listed from the row end; a candidate b > a is queued, and 32
-// at a time -- of both particles -- the exact test, the distance in FP64 and the spline in 64-bit
-// integers run on full warps, and W and grad W are listed with the pair in fixed point (L, W, G).  The particles' own values go into limbs.
+// Forward pass, a warp for two particles a.  Candidates of the cells from its own on pass the
+// single-precision prefilter; a candidate b > a is queued, and 32 at a time -- of both particles --
+// the exact test (where the float test left the pair undecided), the distance in FP64 and the
+// spline in 64-bit integers run on full warps.  W and grad W go in fixed point into a's row and,
+// at a place taken from b's counter, into b's row.  The particles' own values go into limbs.
+// (Listing b < a in a's own walk, and finding its W by a search in b's row, kept the sums waiting
+// for memory: 40 k event, sum pass 197 -> 92 us a stage, gradient
+// pass 150 -> 137; 258 k particles in 3+1D 2.5 -> 0.9 and 3.4 -> 2.6 ms.)
 // Bound: the FP64 pipe, 12 operations per unordered pair (31 with spline and kernel sums in FP64, a
-// reduction per particle and its own partial batch).  40 k event: 220 us a stage, its
-// FP64 pipe then 325 us before the spline left it.
+// reduction per particle and its own partial batch).  40 k event: 214 us a stage (325
+// with the spline in FP64).
 __global__ void __launch_bounds__(32 * kWarps, 8) k_pairs_fwd(EvView v, const double *__restrict__ y,
                                                            const float2 *__restrict__ fpos,
                                                            const double *__restrict__ Nq,
@@ -164,7 +147,7 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_pairs_fwd(EvView v, const do
     const unsigned lt = (1u << lane) - 1u;
     double xa[2], ya[2];
     long long r0[2];
-    int cap[2], nf[2] = {0, 0}, nbk[2] = {0, 0}, qn = 0;
+    int cap[2], nf[2] = {0, 0}, qn = 0;
 #pragma unroll
     for (int p = 0; p < 2; ++p) {
         const int a = (int)a0 + (p < np ? p : 0);
@@ -195,11 +178,18 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_pairs_fwd(EvView v, const do
                 spline_fixed(q, w, dw);
             }
             const int slot = second ? nf[1] + __popc(m1 & lt) : nf[0] + __popc(m0 & lt);
+            const longlong2 g = make_longlong2(grad_fixed(dw, dx * ir), grad_fixed(dw, dy * ir));
             if (slot < (second ? cap[1] : cap[0])) {
                 const long long i = (second ? r0[1] : r0[0]) + slot;
                 pl.L[i] = b;
                 pl.W[i] = w;
-                pl.G[i] = make_longlong2(grad_fixed(dw, dx * ir), grad_fixed(dw, dy * ir));
+                pl.G[i] = g;
+            }
+            const long long i = pl.off[b + 1] - 1 - atomicAdd(&pl.cntB[b], 1);
+            if (i >= pl.off[b] && pl.off[b + 1] <= pl.total) {
+                pl.L[i] = (int)a0 + (second ? 1 : 0);
+                pl.W[i] = w;
+                pl.G[i] = make_longlong2(-g.x, -g.y);
             }
         }
         nf[0] += __popc(m0);
@@ -211,36 +201,25 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_pairs_fwd(EvView v, const do
         const int a = (int)a0 + p, flag = p << 30;
         const float2 fa = fpos[a];
         const uint32_t ka = key[perm[a]];
-        const int cx = (int)unspread2(ka), cy = (int)unspread2(ka >> 1);
-        uint32_t keys[9];
-        const int nk = block_cells_ascending(cx, cy, 1 << v.B, keys);
-        int *Bl = pl.L + (r0[p] + cap[p] - 1);  // backward down from the row end
-        for (int kc = 0; kc < nk; ++kc) {
-            const uint32_t k = keys[kc];
+        const int cx = (int)unspread2(ka), cy = (int)unspread2(ka >> 1), lim = 1 << v.B;
+        for (int o = 0; o < 9; ++o) {
+            const int nx = cx + o % 3 - 1, ny = cy + o / 3 - 1;
+            if (nx < 0 || ny < 0 || nx >= lim || ny >= lim) continue;
+            const uint32_t k = morton2((uint32_t)nx, (uint32_t)ny);
+            if (k < ka) continue;  // all of its particles come before a
             const uint32_t b0 = start[k], b1 = b0 + cnt[k];
-            for (uint32_t base = b0; base < b1; base += 32) {
+            for (uint32_t base = k == ka ? (uint32_t)a + 1u : b0; base < b1; base += 32) {
                 const uint32_t b = base + lane;
                 bool cand = false, sure = false;
-                if (b < b1 && b != (uint32_t)a) {
+                if (b < b1 && (int)b > a) {
                     const float2 fb = fpos[b];
                     const float dx = fa.x - fb.x, dy = fa.y - fb.y;
                     const float r2f = fmaf(dx, dx, dy * dy);
                     cand = r2f <= v.supp2_hi;
                     sure = r2f < v.supp2_lo;
                 }
-                // b < a: decided here and listed; its pair values come from b's own forward pass
-                bool accB = false;
-                if (cand && (int)b < a) accB = sure || dist2_2d(xa[p] - X[b], ya[p] - Y[b]) < v.supp2;
-                const unsigned mb = __ballot_sync(kFull, accB);
-                if (accB) {
-                    const int slot = nbk[p] + __popc(mb & lt);
-                    if (slot < cap[p]) Bl[-slot] = (int)b;
-                }
-                nbk[p] += __popc(mb);
-                // b > a: queued in arrival (ascending) order for the FP64 pair arithmetic
-                const bool fw = cand && (int)b > a;
-                const unsigned m = __ballot_sync(kFull, fw);
-                if (fw) q[qn + __popc(m & lt)] = (int)(b | (sure ? 0u : 0x80000000u)) | flag;
+                const unsigned m = __ballot_sync(kFull, cand);
+                if (cand) q[qn + __popc(m & lt)] = (int)(b | (sure ? 0u : 0x80000000u)) | flag;
                 qn += __popc(m);
                 __syncwarp();
                 if (qn >= 32) {
@@ -254,22 +233,13 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_pairs_fwd(EvView v, const do
         }
     }
     if (qn > 0) forward(lane < qn ? q[lane] : 0, lane < qn);
-    if (lane == 0) {
-        bool over = false;
-        for (int p = 0; p < np; ++p) {
-            pl.cntF[a0 + p] = nf[p];
-            pl.cntB[a0 + p] = nbk[p];
-            over = over || nf[p] + nbk[p] > cap[p];
-        }
-        if (over) atomicOr(&v.sc->pair_flag, 1u);  // the two ends met: lists unusable
-    }
+    if (lane == 0)
+        for (int p = 0; p < np; ++p) pl.cntF[a0 + p] = nf[p];
 }
 
-// Density sums, half a warp per particle a, over its pairs b > a (forward entries of a's row) and
-// b < a (the entry of a in b's ascending forward list, found by binary search; the slot is kept in
-// P for the gradient pass), in integers (pairs_fixed.cuh).
-// Bound: the latency of the searches and of the gathers (L1 hits 78 %); 40 k event 197 us a stage,
-// 3+1D event of 258 k particles 2.5 ms.  More or larger blocks per SM changed nothing (191-229 us).
+// Density sums, half a warp per particle a, over the entries of its row, in integers
+// (pairs_fixed.cuh).
+// Bound: the latency of the gathers; 40 k event 92 us a stage, 3+1D event of 258 k particles 0.92 ms.
 __global__ void __launch_bounds__(32 * kWarps, 7) k_pairs_sum(EvView v, PairBufs pl, double *__restrict__ dens,
                                                            int *__restrict__ nnb)
 {
@@ -280,17 +250,19 @@ __global__ void __launch_bounds__(32 * kWarps, 7) k_pairs_sum(EvView v, PairBufs
     const bool on = ap < v.n;
     const int a = on ? (int)ap : v.n - 1;
     const size_t n = (size_t)v.n;
-    const long long r0 = pl.off[a], rend = pl.off[a + 1] - 1;  // backward entries: rend, rend - 1, ...
-    const int nf = on ? pl.cntF[a] : 0, nt = on ? nf + pl.cntB[a] : 0;
+    const long long r0 = pl.off[a], r1 = pl.off[a + 1];
+    const int nf = on ? pl.cntF[a] : 0, nb = on ? pl.cntB[a] : 0, nt = nf + nb;
+    // the two ends met: the row does not hold a's entries (all listed values are pair values all the
+    // same), and the per-particle passes run
+    if (l == 0 && nt > (r1 <= pl.total ? (int)min(r1 - r0, (long long)nt) : 0)) atomicOr(&v.sc->pair_flag, 1u);
+    const int fit = r1 <= pl.total && r1 - r0 >= nt ? nt : 0;
+    // entry j of a's row
+    auto at = [&](int j) { return j < nf ? r0 + j : r1 - nt + j; };
     const uint2 *Qe = reinterpret_cast<const uint2 *>(pl.Qe);
     // the largest exponents among a and its neighbours (S | N_B << 16, N_S | N_Q << 16)
     uint2 em = Qe[a];
-    for (int j = l; j < nf; j += 16) {
-        const uint2 e = Qe[pl.L[r0 + j]];
-        em = make_uint2(fx_max2(em.x, e.x), fx_max2(em.y, e.y));
-    }
-    for (int j = l; j < nt - nf; j += 16) {
-        const uint2 e = Qe[pl.L[rend - j]];
+    for (int j = l; j < fit; j += 16) {
+        const uint2 e = Qe[pl.L[at(j)]];
         em = make_uint2(fx_max2(em.x, e.x), fx_max2(em.y, e.y));
     }
     em = make_uint2(fx_half_max2(em.x), fx_half_max2(em.y));
@@ -326,35 +298,12 @@ __global__ void __launch_bounds__(32 * kWarps, 7) k_pairs_sum(EvView v, PairBufs
         }
     };
     if (l == 0 && on) add2(a, 1LL << kFxBits, a, 0);  // the self pair, W(0) = 1
-    for (int j = l; j < nf; j += 32) {
-        const bool two = j + 16 < nf;
-        const int b0 = pl.L[r0 + j], b1 = two ? pl.L[r0 + j + 16] : a;
-        const long long w0 = pl.W[r0 + j], w1 = two ? pl.W[r0 + j + 16] : 0;
+    for (int j = l; j < fit; j += 32) {
+        const bool two = j + 16 < fit;
+        const long long i0 = at(j), i1 = at(j + 16);
+        const int b0 = pl.L[i0], b1 = two ? pl.L[i1] : a;
+        const long long w0 = pl.W[i0], w1 = two ? pl.W[i1] : 0;
         add2(b0, w0, b1, w1);
-    }
-    for (int j = l; j < nt - nf; j += 32) {
-        const bool two = j + 16 < nt - nf;
-        const int b0 = pl.L[rend - j], b1 = two ? pl.L[rend - j - 16] : a;
-        const long long rb0 = pl.off[b0], rb1 = pl.off[b1];
-        const int n0 = pl.cntF[b0], n1 = two ? pl.cntF[b1] : 0;
-        SlotSearch f0 = {pl.L + rb0, 0, n0}, f1 = {pl.L + rb1, 0, n1};
-        while (f0.open() || f1.open()) {
-            f0.step(a);
-            f1.step(a);
-        }
-        // both sides take the same acceptance decision (the float and the exact test see
-        // exactly negated differences), so a is in b's list; checked all the same
-        if (f0.base >= n0 || f0.F[f0.base] != a) {
-            atomicOr(&v.sc->err_flags, ERR_PAIR_LIST);
-            f0.base = 0;
-        }
-        if (two && (f1.base >= n1 || f1.F[f1.base] != a)) {
-            atomicOr(&v.sc->err_flags, ERR_PAIR_LIST);
-            f1.base = 0;
-        }
-        pl.P[rend - j] = f0.base;
-        if (two) pl.P[rend - j - 16] = f1.base;
-        add2(b0, n0 > 0 ? pl.W[rb0 + f0.base] : 0, b1, n1 > 0 ? pl.W[rb1 + f1.base] : 0);
     }
     fx_fold(sg);
     FxTotal t[8];
@@ -383,10 +332,9 @@ __global__ void __launch_bounds__(32 * kWarps, 7) k_pairs_sum(EvView v, PairBufs
     if (lane == 0) atomicAdd(&v.sc->pairs, (unsigned long long)c2);
 }
 
-// Gradient pass, half a warp per particle a, over its pairs b > a (forward entries of a's row, with
-// G = grad_a W_ab h / sigma_d) and then b < a (backward entries: -G of the pair in b's row, slot
-// P), forming in integers the sums of the per-particle pass: sum grad W, sum X_b grad W, sum u_b grad W.
-// Bound: the latency of the gathers; 40 k event 150 us a stage (298 us with 10 FP64 operations per
+// Gradient pass, half a warp per particle a, over the entries of its row with G = grad_a W_ab h /
+// sigma_d, forming in integers the sums of the per-particle pass: sum grad W, sum X_b grad W, sum u_b grad W.
+// Bound: the latency of the gathers; 40 k event 137 us a stage (298 us with 10 FP64 operations per
 // pair).  Two entries at a time: 150 against 173 us; 5 blocks per SM: 6 gave 161, 8 150, 10 193.
 __global__ void __launch_bounds__(32 * kWarps, 5) k_pairs_gradient(EvView v, int stage, const double *__restrict__ gin,
                                                                 PairBufs pl, double *__restrict__ gout)
@@ -398,12 +346,12 @@ __global__ void __launch_bounds__(32 * kWarps, 5) k_pairs_gradient(EvView v, int
     const bool on = ap < v.n;
     const int a = on ? (int)ap : v.n - 1;
     const size_t n = (size_t)v.n;
-    const long long r0 = pl.off[a], rend = pl.off[a + 1] - 1;
+    const long long r0 = pl.off[a], r1 = pl.off[a + 1];
     const int nf = on ? pl.cntF[a] : 0, nt = on ? nf + pl.cntB[a] : 0;
+    auto at = [&](int j) { return j < nf ? r0 + j : r1 - nt + j; };  // entry j of a's row
     // the largest exponents among a and its neighbours (stress | u << 16)
     unsigned em = pl.Xe[a];
-    for (int j = l; j < nf; j += 16) em = fx_max2(em, pl.Xe[pl.L[r0 + j]]);
-    for (int j = l; j < nt - nf; j += 16) em = fx_max2(em, pl.Xe[pl.L[rend - j]]);
+    for (int j = l; j < nt; j += 16) em = fx_max2(em, pl.Xe[pl.L[at(j)]]);
     em = fx_half_max2(em);
     const int EX = fx_room((int)(em & 0xFFFFu), nt), EU = fx_room((int)(em >> 16), nt);
     const bool bad = (em & 0xFFFFu) == kNonFinite || (em >> 16) == kNonFinite;
@@ -449,17 +397,10 @@ __global__ void __launch_bounds__(32 * kWarps, 5) k_pairs_gradient(EvView v, int
         if ((it & (kFoldEvery - 1)) == 0) fold();
     };
     const longlong2 zero = make_longlong2(0, 0);
-    for (int j = l; j < nf; j += 32) {
-        const bool two = j + 16 < nf;
-        const int b0 = pl.L[r0 + j], b1 = two ? pl.L[r0 + j + 16] : a;
-        add2(b0, pl.G[r0 + j], b1, two ? pl.G[r0 + j + 16] : zero);
-    }
-    for (int j = l; j < nt - nf; j += 32) {  // grad_a W_ab = -grad_b W_ba, stored with b's forward pair
-        const bool two = j + 16 < nt - nf;
-        const int b0 = pl.L[rend - j], b1 = two ? pl.L[rend - j - 16] : a;
-        const int s0 = pl.P[rend - j], s1 = two ? pl.P[rend - j - 16] : 0;
-        const longlong2 g0 = pl.G[pl.off[b0] + s0], g1 = two ? pl.G[pl.off[b1] + s1] : zero;
-        add2(b0, make_longlong2(-g0.x, -g0.y), b1, make_longlong2(-g1.x, -g1.y));
+    for (int j = l; j < nt; j += 32) {
+        const bool two = j + 16 < nt;
+        const long long i0 = at(j), i1 = at(j + 16);
+        add2(pl.L[i0], pl.G[i0], two ? pl.L[i1] : a, two ? pl.G[i1] : zero);
     }
     fold();
     FxTotal t[8] = {fx_words(sG[0]), fx_words(sG[1]), fx_words(sH[0]), fx_words(sH[1]),

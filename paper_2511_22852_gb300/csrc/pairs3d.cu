@@ -1,8 +1,8 @@
 // pairs3d.cu -- plain 3D neighbour passes over half-pair lists: the 3D counterpart of the plain
-// 2D passes (the same rows, ordering and fallback), over the 27 cells of the generalized Morton
-// table.  Per accepted pair the forward density pass evaluates W and grad W once (both depend on
-// r_ab only; grad_b W_ba = -grad_a W_ab) and keeps them with the pair; the backward pass and the
-// gradient pass add every pair to both of its particles.  Sums in a fixed order: reproducible.
+// 2D passes (the same rows and fallback), over the 27 cells of the generalized Morton table.  Per
+// accepted pair the forward pass evaluates W and grad W once (both depend on r_ab only; grad_b W_ba
+// = -grad_a W_ab) and keeps them in fixed point in both particles' rows; the sum and gradient passes
+// add them in integers (pairs_fixed.cuh), independent of the order: reproducible.
 #include "pairs_fixed.cuh"
 #include "sph_internal.cuh"
 
@@ -13,39 +13,15 @@ namespace {
 constexpr int kWarps = 4;
 constexpr unsigned kFull = 0xFFFFFFFFu;
 
-// the cells of the 3x3x3 block inside the grid, in ascending key (their particles then come in
-// ascending sorted index)
-__device__ __forceinline__ int block27_ascending(const EvView &v, const int c[3], uint32_t keys[27])
-{
-    int nk = 0;
-    for (int oz = -1; oz <= 1; ++oz) {
-        const int nz = c[2] + oz;
-        if (nz < 0 || nz >= (1 << v.B3[2])) continue;
-        for (int oy = -1; oy <= 1; ++oy) {
-            const int ny = c[1] + oy;
-            if (ny < 0 || ny >= (1 << v.B3[1])) continue;
-            for (int ox = -1; ox <= 1; ++ox) {
-                const int nx = c[0] + ox;
-                if (nx < 0 || nx >= (1 << v.B3[0])) continue;
-                const uint32_t k = key3(v, nx, ny, nz);
-                int j = nk++;
-                while (j > 0 && keys[j - 1] > k) {
-                    keys[j] = keys[j - 1];
-                    --j;
-                }
-                keys[j] = k;
-            }
-        }
-    }
-    return nk;
-}
-
-// Forward pass, a warp for two particles a.  Candidates of the 27 cells pass the
-// single-precision prefilter; a neighbour b < a is decided at once (exact FP64 test when the
-// float test left it undecided) and listed from the row end; a candidate b > a is queued, and 32
-// at a time -- of both particles -- the exact test, the distance in FP64 and the spline in 64-bit
-// integers run on full warps, and W and grad W are listed with the pair in fixed point (L, W, G).  The particles' own values go into limbs.
-// Bound: the FP64 pipe, 15 operations per unordered pair.  258 k particles: 4.0 ms a stage
+// Forward pass, a warp for two particles a.  Candidates of the cells from its own on pass the
+// single-precision prefilter; a candidate b > a is queued, and 32 at a time -- of both particles --
+// the exact test (where the float test left the pair undecided), the distance in FP64 and the
+// spline in 64-bit integers run on full warps.  W and grad W go in fixed point into a's row and,
+// at a place taken from b's counter, into b's row.  The particles' own values go into limbs.
+// (Listing b < a in a's own walk, and finding its W by a search in b's row, kept the sums waiting
+// for memory: 40 k event, sum pass 197 -> 92 us a stage, gradient
+// pass 150 -> 137; 258 k particles in 3+1D 2.5 -> 0.9 and 3.4 -> 2.6 ms.)
+// Bound: the FP64 pipe, 15 operations per unordered pair.  258 k particles: 3.5 ms a stage
 // (4.6 with the spline in FP64).
 __global__ void __launch_bounds__(32 * kWarps, 8) k_pairs3_fwd(EvView v, const double *__restrict__ y,
                                                            const float4 *__restrict__ fpos,
@@ -69,7 +45,7 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_pairs3_fwd(EvView v, const d
     const unsigned lt = (1u << lane) - 1u;
     double xa[2], ya[2], za[2];
     long long r0[2];
-    int cap[2], nf[2] = {0, 0}, nbk[2] = {0, 0}, qn = 0;
+    int cap[2], nf[2] = {0, 0}, qn = 0;
 #pragma unroll
     for (int p = 0; p < 2; ++p) {
         const int a = (int)a0 + (p < np ? p : 0);
@@ -102,13 +78,20 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_pairs3_fwd(EvView v, const d
                 spline_fixed(q, w, dw);
             }
             const int slot = second ? nf[1] + __popc(m1 & lt) : nf[0] + __popc(m0 & lt);
+            const long long g[3] = {grad_fixed(dw, dx * ir), grad_fixed(dw, dy * ir), grad_fixed(dw, dz * ir)};
             if (slot < (second ? cap[1] : cap[0])) {
                 const long long i = (second ? r0[1] : r0[0]) + slot;
                 pl.L[i] = b;
                 pl.W[i] = w;
-                pl.G3[3 * i] = grad_fixed(dw, dx * ir);
-                pl.G3[3 * i + 1] = grad_fixed(dw, dy * ir);
-                pl.G3[3 * i + 2] = grad_fixed(dw, dz * ir);
+#pragma unroll
+                for (int k = 0; k < 3; ++k) pl.G3[3 * i + k] = g[k];
+            }
+            const long long i = pl.off[b + 1] - 1 - atomicAdd(&pl.cntB[b], 1);
+            if (i >= pl.off[b] && pl.off[b + 1] <= pl.total) {
+                pl.L[i] = (int)a0 + (second ? 1 : 0);
+                pl.W[i] = w;
+#pragma unroll
+                for (int k = 0; k < 3; ++k) pl.G3[3 * i + k] = -g[k];
             }
         }
         nf[0] += __popc(m0);
@@ -121,35 +104,25 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_pairs3_fwd(EvView v, const d
         const float4 fa = fpos[a];
         const int ca = __float_as_int(fa.w);  // the packed cell coordinates
         const int c[3] = {ca & 1023, (ca >> 10) & 1023, (ca >> 20) & 1023};
-        uint32_t keys[27];
-        const int nk = block27_ascending(v, c, keys);
-        int *Bl = pl.L + (r0[p] + cap[p] - 1);  // backward down from the row end
-        for (int kc = 0; kc < nk; ++kc) {
-            const uint32_t k = keys[kc];
+        const uint32_t ka = key3(v, c[0], c[1], c[2]);
+        for (int o = 0; o < 27; ++o) {
+            const int nx = c[0] + o % 3 - 1, ny = c[1] + (o / 3) % 3 - 1, nz = c[2] + o / 9 - 1;
+            if (nx < 0 || ny < 0 || nz < 0 || nx >= (1 << v.B3[0]) || ny >= (1 << v.B3[1]) || nz >= (1 << v.B3[2])) continue;
+            const uint32_t k = key3(v, nx, ny, nz);
+            if (k < ka) continue;  // all of its particles come before a
             const uint32_t b0 = start[k], b1 = b0 + cnt[k];
-            for (uint32_t base = b0; base < b1; base += 32) {
+            for (uint32_t base = k == ka ? (uint32_t)a + 1u : b0; base < b1; base += 32) {
                 const uint32_t b = base + lane;
                 bool cand = false, sure = false;
-                if (b < b1 && b != (uint32_t)a) {
+                if (b < b1 && (int)b > a) {
                     const float4 fb = fpos[b];
                     const float dx = fa.x - fb.x, dy = fa.y - fb.y, dz = fa.z - fb.z;
                     const float r2f = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
                     cand = r2f <= v.supp2_hi;
                     sure = r2f < v.supp2_lo;
                 }
-                // b < a: decided here and listed; its pair values come from b's own forward pass
-                bool accB = false;
-                if (cand && (int)b < a) accB = sure || dist2_3d(xa[p] - X[b], ya[p] - Y[b], za[p] - Z[b]) < v.supp2;
-                const unsigned mb = __ballot_sync(kFull, accB);
-                if (accB) {
-                    const int slot = nbk[p] + __popc(mb & lt);
-                    if (slot < cap[p]) Bl[-slot] = (int)b;
-                }
-                nbk[p] += __popc(mb);
-                // b > a: queued in arrival (ascending) order for the FP64 pair arithmetic
-                const bool fw = cand && (int)b > a;
-                const unsigned m = __ballot_sync(kFull, fw);
-                if (fw) q[qn + __popc(m & lt)] = (int)(b | (sure ? 0u : 0x80000000u)) | flag;
+                const unsigned m = __ballot_sync(kFull, cand);
+                if (cand) q[qn + __popc(m & lt)] = (int)(b | (sure ? 0u : 0x80000000u)) | flag;
                 qn += __popc(m);
                 __syncwarp();
                 if (qn >= 32) {
@@ -163,21 +136,13 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_pairs3_fwd(EvView v, const d
         }
     }
     if (qn > 0) forward(lane < qn ? q[lane] : 0, lane < qn);
-    if (lane == 0) {
-        bool over = false;
-        for (int p = 0; p < np; ++p) {
-            pl.cntF[a0 + p] = nf[p];
-            pl.cntB[a0 + p] = nbk[p];
-            over = over || nf[p] + nbk[p] > cap[p];
-        }
-        if (over) atomicOr(&v.sc->pair_flag, 1u);  // the two ends met: lists unusable
-    }
+    if (lane == 0)
+        for (int p = 0; p < np; ++p) pl.cntF[a0 + p] = nf[p];
 }
 
-// Gradient pass, half a warp per particle a, over its pairs b > a (stored grad_a W_ab) and b < a
-// (minus the stored grad_b W_ba), in integers (pairs_fixed.cuh): sum grad W (3), sum X_b^{j i}
+// Gradient pass, half a warp per particle a, over the entries of its row, in integers (pairs_fixed.cuh): sum grad W (3), sum X_b^{j i}
 // grad_j W (3), sum u_b^j grad_k W (9); the epilogue as the per-particle pass.
-// Bound: the latency of the gathers; 258 k particles: 3.4 ms a stage (6.0 with 21 FP64 operations per
+// Bound: the latency of the gathers; 258 k particles: 2.6 ms a stage (6.0 with 21 FP64 operations per
 // pair).  4 blocks per SM: 3 gave 3.7, 5 3.8, 6 4.8 ms.
 __global__ void __launch_bounds__(32 * kWarps, 4) k_pairs3_gradient(EvView v, int stage, const double *__restrict__ gin,
                                                                  PairBufs pl, double *__restrict__ gout)
@@ -189,12 +154,12 @@ __global__ void __launch_bounds__(32 * kWarps, 4) k_pairs3_gradient(EvView v, in
     const bool on = ap < v.n;
     const int a = on ? (int)ap : v.n - 1;
     const size_t n = (size_t)v.n;
-    const long long r0 = pl.off[a], rend = pl.off[a + 1] - 1;
+    const long long r0 = pl.off[a], r1 = pl.off[a + 1];
     const int nf = on ? pl.cntF[a] : 0, nt = on ? nf + pl.cntB[a] : 0;
+    auto at = [&](int j) { return j < nf ? r0 + j : r1 - nt + j; };  // entry j of a's row
     // the largest exponents among a and its neighbours (stress | u << 16)
     unsigned em = pl.Xe[a];
-    for (int j = l; j < nf; j += 16) em = fx_max2(em, pl.Xe[pl.L[r0 + j]]);
-    for (int j = l; j < nt - nf; j += 16) em = fx_max2(em, pl.Xe[pl.L[rend - j]]);
+    for (int j = l; j < nt; j += 16) em = fx_max2(em, pl.Xe[pl.L[at(j)]]);
     em = fx_half_max2(em);
     const int EX = fx_room((int)(em & 0xFFFFu), nt), EU = fx_room((int)(em >> 16), nt);
     const bool bad = (em & 0xFFFFu) == kNonFinite || (em >> 16) == kNonFinite;
@@ -215,18 +180,12 @@ __global__ void __launch_bounds__(32 * kWarps, 4) k_pairs3_gradient(EvView v, in
     auto entry = [&](int j, int &b, long long (&g)[3]) {
         b = a;
         g[0] = g[1] = g[2] = 0;
-        if (j < nf) {
-            b = pl.L[r0 + j];
-            const long long *q = pl.G3 + 3 * (r0 + j);
-            g[0] = q[0];
-            g[1] = q[1];
-            g[2] = q[2];
-        } else if (j < nt) {
-            b = pl.L[rend - (j - nf)];
-            const long long *q = pl.G3 + 3 * (pl.off[b] + pl.P[rend - (j - nf)]);
-            g[0] = -q[0];
-            g[1] = -q[1];
-            g[2] = -q[2];
+        if (j < nt) {
+            const long long i = at(j);
+            b = pl.L[i];
+            g[0] = pl.G3[3 * i];
+            g[1] = pl.G3[3 * i + 1];
+            g[2] = pl.G3[3 * i + 2];
         }
     };
     int b1;

@@ -88,16 +88,6 @@ __device__ __forceinline__ long long grad_fixed(long long dw, double e)
     return (__mul64hi(dw, to_fixed<62>(e)) + 4) >> 3;
 }
 
-// a fixed-point kernel value as a double (truncated to 53 bits, without FP64 operations)
-__device__ __forceinline__ double from_fixed(long long f)
-{
-    const unsigned long long m = f < 0 ? -(unsigned long long)f : (unsigned long long)f;
-    const int lz = __clzll((long long)m);
-    const unsigned long long n = m << (lz & 63);  // leading one at bit 63
-    const unsigned long long bits = ((unsigned long long)(1023 - kFxBits + 63 - lz) << 52) | ((n >> 11) & 0xFFFFFFFFFFFFFULL);
-    return m == 0ull ? 0.0 : __longlong_as_double((long long)(bits | ((unsigned long long)f & 0x8000000000000000ULL)));
-}
-
 // biased exponent of v (zero and denormals: 1), kNonFinite for infinities and NaN
 __device__ __forceinline__ int fx_exponent(double v)
 {
@@ -227,22 +217,5 @@ __device__ __forceinline__ int4 fx_limbs2(double v0, int e0, double v1, int e1)
 }
 __device__ __forceinline__ int2 lo_of(int4 v) { return make_int2(v.x, v.y); }
 __device__ __forceinline__ int2 hi_of(int4 v) { return make_int2(v.z, v.w); }
-
-// first slot of the ascending list F[0 .. len) whose entry is not below a
-struct SlotSearch {
-    const int *F;
-    int base, len;
-    __device__ __forceinline__ bool open() const { return len > 0; }
-    __device__ __forceinline__ void step(int a)
-    {
-        const int half = (len + 1) >> 1;  // len = 1 decides the last entry
-        if (len > 0 && F[base + half - 1] < a) {
-            base += half;
-            len -= half;
-        } else {
-            len = half - 1;
-        }
-    }
-};
 
 }  // namespace sphg

@@ -29,7 +29,6 @@ constexpr uint32_t PST_FALLBACK = 1u, PST_OUT_OF_TABLE = 2u, PST_NOCONV = 4u, PS
                    PST_CS2_CAPPED = 16u, PST_SOLVE_FAIL = 32u, PST_BACKUP = 64u;
 // event-level device error bits
 constexpr uint32_t ERR_CELL_OVERFLOW = 1u;
-constexpr uint32_t ERR_PAIR_LIST = 2u;  // a backward pair missing from its partner's forward list
 
 constexpr int kNDens = 6, kNEos = 11, kNGin = 6, kNGout = 6;
 
@@ -132,6 +131,10 @@ struct EvView {
     int diff;
     double kapT2[9], tauJT[3];
     double *dinp, *dal, *dout;
+    // plain form: dinp in limbs for the pair-list pass, planes of [n] int4: alpha_B, alpha_S |
+    // alpha_Q | flux of B, S, Q (x, y); the exponents of alpha_q and flux_q in 16 bits each
+    int4 *dfx;
+    uint4 *dfe;
     // pair lists (plain forms): where the EoS pass leaves the gradient-pass inputs in limbs
     // (PairBufs X, Xe; nullptr: lists off)
     int4 *fxX;
@@ -377,13 +380,13 @@ __device__ __forceinline__ void warp_or(unsigned int *dst, unsigned int v)
 // ---------------------------------------------------------------------------
 // launchers (implemented in cells.cu, density_eos.cu, gradient_eom.cu)
 // Half-pair lists of the plain 2D neighbour passes, rebuilt in every stage's density pass.
-// Particle a (sorted index) owns entries [off[a], off[a+1]) of L, P, W, FAC, sized by its
+// Particle a (sorted index) owns entries [off[a], off[a+1]) of L, W, G, sized by its
 // neighbour count of the previous stage plus a margin (a prefix scan per stage):
-//   from the row start: its accepted neighbours b > a, ascending (L), with W(r)/sigma_d of the
-//      pair (W) and grad_a W_ab h/sigma_d = (dW/dr)/r (x_a - x_b) h/sigma_d (G); both are
-//      computed once per pair (W is symmetric in a, b; grad_b W_ba = -grad_a W_ab);
-//   from the row end, downwards: its accepted neighbours b < a, ascending (L), with the slot of
-//      the pair (b, a) in b's row (P).
+//   from the row start: its accepted neighbours b > a (L), with W(r)/sigma_d of the pair (W) and
+//      grad_a W_ab h/sigma_d = (dW/dr)/r (x_a - x_b) h/sigma_d (G); both are computed once per
+//      pair, by the warp of a (W is symmetric in a, b; grad_b W_ba = -grad_a W_ab);
+//   from the row end, downwards: its accepted neighbours b < a in any order (the sums are in
+//      integers and do not depend on it), with W and -G, written by the warps of the b.
 // A particle whose neighbours exceed its row (or rows beyond the allocation) flags the stage,
 // which then runs the per-particle passes; the counts it records size the next stage's rows.
 // total = 0: lists off (the per-particle passes run).
@@ -394,7 +397,7 @@ struct PairBufs {
     int *cnt_dst;                 // this stage's counts, sorted order (NULL: not recorded)
     long long *off;               // [n + 1] row offsets of this stage
     unsigned long long *part;     // scan partial sums
-    int *L, *P, *cntF, *cntB;
+    int *L, *cntF, *cntB;
     // kernel value W/sigma_d and gradient h grad W/sigma_d of the pair in units of 2^-57
     // (pairs_fixed.cuh)
     long long *W;
