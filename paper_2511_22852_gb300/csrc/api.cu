@@ -199,7 +199,7 @@ static EvView make_view(const sph_event *ev)
     v.dout = ev->dout;
     v.dfx = ev->dfx;
     v.dfe = ev->dfe;
-    v.fxX = ev->cb.pl.total > 0 ? ev->cb.pl.X : nullptr;
+    v.fxX = ev->cb.pl.total > 0 && !ev->mixed ? ev->cb.pl.X : nullptr;
     v.fxE = ev->cb.pl.Xe;
     v.fX = ev->cb.fx;
     return v;
@@ -721,18 +721,22 @@ sph_status sph_init_event(sph_event **out, const sph_event_desc *d, const sph_eo
     return SPH_OK;
 }
 
-// Sizes (or grows) the half-pair lists of the plain passes (2D and 3D).  Each stage gives particle a a row
-// of (its previous neighbour count - 1 + margin) entries; the allocation holds 1.5 x those rows
-// for the current state (at least 1.5 x the old allocation when growing), margin = 32.  Counts
-// are carried from stage to stage in the state order (pcnt[0] with Y[0], pcnt[1] with Y1[0]);
-// here they are taken from a read-out evaluation of the current state.  The lists stay off (the
-// per-particle passes run) for other forms, when SPH_PAIR_LISTS=0, or when they would take more
-// than a quarter of the free device memory.  SPH_PAIR_MARGIN and SPH_PAIR_TOTAL override the
+// Sizes (or grows) the half-pair lists of the plain passes (2D and 3D) and the neighbour lists of
+// the mixed 3+1D ones (indices alone).  Each stage gives particle a a row of (its previous
+// neighbour count - 1 + margin) entries; the allocation holds 1.5 x those rows for the current
+// state (at least 1.5 x the old allocation when growing), margin = 32.  Counts are carried from
+// stage to stage in the state order (pcnt[0] with Y[0], pcnt[1] with Y1[0]); here they are taken
+// from a read-out evaluation of the current state.  The lists stay off (the per-particle passes
+// run) for other forms, when SPH_PAIR_LISTS=0, or when they would take more than a quarter of the
+// free device memory.  SPH_PAIR_MARGIN and SPH_PAIR_TOTAL override the
 // margin and the first allocation (tests of the overflow paths).
 static sph_status size_pair_lists(sph_event *ev)
 {
-    if (ev->pairs_off || ev->mixed || ev->n == 0) return SPH_OK;
-    if (ev->n > (1 << 30)) ev->pairs_off = true;  // the passes pack an index and two flags in a word
+    if (ev->pairs_off || ev->n == 0 || (ev->mixed && ev->dim == 2)) return SPH_OK;
+    // the passes pack an index and two flags (mixed: the neighbour cell's number) in a word.  In the
+    // mixed 2+1D form lists gain nothing: 40,000 particles of the table background, density +
+    // gradient 362 us a step with them and 368 without (its walk is short)
+    if (ev->n > (ev->mixed ? 1 << 27 : 1 << 30)) ev->pairs_off = true;
     if (ev->pairs_off) return SPH_OK;
     if (ev->cb.pl.total > 0 && ev->pair_ovf_host && *ev->pair_ovf_host > ev->pair_ovf_seen) {
         ev->pair_ovf_seen = *ev->pair_ovf_host;
@@ -747,29 +751,36 @@ static sph_status size_pair_lists(sph_event *ev)
     const int n = ev->n;
     int margin = 32;
     if (const char *t = getenv("SPH_PAIR_MARGIN")) margin = std::max(0, atoi(t));
-    // neighbour counts of the current state, moved from the evaluation's sorted order to the state
-    // order (the sort's gather map: sorted j <- state perm[j])
+    // neighbour counts of the current state: a read-out evaluation leaves them in its sorted order (moved
+    // to the state order below), and its pair counter gives their sum
+    DevScalars before, after;
+    sph_status s = fetch(ev, &before, ev->sc, sizeof(before));
+    if (s != SPH_OK) return s;
     enqueue_observe(ev);
     CK(cudaGetLastError());
     ev->observed = true;
-    std::vector<int> cnt(n), perm(n), state(n);
-    sph_status s = fetch(ev, cnt.data(), ev->nnb, sizeof(int) * (size_t)n);
-    if (s != SPH_OK) return s;
-    if ((s = fetch(ev, perm.data(), ev->cb.perm, sizeof(int) * (size_t)n)) != SPH_OK) return s;
-    long long rows = 0;
-    for (int j = 0; j < n; ++j) {
-        state[perm[j]] = cnt[j];
-        rows += std::max(cnt[j] - 1, 0) + margin;
+    if ((s = fetch(ev, &after, ev->sc, sizeof(after))) != SPH_OK) return s;
+    const long long rows = (long long)(after.pairs - before.pairs) - n + (long long)margin * n;
+    if (ev->mixed) {  // the mixed form's totals count its steps' and read-outs' work alone
+        after.pairs = before.pairs;
+        after.eos_resid = before.eos_resid;
+        after.eos_solve = before.eos_solve;
+        after.eos_g = before.eos_g;
+        after.shell_tests = before.shell_tests;
+        CK(cudaMemcpyAsync(ev->sc, &after, sizeof(after), cudaMemcpyHostToDevice, ev->stream));
+        if ((s = wait_stream(ev)) != SPH_OK) return s;
     }
     long long total = rows * 3 / 2 + 1024;
     if (ev->pairs_grow) total = std::max<long long>(total, ev->cb.pl.total * 3 / 2);
     else if (const char *t = getenv("SPH_PAIR_TOTAL")) total = std::max<long long>(1, atoll(t));
     const int nparts = (n + 2047) / 2048;
     // per entry: L (int), W and the kernel gradient (2 or 3 64-bit integers)
-    const size_t per_entry = sizeof(int) + (1 + (size_t)ev->dim) * sizeof(double);
+    const size_t per_entry = sizeof(int) + (ev->mixed ? 0 : 1) * (1 + (size_t)ev->dim) * sizeof(double);
     // per particle: two counts and two carried counts, the values in limbs and their exponents
-    const int nx = ev->dim == 2 ? 3 : 6;  // planes of the gradient-pass inputs
-    const size_t per_particle = 5 * sizeof(int) + 4 * sizeof(unsigned short) + (size_t)(2 + nx) * sizeof(int4);
+    // (the mixed form keeps the indices alone)
+    const int nx = ev->mixed ? 0 : (ev->dim == 2 ? 3 : 6);  // planes of the gradient-pass inputs
+    const int nq = ev->mixed ? 0 : 2;
+    const size_t per_particle = 5 * sizeof(int) + 4 * sizeof(unsigned short) + (size_t)(nq + nx) * sizeof(int4);
     const size_t bytes = (size_t)total * per_entry + (size_t)(n + 1) * sizeof(long long) +
                          (size_t)nparts * sizeof(unsigned long long) + per_particle * (size_t)n + 1024;
     size_t fr = 0, tot = 0;
@@ -798,11 +809,15 @@ static sph_status size_pair_lists(sph_event *ev)
     pl.margin = margin;
     pl.X = static_cast<int4 *>(m);  // the 16-byte aligned arrays first
     pl.Q = pl.X + (size_t)nx * n;
-    long long *gbuf = reinterpret_cast<long long *>(pl.Q + 2 * (size_t)n);  // the kernel gradients
-    if (ev->dim == 2) pl.G = reinterpret_cast<longlong2 *>(gbuf);
-    else pl.G3 = gbuf;
-    pl.W = gbuf + (size_t)ev->dim * total;
-    pl.off = reinterpret_cast<long long *>(pl.W + total);
+    long long *gbuf = reinterpret_cast<long long *>(pl.Q + (size_t)nq * n);  // the kernel gradients
+    if (ev->mixed) {
+        pl.off = gbuf;
+    } else {
+        if (ev->dim == 2) pl.G = reinterpret_cast<longlong2 *>(gbuf);
+        else pl.G3 = gbuf;
+        pl.W = gbuf + (size_t)ev->dim * total;
+        pl.off = pl.W + total;
+    }
     pl.part = reinterpret_cast<unsigned long long *>(pl.off + (n + 1));
     pl.Qe = reinterpret_cast<unsigned short *>(pl.part + nparts);  // read 8 bytes at a time
     pl.L = reinterpret_cast<int *>(pl.Qe + 4 * (size_t)n);
@@ -811,8 +826,7 @@ static sph_status size_pair_lists(sph_event *ev)
     ev->pcnt[0] = pl.cntB + n;
     ev->pcnt[1] = ev->pcnt[0] + n;
     pl.Xe = reinterpret_cast<unsigned int *>(ev->pcnt[1] + n);
-    CK(cudaMemcpyAsync(ev->pcnt[0], state.data(), sizeof(int) * (size_t)n, cudaMemcpyHostToDevice, ev->stream));
-    if ((s = wait_stream(ev)) != SPH_OK) return s;
+    launch_counts_to_state(ev->nnb, ev->cb.perm, ev->pcnt[0], n, ev->stream);
     pl.cnt_src = ev->pcnt[0];
     ev->cb.pl = pl;
     ev->pairs_grow = false;

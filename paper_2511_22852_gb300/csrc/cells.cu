@@ -24,6 +24,7 @@ __global__ void k_bbox_init(DevScalars *sc)
     if (threadIdx.x == 0) {
         sc->pair_flag = 0u;
         sc->eos_claim = 0u;
+        sc->pairs_stage = 0ull;
     }
 }
 
@@ -353,6 +354,13 @@ __global__ void k_scatter_orig_u32(const uint32_t *__restrict__ src, uint32_t *d
     dst[id[j]] = src[j];
 }
 
+// neighbour counts from the sorted order to the state order (sorted j <- state perm[j])
+__global__ void k_counts_to_state(const int *__restrict__ nnb, const uint32_t *__restrict__ perm, int *out, int n)
+{
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j < n) out[perm[j]] = nnb[j];
+}
+
 __global__ void k_cell_coords(EvView v, const double *__restrict__ y, const int *__restrict__ id, int *cell_orig)
 {
     int j = blockIdx.x * blockDim.x + threadIdx.x;
@@ -433,6 +441,11 @@ void launch_scatter_orig(const double *src, double *dst, const int *id, int n, i
 void launch_scatter_orig_u32(const uint32_t *src, uint32_t *dst, const int *id, int n, cudaStream_t st)
 {
     k_scatter_orig_u32<<<nblk(n, 256), 256, 0, st>>>(src, dst, id, n);
+}
+
+void launch_counts_to_state(const int *nnb, const uint32_t *perm, int *out, int n, cudaStream_t st)
+{
+    k_counts_to_state<<<nblk(n, 256), 256, 0, st>>>(nnb, perm, out, n);
 }
 
 void launch_cell_coords(const EvView &v, const double *y, const int *id, int *cell_orig, cudaStream_t st)

@@ -329,7 +329,8 @@ __global__ void __launch_bounds__(32 * kWarps, 7) k_pairs_sum(EvView v, PairBufs
         if (pl.cnt_dst) pl.cnt_dst[a] = c;  // sizes this particle's row in the next stage
     }
     const unsigned c2 = __reduce_add_sync(kFull, on && l == 0 ? 1u + (unsigned)nt : 0u);
-    if (lane == 0) atomicAdd(&v.sc->pairs, (unsigned long long)c2);
+    // added to the event's counter by the pass that follows, unless a list overflowed
+    if (lane == 0) atomicAdd(&v.sc->pairs_stage, (unsigned long long)c2);
 }
 
 // Gradient pass, half a warp per particle a, over the entries of its row with G = grad_a W_ab h /

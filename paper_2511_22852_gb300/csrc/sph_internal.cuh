@@ -54,6 +54,7 @@ struct DevScalars {
     unsigned int pair_ovf;
     unsigned int eos_claim;  // particle counter of the lane-refill EoS pass (reset with the bounding box)
     unsigned int pad_;
+    unsigned long long pairs_stage;  // pair-list passes: this stage's pairs (counted when no list overflowed)
 };
 
 struct EosDev {
@@ -419,7 +420,7 @@ struct CellBufs {
     float4 *fq, *fx;  // mixed: (S, N_B, N_S, N_Q) and the gradient inputs in single precision
     uint32_t *part; // scan partial sums (multi-block scan of large bucket tables)
     int nb;         // number of buckets: 1 << (2 B) in 2D, 1 << (B3[0] + B3[1] + B3[2]) in 3D
-    PairBufs pl;    // plain 2D: half-pair lists (pl.total = 0: off)
+    PairBufs pl;    // half-pair lists, mixed 3D: neighbour lists (pl.total = 0: off)
 };
 
 // Bound for the single-precision candidate prefilter of the neighbour passes.  With
@@ -492,6 +493,7 @@ void launch_totals(const EvView &v, const double *y, const double *Nq, const int
                    const double *eos, double *contrib, cudaStream_t st);
 void launch_sum_fixed(const double *vals, int n, int nfield, double *out, cudaStream_t st);
 void launch_scatter_orig(const double *src, double *dst, const int *id, int n, int nrows, cudaStream_t st);
+void launch_counts_to_state(const int *nnb, const uint32_t *perm, int *out, int n, cudaStream_t st);
 void launch_scatter_orig_u32(const uint32_t *src, uint32_t *dst, const int *id, int n, cudaStream_t st);
 void launch_cell_coords(const EvView &v, const double *y, const int *id, int *cell_orig, cudaStream_t st);
 int device_sm_count();  // SMs of the current device (cached after the first call)

@@ -119,7 +119,10 @@ __global__ void __launch_bounds__(32 * kWarps3) k_density3(EvView v, const doubl
     // fallback = 1: the pair-list passes ran first; this pass only runs if one of their lists
     // overflowed (and counts such stages)
     if (fallback) {
-        if (!v.sc->pair_flag) return;
+        if (!v.sc->pair_flag) {
+            if (blockIdx.x == 0 && threadIdx.x == 0) v.sc->pairs += v.sc->pairs_stage;
+            return;
+        }
         if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&v.sc->pair_ovf, 1u);
     }
     __shared__ int queue[kWarps3][64];
