@@ -774,8 +774,9 @@ static sph_status size_pair_lists(sph_event *ev)
     if (ev->pairs_grow) total = std::max<long long>(total, ev->cb.pl.total * 3 / 2);
     else if (const char *t = getenv("SPH_PAIR_TOTAL")) total = std::max<long long>(1, atoll(t));
     const int nparts = (n + 2047) / 2048;
-    // per entry: L (int), W and the kernel gradient (2 or 3 64-bit integers)
-    const size_t per_entry = sizeof(int) + (ev->mixed ? 0 : 1) * (1 + (size_t)ev->dim) * sizeof(double);
+    // per entry: L (int), W and the kernel gradient (2 64-bit integers, 3D: 3 padded to 4)
+    const size_t gsize = ev->mixed ? 0 : (ev->dim == 2 ? sizeof(longlong2) : sizeof(longlong4_32a));
+    const size_t per_entry = sizeof(int) + (ev->mixed ? 0 : sizeof(long long)) + gsize;
     // per particle: two counts and two carried counts, the values in limbs and their exponents
     // (the mixed form keeps the indices alone)
     const int nx = ev->mixed ? 0 : (ev->dim == 2 ? 3 : 6);  // planes of the gradient-pass inputs
@@ -807,17 +808,15 @@ static sph_status size_pair_lists(sph_event *ev)
     PairBufs pl{};
     pl.total = total;
     pl.margin = margin;
-    pl.X = static_cast<int4 *>(m);  // the 16-byte aligned arrays first
+    // the most aligned arrays first (32 bytes: the 3D gradients; 16: the others)
+    char *p = static_cast<char *>(m);
+    if (ev->dim == 2) pl.G = reinterpret_cast<longlong2 *>(p);
+    else pl.G3 = reinterpret_cast<longlong4_32a *>(p);
+    pl.X = reinterpret_cast<int4 *>(p + gsize * (size_t)total);
     pl.Q = pl.X + (size_t)nx * n;
-    long long *gbuf = reinterpret_cast<long long *>(pl.Q + (size_t)nq * n);  // the kernel gradients
-    if (ev->mixed) {
-        pl.off = gbuf;
-    } else {
-        if (ev->dim == 2) pl.G = reinterpret_cast<longlong2 *>(gbuf);
-        else pl.G3 = gbuf;
-        pl.W = gbuf + (size_t)ev->dim * total;
-        pl.off = pl.W + total;
-    }
+    long long *wbuf = reinterpret_cast<long long *>(pl.Q + (size_t)nq * n);
+    if (!ev->mixed) pl.W = wbuf;
+    pl.off = ev->mixed ? wbuf : wbuf + total;
     pl.part = reinterpret_cast<unsigned long long *>(pl.off + (n + 1));
     pl.Qe = reinterpret_cast<unsigned short *>(pl.part + nparts);  // read 8 bytes at a time
     pl.L = reinterpret_cast<int *>(pl.Qe + 4 * (size_t)n);

@@ -112,17 +112,17 @@ __global__ void __launch_bounds__(kScanThreads) k_rows_apply(int n, const uint32
     }
 }
 
-// Forward pass, a warp for two particles a.  Candidates of the cells from its own on pass the
-// single-precision prefilter; a candidate b > a is queued, and 32 at a time -- of both particles --
-// the exact test (where the float test left the pair undecided), the distance in FP64 and the
-// spline in 64-bit integers run on full warps.  W and grad W go in fixed point into a's row and,
-// at a place taken from b's counter, into b's row.  The particles' own values go into limbs.
+// Forward pass, a warp for two particles a.  Candidates of the cells from its own on (those within
+// 2h of a) pass the single-precision prefilter; a candidate b > a is queued, and 32 at a time -- of
+// both particles -- the exact test (where the float test left the pair undecided) and the kernel in
+// fixed point (pair_fixed) run on full warps.  W and grad W go into a's row and, at a place taken
+// from b's counter, into b's row.  The particles' own values go into limbs.
 // (Listing b < a in a's own walk, and finding its W by a search in b's row, kept the sums waiting
-// for memory: 40 k event, sum pass 197 -> 92 us a stage, gradient
-// pass 150 -> 137; 258 k particles in 3+1D 2.5 -> 0.9 and 3.4 -> 2.6 ms.)
-// Bound: the FP64 pipe, 12 operations per unordered pair (31 with spline and kernel sums in FP64, a
-// reduction per particle and its own partial batch).  40 k event: 214 us a stage (325
-// with the spline in FP64).
+// for memory: 40 k event, sum pass 197 -> 92 us a stage, gradient pass 150 -> 137.)
+// Bound: latency and the L2 sectors of the scattered writes (b's row: three sectors a pair).  4 FP64
+// operations per unordered pair (12 with the kernel's distance in FP64, 31 with spline and sums).
+// 40 k event: 192 us a stage (212 with the distance in FP64 and every cell walked, 325 with the
+// spline in FP64).
 __global__ void __launch_bounds__(32 * kWarps, 8) k_pairs_fwd(EvView v, const double *__restrict__ y,
                                                            const float2 *__restrict__ fpos,
                                                            const double *__restrict__ Nq,
@@ -132,6 +132,10 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_pairs_fwd(EvView v, const do
                                                            const uint32_t *__restrict__ perm, PairBufs pl)
 {
     __shared__ int queue[kWarps][64];
+    // the two particles of a warp: position, first entry and size of the row
+    __shared__ double pos_[kWarps][2][2];
+    __shared__ long long row_[kWarps][2];
+    __shared__ int cap_[kWarps][2];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int n = v.n;
     const long long a0 = 2 * ((long long)blockIdx.x * kWarps + wid);
@@ -145,49 +149,49 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_pairs_fwd(EvView v, const do
         fx_store_value(pl.Q, pl.Qe, (size_t)n, a, k, k == 0 ? S[a] : Nq[(size_t)(k - 1) * n + a]);
     }
     const unsigned lt = (1u << lane) - 1u;
-    double xa[2], ya[2];
-    long long r0[2];
-    int cap[2], nf[2] = {0, 0}, qn = 0;
-#pragma unroll
-    for (int p = 0; p < 2; ++p) {
-        const int a = (int)a0 + (p < np ? p : 0);
-        xa[p] = X[a];
-        ya[p] = Y[a];
-        r0[p] = pl.off[a];
-        const long long r1 = pl.off[a + 1];
-        cap[p] = r1 <= pl.total ? (int)(r1 - r0[p]) : 0;  // rows beyond the allocation write nothing
+    const double (*pos)[2] = pos_[wid];
+    const long long *row = row_[wid];
+    const int *cap = cap_[wid];
+    int nf[2] = {0, 0}, qn = 0;
+    if (lane < 2) {
+        const int a = (int)a0 + (lane < np ? lane : 0);
+        pos_[wid][lane][0] = X[a];
+        pos_[wid][lane][1] = Y[a];
+        const long long r0 = pl.off[a], r1 = pl.off[a + 1];
+        row_[wid][lane] = r0;
+        cap_[wid][lane] = r1 <= pl.total ? (int)(r1 - r0) : 0;  // rows beyond the allocation write nothing
     }
+    __syncwarp();
     // queued word: bit 31: the float test left the pair undecided (exact test needed), bit 30: of a0 + 1
     auto forward = [&](int qb, bool valid) {
         const int b = qb & 0x3FFFFFFF;
-        const bool second = qb & 0x40000000;
+        const int p = qb >> 30 & 1;
         double dx = 0.0, dy = 0.0;
         bool acc = false;
         if (valid) {
-            dx = (second ? xa[1] : xa[0]) - X[b];
-            dy = (second ? ya[1] : ya[0]) - Y[b];
+            dx = pos[p][0] - X[b];
+            dy = pos[p][1] - Y[b];
             acc = qb >= 0 || dist2_2d(dx, dy) < v.supp2;
         }
-        const unsigned m0 = __ballot_sync(kFull, acc && !second), m1 = __ballot_sync(kFull, acc && second);
+        const unsigned m0 = __ballot_sync(kFull, acc && p == 0), m1 = __ballot_sync(kFull, acc && p == 1);
         if (acc) {
+            // b's row and the place in it first: the loads and the atomic wait behind the arithmetic
+            const long long rb = pl.off[b], rb1 = pl.off[b + 1];
+            const int place = atomicAdd(&pl.cntB[b], 1);
             const double r2 = fma(dx, dx, dy * dy);
-            long long w = 1LL << kFxBits, dw = 0;  // coincident particles: W(0), no gradient
-            double ir = 0.0, q;
-            if (nonzero_nonneg(r2)) {
-                pair_distance(r2, v.inv_h, ir, q);
-                spline_fixed(q, w, dw);
-            }
-            const int slot = second ? nf[1] + __popc(m1 & lt) : nf[0] + __popc(m0 & lt);
-            const longlong2 g = make_longlong2(grad_fixed(dw, dx * ir), grad_fixed(dw, dy * ir));
-            if (slot < (second ? cap[1] : cap[0])) {
-                const long long i = (second ? r0[1] : r0[0]) + slot;
+            long long w, gk[2];
+            pair_fixed<2>({dx, dy}, r2, v.inv_h, w, gk);
+            const int slot = (p ? nf[1] : nf[0]) + __popc((p ? m1 : m0) & lt);
+            const longlong2 g = make_longlong2(gk[0], gk[1]);
+            if (slot < cap[p]) {
+                const long long i = row[p] + slot;
                 pl.L[i] = b;
                 pl.W[i] = w;
                 pl.G[i] = g;
             }
-            const long long i = pl.off[b + 1] - 1 - atomicAdd(&pl.cntB[b], 1);
-            if (i >= pl.off[b] && pl.off[b + 1] <= pl.total) {
-                pl.L[i] = (int)a0 + (second ? 1 : 0);
+            const long long i = rb1 - 1 - place;
+            if (i >= rb && rb1 <= pl.total) {
+                pl.L[i] = (int)a0 + p;
                 pl.W[i] = w;
                 pl.G[i] = make_longlong2(-g.x, -g.y);
             }
@@ -202,33 +206,54 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_pairs_fwd(EvView v, const do
         const float2 fa = fpos[a];
         const uint32_t ka = key[perm[a]];
         const int cx = (int)unspread2(ka), cy = (int)unspread2(ka >> 1), lim = 1 << v.B;
-        for (int o = 0; o < 9; ++o) {
-            const int nx = cx + o % 3 - 1, ny = cy + o / 3 - 1;
-            if (nx < 0 || ny < 0 || nx >= lim || ny >= lim) continue;
-            const uint32_t k = morton2((uint32_t)nx, (uint32_t)ny);
-            if (k < ka) continue;  // all of its particles come before a
-            const uint32_t b0 = start[k], b1 = b0 + cnt[k];
-            for (uint32_t base = k == ka ? (uint32_t)a + 1u : b0; base < b1; base += 32) {
-                const uint32_t b = base + lane;
-                bool cand = false, sure = false;
-                if (b < b1 && (int)b > a) {
-                    const float2 fb = fpos[b];
-                    const float dx = fa.x - fb.x, dy = fa.y - fb.y;
-                    const float r2f = fmaf(dx, dx, dy * dy);
-                    cand = r2f <= v.supp2_hi;
-                    sure = r2f < v.supp2_lo;
-                }
-                const unsigned m = __ballot_sync(kFull, cand);
-                if (cand) q[qn + __popc(m & lt)] = (int)(b | (sure ? 0u : 0x80000000u)) | flag;
-                qn += __popc(m);
+        // lane o < 9: the neighbour cell o, kept when it holds particles behind a within 2h of it
+        uint32_t k = 0u, st = 0u, len = 0u;
+        if (lane < 9) {
+            const int ox = lane % 3 - 1, oy = lane / 3 - 1, nx = cx + ox, ny = cy + oy;
+            const float gx = cell_gap(ox, fa.x, cx, v.cell_f), gy = cell_gap(oy, fa.y, cy, v.cell_f);
+            if (nx >= 0 && ny >= 0 && nx < lim && ny < lim && !(fmaf(gx, gx, gy * gy) > v.supp2_hi)) {
+                k = morton2((uint32_t)nx, (uint32_t)ny);
+                st = start[k];
+                len = k < ka ? 0u : cnt[k];  // below ka: all of its particles come before a
+            }
+        }
+        // batches of 32 candidates, each loaded while the one before is tested; b > a in all of them
+        // (lanes past a cell's end hold NaN: never candidates)
+        const float kNaN = __int_as_float(0x7FFFFFFF);
+        unsigned cells = __ballot_sync(kFull, len > 0u);
+        uint32_t base = 0u, b1 = 0u;
+        auto next = [&]() {
+            base += 32u;
+            while (base >= b1 && cells) {
+                const int o = __ffs(cells) - 1;
+                cells &= cells - 1u;
+                base = __shfl_sync(kFull, st, o);
+                b1 = base + __shfl_sync(kFull, len, o);
+                if (__shfl_sync(kFull, k, o) == ka) base = (uint32_t)a + 1u;
+            }
+            return base < b1;
+        };
+        auto load = [&](bool on) { return on && base + lane < b1 ? fpos[base + lane] : make_float2(kNaN, 0.0f); };
+        bool more = next();
+        float2 fn = load(more);
+        while (more) {
+            const uint32_t b = base + lane;
+            const float2 fb = fn;
+            more = next();
+            fn = load(more);
+            const float dx = fa.x - fb.x, dy = fa.y - fb.y;
+            const float r2f = fmaf(dx, dx, dy * dy);
+            const bool cand = r2f <= v.supp2_hi, sure = r2f < v.supp2_lo;
+            const unsigned m = __ballot_sync(kFull, cand);
+            if (cand) q[qn + __popc(m & lt)] = (int)(b | (sure ? 0u : 0x80000000u)) | flag;
+            qn += __popc(m);
+            __syncwarp();
+            if (qn >= 32) {
+                forward(q[lane], true);
+                qn -= 32;
                 __syncwarp();
-                if (qn >= 32) {
-                    forward(q[lane], true);
-                    qn -= 32;
-                    __syncwarp();
-                    if (lane < qn) q[lane] = q[32 + lane];
-                    __syncwarp();
-                }
+                if (lane < qn) q[lane] = q[32 + lane];
+                __syncwarp();
             }
         }
     }

@@ -13,16 +13,20 @@ namespace {
 constexpr int kWarps = 4;
 constexpr unsigned kFull = 0xFFFFFFFFu;
 
-// Forward pass, a warp for two particles a.  Candidates of the cells from its own on pass the
-// single-precision prefilter; a candidate b > a is queued, and 32 at a time -- of both particles --
-// the exact test (where the float test left the pair undecided), the distance in FP64 and the
-// spline in 64-bit integers run on full warps.  W and grad W go in fixed point into a's row and,
-// at a place taken from b's counter, into b's row.  The particles' own values go into limbs.
+// Forward pass, a warp for two particles a.  Candidates of the cells from its own on (those within
+// 2h of a) pass the single-precision prefilter; a candidate b > a is queued, and 32 at a time -- of
+// both particles -- the exact test (where the float test left the pair undecided) and the kernel in
+// fixed point (pair_fixed) run on full warps.  W and grad W go into a's row and, at a place taken
+// from b's counter, into b's row.  The particles' own values go into limbs.
 // (Listing b < a in a's own walk, and finding its W by a search in b's row, kept the sums waiting
-// for memory: 40 k event, sum pass 197 -> 92 us a stage, gradient
-// pass 150 -> 137; 258 k particles in 3+1D 2.5 -> 0.9 and 3.4 -> 2.6 ms.)
-// Bound: the FP64 pipe, 15 operations per unordered pair.  258 k particles: 3.5 ms a stage
-// (4.6 with the spline in FP64).
+// for memory: 40 k event, sum pass 197 -> 92 us a stage, gradient pass 150 -> 137; 258 k particles
+// in 3+1D 2.5 -> 0.9 and 3.4 -> 2.6 ms.)
+// Bound: the L2 sectors of the scattered writes to b's row.  The three components of grad W lie in
+// one 32-byte sector and are written by one store (three 8-byte stores at a stride of 24 bytes
+// wrote 7.6 sectors a pair against 4.4); with that and 6 FP64 operations per unordered pair (15
+// with the kernel's distance in FP64), 258 k particles: density pass 4.36 -> 3.24 ms a stage, the
+// gradient pass, which reads 36 instead of 28 bytes an entry, 2.6 -> 2.9.  The integers alone gave
+// nothing here (the stores bound it), the layout alone was not measured.
 __global__ void __launch_bounds__(32 * kWarps, 8) k_pairs3_fwd(EvView v, const double *__restrict__ y,
                                                            const float4 *__restrict__ fpos,
                                                            const double *__restrict__ Nq,
@@ -30,6 +34,10 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_pairs3_fwd(EvView v, const d
                                                            const uint32_t *__restrict__ cnt, PairBufs pl)
 {
     __shared__ int queue[kWarps][64];
+    // the two particles of a warp: position, first entry and size of the row
+    __shared__ double pos_[kWarps][2][3];
+    __shared__ long long row_[kWarps][2];
+    __shared__ int cap_[kWarps][2];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int n = v.n;
     const long long a0 = 2 * ((long long)blockIdx.x * kWarps + wid);
@@ -43,55 +51,52 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_pairs3_fwd(EvView v, const d
         fx_store_value(pl.Q, pl.Qe, (size_t)n, a, k, k == 0 ? S[a] : Nq[(size_t)(k - 1) * n + a]);
     }
     const unsigned lt = (1u << lane) - 1u;
-    double xa[2], ya[2], za[2];
-    long long r0[2];
-    int cap[2], nf[2] = {0, 0}, qn = 0;
-#pragma unroll
-    for (int p = 0; p < 2; ++p) {
-        const int a = (int)a0 + (p < np ? p : 0);
-        xa[p] = X[a];
-        ya[p] = Y[a];
-        za[p] = Z[a];
-        r0[p] = pl.off[a];
-        const long long r1 = pl.off[a + 1];
-        cap[p] = r1 <= pl.total ? (int)(r1 - r0[p]) : 0;  // rows beyond the allocation write nothing
+    const double (*pos)[3] = pos_[wid];
+    const long long *row = row_[wid];
+    const int *cap = cap_[wid];
+    int nf[2] = {0, 0}, qn = 0;
+    if (lane < 2) {
+        const int a = (int)a0 + (lane < np ? lane : 0);
+        pos_[wid][lane][0] = X[a];
+        pos_[wid][lane][1] = Y[a];
+        pos_[wid][lane][2] = Z[a];
+        const long long r0 = pl.off[a], r1 = pl.off[a + 1];
+        row_[wid][lane] = r0;
+        cap_[wid][lane] = r1 <= pl.total ? (int)(r1 - r0) : 0;  // rows beyond the allocation write nothing
     }
+    __syncwarp();
     // queued word: bit 31: the float test left the pair undecided (exact test needed), bit 30: of a0 + 1
     auto forward = [&](int qb, bool valid) {
         const int b = qb & 0x3FFFFFFF;
-        const bool second = qb & 0x40000000;
+        const int p = qb >> 30 & 1;
         double dx = 0.0, dy = 0.0, dz = 0.0;
         bool acc = false;
         if (valid) {
-            dx = (second ? xa[1] : xa[0]) - X[b];
-            dy = (second ? ya[1] : ya[0]) - Y[b];
-            dz = (second ? za[1] : za[0]) - Z[b];
+            dx = pos[p][0] - X[b];
+            dy = pos[p][1] - Y[b];
+            dz = pos[p][2] - Z[b];
             acc = qb >= 0 || dist2_3d(dx, dy, dz) < v.supp2;
         }
-        const unsigned m0 = __ballot_sync(kFull, acc && !second), m1 = __ballot_sync(kFull, acc && second);
+        const unsigned m0 = __ballot_sync(kFull, acc && p == 0), m1 = __ballot_sync(kFull, acc && p == 1);
         if (acc) {
+            // b's row and the place in it first: the loads and the atomic wait behind the arithmetic
+            const long long rb = pl.off[b], rb1 = pl.off[b + 1];
+            const int place = atomicAdd(&pl.cntB[b], 1);
             const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
-            long long w = 1LL << kFxBits, dw = 0;  // coincident particles: W(0), no gradient
-            double ir = 0.0, q;
-            if (nonzero_nonneg(r2)) {
-                pair_distance(r2, v.inv_h, ir, q);
-                spline_fixed(q, w, dw);
-            }
-            const int slot = second ? nf[1] + __popc(m1 & lt) : nf[0] + __popc(m0 & lt);
-            const long long g[3] = {grad_fixed(dw, dx * ir), grad_fixed(dw, dy * ir), grad_fixed(dw, dz * ir)};
-            if (slot < (second ? cap[1] : cap[0])) {
-                const long long i = (second ? r0[1] : r0[0]) + slot;
+            long long w, g[3];
+            pair_fixed<3>({dx, dy, dz}, r2, v.inv_h, w, g);
+            const int slot = (p ? nf[1] : nf[0]) + __popc((p ? m1 : m0) & lt);
+            if (slot < cap[p]) {
+                const long long i = row[p] + slot;
                 pl.L[i] = b;
                 pl.W[i] = w;
-#pragma unroll
-                for (int k = 0; k < 3; ++k) pl.G3[3 * i + k] = g[k];
+                pl.G3[i] = longlong4_32a{g[0], g[1], g[2], 0};
             }
-            const long long i = pl.off[b + 1] - 1 - atomicAdd(&pl.cntB[b], 1);
-            if (i >= pl.off[b] && pl.off[b + 1] <= pl.total) {
-                pl.L[i] = (int)a0 + (second ? 1 : 0);
+            const long long i = rb1 - 1 - place;
+            if (i >= rb && rb1 <= pl.total) {
+                pl.L[i] = (int)a0 + p;
                 pl.W[i] = w;
-#pragma unroll
-                for (int k = 0; k < 3; ++k) pl.G3[3 * i + k] = -g[k];
+                pl.G3[i] = longlong4_32a{-g[0], -g[1], -g[2], 0};
             }
         }
         nf[0] += __popc(m0);
@@ -105,33 +110,64 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_pairs3_fwd(EvView v, const d
         const int ca = __float_as_int(fa.w);  // the packed cell coordinates
         const int c[3] = {ca & 1023, (ca >> 10) & 1023, (ca >> 20) & 1023};
         const uint32_t ka = key3(v, c[0], c[1], c[2]);
-        for (int o = 0; o < 27; ++o) {
-            const int nx = c[0] + o % 3 - 1, ny = c[1] + (o / 3) % 3 - 1, nz = c[2] + o / 9 - 1;
-            if (nx < 0 || ny < 0 || nz < 0 || nx >= (1 << v.B3[0]) || ny >= (1 << v.B3[1]) || nz >= (1 << v.B3[2])) continue;
-            const uint32_t k = key3(v, nx, ny, nz);
-            if (k < ka) continue;  // all of its particles come before a
-            const uint32_t b0 = start[k], b1 = b0 + cnt[k];
-            for (uint32_t base = k == ka ? (uint32_t)a + 1u : b0; base < b1; base += 32) {
-                const uint32_t b = base + lane;
-                bool cand = false, sure = false;
-                if (b < b1 && (int)b > a) {
-                    const float4 fb = fpos[b];
-                    const float dx = fa.x - fb.x, dy = fa.y - fb.y, dz = fa.z - fb.z;
-                    const float r2f = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                    cand = r2f <= v.supp2_hi;
-                    sure = r2f < v.supp2_lo;
-                }
-                const unsigned m = __ballot_sync(kFull, cand);
-                if (cand) q[qn + __popc(m & lt)] = (int)(b | (sure ? 0u : 0x80000000u)) | flag;
-                qn += __popc(m);
+        // lane o < 27: the neighbour cell o, kept when it holds particles behind a within 2h of it
+        uint32_t k = 0u, st = 0u, len = 0u;
+        if (lane < 27) {
+            const int o[3] = {lane % 3 - 1, (lane / 3) % 3 - 1, lane / 9 - 1};
+            const float f[3] = {fa.x, fa.y, fa.z};
+            bool in = true;
+            float d = 0.0f;
+            int m[3];
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                m[i] = c[i] + o[i];
+                in = in && m[i] >= 0 && m[i] < (1 << v.B3[i]);
+                const float g = cell_gap(o[i], f[i], c[i], v.cell_f);
+                d = fmaf(g, g, d);
+            }
+            if (in && !(d > v.supp2_hi)) {
+                k = key3(v, m[0], m[1], m[2]);
+                st = start[k];
+                len = k < ka ? 0u : cnt[k];  // below ka: all of its particles come before a
+            }
+        }
+        // batches of 32 candidates, each loaded while the one before is tested; b > a in all of them
+        // (lanes past a cell's end hold NaN: never candidates)
+        const float kNaN = __int_as_float(0x7FFFFFFF);
+        unsigned cells = __ballot_sync(kFull, len > 0u);
+        uint32_t base = 0u, b1 = 0u;
+        auto next = [&]() {
+            base += 32u;
+            while (base >= b1 && cells) {
+                const int o = __ffs(cells) - 1;
+                cells &= cells - 1u;
+                base = __shfl_sync(kFull, st, o);
+                b1 = base + __shfl_sync(kFull, len, o);
+                if (__shfl_sync(kFull, k, o) == ka) base = (uint32_t)a + 1u;
+            }
+            return base < b1;
+        };
+        auto load = [&](bool on) { return on && base + lane < b1 ? fpos[base + lane] : make_float4(kNaN, 0.0f, 0.0f, 0.0f); };
+        bool more = next();
+        float4 fn = load(more);
+        while (more) {
+            const uint32_t b = base + lane;
+            const float4 fb = fn;
+            more = next();
+            fn = load(more);
+            const float dx = fa.x - fb.x, dy = fa.y - fb.y, dz = fa.z - fb.z;
+            const float r2f = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+            const bool cand = r2f <= v.supp2_hi, sure = r2f < v.supp2_lo;
+            const unsigned m = __ballot_sync(kFull, cand);
+            if (cand) q[qn + __popc(m & lt)] = (int)(b | (sure ? 0u : 0x80000000u)) | flag;
+            qn += __popc(m);
+            __syncwarp();
+            if (qn >= 32) {
+                forward(q[lane], true);
+                qn -= 32;
                 __syncwarp();
-                if (qn >= 32) {
-                    forward(q[lane], true);
-                    qn -= 32;
-                    __syncwarp();
-                    if (lane < qn) q[lane] = q[32 + lane];
-                    __syncwarp();
-                }
+                if (lane < qn) q[lane] = q[32 + lane];
+                __syncwarp();
             }
         }
     }
@@ -140,10 +176,12 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_pairs3_fwd(EvView v, const d
         for (int p = 0; p < np; ++p) pl.cntF[a0 + p] = nf[p];
 }
 
-// Gradient pass, half a warp per particle a, over the entries of its row, in integers (pairs_fixed.cuh): sum grad W (3), sum X_b^{j i}
-// grad_j W (3), sum u_b^j grad_k W (9); the epilogue as the per-particle pass.
-// Bound: the latency of the gathers; 258 k particles: 2.6 ms a stage (6.0 with 21 FP64 operations per
-// pair).  4 blocks per SM: 3 gave 3.7, 5 3.8, 6 4.8 ms.
+// Gradient pass, half a warp per particle a, over the entries of its row, in integers
+// (pairs_fixed.cuh): sum grad W (3), sum X_b^{j i} grad_j W (3), sum u_b^j grad_k W (9); the
+// epilogue as the per-particle pass.
+// Bound: the latency of the gathers; 258 k particles: 2.9 ms a stage (6.0 with 21 FP64 operations per
+// pair).  4 blocks per SM (of the 2.6 ms with 24-byte entries: 3 gave 3.7, 5 3.8, 6 4.8 ms).  Entries
+// kept out of L1, or the index taken from the padding of the 32-byte entry: no difference.
 __global__ void __launch_bounds__(32 * kWarps, 4) k_pairs3_gradient(EvView v, int stage, const double *__restrict__ gin,
                                                                  PairBufs pl, double *__restrict__ gout)
 {
@@ -183,9 +221,10 @@ __global__ void __launch_bounds__(32 * kWarps, 4) k_pairs3_gradient(EvView v, in
         if (j < nt) {
             const long long i = at(j);
             b = pl.L[i];
-            g[0] = pl.G3[3 * i];
-            g[1] = pl.G3[3 * i + 1];
-            g[2] = pl.G3[3 * i + 2];
+            const longlong4_32a e = pl.G3[i];
+            g[0] = e.x;
+            g[1] = e.y;
+            g[2] = e.z;
         }
     };
     int b1;

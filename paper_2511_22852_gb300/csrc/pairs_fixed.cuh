@@ -3,8 +3,8 @@
 // On GB300 an FP64 operation occupies its pipe for 64 cycles per warp and quadrant, a 32-bit
 // integer multiply-add into 64 bits for about 3.  The pair passes therefore form their sums
 // sum_b q_b w_ab in integers, at or above FP64 precision:
-//   * the pair's kernel value or gradient (dimensionless, |w| <= 1), computed in FP64, as a
-//     fixed-point integer in units of 2^-57;
+//   * the pair's kernel value or gradient (dimensionless, |w| <= 1) as a fixed-point integer in
+//     units of 2^-57, from the FP64 separation (pair_fixed);
 //   * the particle's value q_b as its exact 53-bit mantissa (times 2) in two limbs
 //     hi 2^29 + lo (lo balanced around 0) and its exponent;
 //   * the particle's sums in units of the largest exponent E among its neighbours (a first look
@@ -28,64 +28,66 @@ constexpr int kNonFinite = 0x7FF;
 constexpr int kFoldEvery = 16;     // terms between folds of the cross accumulators
 constexpr int kHeadroom = 128;     // terms a lane's high accumulator holds without a larger unit
 
-// v in units of 2^-BITS (|v| 2^BITS < 2^63), rounded to nearest (halves away from zero)
-template <int BITS>
-__device__ __forceinline__ long long to_fixed(double v)
+// A lower bound of the distance along one axis from x, in cell c of side cell, to the cell c + o: 0
+// for o = 0; the margin covers the rounding of the single-precision position and of c cell (each
+// below 2^-24 of the position), so a cell left out at gap^2 > supp2_hi holds no neighbour.  NaN stays.
+__device__ __forceinline__ float cell_gap(int o, float x, int c, float cell)
 {
-    const long long b = __double_as_longlong(v);
-    const int e = (int)(b >> 52) & 0x7FF;
-    long long m = (b & 0xFFFFFFFFFFFFFLL) | (1LL << 52);
-    const int s = e - (1075 - BITS);
-    m = s >= 0 ? m << min(s, 10) : (s > -60 ? (m + (1LL << (-s - 1))) >> -s : 0LL);
-    return b < 0 ? -m : m;
+    if (o == 0) return 0.0f;
+    const float g = o < 0 ? x - (float)c * cell : (float)(c + 1) * cell - x;
+    const float m = g - 1e-6f * (fabsf(x) + cell);
+    return m < 0.0f ? 0.0f : m;
 }
 
-// 1/r, r/h of a pair from r^2 > 0: a single-precision reciprocal square root y (relative error
-// below 2^-21) refined by one third-order Householder step, e = 1 - r^2 y^2, c = e/2 + 3 e^2/8,
-// 1/r = y (1 + c), r = r^2 y (1 + c), with the remainder of order e^3 below 2^-62.  Six FP64
-// operations for both and the division by h (rsqrt and two products: about nine); 3 e^2/8 is
-// below 2^-44 and is taken in single precision.  Outside the single-precision range: rsqrt.
-__device__ __forceinline__ void pair_distance(double r2, double inv_h, double &ir, double &q)
+// |v| 2^-s in units of 2^-61 (below 2^62), rounded to nearest
+__device__ __forceinline__ unsigned long long abs_fixed(double v, int s)
 {
-    const unsigned hi = (unsigned)__double2hiint(r2);
-    if (hi - 0x3B000000u < 0x08000000u) {  // 2^-79 <= r^2 < 2^49
-        const float f = __uint_as_float(__funnelshift_l((unsigned)__double2loint(r2), hi - 0x38000000u, 3));
-        const float y = rsqrt_apx(f);
-        const unsigned yb = __float_as_uint(y);
-        const double y0 = __hiloint2double((int)((yb >> 3) + 0x38000000u), (int)(yb << 29));
-        const double t = r2 * y0;
-        const double e = fma(-t, y0, 1.0);
-        // (3/8) e^2 from e's leading bits: |e| < 2^-19, so a float holds it (zero below 2^-126)
-        const unsigned eh = (unsigned)__double2hiint(e) & 0x7FFFFFFFu;
-        const float ef = eh < 0x3C000000u ? 0.0f : __uint_as_float(__funnelshift_l((unsigned)__double2loint(e), eh - 0x38000000u, 3));
-        const unsigned cb = __float_as_uint(0.375f * ef * ef);
-        const double c2 = cb < 0x00800000u ? 0.0 : __hiloint2double((int)((cb >> 3) + 0x38000000u), (int)(cb << 29));
-        const double c = fma(e, 0.5, c2);
-        ir = fma(y0, c, y0);
-        q = fma(t, c, t) * inv_h;
-    } else {
-        ir = rsqrt(r2);
-        q = r2 * ir * inv_h;
-    }
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    const int k = (int)(b >> 52 & 0x7FF) - (1075 - 61) - s;
+    const unsigned long long m = (b & 0xFFFFFFFFFFFFFULL) | (1ULL << 52);
+    return k >= 0 ? m << min(k, 9) : (k > -60 ? (m + (1ULL << (-k - 1))) >> -k : 0ULL);
 }
 
-// The cubic spline in fixed point from q = r/h in [0, 2]: w = (2-q)^3/4 - max(1-q, 0)^3 in units of
-// 2^-kFxBits and w' = 3 max(1-q, 0)^2 - 3 (2-q)^2/4 in units of 2^-62 (|w'| <= 1).  t = 2 - q and
-// u = max(1 - q, 0) in units of 2^-61; 64-bit high products instead of FP64 ones (about 10 integer
-// instructions against one operation of 64 cycles), errors below 2^-56.
-__device__ __forceinline__ void spline_fixed(double q, long long &w, long long &dw)
+// A pair's kernel value and gradient in fixed point from its separation d and r2 = |d|^2 <= 4 h^2:
+// w = (2-q)^3/4 - max(1-q, 0)^3 and g_k = w' d_k/r, w' = 3 max(1-q, 0)^2 - 3 (2-q)^2/4 <= 0, q = r/h,
+// all in units of 2^-kFxBits.  r2 = m 4^s with m in [1, 4): a single-precision reciprocal square
+// root y of m (relative error below 2^-21) is refined by one third-order Householder step, e =
+// 1 - m y^2, c = e/2 + 3 e^2/8, 1/sqrt(m) = y (1 + c), with the remainder of order e^3 below 2^-60.
+// Everything behind r2 is in 64-bit integers: a high product is about 10 integer instructions
+// (25 cycles a warp), an FP64 operation 64 cycles; errors below 2^-56 of the kernel's maximum.
+template <int D>
+__device__ __forceinline__ void pair_fixed(const double (&d)[D], double r2, double inv_h, long long &w, long long (&g)[D])
 {
-    const long long Q = to_fixed<61>(q);
+    const unsigned hi = (unsigned)__double2hiint(r2), lo = (unsigned)__double2loint(r2);
+    w = 1LL << kFxBits;  // coincident particles: W(0), no gradient
+#pragma unroll
+    for (int k = 0; k < D; ++k) g[k] = 0;
+    if (hi - 0x00100000u >= 0x7FE00000u) return;  // zero (or below 2^-1022)
+    const int E = (int)(hi >> 20) - 1023, s = E >> 1, odd = E & 1;
+    const unsigned long long M = (((unsigned long long)(hi & 0xFFFFFu) | 0x100000u) << 32 | lo) << (10 + odd);  // m, 2^-62
+    const float y = rsqrt_apx(__uint_as_float((__funnelshift_l(lo, hi, 3) & 0x7FFFFFu) | (unsigned)(127 + odd) << 23));
+    const unsigned Y = __float2uint_rz(y * 33554432.0f);  // 2^-25, exact
+    const long long e = (1LL << 61) - (long long)__umul64hi(M, (unsigned long long)Y * Y << 13);  // 2^-61, |e| < 2^-19
+    const int e0 = (int)(e >> 21);
+    const long long c = (e >> 1) + (((long long)e0 * e0 * 3) >> 22);
+    const unsigned long long R = __umul64hi((unsigned long long)Y << 38, (1ULL << 63) + (unsigned long long)(c * 4)) << 1;  // 1/sqrt(m), 2^-63
+    const unsigned long long hb = (unsigned long long)__double_as_longlong(inv_h);
+    const unsigned long long H = (hb << 11) | (1ULL << 63);  // 1/h = H 2^t, 2^-63
+    const int sh = s + (int)(hb >> 52 & 0x7FF) - 1023;
+    const unsigned long long qr = __umul64hi(__umul64hi(M, R) << 1, H);  // q 2^-sh, 2^-61
+    const long long Q = (long long)(sh >= 0 ? qr << min(sh, 63) : qr >> min(-sh, 63));
+    // t = 2 - q and u = max(1 - q, 0), 2^-61
     const unsigned long long T = (unsigned long long)max((1LL << 62) - Q, 0LL), U = (unsigned long long)max((1LL << 61) - Q, 0LL);
-    const unsigned long long T2 = __umul64hi(T, T), U2 = __umul64hi(U, U);  // units of 2^-58
+    const unsigned long long T2 = __umul64hi(T, T), U2 = __umul64hi(U, U);  // 2^-58
     const unsigned long long T3 = __umul64hi(T2 << 3, T), U3 = __umul64hi(U2 << 3, U);
     w = ((long long)T3 - 4 * (long long)U3 + 4) >> 3;
-    dw = 48 * ((long long)U2 - (long long)(T2 >> 2));  // 3 (u^2 - t^2/4), 2^-58 -> 2^-62
-}
-// w' times the unit vector's component e in [-1, 1], in units of 2^-kFxBits
-__device__ __forceinline__ long long grad_fixed(long long dw, double e)
-{
-    return (__mul64hi(dw, to_fixed<62>(e)) + 4) >> 3;
+    const unsigned long long n = (unsigned long long)max(48 * ((long long)(T2 >> 2) - (long long)U2), 0LL);  // -w', 2^-62
+    const unsigned long long P = __umul64hi(n << 1, R) << 1;  // -w'/sqrt(m), 2^-63
+#pragma unroll
+    for (int k = 0; k < D; ++k) {
+        const long long a = (long long)((__umul64hi(P, abs_fixed(d[k], s) << 1) + 8) >> 4);
+        g[k] = __double2hiint(d[k]) < 0 ? a : -a;
+    }
 }
 
 // biased exponent of v (zero and denormals: 1), kNonFinite for infinities and NaN

@@ -403,7 +403,7 @@ struct PairBufs {
     // (pairs_fixed.cuh)
     long long *W;
     longlong2 *G;   // 2D
-    long long *G3;  // 3D: three components per entry
+    longlong4_32a *G3;  // 3D: three components, padded to a 32-byte sector
     // particle values in limbs (sorted order), planes of [n] int4 with two values each: S, N_B |
     // N_S, N_Q with an exponent each (Qe[n][4]); the rows of gin, two at a time, with their two
     // exponents (stress, u) packed in Xe
