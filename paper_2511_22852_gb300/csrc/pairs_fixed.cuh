@@ -90,6 +90,33 @@ __device__ __forceinline__ void pair_fixed(const double (&d)[D], double r2, doub
     }
 }
 
+// w >= 0 in units of 2^-kFxBits as a double, rounded to nearest (in integers: a conversion instruction
+// occupies the FP64 pipe like an operation)
+__device__ __forceinline__ double fixed_value(long long w)
+{
+    if (w <= 0) return 0.0;
+    const int s = __clzll(w);
+    const unsigned long long m = (unsigned long long)w << s;
+    const unsigned long long b = ((unsigned long long)(1022 + 63 - kFxBits - s) << 52) + (m >> 11) + (m >> 10 & 1u);
+    return __longlong_as_double((long long)b);
+}
+
+// The lanes' sums of up to 8 values: value k (of t[0..7]) over the warp in lane 4 k (and 4 k + 1 to
+// 4 k + 3).  Halves exchange values first: 9 additions instead of 5 a value, in a fixed order.
+__device__ __forceinline__ double warp_sums8(double (&t)[8], int lane)
+{
+#pragma unroll
+    for (int h = 4, o = 16; h > 0; h >>= 1, o >>= 1)
+#pragma unroll
+        for (int k = 0; k < h; ++k) {
+            const bool up = lane & o;
+            const double send = up ? t[k] : t[k + h];
+            t[k] = (up ? t[k + h] : t[k]) + __shfl_xor_sync(0xFFFFFFFFu, send, o);
+        }
+    t[0] += __shfl_xor_sync(0xFFFFFFFFu, t[0], 2);
+    return t[0] + __shfl_xor_sync(0xFFFFFFFFu, t[0], 1);
+}
+
 // biased exponent of v (zero and denormals: 1), kNonFinite for infinities and NaN
 __device__ __forceinline__ int fx_exponent(double v)
 {

@@ -108,7 +108,8 @@ __device__ __forceinline__ double warp_sum(double x)
 }
 
 // ---------------------------------------------------------------------------
-// a3: kernel sums (lab frame); u^0 and the rest-frame division happen in the EoS pass
+// a3: kernel sums (lab frame); u^0 and the rest-frame division happen in the EoS pass.  Kernel values
+// in integers and the lanes' sums by halves as in the 2D pass: 11 FP64 operations per pair (25).
 __global__ void __launch_bounds__(32 * kWarps3) k_density3(EvView v, const double *__restrict__ y,
                                                            const float4 *__restrict__ fpos,
                                                            const double *__restrict__ Nq,
@@ -141,8 +142,9 @@ __global__ void __launch_bounds__(32 * kWarps3) k_density3(EvView v, const doubl
             if (qb < 0 && !(dist2_3d(dx, dy, dz) < v.supp2)) return;
             {
                 const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
-                double q = r2 > 0.0 ? r2 * inv_sqrt(r2) * v.inv_h : 0.0;
-                double w = kernel_w(q);
+                long long wf, g[3];
+                pair_fixed<3>({dx, dy, dz}, r2, v.inv_h, wf, g);
+                const double w = fixed_value(wf);
                 sg += w;
                 ss = fma(S[b], w, ss);
                 sb = fma(Nq[b], w, sb);
@@ -152,19 +154,11 @@ __global__ void __launch_bounds__(32 * kWarps3) k_density3(EvView v, const doubl
             }
         };
         walk27(v, start, cnt, fpos, a, xa, queue[wid], pair);
-        sg = warp_sum(sg);
-        ss = warp_sum(ss);
-        sb = warp_sum(sb);
-        sS = warp_sum(sS);
-        sq = warp_sum(sq);
-        for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xFFFFFFFFu, c, o);
+        double t[8] = {sg, ss, sb, sS, sq, 0.0, 0.0, 0.0};
+        const double tot = warp_sums8(t, lane);
+        c = (int)__reduce_add_sync(0xFFFFFFFFu, (unsigned)c);
+        if ((lane & 3) == 0 && lane < 20) dens[(size_t)(lane >> 2) * n + a] = v.sigma_d * tot;
         if (lane == 0) {
-            const double sd = v.sigma_d;
-            dens[a] = sd * sg;
-            dens[n + a] = sd * ss;
-            dens[2 * n + a] = sd * sb;
-            dens[3 * n + a] = sd * sS;
-            dens[4 * n + a] = sd * sq;
             nnb[a] = c;
             if (cnt_dst) cnt_dst[a] = c;  // sizes the pair-list rows of the next stage
             atomicAdd(&v.sc->pairs, (unsigned long long)c);

@@ -58,3 +58,20 @@ def test_fixed_sums_against_oracle(dim, n, extent, decades, coincident):
     for rows in (slice(0, dim * dim), slice(dim * dim, dim * dim + dim)):
         assert np.max(np.abs(grad[rows] - og[rows])) <= 10 * TOL * max(np.max(np.abs(og[rows])), 1e-300)
     g.free()
+
+
+@pytest.mark.parametrize("dim", [2, 3])
+@pytest.mark.parametrize("n,extent,decades,coincident", [(1, 0.1, 0.0, False), (3, 3.0, 0.0, False), (64, 0.5, 0.0, True),
+                                                         (501, 0.8, 8.0, False), (2501, 0.17, 1.0, False)])
+def test_densities_without_lists_against_oracle(dim, n, extent, decades, coincident):
+    """A new state's read-out (no lists yet): the per-particle density pass."""
+    ev = _event(dim, n, extent, decades, coincident)
+    g = Bd.GpuEvent(ev)
+    f = g.read(("NNB", "SIGMA_STAR", "S_DENS", "N_DENS"))
+    aux, _ = O.OracleRun.start(ev).observe()
+    A = O.AUX
+    assert np.array_equal(f["NNB"], aux[A["nnb"]].astype(np.int32))
+    assert np.max(np.abs(f["SIGMA_STAR"] / aux[A["sigstar"]] - 1.0)) < TOL
+    assert np.max(np.abs(f["S_DENS"] / aux[A["s"]] - 1.0)) < TOL
+    assert np.max(np.abs(f["N_DENS"] - aux[A["nB"]:A["nQ"] + 1]) / aux[A["s"]]) < 0.01 * TOL
+    g.free()
