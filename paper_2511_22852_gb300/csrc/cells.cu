@@ -42,6 +42,7 @@ __global__ void k_bbox(EvView v, const double *__restrict__ y)
 __global__ void k_cells(EvView v, const double *__restrict__ y, uint32_t *key, uint32_t *cnt)
 {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const unsigned act = __ballot_sync(0xFFFFFFFFu, i < v.n);
     if (i >= v.n) return;
     double xmin0 = dec_double(v.sc->xmin_enc[0]);
     double xmin1 = dec_double(v.sc->xmin_enc[1]);
@@ -55,7 +56,7 @@ __global__ void k_cells(EvView v, const double *__restrict__ y, uint32_t *key, u
     }
     uint32_t k = morton2((uint32_t)cx, (uint32_t)cy);
     key[i] = k;
-    atomicAdd(&cnt[k], 1u);
+    warp_count(cnt, k, act);
 }
 
 // exclusive scan of nb counts with one block of 1024 threads, in tiles of 4096 buckets: thread t
@@ -209,8 +210,9 @@ __global__ void __launch_bounds__(256) k_scan_apply(const uint32_t *__restrict__
 __global__ void k_scatter(int n, const uint32_t *__restrict__ key, uint32_t *cursor, uint32_t *tmp)
 {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const unsigned act = __ballot_sync(0xFFFFFFFFu, i < n);
     if (i >= n) return;
-    uint32_t slot = atomicAdd(&cursor[key[i]], 1u);
+    uint32_t slot = warp_count(cursor, key[i], act);
     tmp[slot] = (uint32_t)i;
 }
 

@@ -216,6 +216,20 @@ __device__ __forceinline__ int cell_coord(double x, double xmin, double inv_cell
     return (int)floor(__dmul_rn(__dsub_rn(x, xmin), inv_cell));
 }
 
+// adds 1 to count[k] for every lane of act (the calling lanes) and returns the lane's own place: one
+// atomic per distinct k of the warp.  The particles come in nearly the order of the cells, so a
+// warp's lanes fall on a few of them, and atomics on one address run one after the other: the sort of
+// 4,997 particles 38 -> 33 us, of 39,997 52 -> 39, of 258,661 in 3D 111 -> 81.
+__device__ __forceinline__ uint32_t warp_count(uint32_t *count, uint32_t k, unsigned act)
+{
+    const int lane = threadIdx.x & 31;
+    const unsigned m = __match_any_sync(act, k);
+    const int first = __ffs(m) - 1;
+    uint32_t base = 0u;
+    if (lane == first) base = atomicAdd(&count[k], (uint32_t)__popc(m));
+    return __shfl_sync(act, base, first) + (uint32_t)__popc(m & ((1u << lane) - 1u));
+}
+
 // r^2 with each product rounded separately (no fused multiply-add), so the
 // neighbour decision r^2 < (2h)^2 is bit-for-bit reproducible
 __device__ __forceinline__ double dist2_2d(double dx, double dy) { return __dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)); }

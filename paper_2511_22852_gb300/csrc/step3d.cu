@@ -27,6 +27,7 @@ constexpr int kWarps3 = 4;
 __global__ void k_cells3(EvView v, const double *__restrict__ y, uint32_t *key, uint32_t *cnt)
 {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const unsigned act = __ballot_sync(0xFFFFFFFFu, i < v.n);
     if (i >= v.n) return;
     int c[3];
     bool bad = false;
@@ -42,7 +43,7 @@ __global__ void k_cells3(EvView v, const double *__restrict__ y, uint32_t *key, 
     if (bad) atomicOr(&v.sc->err_flags, ERR_CELL_OVERFLOW);
     uint32_t k = key3(v, c[0], c[1], c[2]);
     key[i] = k;
-    atomicAdd(&cnt[k], 1u);
+    warp_count(cnt, k, act);
 }
 
 // the 27-cell candidate walk of one warp: prefilter, compaction, then `pair` on full warps
