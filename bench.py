@@ -794,7 +794,7 @@ def run_ours(args):
         peak32 = f"measured FP32 FMA rate of this GPU ({fp32_gflops:.0f} GFLOP/s, sph_measure_fma_peak)"
         ppl = psteps / max(1, batch_steps)  # mean particles per launch (resident per batch step)
         rooflines = {
-            "eos": alu_roof("eos", flops["eos"], g_ms["eos"], launches_g, fp64_gflops, peak64, "k_eos2_seg",
+            "eos": alu_roof("eos", flops["eos"], g_ms["eos"], launches_g, fp64_gflops, peak64, "k_eos2_seg_find+finish",
                             traffic_of("k_eos2_seg", ppl)),
             "density": alu_roof("density", flops["density"], g_ms["density"], launches_g, fp32_gflops, peak32,
                                 "k_seg_density", traffic_of("k_seg_density", ppl)),
@@ -817,7 +817,7 @@ def run_ours(args):
         fp64ev.pop("_launches")
         fp64ev["kernel_rooflines"] = {
             k: alu_roof(k, f64[k], t64[k][0], t64[k][1], fp64_gflops, peak64,
-                        {"density": "k_pairs_density_fwd+bwd", "gradient": "k_pairs_gradient", "eos": "k_eos2"}[k],
+                        {"density": "k_pairs_fwd+sum", "gradient": "k_pairs_gradient", "eos": "k_eos2_find+finish"}[k],
                         traffic_of({"density": "k_pairs_density", "gradient": "k_pairs_gradient", "eos": "k_eos2"}[k]))
             for k in f64}
         events_hr = 3600.0 * args.events / res["wall"]

@@ -690,9 +690,9 @@ __device__ EosOut eos_invert(const EosDev &E, double cs2_cap, double s, const do
 // across a cell boundary, rarely) goes through the general FP64 inversion from that point.
 //
 // Bound: the FP64 pipe (64 cycles per warp instruction and quadrant).  Measured per stage on the
-// 40 k viscous BSQ event: 103 us (196 in one pass with the
-// derivatives and the solve of every evaluation in FP64), ideal Gubser lattice 31 (303), eight served
-// events (437 k particles) 616 (772), 3+1D Milne event of 258 k particles 595 (1,100).
+// 40 k viscous BSQ event: 106 us (196 in one pass with the derivatives and the solve of every
+// evaluation in FP64), ideal Gubser lattice 31 (303), eight served events (437 k particles) 588 (772),
+// 3+1D Milne event of 258 k particles, mixed form, 502 (976).
 //
 // Hand-over bounds on max |residual| / s: 1e-10 where the point has to be the root to rounding
 // (polish), 1e-6 for the 1e-10 tolerance of the mixed and serving forms.

@@ -9,7 +9,7 @@
 // depend on the order, so results are reproducible run to run.
 //
 // FP64 operations per unordered pair fall from 56 (26 for the kernel, 10 for the density and 20 for
-// the gradient sums of its two particles) to 12; the 40 k event's step 2,038 -> 1,310 us.
+// the gradient sums of its two particles) to 4; the 40 k event's step 2,038 -> 1,205 us.
 //
 // Rows: a particle's row holds its previous neighbour count plus a margin (a prefix scan per
 // stage); forward entries fill it from the start, backward entries from the end.

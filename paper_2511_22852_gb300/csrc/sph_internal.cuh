@@ -394,7 +394,8 @@ __device__ __forceinline__ void warp_or(unsigned int *dst, unsigned int v)
 
 // ---------------------------------------------------------------------------
 // launchers (implemented in cells.cu, density_eos.cu, gradient_eom.cu)
-// Half-pair lists of the plain 2D neighbour passes, rebuilt in every stage's density pass.
+// Half-pair lists of the plain neighbour passes, rebuilt in every stage's density pass (in the mixed
+// 3D form a plain neighbour list: L alone, filled from the row start).
 // Particle a (sorted index) owns entries [off[a], off[a+1]) of L, W, G, sized by its
 // neighbour count of the previous stage plus a margin (a prefix scan per stage):
 //   from the row start: its accepted neighbours b > a (L), with W(r)/sigma_d of the pair (W) and

@@ -1,4 +1,4 @@
-// tiled_common.cuh -- device helpers of the cell-tiled FP32 neighbour passes (the serving form's
+// tiled_common.cuh -- device helpers of the FP32 neighbour passes (the serving form's cell-tiled ones
 // and the per-event mixed form's): compensated single-precision sums, the error-free combination
 // of a particle's lanes, the lanes-per-particle rule, and the packed two-wide candidate layout.
 #pragma once
