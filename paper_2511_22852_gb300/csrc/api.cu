@@ -248,7 +248,7 @@ static void enqueue_step(sph_event *ev)
         const double *src[4] = {ev->Y[0], ev->Nq[0], ev->wguess, ev->eprev[0]};
         double *dst[4] = {ev->Y[1], ev->Nq[1], ev->guess_in, ev->eprev[1]};
         int rows[4] = {ev->nv, 3, 4, 1};
-        launch_permute(v, ev->cb, src, dst, rows, ev->fo_on ? 4 : 3, ev->id[0], ev->id[1], ev->dens, st);
+        launch_permute(v, ev->cb, src, dst, rows, ev->fo_on ? 4 : 3, src[0], src[0] + ev->dim * (size_t)ev->n, ev->id[0], ev->id[1], ev->dens, st);
     }
     mark(ev, G_PERMUTE, 1, 1);
     mark(ev, G_DENSITY, 1, 0);
@@ -285,7 +285,7 @@ static void enqueue_step(sph_event *ev)
         int ng = 4;
         if (ev->charges) src[ng] = ev->NqS[0], dst[ng] = ev->NqS[1], rows[ng++] = 3;
         if (ev->fo_on) src[ng] = ev->eprev[1], dst[ng] = ev->eprev[0], rows[ng++] = 1;
-        launch_permute(v, ev->cb, src, dst, rows, ng, ev->id[1], ev->id[0], ev->dens, st);
+        launch_permute(v, ev->cb, src, dst, rows, ng, src[0], src[0] + ev->dim * (size_t)ev->n, ev->id[1], ev->id[0], ev->dens, st);
     }
     mark(ev, G_PERMUTE, 2, 1);
     mark(ev, G_DENSITY, 2, 0);
@@ -335,7 +335,7 @@ static void enqueue_observe(sph_event *ev)
     const double *src[3] = {ev->Y[0], ev->Nq[0], ev->wguess};
     double *dst[3] = {ev->Y[1], ev->Nq[1], ev->guess_in};
     int rows[3] = {ev->nv, 3, 4};
-    launch_permute(v, ev->cb, src, dst, rows, 3, ev->id[0], ev->id[1], ev->dens, st);
+    launch_permute(v, ev->cb, src, dst, rows, 3, src[0], src[0] + ev->dim * (size_t)ev->n, ev->id[0], ev->id[1], ev->dens, st);
     launch_density(v, ev->Y[1], ev->Nq[1], stage_cb(ev, 0, -1), ev->dens, ev->nnb, st);
     launch_eos(v, 1, ev->Y[1], ev->dens, ev->eosf, ev->gin, ev->status, ev->wpart, ev->guess_in, ev->wguess_obs, st);
 }

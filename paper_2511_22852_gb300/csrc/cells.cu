@@ -236,6 +236,7 @@ struct PermArgs {
     double *dst[8];
     int rows[8];
     int ngroups;
+    const double *x, *u;  // position rows, and velocity rows for u0 (nullptr: no u0), before the sort
 };
 
 // Gathers the rows into the cell order.  Block row 0 writes the ids and what the neighbour passes
@@ -270,8 +271,8 @@ __global__ void k_permute(EvView v, const uint32_t *__restrict__ perm, PermArgs 
         return;
     }
     id_out[j] = id_in[s];
-    // what the neighbour passes read per particle in single precision, from the state (rows src[0] on)
-    const double *y = a.src[0] + s;
+    // what the neighbour passes read per particle in single precision
+    const double *y = a.x + s;
     if (v.dim == 3) {
         if (v.mixed) return;  // k_relpos3
         float f[3];
@@ -294,8 +295,8 @@ __global__ void k_permute(EvView v, const uint32_t *__restrict__ perm, PermArgs 
         f[d] = __double2float_rn(r);
     }
     fpos[j] = make_float2(f[0], f[1]);
-    if (!v.mixed) {  // u0 = sqrt(1 + u.u) (density row 5)
-        const double ux = y[2 * (size_t)n], uy = y[3 * (size_t)n];
+    if (a.u) {  // u0 = sqrt(1 + u.u) (density row 5)
+        const double ux = a.u[s], uy = a.u[(size_t)n + s];
         dens[5 * (size_t)n + j] = sqrt(fma(ux, ux, fma(uy, uy, 1.0)));
     }
 }
@@ -428,10 +429,13 @@ void launch_cells(const EvView &v, const double *y, const int *id, CellBufs cb, 
 }
 
 void launch_permute(const EvView &v, const CellBufs &cb, const double *const *src, double *const *dst,
-                    const int *nrows, int ngroups, const int *id_in, int *id_out, double *dens, cudaStream_t st)
+                    const int *nrows, int ngroups, const double *x, const double *u, const int *id_in, int *id_out,
+                    double *dens, cudaStream_t st)
 {
     PermArgs a;
     a.ngroups = ngroups;
+    a.x = x;
+    a.u = v.dim == 2 && !v.mixed ? u : nullptr;  // the other forms' passes write u0 themselves
     int total = 0;
     for (int g = 0; g < ngroups; ++g) {
         a.src[g] = src[g];

@@ -128,11 +128,9 @@ __global__ void __launch_bounds__(32 * kWarps) k_density2(EvView v, const double
         double t[8] = {sg, ss, sb, sS, sq, 0.0, 0.0, 0.0};
         const double tot = warp_sums8(t, lane);
         c = (int)__reduce_add_sync(0xFFFFFFFFu, (unsigned)c);
-        // rows sigma*, lab-frame s* (divided by u0 sqrt(-g) in the EoS pass), n*_B, n*_S, n*_Q, u0
+        // rows sigma*, lab-frame s* (divided by u0 sqrt(-g) in the EoS pass), n*_B, n*_S, n*_Q
         if ((lane & 3) == 0 && lane < 20) dens[(size_t)(lane >> 2) * n + a] = v.sigma_d * tot;
         if (lane == 0) {
-            const double ux = y[2 * (size_t)n + a], uy = y[3 * (size_t)n + a];
-            dens[5 * (size_t)n + a] = sqrt(fma(ux, ux, fma(uy, uy, 1.0)));
             nnb[a] = c;
             if (cnt_dst) cnt_dst[a] = c;  // sizes the pair-list rows of the next stage
             atomicAdd(&v.sc->pairs, (unsigned long long)c);

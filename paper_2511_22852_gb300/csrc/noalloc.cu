@@ -217,7 +217,7 @@ extern "C" sph_status sph_density_noalloc(const double *x, const double *u, cons
         const double *src[4] = {x, u, S, Nq};
         double *dst[4] = {ys, ys + 2 * (size_t)nn, ys + 4 * (size_t)nn, nqs};
         int rows[4] = {2, 2, 1, 3};
-        launch_permute(v, cb, src, dst, rows, 4, id_in, id_out, dens, st);
+        launch_permute(v, cb, src, dst, rows, 4, x, u, id_in, id_out, dens, st);
     }
     launch_density(v, ys, nqs, cb, dens, nnb, st);
     k_unsort<<<(nn + 255) / 256, 256, 0, st>>>(dens, id_out, nn, milne ? tau : 1.0, out);

@@ -472,10 +472,12 @@ inline float prefilter_bound(double h, int B, int dim = 2)
 
 void launch_bbox(const EvView &v, const double *y, cudaStream_t st);
 void launch_cells(const EvView &v, const double *y, const int *id, CellBufs cb, cudaStream_t st);
-// dst[0] on holds the state: its sorted single-precision positions (and u0, plain 2D: density row 5) are
-// written for the neighbour passes
+// x, u: the position and velocity rows before the sort (n apart, each in its own array where the
+// caller's are); from them the sorted single-precision positions and, in the plain 2D form, u0 (density
+// row 5: its only writer) for the neighbour passes
 void launch_permute(const EvView &v, const CellBufs &cb, const double *const *src, double *const *dst,
-                    const int *nrows, int ngroups, const int *id_in, int *id_out, double *dens, cudaStream_t st);
+                    const int *nrows, int ngroups, const double *x, const double *u, const int *id_in, int *id_out,
+                    double *dens, cudaStream_t st);
 // plain 2D neighbour passes over the half-pair lists (cb.pl.total > 0): row offsets from the
 // previous counts, then the forward and backward density passes
 void launch_pairs_density(const EvView &v, const double *y, const double *Nq, CellBufs cb, double *dens, int *nnb,

@@ -64,6 +64,38 @@ def test_noalloc_density_matches_event_path_on_consecutive_calls():
             assert not np.any(o[2:5])
 
 
+@pytest.mark.parametrize("order", ["x S Nq u", "u x Nq S"])
+def test_noalloc_reads_each_array_by_itself(order):
+    """The four arrays in one allocation, with other rows than u behind x: s = s*/(u0 sqrt(-g)) takes u0
+    from the caller's u, and no array is read beyond its rows."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2511_22852_gb300 import binding as Bd
+    from paper_2511_22852_gb300 import build_lib
+    build_lib.build()
+    f = _noalloc(Bd)
+    n, h, tau = 1500, 0.3, 0.8
+    a = {"x": I.random_points(n, 2, 1.5, 5), "u": 2.0 * I.random_points(n, 2, 1.0, 6),
+         "S": 0.5 + I.uniform01(7, n).reshape(1, n), "Nq": I.uniform01(8, 3 * n).reshape(3, n)}
+    names = order.split()
+    # 4 rows that no array may reach, behind the last one
+    big = torch.tensor(np.concatenate([a[k] for k in names] + [np.full((4, n), 1e3)]), dtype=torch.float64, device="cuda")
+    first = dict(zip(names, np.cumsum([0] + [a[k].shape[0] for k in names])))
+    out = torch.full((5, n), float("nan"), dtype=torch.float64, device="cuda")
+    rc = f(*[big[first[k]].data_ptr() for k in ("x", "u", "S", "Nq")], n, h, tau, 1, out.data_ptr(),
+           torch.cuda.current_stream().cuda_stream)
+    assert rc == Bd.SPH_OK, Bd.lib().sph_last_error().decode()
+    d = a["x"][:, :, None] - a["x"][:, None, :]
+    q = np.sqrt(np.sum(d * d, axis=0)) / h
+    w = np.where(q < 2.0, 0.25 * (2.0 - q) ** 3 - np.maximum(1.0 - q, 0.0) ** 3, 0.0) * 10.0 / (7.0 * np.pi * h * h)
+    vol = np.sqrt(1.0 + np.sum(a["u"] ** 2, axis=0)) * tau
+    o = out.cpu().numpy()
+    assert _relerr(o[0], np.sum(w, axis=1)) < TOL
+    for k, row in ((1, a["S"][0]), (2, a["Nq"][0]), (3, a["Nq"][1]), (4, a["Nq"][2])):
+        assert np.max(np.abs(o[k] * vol / (w @ row) - 1.0)) < TOL
+
+
 def test_noalloc_rejects_sizes_beyond_its_limit():
     torch = pytest.importorskip("torch")
     if not torch.cuda.is_available():
