@@ -78,7 +78,7 @@ struct sph_event {
     int diff = 0;
     double kapT2[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0}, tauJT[3] = {0, 0, 0};
     double *dinp = nullptr, *dal = nullptr, *dout = nullptr;
-    int4 *dfx = nullptr;
+    longlong2 *dfx = nullptr;
     uint4 *dfe = nullptr;
     cudaStream_t stream = nullptr;
     bool own_stream = false;
@@ -200,7 +200,6 @@ static EvView make_view(const sph_event *ev)
     v.dfx = ev->dfx;
     v.dfe = ev->dfe;
     v.fxX = ev->cb.pl.total > 0 && !ev->mixed ? ev->cb.pl.X : nullptr;
-    v.fxE = ev->cb.pl.Xe;
     v.fX = ev->cb.fx;
     return v;
 }
@@ -674,7 +673,7 @@ sph_status sph_init_event(sph_event **out, const sph_event_desc *d, const sph_eo
         AL(ev->dal, dv * 12);
         AL(ev->dout, dv * 9);
         if (!ev->mixed) {
-            AL(ev->dfx, sizeof(int4) * 5 * N);
+            AL(ev->dfx, sizeof(longlong2) * 5 * N);
             AL(ev->dfe, sizeof(uint4) * N);
         }
         ev->charges = true;
@@ -774,14 +773,14 @@ static sph_status size_pair_lists(sph_event *ev)
     if (ev->pairs_grow) total = std::max<long long>(total, ev->cb.pl.total * 3 / 2);
     else if (const char *t = getenv("SPH_PAIR_TOTAL")) total = std::max<long long>(1, atoll(t));
     const int nparts = (n + 2047) / 2048;
-    // per entry: L (int), W and the kernel gradient (2 64-bit integers, 3D: 3 padded to 4)
-    const size_t gsize = ev->mixed ? 0 : (ev->dim == 2 ? sizeof(longlong2) : sizeof(longlong4_32a));
-    const size_t per_entry = sizeof(int) + (ev->mixed ? 0 : sizeof(long long)) + gsize;
+    // per entry: L (int), W and the kernel gradient (2 doubles, 3D: 3 padded to 4)
+    const size_t gsize = ev->mixed ? 0 : (ev->dim == 2 ? sizeof(double2) : sizeof(double4_32a));
+    const size_t per_entry = sizeof(int) + (ev->mixed ? 0 : sizeof(double)) + gsize;
     // per particle: two counts and two carried counts, the values in limbs and their exponents
     // (the mixed form keeps the indices alone)
-    const int nx = ev->mixed ? 0 : (ev->dim == 2 ? 3 : 6);  // planes of the gradient-pass inputs
-    const int nq = ev->mixed ? 0 : 2;
-    const size_t per_particle = 5 * sizeof(int) + 4 * sizeof(unsigned short) + (size_t)(nq + nx) * sizeof(int4);
+    const int nx = ev->mixed ? 0 : (ev->dim == 2 ? 2 : 4);  // planes of the gradient-pass inputs
+    const int nq = ev->mixed ? 0 : 1;
+    const size_t per_particle = 4 * sizeof(int) + 4 * sizeof(unsigned short) + (size_t)(nq + nx) * sizeof(Limb4);
     const size_t bytes = (size_t)total * per_entry + (size_t)(n + 1) * sizeof(long long) +
                          (size_t)nparts * sizeof(unsigned long long) + per_particle * (size_t)n + 1024;
     size_t fr = 0, tot = 0;
@@ -808,15 +807,16 @@ static sph_status size_pair_lists(sph_event *ev)
     PairBufs pl{};
     pl.total = total;
     pl.margin = margin;
-    // the most aligned arrays first (32 bytes: the 3D gradients; 16: the others)
+    // the most aligned arrays first (32 bytes: the limbs and the 3D gradients; 16: the 2D gradients)
     char *p = static_cast<char *>(m);
-    if (ev->dim == 2) pl.G = reinterpret_cast<longlong2 *>(p);
-    else pl.G3 = reinterpret_cast<longlong4_32a *>(p);
-    pl.X = reinterpret_cast<int4 *>(p + gsize * (size_t)total);
+    pl.X = reinterpret_cast<Limb4 *>(p);
     pl.Q = pl.X + (size_t)nx * n;
-    long long *wbuf = reinterpret_cast<long long *>(pl.Q + (size_t)nq * n);
-    if (!ev->mixed) pl.W = wbuf;
-    pl.off = ev->mixed ? wbuf : wbuf + total;
+    p = reinterpret_cast<char *>(pl.Q + (size_t)nq * n);
+    if (ev->dim == 2) pl.G = reinterpret_cast<double2 *>(p);
+    else pl.G3 = reinterpret_cast<double4_32a *>(p);
+    p += gsize * (size_t)total;
+    if (!ev->mixed) pl.W = reinterpret_cast<double *>(p);
+    pl.off = reinterpret_cast<long long *>(p + (ev->mixed ? 0 : sizeof(double) * (size_t)total));
     pl.part = reinterpret_cast<unsigned long long *>(pl.off + (n + 1));
     pl.Qe = reinterpret_cast<unsigned short *>(pl.part + nparts);  // read 8 bytes at a time
     pl.L = reinterpret_cast<int *>(pl.Qe + 4 * (size_t)n);
@@ -824,7 +824,6 @@ static sph_status size_pair_lists(sph_event *ev)
     pl.cntB = pl.cntF + n;
     ev->pcnt[0] = pl.cntB + n;
     ev->pcnt[1] = ev->pcnt[0] + n;
-    pl.Xe = reinterpret_cast<unsigned int *>(ev->pcnt[1] + n);
     launch_counts_to_state(ev->nnb, ev->cb.perm, ev->pcnt[0], n, ev->stream);
     pl.cnt_src = ev->pcnt[0];
     ev->cb.pl = pl;

@@ -35,7 +35,7 @@ constexpr int kWarps = 4;  // warps (particles in flight) per block of the neigh
 // candidates at a time through a single-precision prefilter; survivors are compacted
 // (ballot) into a per-warp queue and, 32 at a time, go through the exact FP64 test
 // r^2 < (2h)^2 and the kernel sum with every lane busy.  The kernel value is formed in integers
-// (pair_fixed), and the lanes' sums exchange halves before they are added: the order is fixed, so
+// (pair_kernel), and the lanes' sums exchange halves before they are added: the order is fixed, so
 // results are reproducible.
 // Runs for events without lists: read-outs of new states, and stages whose lists overflowed.
 // Bound: the FP64 pipe, 9 operations per pair (22 with distance and kernel in FP64) and 9 additions a
@@ -81,9 +81,8 @@ __global__ void __launch_bounds__(32 * kWarps) k_density2(EvView v, const double
             if (qb < 0 && !(dist2_2d(dx, dy) < v.supp2)) return;
             {
                 const double r2 = fma(dx, dx, dy * dy);
-                long long wf, g[2];
-                pair_fixed<2>({dx, dy}, r2, v.inv_h, wf, g);
-                const double w = fixed_value(wf);
+                double w, g[2];
+                pair_kernel<2>({dx, dy}, r2, v.inv_h, w, g);
                 sg += w;
                 ss = fma(S[b], w, ss);
                 sb = fma(NB[b], w, sb);
@@ -238,11 +237,12 @@ __device__ __forceinline__ double eos2_store(const EvView &v, int stage, size_t 
         reinterpret_cast<float2 *>(v.fX + n)[a] = make_float2((float)us[0], (float)us[1]);
     }
     if (LIMBS && v.fxX) {  // the same in limbs for the pair-list gradient pass
-        const int eX = fx_shared_exponent(X), eu = fx_shared_exponent(us);
-        v.fxX[a] = fx_limbs2(X[0], eX, X[1], eX);
-        v.fxX[n + a] = fx_limbs2(X[2], eX, X[3], eX);
-        v.fxX[2 * n + a] = fx_limbs2(us[0], eu, us[1], eu);
-        v.fxE[a] = (unsigned)eX | ((unsigned)eu << 16);
+        const int e0 = fx_exponent(X[0]), e1 = fx_exponent(X[1]), e2 = fx_exponent(X[2]), e3 = fx_exponent(X[3]);
+        const int eu0 = fx_exponent(us[0]), eu1 = fx_exponent(us[1]);
+        v.fxX[a] = Limb4{fx_word(fx_limbs(X[0], e0)), fx_word(fx_limbs(X[1], e1)), fx_word(fx_limbs(X[2], e2)),
+                         fx_word(fx_limbs(X[3], e3))};
+        v.fxX[n + a] = Limb4{fx_word(fx_limbs(us[0], eu0)), fx_word(fx_limbs(us[1], eu1)),
+                             fx_word(fx_pair(e0, e1), fx_pair(e2, e3)), fx_word(fx_pair(eu0, eu1), 0u)};
     }
     double wcontrib = 0.0;
     if (v.milne) {

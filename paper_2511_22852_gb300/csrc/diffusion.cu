@@ -52,18 +52,17 @@ __global__ void __launch_bounds__(128) k_diff_prep(EvView v, int stage, const do
         v.dinp[(3 + 2 * q) * n + a] = Fq[q][0];
         v.dinp[(4 + 2 * q) * n + a] = Fq[q][1];
     }
-    if (v.dfx) {  // the same in limbs for the pair-list pass
-        int ea[3], ef[3];
+    if (v.dfx) {  // for the pair-list pass: alpha, and the fluxes in limbs
+        unsigned ef[3];
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
-            ea[q] = fx_exponent(al[q]);
-            ef[q] = fx_shared_exponent(Fq[q]);
-            v.dfx[(2 + q) * n + a] = fx_limbs2(Fq[q][0], ef[q], Fq[q][1], ef[q]);
+            const int e0 = fx_exponent(Fq[q][0]), e1 = fx_exponent(Fq[q][1]);
+            v.dfx[(2 + q) * n + a] = make_longlong2(fx_word(fx_limbs(Fq[q][0], e0)), fx_word(fx_limbs(Fq[q][1], e1)));
+            ef[q] = fx_pair(e0, e1);
         }
-        v.dfx[a] = fx_limbs2(al[0], ea[0], al[1], ea[1]);
-        v.dfx[n + a] = fx_limbs2(al[2], ea[2], 0.0, ea[2]);
-        v.dfe[a] = make_uint4((unsigned)ea[0] | ((unsigned)ea[1] << 16), (unsigned)ea[2] | ((unsigned)ef[0] << 16),
-                              (unsigned)ef[1] | ((unsigned)ef[2] << 16), 0u);
+        v.dfx[a] = make_longlong2(__double_as_longlong(al[0]), __double_as_longlong(al[1]));
+        v.dfx[n + a] = make_longlong2(__double_as_longlong(al[2]), 0);
+        v.dfe[a] = make_uint4(ef[0], ef[1], ef[2], 0u);
     }
     double dal[3][4];
 #pragma unroll
@@ -160,9 +159,8 @@ __device__ __forceinline__ void diff_finish(const EvView &v, int stage, const do
 }
 
 // pair-list form (plain 2D events): half a warp per particle over the entries of its row with the
-// kernel gradient stored there (grad_a W_ab h / sigma_d), in integers (pairs_fixed.cuh): alpha_b -
-// alpha_a is formed in units of the neighbours' largest alpha (zero for a uniform alpha), the fluxes
-// are summed as the gradient pass sums the stresses.
+// kernel gradient stored there (grad_a W_ab h / sigma_d), in integers (pairs_fixed.cuh) but for
+// alpha_b - alpha_a, an FP64 subtraction; the fluxes are summed as the gradient pass sums the stresses.
 // Bound: the latency of the gathers; 40 k event, diffusion and EoS passes per step 1,561 -> 860 us
 // (17 FP64 operations per pair before).
 __global__ void __launch_bounds__(32 * kDiffWarps, 4) k_diff_pairs(EvView v, int stage, const double *__restrict__ dens,
@@ -178,30 +176,36 @@ __global__ void __launch_bounds__(32 * kDiffWarps, 4) k_diff_pairs(EvView v, int
     const long long r0 = pl.off[a], r1 = pl.off[a + 1];
     const int nf = on ? pl.cntF[a] : 0, nt = on ? nf + pl.cntB[a] : 0;
     auto at = [&](int j) { return j < nf ? r0 + j : r1 - nt + j; };  // entry j of a's row
-    uint4 em = v.dfe[a];
+    const double2 *alpha = reinterpret_cast<const double2 *>(v.dfx);
+    const double aa[3] = {alpha[a].x, alpha[a].y, alpha[n + a].x};
+    // the largest exponents among the terms of each sum, two in 16-bit halves: g_x | g_y, (alpha_b - alpha_a)_q
+    // g_x | g_y, F_q^x g_x | F_q^y g_y
+    unsigned mG = 0u, mA[3] = {0u, 0u, 0u}, mF[3] = {0u, 0u, 0u};
     for (int j = l; j < nt; j += 16) {
-        const uint4 e = v.dfe[pl.L[at(j)]];
-        em = make_uint4(fx_max2(em.x, e.x), fx_max2(em.y, e.y), fx_max2(em.z, e.z), 0u);
+        const long long i = at(j);
+        const int b = pl.L[i];
+        const double2 g = pl.G[i], al0 = alpha[b], al1 = alpha[n + b];
+        const uint4 e = v.dfe[b];
+        const unsigned eg = fx_pair(fx_kexp(g.x), fx_kexp(g.y)), ef[3] = {e.x, e.y, e.z};
+        const double al[3] = {al0.x, al0.y, al1.x};
+        mG = fx_max2(mG, eg);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const int ea = fx_exponent(al[q] - aa[q]);
+            mA[q] = fx_max2(mA[q], fx_pair(ea, ea) + eg);
+            mF[q] = fx_max2(mF[q], ef[q] + eg);
+        }
     }
-    em = make_uint4(fx_half_max2(em.x), fx_half_max2(em.y), fx_half_max2(em.z), 0u);
-    const int m[6] = {(int)(em.x & 0xFFFFu), (int)(em.x >> 16), (int)(em.y & 0xFFFFu),
-                      (int)(em.y >> 16), (int)(em.z & 0xFFFFu), (int)(em.z >> 16)};
-    int E[6];
+    mG = fx_half_max2(mG);
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
-        E[q] = fx_room(m[q] + 1, nt);  // the difference of two values
-        E[3 + q] = fx_room(m[3 + q], nt);
+        mA[q] = fx_half_max2(mA[q]);
+        mF[q] = fx_half_max2(mF[q]);
     }
-    // a value's mantissa in units of 2^(E - 1076)
-    auto mantissa = [](int2 q, int d) { return ((long long)q.x * (1LL << kLimb) + q.y) >> min(d, 63); };
-    long long ma[3];
-    {
-        const int4 x0 = v.dfx[a], x1 = v.dfx[n + a];
-        const uint4 e = v.dfe[a];
-        ma[0] = mantissa(lo_of(x0), E[0] - (int)(e.x & 0xFFFFu));
-        ma[1] = mantissa(hi_of(x0), E[1] - (int)(e.x >> 16));
-        ma[2] = mantissa(lo_of(x1), E[2] - (int)(e.y & 0xFFFFu));
-    }
+    // exponents of the 11 sums: g (2), 2 + 2 q + i: (alpha_b - alpha_a) g_i, 8 + q: F_b . g
+    const int Em[11] = {fx_lo(mG), fx_hi(mG), fx_lo(mA[0]), fx_hi(mA[0]), fx_lo(mA[1]), fx_hi(mA[1]), fx_lo(mA[2]), fx_hi(mA[2]),
+                        max(fx_lo(mF[0]), fx_hi(mF[0])), max(fx_lo(mF[1]), fx_hi(mF[1])), max(fx_lo(mF[2]), fx_hi(mF[2]))};
+    const int room = fx_room(0, nt);
     FxSum sG[2] = {{0, 0}, {0, 0}}, sA[3][2], sF[3];
 #pragma unroll
     for (int q = 0; q < 3; ++q) sA[q][0] = sA[q][1] = sF[q] = FxSum{0, 0};
@@ -218,30 +222,28 @@ __global__ void __launch_bounds__(32 * kDiffWarps, 4) k_diff_pairs(EvView v, int
     for (int j = l, it = 1; j < nt; j += 16, ++it) {
         const long long i = at(j);
         const int b = pl.L[i];
-        const longlong2 g = pl.G[i];
-        const int4 x0 = v.dfx[b], x1 = v.dfx[n + b];
+        const double2 g = pl.G[i], al0 = alpha[b], al1 = alpha[n + b];
         const uint4 e = v.dfe[b];
-        const int eb[6] = {(int)(e.x & 0xFFFFu), (int)(e.x >> 16), (int)(e.y & 0xFFFFu),
-                           (int)(e.y >> 16), (int)(e.z & 0xFFFFu), (int)(e.z >> 16)};
-        const int2 al[3] = {lo_of(x0), hi_of(x0), lo_of(x1)};
-        sG[0].x += g.x;
-        sG[1].x += g.y;
-        int gxh, gxl, gyh, gyl;
-        fx_split(g.x, 0, gxh, gxl);
-        fx_split(g.y, 0, gyh, gyl);
+        const unsigned ef[3] = {e.x, e.y, e.z};
+        const double al[3] = {al0.x, al0.y, al1.x};
+        const long long m[2] = {fx_kmant(g.x), fx_kmant(g.y)};
+        const int eg[2] = {fx_kexp(g.x) - room, fx_kexp(g.y) - room};
+        int hi, lo;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) sG[k].x += fx_shift(m[k], Em[k] - eg[k] + kGuard);
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
-            const long long d = mantissa(al[q], E[q] - eb[q]) - ma[q];
-            const int lo = (int)((unsigned)d << (32 - kLimb)) >> (32 - kLimb);
-            const int2 da = make_int2((int)((d - lo) >> kLimb), lo);
-            fx_add(sA[q][0], gxh, gxl, da);
-            fx_add(sA[q][1], gyh, gyl, da);
-            const int4 F = v.dfx[(2 + q) * n + b];
-            int hi, lo2;
-            fx_split(g.x, E[3 + q] - eb[3 + q], hi, lo2);
-            fx_add(sF[q], hi, lo2, lo_of(F));
-            fx_split(g.y, E[3 + q] - eb[3 + q], hi, lo2);
-            fx_add(sF[q], hi, lo2, hi_of(F));
+            const double d = al[q] - aa[q];
+            const int ea = fx_exponent(d);
+            const int2 da = fx_limbs(d, ea);
+            const longlong2 F = v.dfx[(2 + q) * n + b];
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                fx_split(m[k], Em[2 + 2 * q + k] - eg[k] - ea, hi, lo);
+                fx_add(sA[q][k], hi, lo, da);
+                fx_split(m[k], Em[8 + q] - eg[k] - (k ? fx_hi(ef[q]) : fx_lo(ef[q])), hi, lo);
+                fx_add(sF[q], hi, lo, fx_pair_of(k ? F.y : F.x));
+            }
         }
         if ((it & (kFoldEvery - 1)) == 0) fold();
     }
@@ -260,10 +262,12 @@ __global__ void __launch_bounds__(32 * kDiffWarps, 4) k_diff_pairs(EvView v, int
     const FxTotal tt = fx_reduce16(t, lane);
     // lane l: 0, 1 sum grad W; 2 + 2 q + i sum (alpha_b - alpha_a) grad_i W; 8 + q sum F_b . grad W
     const int q = l < 8 ? (l - 2) >> 1 : l - 8;
-    const int Eq = l < 8 ? (q <= 0 ? E[0] : (q == 1 ? E[1] : E[2])) : (q == 0 ? E[3] : (q == 1 ? E[4] : E[5]));
-    const int mq = l < 8 ? (q <= 0 ? m[0] : (q == 1 ? m[1] : m[2])) : (q == 0 ? m[3] : (q == 1 ? m[4] : m[5]));
-    double tot = fx_value(tt, l < 2 ? -kFxBits : fx_unit(Eq));
-    if (l >= 2 && mq == kNonFinite) tot = fx_nan();
+    int El = Em[0];
+#pragma unroll
+    for (int i = 1; i < 11; ++i)
+        if (l == i) El = Em[i];
+    double tot = fx_value(tt, l < 2 ? fx_kunit(El + room) : fx_unit(El + room));
+    if (El >= kNonFinite) tot = fx_nan();
     const double Gx = __shfl_sync(kFull, tot, lane & 16), Gy = __shfl_sync(kFull, tot, (lane & 16) + 1);
     if (on && l >= 2 && l < 11) {
         const double c = v.sigma_d * v.inv_h;

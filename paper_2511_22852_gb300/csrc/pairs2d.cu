@@ -9,7 +9,7 @@
 // depend on the order, so results are reproducible run to run.
 //
 // FP64 operations per unordered pair fall from 56 (26 for the kernel, 10 for the density and 20 for
-// the gradient sums of its two particles) to 4; the 40 k event's step 2,038 -> 1,205 us.
+// the gradient sums of its two particles) to 4; the 40 k event's step 2,038 -> 1,262 us.
 //
 // Rows: a particle's row holds its previous neighbour count plus a margin (a prefix scan per
 // stage); forward entries fill it from the start, backward entries from the end.
@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(kScanThreads) k_rows_apply(int n, const uint32
 // Forward pass, a warp for two particles a.  Candidates of the cells from its own on (those within
 // 2h of a) pass the single-precision prefilter; a candidate b > a is queued, and 32 at a time -- of
 // both particles -- the exact test (where the float test left the pair undecided) and the kernel in
-// fixed point (pair_fixed) run on full warps.  W and grad W go into a's row and, at a place taken
+// integers (pair_kernel) run on full warps.  W and grad W go into a's row and, at a place taken
 // from b's counter, into b's row.  The particles' own values go into limbs.
 // (Listing b < a in a's own walk, and finding its W by a search in b's row, kept the sums waiting
 // for memory: 40 k event, sum pass 197 -> 92 us a stage, gradient pass 150 -> 137.)
@@ -147,7 +147,7 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_pairs_fwd(EvView v, const do
     if (lane < 4 * np) {
         const size_t a = (size_t)a0 + (lane >> 2);
         const int k = lane & 3;
-        fx_store_value(pl.Q, pl.Qe, (size_t)n, a, k, k == 0 ? S[a] : Nq[(size_t)(k - 1) * n + a]);
+        fx_store_value(pl.Q, pl.Qe, a, k, k == 0 ? S[a] : Nq[(size_t)(k - 1) * n + a]);
     }
     const unsigned lt = (1u << lane) - 1u;
     const double (*pos)[2] = pos_[wid];
@@ -180,10 +180,10 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_pairs_fwd(EvView v, const do
             const long long rb = pl.off[b], rb1 = pl.off[b + 1];
             const int place = atomicAdd(&pl.cntB[b], 1);
             const double r2 = fma(dx, dx, dy * dy);
-            long long w, gk[2];
-            pair_fixed<2>({dx, dy}, r2, v.inv_h, w, gk);
+            double w, gk[2];
+            pair_kernel<2>({dx, dy}, r2, v.inv_h, w, gk);
             const int slot = (p ? nf[1] : nf[0]) + __popc((p ? m1 : m0) & lt);
-            const longlong2 g = make_longlong2(gk[0], gk[1]);
+            const double2 g = make_double2(gk[0], gk[1]);
             if (slot < cap[p]) {
                 const long long i = row[p] + slot;
                 pl.L[i] = b;
@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_pairs_fwd(EvView v, const do
             if (i >= rb && rb1 <= pl.total) {
                 pl.L[i] = (int)a0 + p;
                 pl.W[i] = w;
-                pl.G[i] = make_longlong2(-g.x, -g.y);
+                pl.G[i] = make_double2(-g.x, -g.y);
             }
         }
         nf[0] += __popc(m0);
@@ -263,8 +263,8 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_pairs_fwd(EvView v, const do
         for (int p = 0; p < np; ++p) pl.cntF[a0 + p] = nf[p];
 }
 
-// Density sums, half a warp per particle a, over the entries of its row, in integers
-// (pairs_fixed.cuh).
+// Density sums, half a warp per particle a, over the entries of its row, in integers, each in the unit
+// of its own largest term (pairs_fixed.cuh).
 // Bound: the latency of the gathers; 40 k event 92 us a stage, 3+1D event of 258 k particles 0.92 ms.
 __global__ void __launch_bounds__(32 * kWarps, 7) k_pairs_sum(EvView v, PairBufs pl, double *__restrict__ dens,
                                                            int *__restrict__ nnb)
@@ -285,37 +285,44 @@ __global__ void __launch_bounds__(32 * kWarps, 7) k_pairs_sum(EvView v, PairBufs
     // entry j of a's row
     auto at = [&](int j) { return j < nf ? r0 + j : r1 - nt + j; };
     const uint2 *Qe = reinterpret_cast<const uint2 *>(pl.Qe);
-    // the largest exponents among a and its neighbours (S | N_B << 16, N_S | N_Q << 16)
-    uint2 em = Qe[a];
+    // the largest exponents among the products q_b W of a (W = 1) and its neighbours (S | N_B << 16,
+    // N_S | N_Q << 16)
+    const unsigned one2 = fx_pair(1023, 1023);
+    uint2 em = make_uint2(Qe[a].x + one2, Qe[a].y + one2);
     for (int j = l; j < fit; j += 16) {
-        const uint2 e = Qe[pl.L[at(j)]];
-        em = make_uint2(fx_max2(em.x, e.x), fx_max2(em.y, e.y));
+        const long long i = at(j);
+        const uint2 e = Qe[pl.L[i]];
+        const int ew = fx_kexp(pl.W[i]);
+        const unsigned w2 = fx_pair(ew, ew);
+        em = make_uint2(fx_max2(em.x, e.x + w2), fx_max2(em.y, e.y + w2));
     }
     em = make_uint2(fx_half_max2(em.x), fx_half_max2(em.y));
-    const int Em[4] = {(int)(em.x & 0xFFFFu), (int)(em.x >> 16), (int)(em.y & 0xFFFFu), (int)(em.y >> 16)};
+    const int Em[4] = {fx_lo(em.x), fx_hi(em.x), fx_lo(em.y), fx_hi(em.y)};
     int E[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) E[k] = fx_room(Em[k], nt);
-    FxSum sg = {0, 0};  // x in units of 2^-kFxBits
+    FxSum sg = {0, 0};  // of W alone, the largest W(0) = 1: x in units of 2^-kMant
     FxSum s[4] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
     int it = 0;
-    auto add = [&](long long w, int4 q0, int4 q1, uint2 e2) {
-        const int e[4] = {(int)(e2.x & 0xFFFFu), (int)(e2.x >> 16), (int)(e2.y & 0xFFFFu), (int)(e2.y >> 16)};
-        const int2 qv[4] = {lo_of(q0), hi_of(q0), lo_of(q1), hi_of(q1)};
-        sg.x += w;
+    auto add = [&](double w, Limb4 q, uint2 e2) {
+        const int e[4] = {fx_lo(e2.x), fx_hi(e2.x), fx_lo(e2.y), fx_hi(e2.y)};
+        const long long qv[4] = {q.x, q.y, q.z, q.w};
+        const long long m = fx_kmant(w);
+        const int ew = fx_kexp(w);
+        sg.x += fx_shift(m, 1023 - ew + kGuard);
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             int whi, wlo;
-            fx_split(w, E[k] - e[k], whi, wlo);
-            fx_add(s[k], whi, wlo, qv[k]);
+            fx_split(m, E[k] - e[k] - ew, whi, wlo);
+            fx_add(s[k], whi, wlo, fx_pair_of(qv[k]));
         }
     };
     // two entries at a time, their loads ahead of both; an entry past the end is a with weight 0
-    auto add2 = [&](int b0, long long w0, int b1, long long w1) {
-        const int4 p0 = pl.Q[b0], p1 = pl.Q[n + b0], r0_ = pl.Q[b1], r1_ = pl.Q[n + b1];
+    auto add2 = [&](int b0, double w0, int b1, double w1) {
+        const Limb4 q0 = pl.Q[b0], q1 = pl.Q[b1];
         const uint2 e0 = Qe[b0], e1 = Qe[b1];
-        add(w0, p0, p1, e0);
-        add(w1, r0_, r1_, e1);
+        add(w0, q0, e0);
+        add(w1, q1, e1);
         it += 2;
         if ((it & (kFoldEvery - 1)) == 0) {
             fx_fold(sg);
@@ -323,12 +330,12 @@ __global__ void __launch_bounds__(32 * kWarps, 7) k_pairs_sum(EvView v, PairBufs
             for (int k = 0; k < 4; ++k) fx_fold(s[k]);
         }
     };
-    if (l == 0 && on) add2(a, 1LL << kFxBits, a, 0);  // the self pair, W(0) = 1
+    if (l == 0 && on) add2(a, 1.0, a, 0.0);  // the self pair, W(0) = 1
     for (int j = l; j < fit; j += 32) {
         const bool two = j + 16 < fit;
         const long long i0 = at(j), i1 = at(j + 16);
         const int b0 = pl.L[i0], b1 = two ? pl.L[i1] : a;
-        const long long w0 = pl.W[i0], w1 = two ? pl.W[i1] : 0;
+        const double w0 = pl.W[i0], w1 = two ? pl.W[i1] : 0.0;
         add2(b0, w0, b1, w1);
     }
     fx_fold(sg);
@@ -345,8 +352,8 @@ __global__ void __launch_bounds__(32 * kWarps, 7) k_pairs_sum(EvView v, PairBufs
     if (on && (l & 1) == 0 && k < 5) {
         // rows sigma*, lab-frame s* (divided by u0 sqrt(-g) in the EoS pass), n*_B, n*_S, n*_Q
         const int Ek = k <= 1 ? E[0] : (k == 2 ? E[1] : (k == 3 ? E[2] : E[3]));
-        const bool bad = (k <= 1 ? Em[0] : (k == 2 ? Em[1] : (k == 3 ? Em[2] : Em[3]))) == kNonFinite && k > 0;
-        const double d = fx_value(tot, k == 0 ? -kFxBits : fx_unit(Ek));
+        const bool bad = (k <= 1 ? Em[0] : (k == 2 ? Em[1] : (k == 3 ? Em[2] : Em[3]))) >= kNonFinite && k > 0;
+        const double d = fx_value(tot, k == 0 ? -kMant : fx_unit(Ek));
         dens[(size_t)k * n + a] = bad ? fx_nan() : v.sigma_d * d;
     }
     if (on && l == 0) {
@@ -360,7 +367,8 @@ __global__ void __launch_bounds__(32 * kWarps, 7) k_pairs_sum(EvView v, PairBufs
 }
 
 // Gradient pass, half a warp per particle a, over the entries of its row with G = grad_a W_ab h /
-// sigma_d, forming in integers the sums of the per-particle pass: sum grad W, sum X_b grad W, sum u_b grad W.
+// sigma_d, forming in integers the sums of the per-particle pass: sum grad W, sum X_b grad W, sum u_b grad W, each in
+// the unit of its own largest term (a first look over the exponents).
 // Bound: the latency of the gathers; 40 k event 137 us a stage (298 us with 10 FP64 operations per
 // pair).  Two entries at a time: 150 against 173 us; 5 blocks per SM: 6 gave 161, 8 150, 10 193.
 __global__ void __launch_bounds__(32 * kWarps, 5) k_pairs_gradient(EvView v, int stage, const double *__restrict__ gin,
@@ -376,33 +384,48 @@ __global__ void __launch_bounds__(32 * kWarps, 5) k_pairs_gradient(EvView v, int
     const long long r0 = pl.off[a], r1 = pl.off[a + 1];
     const int nf = on ? pl.cntF[a] : 0, nt = on ? nf + pl.cntB[a] : 0;
     auto at = [&](int j) { return j < nf ? r0 + j : r1 - nt + j; };  // entry j of a's row
-    // the largest exponents among a and its neighbours (stress | u << 16)
-    unsigned em = pl.Xe[a];
-    for (int j = l; j < nt; j += 16) em = fx_max2(em, pl.Xe[pl.L[at(j)]]);
-    em = fx_half_max2(em);
-    const int EX = fx_room((int)(em & 0xFFFFu), nt), EU = fx_room((int)(em >> 16), nt);
-    const bool bad = (em & 0xFFFFu) == kNonFinite || (em >> 16) == kNonFinite;
+    // the largest exponents among the terms of each sum: g_x | g_y, H_x | H_y, d_x u^x | d_x u^y, d_y u^x |
+    // d_y u^y (16-bit halves)
+    uint4 em = make_uint4(0u, 0u, 0u, 0u);
+    for (int j = l; j < nt; j += 16) {
+        const long long i = at(j);
+        const longlong2 e = reinterpret_cast<const longlong2 *>(pl.X + n + pl.L[i])[1];
+        const double2 g = pl.G[i];
+        const int ex = fx_kexp(g.x), ey = fx_kexp(g.y);
+        const unsigned x2 = fx_pair(ex, ex), y2 = fx_pair(ey, ey);
+        em.x = fx_max2(em.x, fx_pair(ex, ey));
+        em.y = fx_max2(em.y, fx_max2(word_lo(e.x) + x2, word_hi(e.x) + y2));
+        em.z = fx_max2(em.z, word_lo(e.y) + x2);
+        em.w = fx_max2(em.w, word_lo(e.y) + y2);
+    }
+    em = make_uint4(fx_half_max2(em.x), fx_half_max2(em.y), fx_half_max2(em.z), fx_half_max2(em.w));
+    const int Em[8] = {fx_lo(em.x), fx_hi(em.x), fx_lo(em.y), fx_hi(em.y), fx_lo(em.z), fx_hi(em.z), fx_lo(em.w), fx_hi(em.w)};
+    int E[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) E[k] = fx_room(Em[k], nt);
     FxSum sG[2] = {{0, 0}, {0, 0}};
     FxSum sH[2] = {{0, 0}, {0, 0}};                  // sum X^{x.} g, sum X^{y.} g
     FxSum sU[4] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};  // d_x u^x, d_x u^y, d_y u^x, d_y u^y
     int it = 0;
-    auto add = [&](longlong2 g, int4 x0, int4 x1, int4 u0, unsigned e) {
-        sG[0].x += g.x;
-        sG[1].x += g.y;
-        int xh, xl, yh, yl, d = EX - (int)(e & 0xFFFFu);
-        fx_split(g.x, d, xh, xl);
-        fx_split(g.y, d, yh, yl);
-        fx_add(sH[0], xh, xl, lo_of(x0));  // X^{xx} g_x
-        fx_add(sH[0], yh, yl, lo_of(x1));  // X^{yx} g_y
-        fx_add(sH[1], xh, xl, hi_of(x0));  // X^{xy} g_x
-        fx_add(sH[1], yh, yl, hi_of(x1));  // X^{yy} g_y
-        d = EU - (int)(e >> 16);
-        fx_split(g.x, d, xh, xl);
-        fx_split(g.y, d, yh, yl);
-        fx_add(sU[0], xh, xl, lo_of(u0));
-        fx_add(sU[1], xh, xl, hi_of(u0));
-        fx_add(sU[2], yh, yl, lo_of(u0));
-        fx_add(sU[3], yh, yl, hi_of(u0));
+    auto add = [&](double2 g, Limb4 x, Limb4 u) {
+        const long long mx = fx_kmant(g.x), my = fx_kmant(g.y);
+        const int ex = fx_kexp(g.x), ey = fx_kexp(g.y);
+        const unsigned eX0 = word_lo(u.z), eX1 = word_hi(u.z), eU = word_lo(u.w);
+        sG[0].x += fx_shift(mx, E[0] - ex + kGuard);
+        sG[1].x += fx_shift(my, E[1] - ey + kGuard);
+        auto term = [&](FxSum &s, long long m, int d, long long q) {
+            int hi, lo;
+            fx_split(m, d, hi, lo);
+            fx_add(s, hi, lo, fx_pair_of(q));
+        };
+        term(sH[0], mx, E[2] - ex - fx_lo(eX0), x.x);  // X^{xx} g_x
+        term(sH[0], my, E[2] - ey - fx_lo(eX1), x.z);  // X^{yx} g_y
+        term(sH[1], mx, E[3] - ex - fx_hi(eX0), x.y);  // X^{xy} g_x
+        term(sH[1], my, E[3] - ey - fx_hi(eX1), x.w);  // X^{yy} g_y
+        term(sU[0], mx, E[4] - ex - fx_lo(eU), u.x);
+        term(sU[1], mx, E[5] - ex - fx_hi(eU), u.y);
+        term(sU[2], my, E[6] - ey - fx_lo(eU), u.x);
+        term(sU[3], my, E[7] - ey - fx_hi(eU), u.y);
     };
     auto fold = [&]() {
 #pragma unroll
@@ -414,16 +437,14 @@ __global__ void __launch_bounds__(32 * kWarps, 5) k_pairs_gradient(EvView v, int
         }
     };
     // two entries at a time, their loads ahead of both; an entry past the end is a with gradient 0
-    auto add2 = [&](int b0, longlong2 g0, int b1, longlong2 g1) {
-        const int4 x0 = pl.X[b0], y0 = pl.X[n + b0], u0 = pl.X[2 * n + b0];
-        const int4 x1 = pl.X[b1], y1 = pl.X[n + b1], u1 = pl.X[2 * n + b1];
-        const unsigned e0 = pl.Xe[b0], e1 = pl.Xe[b1];
-        add(g0, x0, y0, u0, e0);
-        add(g1, x1, y1, u1, e1);
+    auto add2 = [&](int b0, double2 g0, int b1, double2 g1) {
+        const Limb4 x0 = pl.X[b0], u0 = pl.X[n + b0], x1 = pl.X[b1], u1 = pl.X[n + b1];
+        add(g0, x0, u0);
+        add(g1, x1, u1);
         it += 2;
         if ((it & (kFoldEvery - 1)) == 0) fold();
     };
-    const longlong2 zero = make_longlong2(0, 0);
+    const double2 zero = make_double2(0.0, 0.0);
     for (int j = l; j < nt; j += 32) {
         const bool two = j + 16 < nt;
         const long long i0 = at(j), i1 = at(j + 16);
@@ -434,8 +455,12 @@ __global__ void __launch_bounds__(32 * kWarps, 5) k_pairs_gradient(EvView v, int
                     fx_words(sU[0]), fx_words(sU[1]), fx_words(sU[2]), fx_words(sU[3])};
     const FxTotal tt = fx_reduce8(t, lane);
     const int k = l >> 1;
-    double tot = fx_value(tt, k < 2 ? -kFxBits : fx_unit(k < 4 ? EX : EU));
-    if (bad && k >= 2) tot = fx_nan();
+    int Ek = E[0], Emk = Em[0];
+#pragma unroll
+    for (int i = 1; i < 8; ++i)
+        if (k == i) Ek = E[i], Emk = Em[i];
+    double tot = fx_value(tt, k < 2 ? fx_kunit(Ek) : fx_unit(Ek));
+    if (Emk >= kNonFinite) tot = fx_nan();
     // totals of lanes 2 k of the half warp: k = 0, 1: sum grad W; 2, 3: sum X_b grad W; 4-7: sum u_b grad W
     const double Sx = __shfl_sync(kFull, tot, lane & 16), Sy = __shfl_sync(kFull, tot, (lane & 16) + 2);
     if (on && (l & 1) == 0 && k >= 2) {

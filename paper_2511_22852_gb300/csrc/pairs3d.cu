@@ -16,7 +16,7 @@ constexpr unsigned kFull = 0xFFFFFFFFu;
 // Forward pass, a warp for two particles a.  Candidates of the cells from its own on (those within
 // 2h of a) pass the single-precision prefilter; a candidate b > a is queued, and 32 at a time -- of
 // both particles -- the exact test (where the float test left the pair undecided) and the kernel in
-// fixed point (pair_fixed) run on full warps.  W and grad W go into a's row and, at a place taken
+// integers (pair_kernel) run on full warps.  W and grad W go into a's row and, at a place taken
 // from b's counter, into b's row.  The particles' own values go into limbs.
 // (Listing b < a in a's own walk, and finding its W by a search in b's row, kept the sums waiting
 // for memory: 40 k event, sum pass 197 -> 92 us a stage, gradient pass 150 -> 137; 258 k particles
@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_pairs3_fwd(EvView v, const d
     if (lane < 4 * np) {
         const size_t a = (size_t)a0 + (lane >> 2);
         const int k = lane & 3;
-        fx_store_value(pl.Q, pl.Qe, (size_t)n, a, k, k == 0 ? S[a] : Nq[(size_t)(k - 1) * n + a]);
+        fx_store_value(pl.Q, pl.Qe, a, k, k == 0 ? S[a] : Nq[(size_t)(k - 1) * n + a]);
     }
     const unsigned lt = (1u << lane) - 1u;
     const double (*pos)[3] = pos_[wid];
@@ -83,20 +83,20 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_pairs3_fwd(EvView v, const d
             const long long rb = pl.off[b], rb1 = pl.off[b + 1];
             const int place = atomicAdd(&pl.cntB[b], 1);
             const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
-            long long w, g[3];
-            pair_fixed<3>({dx, dy, dz}, r2, v.inv_h, w, g);
+            double w, g[3];
+            pair_kernel<3>({dx, dy, dz}, r2, v.inv_h, w, g);
             const int slot = (p ? nf[1] : nf[0]) + __popc((p ? m1 : m0) & lt);
             if (slot < cap[p]) {
                 const long long i = row[p] + slot;
                 pl.L[i] = b;
                 pl.W[i] = w;
-                pl.G3[i] = longlong4_32a{g[0], g[1], g[2], 0};
+                pl.G3[i] = double4_32a{g[0], g[1], g[2], 0.0};
             }
             const long long i = rb1 - 1 - place;
             if (i >= rb && rb1 <= pl.total) {
                 pl.L[i] = (int)a0 + p;
                 pl.W[i] = w;
-                pl.G3[i] = longlong4_32a{-g[0], -g[1], -g[2], 0};
+                pl.G3[i] = double4_32a{-g[0], -g[1], -g[2], 0.0};
             }
         }
         nf[0] += __popc(m0);
@@ -194,13 +194,51 @@ __global__ void __launch_bounds__(32 * kWarps, 4) k_pairs3_gradient(EvView v, in
     const size_t n = (size_t)v.n;
     const long long r0 = pl.off[a], r1 = pl.off[a + 1];
     const int nf = on ? pl.cntF[a] : 0, nt = on ? nf + pl.cntB[a] : 0;
-    auto at = [&](int j) { return j < nf ? r0 + j : r1 - nt + j; };  // entry j of a's row
-    // the largest exponents among a and its neighbours (stress | u << 16)
-    unsigned em = pl.Xe[a];
-    for (int j = l; j < nt; j += 16) em = fx_max2(em, pl.Xe[pl.L[at(j)]]);
-    em = fx_half_max2(em);
-    const int EX = fx_room((int)(em & 0xFFFFu), nt), EU = fx_room((int)(em >> 16), nt);
-    const bool bad = (em & 0xFFFFu) == kNonFinite || (em >> 16) == kNonFinite;
+    const int *L = pl.L + r0;
+    const double4_32a *G = pl.G3 + r0;
+    const int gap = (int)(r1 - r0) - nt;
+    auto at = [&](int j) { return j + (j < nf ? 0 : gap); };  // entry j of a's row
+    // the largest exponents among the terms of each sum, two in 16-bit halves: mG g_1 | g_2 and g_3, mH H_1 |
+    // H_2, mD[k] H_3 (its terms of k) | u^k g_k, mU[k] the two u^j g_k with j != k, ascending
+    unsigned mG[2] = {0u, 0u}, mH = 0u, mD[3] = {0u, 0u, 0u}, mU[3] = {0u, 0u, 0u};
+    // u^j of j != k from the words (X^{j3} | u^j)
+    auto others = [](const unsigned (&w)[3], int k) { return __byte_perm(w[k == 0 ? 1 : 0], w[k == 2 ? 1 : 2], 0x7632); };
+    for (int j = l; j < nt; j += 16) {
+        const int i = at(j);
+        const int b = L[i];
+        const double4_32a g = G[i];
+        const Limb4 e = pl.X[3 * n + b];
+        const unsigned eA[3] = {word_lo(e.x), word_lo(e.y), word_lo(e.z)}, eB[3] = {word_hi(e.x), word_hi(e.y), word_hi(e.z)};
+        const int eg[3] = {fx_kexp(g.x), fx_kexp(g.y), fx_kexp(g.z)};
+        mG[0] = fx_max2(mG[0], fx_pair(eg[0], eg[1]));
+        mG[1] = fx_max2(mG[1], (unsigned)eg[2]);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const unsigned g2 = fx_pair(eg[k], eg[k]);
+            mH = fx_max2(mH, eA[k] + g2);
+            mD[k] = fx_max2(mD[k], eB[k] + g2);
+            mU[k] = fx_max2(mU[k], others(eB, k) + g2);
+        }
+    }
+    mH = fx_half_max2(mH);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        if (k < 2) mG[k] = fx_half_max2(mG[k]);
+        mD[k] = fx_half_max2(mD[k]);
+        mU[k] = fx_half_max2(mU[k]);
+    }
+    {
+        // one unit for H_3; room for rows of many entries
+        const unsigned h3 = fx_max2(fx_max2(mD[0], mD[1]), mD[2]) & 0xFFFFu, room = (unsigned)fx_room(0, nt) * 0x10001u;
+        mG[0] += room;
+        mG[1] += room;
+        mH += room;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            mD[k] = ((mD[k] & 0xFFFF0000u) | h3) + room;
+            mU[k] += room;
+        }
+    }
     FxSum sG[3], sH[3], sU[9];  // sum g; sum_j X^{j i} g_j; 3 k + j: sum u^j g_k
 #pragma unroll
     for (int k = 0; k < 3; ++k) sG[k] = sH[k] = sU[k] = sU[3 + k] = sU[6 + k] = FxSum{0, 0};
@@ -215,40 +253,47 @@ __global__ void __launch_bounds__(32 * kWarps, 4) k_pairs3_gradient(EvView v, in
         }
     };
     // the next entry's index and gradient are loaded while the current one is added
-    auto entry = [&](int j, int &b, long long (&g)[3]) {
+    auto entry = [&](int j, int &b, double (&g)[3]) {
         b = a;
-        g[0] = g[1] = g[2] = 0;
+        g[0] = g[1] = g[2] = 0.0;
         if (j < nt) {
-            const long long i = at(j);
-            b = pl.L[i];
-            const longlong4_32a e = pl.G3[i];
+            const int i = at(j);
+            b = L[i];
+            const double4_32a e = G[i];
             g[0] = e.x;
             g[1] = e.y;
             g[2] = e.z;
         }
     };
     int b1;
-    long long g1[3];
+    double g1[3];
     entry(l, b1, g1);
     for (int j = l, it = 1; j < nt; j += 16, ++it) {
         const int b = b1;
-        const long long g[3] = {g1[0], g1[1], g1[2]};
-        int4 x4[6];
-#pragma unroll
-        for (int m = 0; m < 6; ++m) x4[m] = pl.X[m * n + b];
-        const unsigned e = pl.Xe[b];
+        const double g[3] = {g1[0], g1[1], g1[2]};
+        const Limb4 x0 = pl.X[b], x1 = pl.X[n + b], x2 = pl.X[2 * n + b], e = pl.X[3 * n + b];
         entry(j + 16, b1, g1);
-        const int dX = EX - (int)(e & 0xFFFFu), dU = EU - (int)(e >> 16);
+        const long long x[12] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w, x2.x, x2.y, x2.z, x2.w};
+        const unsigned eA[3] = {word_lo(e.x), word_lo(e.y), word_lo(e.z)}, eB[3] = {word_hi(e.x), word_hi(e.y), word_hi(e.z)};
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            int hi, lo;
-            sG[k].x += g[k];
-            fx_split(g[k], dX, hi, lo);
-#pragma unroll
-            for (int i = 0; i < 3; ++i) fx_add(sH[i], hi, lo, (3 * k + i) & 1 ? hi_of(x4[(3 * k + i) >> 1]) : lo_of(x4[(3 * k + i) >> 1]));
-            fx_split(g[k], dU, hi, lo);
-#pragma unroll
-            for (int i = 0; i < 3; ++i) fx_add(sU[3 * k + i], hi, lo, (9 + i) & 1 ? hi_of(x4[(9 + i) >> 1]) : lo_of(x4[(9 + i) >> 1]));
+            const long long m = fx_kmant(g[k]);
+            const int eg = fx_kexp(g[k]);
+            const unsigned g2 = fx_pair(eg, eg);
+            // the shifts of the terms X^{k i} g_k and u^j g_k, two in a word (an entry past the end has m = 0)
+            const unsigned dH = mH - eA[k] - g2, dD = mD[k] - eB[k] - g2, dU = mU[k] - others(eB, k) - g2;
+            sG[k].x += fx_shift(m, (k == 0 ? fx_lo(mG[0]) : (k == 1 ? fx_hi(mG[0]) : fx_lo(mG[1]))) - eg + kGuard);
+            auto term = [&](FxSum &s, int d, int i) {
+                int hi, lo;
+                fx_split(m, d, hi, lo);
+                fx_add(s, hi, lo, fx_pair_of(x[i]));
+            };
+            term(sH[0], fx_lo(dH), 3 * k);
+            term(sH[1], fx_hi(dH), 3 * k + 1);
+            term(sH[2], fx_lo(dD), 3 * k + 2);
+            term(sU[4 * k], fx_hi(dD), 9 + k);
+            term(sU[3 * k + (k == 0 ? 1 : 0)], fx_lo(dU), 9 + (k == 0 ? 1 : 0));
+            term(sU[3 * k + (k == 2 ? 1 : 2)], fx_hi(dU), 9 + (k == 2 ? 1 : 2));
         }
         if ((it & (kFoldEvery - 1)) == 0) fold();
     }
@@ -263,8 +308,15 @@ __global__ void __launch_bounds__(32 * kWarps, 4) k_pairs3_gradient(EvView v, in
     for (int k = 0; k < 9; ++k) t[6 + k] = fx_words(sU[k]);
     t[15] = FxTotal{0, 0};
     const FxTotal tt = fx_reduce16(t, lane);
-    double tot = fx_value(tt, l < 3 ? -kFxBits : fx_unit(l < 6 ? EX : EU));
-    if (bad && l >= 3) tot = fx_nan();
+    // the unit of the lane's sum: 0-2 g, 3-5 H, 6 + 3 k + j u^j g_k
+    const int E[15] = {fx_lo(mG[0]), fx_hi(mG[0]), fx_lo(mG[1]), fx_lo(mH), fx_hi(mH), fx_lo(mD[0]), fx_hi(mD[0]), fx_lo(mU[0]),
+                       fx_hi(mU[0]), fx_lo(mU[1]), fx_hi(mD[1]), fx_hi(mU[1]), fx_lo(mU[2]), fx_hi(mU[2]), fx_hi(mD[2])};
+    int El = E[0];
+#pragma unroll
+    for (int i = 1; i < 15; ++i)
+        if (l == i) El = E[i];
+    double tot = fx_value(tt, l < 3 ? fx_kunit(El) : fx_unit(El));
+    if (El >= kNonFinite) tot = fx_nan();
     const int h0 = lane & 16;
     const double G0 = __shfl_sync(kFull, tot, h0), G1 = __shfl_sync(kFull, tot, h0 + 1), G2 = __shfl_sync(kFull, tot, h0 + 2);
     if (on && l >= 3 && l < 15) {

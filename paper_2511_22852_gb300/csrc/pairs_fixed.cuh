@@ -1,30 +1,32 @@
 // pairs_fixed.cuh -- integer accumulation of the plain (FP64) neighbour sums.
 //
 // On GB300 an FP64 operation occupies its pipe for 64 cycles per warp and quadrant, a 32-bit
-// integer multiply-add into 64 bits for about 3.  The pair passes therefore form their sums
-// sum_b q_b w_ab in integers, at or above FP64 precision:
-//   * the pair's kernel value or gradient (dimensionless, |w| <= 1) as a fixed-point integer in
-//     units of 2^-57, from the FP64 separation (pair_fixed);
+// integer multiply-add into 64 bits for about 3.  The pair passes therefore evaluate the kernel and
+// form their sums sum_b q_b w_ab in integers, with the error of FP64 arithmetic or less in every term:
+//   * the pair's kernel value or gradient component as a double, from the FP64 separation by 64-bit
+//     integer operations (pair_kernel): relative error at most 2^-53 + 11 2^-60 / (2 - r/h), also
+//     towards the kernel's rim and for a component much smaller than the others;
 //   * the particle's value q_b as its exact 53-bit mantissa (times 2) in two limbs
 //     hi 2^29 + lo (lo balanced around 0) and its exponent;
-//   * the particle's sums in units of the largest exponent E among its neighbours (a first look
-//     over the exponents alone): w is shifted down by E - e_b and split into limbs, hi hi goes to
-//     one 64-bit accumulator and the two cross products to another; the dropped lo lo is below
-//     2^-54 of the largest q_b, with either sign;
+//   * each sum in units of the largest exponent E among its own terms' products q_b w_ab (a first
+//     look over the exponents alone): w's mantissa is shifted down by E less the term's exponent
+//     and split into limbs, hi hi goes to one 64-bit accumulator and the two cross products to another;
+//     what is dropped is below 2^-53 of the largest term, and a sum in FP64 rounds at 2^-53 of its
+//     partial sums, which reach half the largest term at least;
 //   * the lanes are added in integers, and each total becomes a double once.
-// Against sums in FP64, whose additions round at 2^-53 of the partial sum, the error is smaller
-// (the step's error against 64-bit values: 5.2e-16 of u on the ideal lattice with FP64 sums, 5.0e-16
-// now), and it does not depend on the order of the additions.
-// A non-finite q_b makes the particle's sums NaN.
+// So no value, charge or component is rounded against a larger one of another sum or of a neighbour
+// that hardly counts, and the result does not depend on the order of the additions.
+// A non-finite q_b makes the sums it enters NaN.
 #pragma once
 #include "sph_internal.cuh"
 
 namespace sphg {
 
-constexpr int kFxBits = 57;   // units of the fixed-point kernel values
+constexpr int kMant = 56;     // a kernel value's mantissa in units of its exponent: [2^56, 2^57),
+constexpr int kGuard = 3;     // held times 2^3, so that a 32-bit word boundary parts the limbs
 constexpr int kLimb = 29;
 constexpr long long kLimbMask = (1LL << kLimb) - 1;
-constexpr int kNonFinite = 0x7FF;
+constexpr int kNonFinite = 0x3FFF;  // exponent of infinities and NaN: above every product's
 constexpr int kFoldEvery = 16;     // terms between folds of the cross accumulators
 constexpr int kHeadroom = 128;     // terms a lane's high accumulator holds without a larger unit
 
@@ -39,29 +41,33 @@ __device__ __forceinline__ float cell_gap(int o, float x, int c, float cell)
     return m < 0.0f ? 0.0f : m;
 }
 
-// |v| 2^-s in units of 2^-61 (below 2^62), rounded to nearest
-__device__ __forceinline__ unsigned long long abs_fixed(double v, int s)
+// m 2^e as a double rounded to nearest (in integers: a conversion instruction occupies the FP64 pipe
+// like an operation); m = 0 and results below 2^-1022: 0
+__device__ __forceinline__ double pack_double(unsigned long long m, int e)
 {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-    const int k = (int)(b >> 52 & 0x7FF) - (1075 - 61) - s;
-    const unsigned long long m = (b & 0xFFFFFFFFFFFFFULL) | (1ULL << 52);
-    return k >= 0 ? m << min(k, 9) : (k > -60 ? (m + (1ULL << (-k - 1))) >> -k : 0ULL);
+    const int s = __clzll((long long)m);
+    m <<= s & 63;
+    const int f = e - s + 63 + 1022;
+    const unsigned long long b = ((unsigned long long)(unsigned)f << 52) + (m >> 11) + (m >> 10 & 1u);
+    return __longlong_as_double(m == 0ULL || f < 0 ? 0LL : (long long)b);
 }
 
-// A pair's kernel value and gradient in fixed point from its separation d and r2 = |d|^2 <= 4 h^2:
-// w = (2-q)^3/4 - max(1-q, 0)^3 and g_k = w' d_k/r, w' = 3 max(1-q, 0)^2 - 3 (2-q)^2/4 <= 0, q = r/h,
-// all in units of 2^-kFxBits.  r2 = m 4^s with m in [1, 4): a single-precision reciprocal square
-// root y of m (relative error below 2^-21) is refined by one third-order Householder step, e =
-// 1 - m y^2, c = e/2 + 3 e^2/8, 1/sqrt(m) = y (1 + c), with the remainder of order e^3 below 2^-60.
+// A pair's kernel value and gradient from its separation d and r2 = |d|^2 <= 4 h^2: w = (2-q)^3/4 -
+// max(1-q, 0)^3 and g_k = w' d_k/r, w' = 3 max(1-q, 0)^2 - 3 (2-q)^2/4 <= 0, q = r/h.  r2 = m 4^s with
+// m in [1, 4): a single-precision reciprocal square root y of m (relative error below 2^-21) is refined
+// by one third-order Householder step, e = 1 - m y^2, c = e/2 + 3 e^2/8, 1/sqrt(m) = y (1 + c).
 // Everything behind r2 is in 64-bit integers: a high product is about 10 integer instructions
-// (25 cycles a warp), an FP64 operation 64 cycles; errors below 2^-56 of the kernel's maximum.
+// (25 cycles a warp), an FP64 operation 64 cycles.  q itself (q < 1) or t = 2 - q is normalised before
+// its powers are taken, as are w'/r and d_k, so small results keep their leading bits: relative errors
+// against 200-bit values at 60,000 separations stay below 2^-53 + 11 2^-60/(2 - q) for w and
+// 2^-53 + 7.3 2^-60/(2 - q) for g_k (FP64 arithmetic: several 2^-53/(2 - q)).
 template <int D>
-__device__ __forceinline__ void pair_fixed(const double (&d)[D], double r2, double inv_h, long long &w, long long (&g)[D])
+__device__ __forceinline__ void pair_kernel(const double (&d)[D], double r2, double inv_h, double &w, double (&g)[D])
 {
     const unsigned hi = (unsigned)__double2hiint(r2), lo = (unsigned)__double2loint(r2);
-    w = 1LL << kFxBits;  // coincident particles: W(0), no gradient
+    w = 1.0;  // coincident particles: W(0), no gradient
 #pragma unroll
-    for (int k = 0; k < D; ++k) g[k] = 0;
+    for (int k = 0; k < D; ++k) g[k] = 0.0;
     if (hi - 0x00100000u >= 0x7FE00000u) return;  // zero (or below 2^-1022)
     const int E = (int)(hi >> 20) - 1023, s = E >> 1, odd = E & 1;
     const unsigned long long M = (((unsigned long long)(hi & 0xFFFFFu) | 0x100000u) << 32 | lo) << (10 + odd);  // m, 2^-62
@@ -75,30 +81,28 @@ __device__ __forceinline__ void pair_fixed(const double (&d)[D], double r2, doub
     const unsigned long long H = (hb << 11) | (1ULL << 63);  // 1/h = H 2^t, 2^-63
     const int sh = s + (int)(hb >> 52 & 0x7FF) - 1023;
     const unsigned long long qr = __umul64hi(__umul64hi(M, R) << 1, H);  // q 2^-sh, 2^-61
-    const long long Q = (long long)(sh >= 0 ? qr << min(sh, 63) : qr >> min(-sh, 63));
-    // t = 2 - q and u = max(1 - q, 0), 2^-61
-    const unsigned long long T = (unsigned long long)max((1LL << 62) - Q, 0LL), U = (unsigned long long)max((1LL << 61) - Q, 0LL);
-    const unsigned long long T2 = __umul64hi(T, T), U2 = __umul64hi(U, U);  // 2^-58
-    const unsigned long long T3 = __umul64hi(T2 << 3, T), U3 = __umul64hi(U2 << 3, U);
-    w = ((long long)T3 - 4 * (long long)U3 + 4) >> 3;
-    const unsigned long long n = (unsigned long long)max(48 * ((long long)(T2 >> 2) - (long long)U2), 0LL);  // -w', 2^-62
-    const unsigned long long P = __umul64hi(n << 1, R) << 1;  // -w'/sqrt(m), 2^-63
+    const unsigned long long Q = sh >= 0 ? qr << min(sh, 63) : qr >> min(-sh, 63);  // q, 2^-61
+    const bool in = Q < (1ULL << 61);
+    // v = X 2^ex: q itself for q < 1, t = 2 - q beyond, with all of its leading bits
+    const unsigned long long v0 = in ? qr : (unsigned long long)max((1LL << 62) - (long long)Q, 0LL);
+    const int lv = __clzll((long long)v0) & 63, ex = (in ? sh : 0) - 61 - lv;
+    const unsigned long long X = v0 << lv, A = __umul64hi(X, X);
+    // w = 1 - q^2 (3/2 - 3 q/4)  or  t^3/4;  -w' = 3 q (1 - 3 q/4)  or  3 t^2/4
+    const unsigned long long B = __umul64hi(A, in ? 3 * ((1ULL << 62) - Q) : X);
+    const unsigned long long w61 = (1ULL << 61) - (B >> min(-(126 + 2 * ex), 63));
+    w = in ? pack_double(w61, -61) : pack_double(B, 126 + 3 * ex);
+    unsigned long long N = in ? __umul64hi(X, (1ULL << 63) - 3 * Q) : A;
+    N -= N >> 2;
+    const int ln = __clzll((long long)N) & 63, en = (in ? ex + 1 : 62 + 2 * ex) + 2 - ln;
+    const unsigned long long P = __umul64hi(N << ln, R);  // -w'/r = P 2^(en + 1 - s)
 #pragma unroll
     for (int k = 0; k < D; ++k) {
-        const long long a = (long long)((__umul64hi(P, abs_fixed(d[k], s) << 1) + 8) >> 4);
-        g[k] = __double2hiint(d[k]) < 0 ? a : -a;
+        const unsigned long long db = (unsigned long long)__double_as_longlong(d[k]);
+        const int ed = (int)(db >> 52 & 0x7FF);
+        const unsigned long long G = ed > 0 ? __umul64hi(P, (db << 11) | (1ULL << 63)) : 0ULL;
+        const double a = pack_double(G, en - s + ed - 1021);
+        g[k] = (long long)db < 0 ? a : -a;
     }
-}
-
-// w >= 0 in units of 2^-kFxBits as a double, rounded to nearest (in integers: a conversion instruction
-// occupies the FP64 pipe like an operation)
-__device__ __forceinline__ double fixed_value(long long w)
-{
-    if (w <= 0) return 0.0;
-    const int s = __clzll(w);
-    const unsigned long long m = (unsigned long long)w << s;
-    const unsigned long long b = ((unsigned long long)(1022 + 63 - kFxBits - s) << 52) + (m >> 11) + (m >> 10 & 1u);
-    return __longlong_as_double((long long)b);
 }
 
 // The lanes' sums of up to 8 values: value k (of t[0..7]) over the warp in lane 4 k (and 4 k + 1 to
@@ -121,7 +125,19 @@ __device__ __forceinline__ double warp_sums8(double (&t)[8], int lane)
 __device__ __forceinline__ int fx_exponent(double v)
 {
     const int e = (__double2hiint(v) >> 20) & 0x7FF;
-    return max(e, 1);
+    return e == 0x7FF ? kNonFinite : max(e, 1);
+}
+// two exponents in the 16-bit halves of a word
+__device__ __forceinline__ unsigned fx_pair(int lo, int hi) { return (unsigned)lo | ((unsigned)hi << 16); }
+__device__ __forceinline__ int fx_lo(unsigned e) { return (int)(e & 0xFFFFu); }
+__device__ __forceinline__ int fx_hi(unsigned e) { return (int)(e >> 16); }
+// a kernel value (zero, or normal of magnitude up to 1) as mant 2^(exp - 1023 - kMant - kGuard)
+__device__ __forceinline__ int fx_kexp(double w) { return (__double2hiint(w) >> 20) & 0x7FF; }
+__device__ __forceinline__ long long fx_kmant(double w)
+{
+    const long long b = __double_as_longlong(w);
+    const long long m = ((b & 0xFFFFFFFFFFFFFLL) | (1LL << 52)) << (kMant + kGuard - 52);
+    return fx_kexp(w) == 0 ? 0LL : (b < 0 ? -m : m);
 }
 // v = (hi 2^29 + lo) 2^(E - 1076), E at least v's exponent (rounded down to that unit)
 __device__ __forceinline__ int2 fx_limbs(double v, int E)
@@ -134,7 +150,7 @@ __device__ __forceinline__ int2 fx_limbs(double v, int E)
     return make_int2((int)((m - lo) >> kLimb), lo);
 }
 
-// one sum: value (hh 2^29 + x) 2^29 in units of 2^(E - 1076 - kFxBits)
+// one sum: value (hh 2^29 + x) 2^29 in units of 2^(E - 1076 - 1023 - kMant), E its products' exponent
 struct FxSum {
     long long hh, x;
 };
@@ -160,12 +176,18 @@ __device__ __forceinline__ unsigned fx_half_max2(unsigned e)
 // the unit's exponent for sums over n entries (16 lanes): E, and more where a lane adds over
 // kHeadroom terms
 __device__ __forceinline__ int fx_room(int E, int n) { return E + (32 - __clz((n / 16) / kHeadroom)); }
-// w shifted to a unit d exponents larger, in limbs
-__device__ __forceinline__ void fx_split(long long w, int d, int &hi, int &lo)
+// a mantissa shifted to a unit d exponents larger: as it is (units of kMant), and in limbs
+__device__ __forceinline__ long long fx_shift(long long m, int d)
 {
-    const long long t = w >> min(d, 63);
-    hi = (int)(t >> kLimb);
-    lo = (int)t & (int)kLimbMask;
+    long long t;  // amounts beyond 63 are clamped
+    asm("shr.s64 %0, %1, %2;" : "=l"(t) : "l"(m), "r"(d));
+    return t;
+}
+__device__ __forceinline__ void fx_split(long long m, int d, int &hi, int &lo)
+{
+    const long long t = fx_shift(m, d);
+    hi = (int)(t >> 32);
+    lo = (int)((unsigned)t >> kGuard);
 }
 
 // Sums over the 16 lanes of a half warp.  Each lane's (hh, x) goes into two words that cannot
@@ -210,41 +232,31 @@ __device__ __forceinline__ FxTotal fx_reduce16(const FxTotal (&v)[16], int lane)
     for (int i = 0; i < 2; ++i) g[i] = fx_exchange(fx_sel(b1, h[2 + i], h[i]), fx_sel(b1, h[i], h[2 + i]), 2);
     return fx_exchange(fx_sel(b0, g[1], g[0]), fx_sel(b0, g[0], g[1]), 1);
 }
-// a total p 2^49 + q in units of 2^k as a double: k = fx_unit(E) for a group's sums, -kFxBits for
-// sums of kernel values alone (x counting units of 2^-kFxBits)
-__device__ __forceinline__ int fx_unit(int E) { return E - 1076 - kFxBits + kLimb; }
+// a total p 2^49 + q in units of 2^k as a double: k = fx_unit(E) for a sum of products, fx_kunit(E)
+// for a sum of kernel values alone (x counting units); below 2^-1400 the total is zero as a double
+__device__ __forceinline__ int fx_unit(int E) { return E - 1076 - 1023 - kMant + kLimb; }
+__device__ __forceinline__ int fx_kunit(int E) { return E - 1023 - kMant; }
 __device__ __forceinline__ double fx_value(const FxTotal &t, int k)
 {
     const double v = fma((double)t.p, 562949953421312.0, (double)t.q);  // 2^49
-    const int k1 = k / 2, k2 = k - k1;                                  // two normal factors
+    k = max(k, -1400);
+    const int k1 = k / 2, k2 = k - k1;  // two normal factors
     return v * __hiloint2double((1023 + k1) << 20, 0) * __hiloint2double((1023 + k2) << 20, 0);
 }
 __device__ __forceinline__ double fx_nan() { return __longlong_as_double(0x7FF8000000000000LL); }
 
-// The limbs of particle values for the pair passes, in planes of int4 (two values each) over the
-// particles, so that the lanes' neighbours, mostly consecutive, load from few cache lines: values
-// with an exponent each (S, N_B, N_S, N_Q; lane k < 4 of a group of lanes writes value k)
-__device__ __forceinline__ void fx_store_value(int4 *Q, unsigned short *Qe, size_t n, size_t a, int k, double v)
+// limbs and pairs of words in 64 bits, four of them in a Limb4
+__device__ __forceinline__ long long fx_word(unsigned lo, unsigned hi) { return (long long)(((unsigned long long)hi << 32) | lo); }
+__device__ __forceinline__ long long fx_word(int2 v) { return fx_word((unsigned)v.x, (unsigned)v.y); }
+__device__ __forceinline__ int2 fx_pair_of(long long w) { return make_int2((int)w, (int)(w >> 32)); }
+__device__ __forceinline__ unsigned word_lo(long long w) { return (unsigned)w; }
+__device__ __forceinline__ unsigned word_hi(long long w) { return (unsigned)(w >> 32); }
+// S, N_B, N_S, N_Q (lane k < 4 of a group of lanes writes value k)
+__device__ __forceinline__ void fx_store_value(Limb4 *Q, unsigned short *Qe, size_t a, int k, double v)
 {
     const int e = fx_exponent(v);
-    reinterpret_cast<int2 *>(Q)[2 * ((k >> 1) * n + a) + (k & 1)] = fx_limbs(v, e);
+    reinterpret_cast<int2 *>(Q)[4 * a + k] = fx_limbs(v, e);
     Qe[4 * a + k] = (unsigned short)e;
 }
-// the largest exponent of K components of one tensor or vector
-template <int K>
-__device__ __forceinline__ int fx_shared_exponent(const double (&v)[K])
-{
-    int e = 1;
-#pragma unroll
-    for (int k = 0; k < K; ++k) e = max(e, fx_exponent(v[k]));
-    return e;
-}
-__device__ __forceinline__ int4 fx_limbs2(double v0, int e0, double v1, int e1)
-{
-    const int2 l0 = fx_limbs(v0, e0), l1 = fx_limbs(v1, e1);
-    return make_int4(l0.x, l0.y, l1.x, l1.y);
-}
-__device__ __forceinline__ int2 lo_of(int4 v) { return make_int2(v.x, v.y); }
-__device__ __forceinline__ int2 hi_of(int4 v) { return make_int2(v.z, v.w); }
 
 }  // namespace sphg

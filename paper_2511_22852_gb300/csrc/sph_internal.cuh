@@ -57,6 +57,9 @@ struct DevScalars {
     unsigned long long pairs_stage;  // pair-list passes: this stage's pairs (counted when no list overflowed)
 };
 
+// four 64-bit words of the pair passes, loaded at once (pairs_fixed.cuh)
+typedef longlong4_32a Limb4;
+
 struct EosDev {
     // closed form
     double a0, a1, Tc_GeV, w_GeV, chi[3];
@@ -132,14 +135,13 @@ struct EvView {
     int diff;
     double kapT2[9], tauJT[3];
     double *dinp, *dal, *dout;
-    // plain form: dinp in limbs for the pair-list pass, planes of [n] int4: alpha_B, alpha_S |
-    // alpha_Q | flux of B, S, Q (x, y); the exponents of alpha_q and flux_q in 16 bits each
-    int4 *dfx;
+    // plain form: dinp for the pair-list pass (pairs_fixed.cuh), planes of [n]: alpha_B, alpha_S | alpha_Q, 0
+    // (as doubles) | flux of B, S, Q (x, y: in limbs); the fluxes' six exponents in 16 bits each
+    longlong2 *dfx;
     uint4 *dfe;
     // pair lists (plain forms): where the EoS pass leaves the gradient-pass inputs in limbs
-    // (PairBufs X, Xe; nullptr: lists off)
-    int4 *fxX;
-    unsigned int *fxE;
+    // (PairBufs X; nullptr: lists off)
+    Limb4 *fxX;
     // mixed forms: where the EoS pass leaves the gradient-pass inputs in single precision: 2D
     // [n] float4 (X^{xx}, X^{xy}, X^{yx}, X^{yy}) and [n] float2 (u^x, u^y) behind it, 3D
     // planes [3][n] of four rows each
@@ -414,18 +416,17 @@ struct PairBufs {
     long long *off;               // [n + 1] row offsets of this stage
     unsigned long long *part;     // scan partial sums
     int *L, *cntF, *cntB;
-    // kernel value W/sigma_d and gradient h grad W/sigma_d of the pair in units of 2^-57
-    // (pairs_fixed.cuh)
-    long long *W;
-    longlong2 *G;   // 2D
-    longlong4_32a *G3;  // 3D: three components, padded to a 32-byte sector
-    // particle values in limbs (sorted order), planes of [n] int4 with two values each: S, N_B |
-    // N_S, N_Q with an exponent each (Qe[n][4]); the rows of gin, two at a time, with their two
-    // exponents (stress, u) packed in Xe
-    int4 *Q;
+    // kernel value W/sigma_d and gradient h grad W/sigma_d of the pair (pairs_fixed.cuh)
+    double *W;
+    double2 *G;   // 2D
+    double4_32a *G3;  // 3D: three components, padded to a 32-byte sector
+    // particle values in limbs (sorted order): S, N_B, N_S, N_Q with their exponents in Qe[n][4]; the rows of
+    // gin in planes of [n], exponents in 16 bits each: 2D X^{xx}, X^{xy}, X^{yx}, X^{yy} | u^x, u^y, the
+    // exponents of the X, those of u; 3D X^{11} .. X^{21} | X^{22} .. X^{32} | X^{33}, u | for j = 1, 2, 3 the
+    // exponents of X^{j1}, X^{j2}, X^{j3}, u^j.  32 bytes each, one gather: the passes are bound by their number.
+    Limb4 *Q;
     unsigned short *Qe;
-    int4 *X;
-    unsigned int *Xe;
+    Limb4 *X;
 };
 
 struct CellBufs {

@@ -143,9 +143,8 @@ __global__ void __launch_bounds__(32 * kWarps3) k_density3(EvView v, const doubl
             if (qb < 0 && !(dist2_3d(dx, dy, dz) < v.supp2)) return;
             {
                 const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
-                long long wf, g[3];
-                pair_fixed<3>({dx, dy, dz}, r2, v.inv_h, wf, g);
-                const double w = fixed_value(wf);
+                double w, g[3];
+                pair_kernel<3>({dx, dy, dz}, r2, v.inv_h, w, g);
                 sg += w;
                 ss = fma(S[b], w, ss);
                 sb = fma(Nq[b], w, sb);
@@ -342,12 +341,18 @@ __global__ void __launch_bounds__(64, 5) k_eos3_finish(EvView v, int stage, cons
             v.fX[2 * n + a] = make_float4((float)X[8], (float)us[0], (float)us[1], (float)us[2]);
         }
         if (v.fxX) {  // the same in limbs for the pair-list gradient pass
-            const int eX = fx_shared_exponent(X), eu = fx_shared_exponent(us);
+            int e[12];
+            long long w[12];
 #pragma unroll
-            for (int m = 0; m < 4; ++m) v.fxX[m * n + a] = fx_limbs2(X[2 * m], eX, X[2 * m + 1], eX);
-            v.fxX[4 * n + a] = fx_limbs2(X[8], eX, us[0], eu);
-            v.fxX[5 * n + a] = fx_limbs2(us[1], eu, us[2], eu);
-            v.fxE[a] = (unsigned)eX | ((unsigned)eu << 16);
+            for (int m = 0; m < 12; ++m) {
+                const double x = m < 9 ? X[m] : us[m - 9];
+                e[m] = fx_exponent(x);
+                w[m] = fx_word(fx_limbs(x, e[m]));
+            }
+#pragma unroll
+            for (int m = 0; m < 3; ++m) v.fxX[m * n + a] = Limb4{w[4 * m], w[4 * m + 1], w[4 * m + 2], w[4 * m + 3]};
+            v.fxX[3 * n + a] = Limb4{fx_word(fx_pair(e[0], e[1]), fx_pair(e[2], e[9])), fx_word(fx_pair(e[3], e[4]), fx_pair(e[5], e[10])),
+                                     fx_word(fx_pair(e[6], e[7]), fx_pair(e[8], e[11])), 0};
         }
         if (G.milne) {
             // sqrt(-g) Gamma^0_{33} T^{33} / sigma* = tau^2 T^{eta eta} / sigma*
