@@ -261,11 +261,15 @@ constexpr int kEosWarps = 4;
 #endif
 constexpr int kEosBlocksPerSM = SPH_EOS_BLOCKS_PER_SM;  // resident blocks per SM (the register budget)
 
-__device__ __forceinline__ void put_point(double *__restrict__ guess_out, uint32_t *__restrict__ status, size_t n,
-                                          size_t a, const double x[4], uint32_t st)
+__device__ __forceinline__ void put_guess(double *__restrict__ guess_out, size_t n, size_t a, const double x[4])
 {
 #pragma unroll
     for (int k = 0; k < 4; ++k) guess_out[k * n + a] = x[k];
+}
+__device__ __forceinline__ void put_point(double *__restrict__ guess_out, uint32_t *__restrict__ status, size_t n,
+                                          size_t a, const double x[4], uint32_t st)
+{
+    put_guess(guess_out, n, a, x);
     status[a] = st;
 }
 
@@ -284,6 +288,8 @@ struct Find2Ctx {
         return true;
     }
     __device__ void put(int a, const double x[4], uint32_t st) { put_point(guess_out, status, n, (size_t)a, x, st); }
+    __device__ void keep(int a, const double g[4]) { put_guess(guess_out, n, (size_t)a, g); }
+    __device__ void mark(int a, uint32_t st) { status[a] = st; }
 };
 
 __device__ __forceinline__ void add_eos_work(DevScalars *sc, const EosWork &w, unsigned st_or)
@@ -380,10 +386,21 @@ struct SegFindCtx {
     __device__ void put(int a, const double x[4], uint32_t st)
     {
         put_point(A.wguess, A.status, P, (size_t)a, x, st);
+        count();
+    }
+    // the particle's work so far, to its event's counters
+    __device__ void count()
+    {
         unsigned int *c = sh + 4 * slot;
         if (w->resid != w0.resid) atomicAdd_block(c, w->resid - w0.resid);
         if (w->solve != w0.solve) atomicAdd_block(c + 1, w->solve - w0.solve);
         if (w->g != w0.g) atomicAdd_block(c + 2, w->g - w0.g);
+    }
+    __device__ void keep(int a, const double g[4]) { put_guess(A.wguess, P, (size_t)a, g); }
+    __device__ void mark(int a, uint32_t st)
+    {
+        A.status[a] = st;
+        count();
     }
 };
 

@@ -683,11 +683,15 @@ __device__ EosOut eos_invert(const EosDev &E, double cs2_cap, double s, const do
 // 360 (values, derivatives, p, solve) to about 110, and one evaluation fewer is needed: the last
 // step is taken when the residual is below the hand-over bound, and eos_finish looks at its
 // result.  The Newton's work varies from particle to particle, so the lanes refill: each lane
-// holds its own particle and claims the next one as soon as its own is handed on.
+// holds its own particle and claims the next one as soon as its own is handed on.  Where FP32 does not
+// do (rough_step, exact_step: charges that move together, differences that it does not resolve; a
+// singular system; maxit steps), the particle is left to the general FP64 inversion from its own start.
 //
 // eos_finish evaluates p, e and (p_s, p_n) = H^-T (s, n) at that point in FP64, one thread per
 // particle, all lanes alike.  A table point whose residual misses the tolerance there (a step
-// across a cell boundary, rarely) goes through the general FP64 inversion from that point.
+// across a cell boundary, rarely), or with polish the rounding level (kPolished: the FP32 step did not
+// reduce the residual as an FP64 step does), goes through the general FP64 inversion from that point,
+// and so do, from their starts, the particles that the search left to it.
 //
 // Bound: the FP64 pipe (64 cycles per warp instruction and quadrant).  Measured per stage on the
 // 40 k viscous BSQ event: 106 us (196 in one pass with the derivatives and the solve of every
@@ -696,7 +700,10 @@ __device__ EosOut eos_invert(const EosDev &E, double cs2_cap, double s, const do
 //
 // Hand-over bounds on max |residual| / s: 1e-10 where the point has to be the root to rounding
 // (polish), 1e-6 for the 1e-10 tolerance of the mixed and serving forms.
-constexpr uint32_t kNoVerify = 0x80000000u;  // status bit between the halves: the point is taken as it is
+// status bits between the halves: the point is taken as it is; the general inversion from the start
+constexpr uint32_t kNoVerify = 0x80000000u, kGeneral = 0x40000000u;
+// max |residual| / s of a polished point: the rounding of the interpolant, about 20 operations of 2^-53
+constexpr double kPolished = 4e-15;
 
 // magnitude-truncated single-precision value of a double, from its bits (|v| < 2^-126: zero)
 __device__ __forceinline__ float f32_bits(double v)
@@ -834,40 +841,15 @@ __device__ __forceinline__ bool inside_keys(const EosDev &E, const double *x)
     for (int q = 0; q < 3; ++q) in = in && okey(x[1 + q]) >= okey(E.mu0[q]) && okey(x[1 + q]) <= okey(E.mumax[q]);
     return in;  // NaN keys lie beyond every bound
 }
-__device__ __forceinline__ bool finite_bits(double v) { return mag_bits(v) < kInfBits; }
-
-// max |residual| at grid coordinates xi as an integer magnitude (the line search's trials)
-__device__ __forceinline__ long long tab_resid_norm(const EosDev &E, const double *xi, const double *tgt)
+// max |r| as an integer magnitude; non-finite ones count as infinite
+__device__ __forceinline__ long long resid_norm(const double *r)
 {
-    int i[4];
-    double t[4];
-    locate_steps(xi[0], E.nT, i[0], t[0]);
-#pragma unroll
-    for (int q = 0; q < 3; ++q) locate_steps(xi[1 + q], E.nmu[q], i[1 + q], t[1 + q]);
-    const int n3 = E.nmu[2], n23 = E.nmu[1] * E.nmu[2], n123 = E.nmu[0] * n23;
-    const size_t node0 = (size_t)i[0] * n123 + (size_t)i[1] * n23 + (size_t)i[2] * n3 + i[3];
-    const double2 *sn2 = reinterpret_cast<const double2 *>(E.sn);
-    // the order of operations of tab_resid_steps: the same residuals
-    const double uT = 1.0 - t[0], uB = 1.0 - t[1], uS = 1.0 - t[2], uQ = 1.0 - t[3];
-    const double w00 = uS * uQ, w01 = uS * t[3], w10 = t[2] * uQ, w11 = t[2] * t[3];
-    const double wp[4] = {uT * uB, uT * t[1], t[0] * uB, t[0] * t[1]};
-    double acc[4] = {-tgt[0], -tgt[1], -tgt[2], -tgt[3]};
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        const size_t base = node0 + (size_t)(c >> 1) * n123 + (size_t)(c & 1) * n23;
-#pragma unroll
-        for (int fp = 0; fp < 2; ++fp) {
-            const double2 q00 = __ldg(sn2 + 2 * base + fp), q01 = __ldg(sn2 + 2 * (base + 1) + fp);
-            const double2 q10 = __ldg(sn2 + 2 * (base + n3) + fp), q11 = __ldg(sn2 + 2 * (base + n3 + 1) + fp);
-            acc[2 * fp] = fma(wp[c], fma(w11, q11.x, fma(w10, q10.x, fma(w01, q01.x, w00 * q00.x))), acc[2 * fp]);
-            acc[2 * fp + 1] = fma(wp[c], fma(w11, q11.y, fma(w10, q10.y, fma(w01, q01.y, w00 * q00.y))), acc[2 * fp + 1]);
-        }
-    }
     long long m = 0;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) m = max(m, min(mag_bits(acc[k]), kInfBits));
+    for (int k = 0; k < 4; ++k) m = max(m, min(mag_bits(r[k]), kInfBits));
     return m;
 }
+__device__ __forceinline__ bool finite_bits(double v) { return mag_bits(v) < kInfBits; }
 
 // the closed form as a call of its own: the lane loop keeps its registers for the table Newton
 __device__ __noinline__ uint32_t an_invert_call(const EosDev &E, double s, const double *n, double *x, EosWork &w,
@@ -893,13 +875,54 @@ __device__ __forceinline__ void trial_point(const long long *top, const double *
     }
 }
 
+// Whether the FP32 step d at residual norm r may not decrease the residual where the exact one does.  The
+// Jacobian per grid step in FP32 is off by at most 2^-21 of the node values, and the elimination by about
+// as much, so |J d + r| <= 2^-17 v sum |d_k| with v the node values, which the target and the residual
+// bound (about 4 (|target| + r)): up to r/4 it does.
+__device__ __forceinline__ bool rough_step(const float *d, float r, float target)
+{
+    const float sum = (fabsf(d[0]) + fabsf(d[1])) + (fabsf(d[2]) + fabsf(d[3]));
+    return !(0x1p-15f * (target + r) * sum <= r);
+}
+// Whether the FP32 step d from a point with residual r and FP32 Jacobian J is the exact one to 1/32 of its
+// length, so that a search along the one stalls as along the other: its error is J^-1 (E d) with |E_fk| <=
+// 2^-20 v_f, v_f the node values of field f, bounded by the target, the residual and the differences.
+__device__ __noinline__ bool exact_step(const float (&J)[4][4], const double *r, const double *tgt, const float *d)
+{
+    float err[4] = {0.f, 0.f, 0.f, 0.f}, rn = 0.f, sum = 0.f, top = 0.f;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        rn = fmaxf(rn, fabsf(f32_bits(r[k])));
+        sum += fabsf(d[k]);
+        top = fmaxf(top, fabsf(d[k]));
+    }
+    bool ok = true;
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {  // column f of the inverse
+        float A[4][4], e[4], v = rn + fabsf(f32_bits(tgt[f]));
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            e[i] = i == f ? 1.f : 0.f;
+            v += fabsf(J[f][i]);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) A[i][k] = J[i][k];
+        }
+        ok = solve4f(A, e) && ok;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) err[i] += fabsf(e[i]) * (0x1p-18f * v);
+    }
+    // a step below the single-precision range is zero here
+    return ok && top > 0.f && fmaxf(fmaxf(err[0], err[1]), fmaxf(err[2], err[3])) * sum <= 0x1p-5f * top;
+}
+
 // The line searches of a warp's lanes in todo after a full step without a decrease: the halvings
 // 1/2 .. 1/2^8 of one particle at a time, a lane for each, and the largest that decreases the
-// residual (the first that a search trial by trial would take).  xt: the point found; false: none.
+// residual (the first that a search trial by trial would take).  xt: the point found; false: none, and
+// exact says whether the step is an exact_step (a ninth lane looks, at the point itself).
 // One trial a trip held the whole pass for particles beyond a table edge, whose searches fail
 // every stage: 40 k event with three such particles, EoS pass 341 us per step, now 270.
 __device__ __noinline__ bool line_searches(const EosDev &E, unsigned todo, const double *xi, const float *d,
-                                           const double *tgt, long long rn, double *xt, unsigned &trials)
+                                           const double *tgt, long long rn, double *xt, unsigned &trials, bool &exact)
 {
     const unsigned FULL = 0xFFFFFFFFu;
     const int lane = threadIdx.x & 31;
@@ -917,15 +940,23 @@ __device__ __noinline__ bool line_searches(const EosDev &E, unsigned todo, const
             ds[k] = __shfl_sync(FULL, d[k], src);
         }
         const long long rs = __shfl_sync(FULL, rn, src);
-        bool less = false;
-        if (lane < 8) {
-            trial_point(top, xs, ds, __int_as_float((126 - lane) << 23), xl);
-            less = tab_resid_norm(E, xl, ts) < rs;
+        bool less = false, ex = false;
+        double r[4];
+        float J[4][4];
+        if (lane < 9) {
+            if (lane < 8) trial_point(top, xs, ds, __int_as_float((126 - lane) << 23), xl);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) xl[k] = lane < 8 ? xl[k] : xs[k];
+            tab_resid_steps(E, xl, ts, r, J);
+            less = lane < 8 && resid_norm(r) < rs;
         }
         const unsigned m = __ballot_sync(FULL, less);
+        if (m == 0u && lane == 8) ex = exact_step(J, r, ts, ds);
+        const unsigned mx = __ballot_sync(FULL, ex);
         if (lane == src) {
             trials = m ? (unsigned)__ffs(m) : 8u;
             found = m != 0u;
+            exact = mx != 0u;
             if (m) trial_point(top, xi, d, __int_as_float((127 - __ffs(m)) << 23), xt);  // evaluated and accepted next
         }
     }
@@ -934,8 +965,12 @@ __device__ __noinline__ bool line_searches(const EosDev &E, unsigned todo, const
 
 // First half.  Ctx supplies  bool load(int a, double &s, double n[3], double g[4])  (false: not a
 // particle of this pass; g: the warm start, T > 0 a table solution, T < 0 minus a closed-form T)
-// and  void put(int a, const double x[4], uint32_t st): T > 0 a table point, T < 0 minus the
-// closed form's T, 0 none (st tells why).  claim: the pass's particle counter.
+// void put(int a, const double x[4], uint32_t st): T > 0 a table point, T < 0 minus the closed form's
+// T, 0 none (st tells why), and  void keep(int a, const double g[4]), which leaves the warm start where
+// put leaves the result (kGeneral), and  void mark(int a, uint32_t st), the status alone.
+// claim: the pass's particle counter.
+// Every loop ends: a search takes at most maxit accepted points and one line search after each (its
+// point has to be accepted next), from the warm start and from the closed form.
 template <class Ctx>
 __device__ void eos_find(const EosDev &E, unsigned int *claim, int limit, Ctx &ctx, EosWork &w)
 {
@@ -948,10 +983,10 @@ __device__ void eos_find(const EosDev &E, unsigned int *claim, int limit, Ctx &c
     grid_top(E, top);
     const double hand = E.polish ? 1e-10 : 1e-6;
     int a = -1, it = 0;
-    bool more = true, first = false, cold = false;
+    bool more = true, first = false, cold = false, searched = false;  // searched: xt is a line search's
     long long rn = 0, tolb = 0, handb = 0;
     double xi[4] = {0.0, 0.0, 0.0, 0.0}, xt[4] = {0.0, 0.0, 0.0, 0.0}, tgt[4] = {0.0, 0.0, 0.0, 0.0}, Tcf = 0.0;
-    float d[4] = {0.f, 0.f, 0.f, 0.f};
+    float d[4] = {0.f, 0.f, 0.f, 0.f}, tmax = 0.f;
     for (;;) {
         // lanes without a particle claim the next ones (one atomic per warp)
         const unsigned need = __ballot_sync(FULL, a < 0 && more);
@@ -1006,33 +1041,36 @@ __device__ void eos_find(const EosDev &E, unsigned int *claim, int limit, Ctx &c
                 }
             }
             if (a >= 0 && ((need >> lane) & 1u)) {
+                ctx.keep(a, g);
                 first = true;
+                searched = false;
                 it = 0;
+                tmax = fmaxf(fmaxf(fabsf(f32_bits(tgt[0])), fabsf(f32_bits(tgt[1]))), fmaxf(fabsf(f32_bits(tgt[2])), fabsf(f32_bits(tgt[3]))));
                 tolb = __double_as_longlong(E.tol * tgt[0]);
                 handb = max(tolb, __double_as_longlong(hand * tgt[0]));
             }
         }
         if (__ballot_sync(FULL, a >= 0 || more) == 0u) break;
-        bool fail = false, step_on = false, last = false, search = false;
+        bool fail = false, general = false, step_on = false, last = false, search = false;
         if (a >= 0) {
             // one evaluation at the trial point
             double r[4];
             float J[4][4];
             tab_resid_steps(E, xt, tgt, r, J);
             ++w.resid;
-            long long rnn = 0;
-#pragma unroll
-            for (int k = 0; k < 4; ++k) rnn = max(rnn, min(mag_bits(r[k]), kInfBits));
+            const long long rnn = resid_norm(r);
             if (first || rnn < rn) {
                 it += first ? 0 : 1;
-                first = false;
+                first = searched = false;
 #pragma unroll
                 for (int k = 0; k < 4; ++k) xi[k] = xt[k];
                 rn = rnn;
-                if (rn <= tolb && !E.polish) last = true;
+                if (rn <= tolb && (!E.polish || it >= E.maxit)) last = true;
+                else if (it >= E.maxit) general = true;
                 else if (rn <= handb) last = step_on = true;
-                else if (it >= E.maxit) fail = true;
                 else step_on = true;
+            } else if (searched) {
+                general = true;
             } else {
                 search = true;
             }
@@ -1041,10 +1079,7 @@ __device__ void eos_find(const EosDev &E, unsigned int *claim, int limit, Ctx &c
 #pragma unroll
                 for (int k = 0; k < 4; ++k) d[k] = -f32_bits(r[k]);
                 const bool ok = solve4f(J, d);
-                if (!ok && !last) fail = true;
-                if (!ok)
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) d[k] = 0.0f;
+                general = !ok || rough_step(d, f32_bits(__longlong_as_double(rn)), tmax);
                 trial_point(top, xi, d, 1.0f, xt);
             }
         }
@@ -1056,15 +1091,21 @@ __device__ void eos_find(const EosDev &E, unsigned int *claim, int limit, Ctx &c
 #pragma unroll
             for (int k = 0; k < 4; ++k) xs[k] = xi[k], ts[k] = tgt[k], ds[k] = d[k], xo[k] = xt[k];
             unsigned trials = 0u;
-            const bool found = line_searches(E, todo, xs, ds, ts, rn, xo, trials);
+            bool exact = false;
+            const bool found = line_searches(E, todo, xs, ds, ts, rn, xo, trials, exact);
             w.resid += trials;
             if (search) {
+                searched = true;
                 fail = !found;  // no decrease along the Newton direction: stalled
+                general = fail && !exact;
 #pragma unroll
                 for (int k = 0; k < 4; ++k) xt[k] = xo[k];
             }
         }
-        if (last) {
+        if (general) {
+            ctx.mark(a, kGeneral);
+            a = -1;
+        } else if (last) {
             double x[4];
 #pragma unroll
             for (int k = 0; k < 4; ++k) x[k] = fma(step_on ? xt[k] : xi[k], step[k], org[k]);
@@ -1077,6 +1118,7 @@ __device__ void eos_find(const EosDev &E, unsigned int *claim, int limit, Ctx &c
                 const uint32_t st = an_invert_call(E, tgt[0], tgt + 1, x, w, 0.0);
                 if (!st && inside_keys(E, x)) {
                     cold = first = true;
+                    searched = false;
                     Tcf = x[0];
                     it = 0;
 #pragma unroll
@@ -1114,6 +1156,7 @@ __device__ __forceinline__ EosOut eos_finish(const EosDev &E, double cs2_cap, do
     for (int q = 0; q < 3; ++q) o.mu[q] = o.pn[q] = 0.0;
     o.st = st & ~kNoVerify;
     used_table = false;
+    if (st & kGeneral) return eos_invert_call(E, cs2_cap, s, n, g, used_table, w);
     const long long tb = __double_as_longlong(g[0]);
     if (tb == 0) {
         if (st & PST_BACKUP) return backup_eos(E, s, n);
@@ -1130,7 +1173,7 @@ __device__ __forceinline__ EosOut eos_finish(const EosDev &E, double cs2_cap, do
         long long rn = 0;
 #pragma unroll
         for (int k = 0; k < 4; ++k) rn = max(rn, min(mag_bits(sn[k] - b[k]), kInfBits));
-        if (!(st & kNoVerify) && rn > __double_as_longlong(E.tol * s))
+        if (!(st & kNoVerify) && rn > __double_as_longlong((E.polish ? fmin(E.tol, kPolished) : E.tol) * s))
             return eos_invert_call(E, cs2_cap, s, n, g, used_table, w);
         const double istep[4] = {E.inv_dT, E.inv_dmu[0], E.inv_dmu[1], E.inv_dmu[2]};
 #pragma unroll

@@ -247,6 +247,12 @@ struct Find3Ctx {
         for (int k = 0; k < 4; ++k) guess_out[k * n + a] = x[k];
         status[a] = st;
     }
+    __device__ void keep(int a, const double g[4])
+    {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) guess_out[k * n + a] = g[k];
+    }
+    __device__ void mark(int a, uint32_t st) { status[a] = st; }
 };
 
 __device__ __forceinline__ void add_eos_work3(DevScalars *sc, const EosWork &w, unsigned st_or)
