@@ -186,7 +186,8 @@ sph_status sph_step(sph_event *ev, int32_t nsteps, uint32_t flags);
  * STATUS) are evaluated at the current state (cell list, kernel sums and EoS
  * inversion are rerun if the state changed since the last read).
  * Destinations are host memory unless on_device = 1.  The call synchronises the
- * event's stream.
+ * event's stream, also where it returns SPH_ERR_ARG for a NULL destination: the fields
+ * before that one, in the order x .. Jv, sigstar .. e, Pi, status, nnb, cell, are then complete.
  * ------------------------------------------------------------------------- */
 #define SPH_F_X (1ull << 0)          /* x[dim*n] */
 #define SPH_F_U (1ull << 1)          /* u[dim*n] */

@@ -982,6 +982,13 @@ struct ReadOut {
         used = 0;
         return SPH_OK;
     }
+    // a requested field without a destination: the fields before it are complete when the call returns
+    sph_status refuse()
+    {
+        sph_status s = flush();
+        if (s == SPH_OK) s = wait_stream(ev);
+        return s != SPH_OK ? s : fail(SPH_ERR_ARG, "requested field has a null destination");
+    }
 };
 
 sph_status sph_read_fields(sph_event *ev, uint64_t mask, const sph_field_bufs *o, sph_totals *tot)
@@ -1029,45 +1036,17 @@ sph_status sph_read_fields(sph_event *ev, uint64_t mask, const sph_field_bufs *o
     sph_status rs;
     for (auto &r : rows) {
         if (!(mask & r.bit)) continue;
-        if (!r.dst) return fail(SPH_ERR_ARG, "requested field has a null destination");
+        if (!r.dst) return out.refuse();
         if (n == 0) continue;
         double *at = nullptr;
         if ((rs = out.room(r.rows, &at)) != SPH_OK) return rs;
         launch_scatter_orig(r.src, at, r.state ? ev->id[0] : ev->id[1], n, r.rows, st);
         if ((rs = out.put(r.dst, at, r.rows, dn * r.rows)) != SPH_OK) return rs;
     }
-    if (mask & SPH_F_STATUS) {
-        if (!o->status) return fail(SPH_ERR_ARG, "requested field has a null destination");
-        if (n > 0) {
-            double *at = nullptr;
-            if ((rs = out.room(1, &at)) != SPH_OK) return rs;
-            launch_scatter_orig_u32(ev->status, (uint32_t *)at, ev->id[1], n, st);
-            if ((rs = out.put(o->status, at, 1, sizeof(uint32_t) * n)) != SPH_OK) return rs;
-        }
-    }
-    if (mask & SPH_F_NNB) {
-        if (!o->nnb) return fail(SPH_ERR_ARG, "requested field has a null destination");
-        if (n > 0) {
-            double *at = nullptr;
-            if ((rs = out.room(1, &at)) != SPH_OK) return rs;
-            launch_scatter_orig_u32((const uint32_t *)ev->nnb, (uint32_t *)at, ev->id[1], n, st);
-            if ((rs = out.put(o->nnb, at, 1, sizeof(int) * n)) != SPH_OK) return rs;
-        }
-    }
-    if (mask & SPH_F_CELL) {
-        if (!o->cell) return fail(SPH_ERR_ARG, "requested field has a null destination");
-        if (n > 0) {
-            EvView v = make_view(ev);
-            double *at = nullptr;
-            if ((rs = out.room(ev->dim, &at)) != SPH_OK) return rs;
-            launch_cell_coords(v, ev->Y[1], ev->id[1], (int *)at, st);
-            if ((rs = out.put(o->cell, at, ev->dim, sizeof(int) * ev->dim * n)) != SPH_OK) return rs;
-        }
-    }
-    if ((rs = out.flush()) != SPH_OK) return rs;
     if (mask & SPH_F_PI_BULK) {
-        if (!o->Pi) return fail(SPH_ERR_ARG, "requested field has a null destination");
+        if (!o->Pi) return out.refuse();
         if (n > 0) {
+            if ((rs = out.flush()) != SPH_OK) return rs;  // the scratch rows are used below
             // Pi = sigma * (Pi/sigma) with sigma = sigma* / (u^0 sqrt(-g)), on the host side of the copy
             std::vector<double> bv(n), sg(n), u0(n);
             launch_scatter_orig(ev->Y[1] + (2 * ev->dim + 1) * N, ev->scratch, ev->id[1], n, 1, st);
@@ -1085,6 +1064,35 @@ sph_status sph_read_fields(sph_event *ev, uint64_t mask, const sph_field_bufs *o
             CK(cudaMemcpy(o->Pi, Pi.data(), dn, o->on_device ? cudaMemcpyHostToDevice : cudaMemcpyHostToHost));
         }
     }
+    if (mask & SPH_F_STATUS) {
+        if (!o->status) return out.refuse();
+        if (n > 0) {
+            double *at = nullptr;
+            if ((rs = out.room(1, &at)) != SPH_OK) return rs;
+            launch_scatter_orig_u32(ev->status, (uint32_t *)at, ev->id[1], n, st);
+            if ((rs = out.put(o->status, at, 1, sizeof(uint32_t) * n)) != SPH_OK) return rs;
+        }
+    }
+    if (mask & SPH_F_NNB) {
+        if (!o->nnb) return out.refuse();
+        if (n > 0) {
+            double *at = nullptr;
+            if ((rs = out.room(1, &at)) != SPH_OK) return rs;
+            launch_scatter_orig_u32((const uint32_t *)ev->nnb, (uint32_t *)at, ev->id[1], n, st);
+            if ((rs = out.put(o->nnb, at, 1, sizeof(int) * n)) != SPH_OK) return rs;
+        }
+    }
+    if (mask & SPH_F_CELL) {
+        if (!o->cell) return out.refuse();
+        if (n > 0) {
+            EvView v = make_view(ev);
+            double *at = nullptr;
+            if ((rs = out.room(ev->dim, &at)) != SPH_OK) return rs;
+            launch_cell_coords(v, ev->Y[1], ev->id[1], (int *)at, st);
+            if ((rs = out.put(o->cell, at, ev->dim, sizeof(int) * ev->dim * n)) != SPH_OK) return rs;
+        }
+    }
+    if ((rs = out.flush()) != SPH_OK) return rs;
     if (tot) {
         memset(tot, 0, sizeof(*tot));
         DevScalars hs;
