@@ -726,8 +726,8 @@ sph_status sph_init_event(sph_event **out, const sph_event_desc *d, const sph_eo
 // state (at least 1.5 x the old allocation when growing), margin = 32.  Counts are carried from
 // stage to stage in the state order (pcnt[0] with Y[0], pcnt[1] with Y1[0]); here they are taken
 // from a read-out evaluation of the current state.  The lists stay off (the per-particle passes
-// run) for other forms, when SPH_PAIR_LISTS=0, or when they would take more than a quarter of the
-// free device memory.  SPH_PAIR_MARGIN and SPH_PAIR_TOTAL override the
+// run) for other forms, when SPH_PAIR_LISTS=0, or when they would take more than about a quarter of
+// the free device memory (the limit below).  SPH_PAIR_MARGIN and SPH_PAIR_TOTAL override the
 // margin and the first allocation (tests of the overflow paths).
 static sph_status size_pair_lists(sph_event *ev)
 {
@@ -785,7 +785,11 @@ static sph_status size_pair_lists(sph_event *ev)
                          (size_t)nparts * sizeof(unsigned long long) + per_particle * (size_t)n + 1024;
     size_t fr = 0, tot = 0;
     CK(cudaMemGetInfo(&fr, &tot));
-    if (bytes > fr / 4) {
+    // a quarter of the free memory; the plain 3D entries are padded to 44 bytes (a gradient in one sector), and
+    // the limit holds as many of them as a quarter holds at 40: beyond it a step of the per-particle passes
+    // takes 2.7 times as long (172 against 63 ns a particle)
+    const size_t limit = !ev->mixed && ev->dim == 3 ? fr / 160 * 44 : fr / 4;
+    if (bytes > limit) {
         ev->pairs_off = true;
         ev->pairs_grow = false;
         return SPH_OK;
