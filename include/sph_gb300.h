@@ -154,13 +154,19 @@ typedef struct {
     const double *kappaT2, *tauJT, *Jv;
 } sph_event_desc;
 
-/* Precision of the step.  SPH_FP64: every operation in double precision.  SPH_MIXED (dim 2 or 3):
+/* Precision of the step.  SPH_FP64: state, inputs, outputs, accumulation and every result in double
+ * precision.  Two parts use other units to get there: the neighbour sums are formed in integers
+ * (kernel values of 53 bits with a relative error of 2^-53 + 11 2^-60 / (2 - r/h), also towards the
+ * kernel's rim; each sum in units of its own largest term, 2^-53 of it per term), and the table
+ * search takes FP64 residuals with the Newton step's Jacobian and 4x4 solve in single precision, or in
+ * double where that does not resolve the system; the point it ends at is accepted and polished on FP64
+ * residuals, and everything evaluated there is FP64.  SPH_MIXED (dim 2 or 3):
  * the neighbour passes (kernel sums and gradients) run in single precision with positions
  * relative to their cell's origin and compensated (two-sum) accumulation, combined per particle
  * without loss (two particles of a cell per warp, packed two-wide FP32 instructions); the neighbour set
  * stays exactly that of the FP64 test (a proven float error band, the FP64 test inside it); the
  * EoS inversion (to max(newton_tol, 1e-10) without the polishing step, as its inputs carry the
- * single-precision sums' rounding), equations of motion, Heun update and reductions stay FP64.
+ * single-precision sums' rounding), equations of motion, Heun update and reductions are those of SPH_FP64.
  * Results differ from SPH_FP64 at the ~1e-7 relative level. */
 #define SPH_FP64 0
 #define SPH_MIXED 1
@@ -175,7 +181,14 @@ void sph_free_event(sph_event *ev);
 /* Advances nsteps full Heun steps (2 stages each) of size dtau on the event's
  * stream.  Asynchronous unless flags & SPH_SYNC; with SPH_SYNC the call waits
  * (bounded by the event's timeout, SPH_ERR_TIMEOUT if exceeded) and checks the
- * per-particle status against fatal_mask.  nsteps < 0: SPH_ERR_ARG. */
+ * per-particle status against fatal_mask.  nsteps < 0: SPH_ERR_ARG.
+ * Forms with pair lists (SPH_FP64, and SPH_MIXED with dim = 3) size them in the first call with
+ * nsteps > 0, and again in the call after a step whose lists overflowed: these calls run a read-out
+ * evaluation and wait for the stream before they enqueue.  The lists hold 1.5 times the entries of
+ * the current state: 28 bytes per ordered neighbour pair in 2D, 44 in 3D, 4 in the mixed 3D form (30 GB
+ * for 8 M particles of 600 neighbours), if that is at most a quarter (plain 3D: 11/40) of the free device
+ * memory, else none are kept and each pass finds its neighbours by itself.  They are given back by
+ * sph_free_event.  SPH_PAIR_LISTS=0 in the environment leaves them out. */
 #define SPH_SYNC 1u
 sph_status sph_step(sph_event *ev, int32_t nsteps, uint32_t flags);
 
