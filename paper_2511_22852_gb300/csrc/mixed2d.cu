@@ -86,8 +86,8 @@ __device__ __forceinline__ double total2(const CSum &t)
 }
 
 // The walk of one warp over the candidates of particles a0 and a1 = a0 + 1 of cell (cx, cy) (two =
-// false: a0 alone).  pair(which, entry) receives an accepted pair per lane; flush() is called after
-// every kRun batches and at the end, with empty queues.
+// false: a0 alone).  pair(which, entry) receives an accepted pair per lane; flush() is called before a
+// particle has kRun batches behind it and at the end, with empty queues.
 // nacc: accepted candidates (self included); shell: candidates decided by the FP64 test.
 template <class Pair, class Flush>
 __device__ __forceinline__ void walk9_two(const EvView &v, const double *__restrict__ y,
@@ -172,7 +172,7 @@ __device__ __forceinline__ void walk9_two(const EvView &v, const double *__restr
                 if (lane < qn1) M.q[1][lane] = rest;
                 ++nb;
             }
-            if (nb >= kRun) {  // at most kRun plain terms per lane
+            if (nb >= kRun - 1) {  // at most kRun plain terms per lane and particle, these partial batches included
                 __syncwarp();
                 if (lane < qn0) pair(0, M.q[0][lane]);
                 if (lane < qn1) pair(1, M.q[1][lane]);
