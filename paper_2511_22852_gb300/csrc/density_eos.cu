@@ -7,18 +7,19 @@
 // with every product rounded separately, so the neighbour set is identical to a
 // plain FP64 evaluation on any platform.
 //
-// EoS pass (Sec. "EoS inverter", online inversion done on the device):
+// EoS pass (Sec. "EoS inverter", online inversion done on the device), in two halves (eos_device.cuh):
+//   find:
 //   0. damped Newton on the quadrilinear table interpolant warm-started from this
 //      particle's previous-stage table solution, when there is one in the table;
 //   1. otherwise: closed-form EoS solved for T on its upper branch
 //      (mu_q = n_q/(chi_q T^2)), bracketed Newton with bisection safeguard;
-//   2. if that point lies in the table, damped Newton on the quadrilinear
-//      interpolant of (s, n_B, n_S, n_Q), residual scaled by s, 4x4 Jacobian from
-//      the same 16-corner stencil, one polishing step after convergence;
-//      otherwise (or without convergence) the closed form is kept and flagged;
-//   3. p, e = T s + mu.n - p, and (dp/ds, dp/dn_q) = H^-T (s, n) with H the
-//      Jacobian d(s, n)/d(T, mu) of the EoS used; c_s^2 above the cap scales
-//      them down (flagged).
+//   2. if that point lies in the table, the damped Newton from it; otherwise (or without
+//      convergence) the closed form is kept and flagged;
+//   finish:
+//   3. the interpolant and its derivatives there in FP64 (the general FP64 inversion where the
+//      search's point does not meet the tolerance, or left it to that); p, e = T s + mu.n - p, and
+//      (dp/ds, dp/dn_q) = H^-T (s, n) with H the Jacobian d(s, n)/d(T, mu) of the EoS used;
+//      c_s^2 above the cap scales them down (flagged).
 #include <algorithm>
 
 #include "sph_internal.cuh"
@@ -291,20 +292,6 @@ struct Find2Ctx {
     __device__ void keep(int a, const double g[4]) { put_guess(guess_out, n, (size_t)a, g); }
     __device__ void mark(int a, uint32_t st) { status[a] = st; }
 };
-
-__device__ __forceinline__ void add_eos_work(DevScalars *sc, const EosWork &w, unsigned st_or)
-{
-    const unsigned wres = __reduce_add_sync(0xFFFFFFFFu, w.resid);
-    const unsigned wsol = __reduce_add_sync(0xFFFFFFFFu, w.solve);
-    const unsigned wg = __reduce_add_sync(0xFFFFFFFFu, w.g);
-    const unsigned sor = __reduce_or_sync(0xFFFFFFFFu, st_or);
-    if ((threadIdx.x & 31) == 0) {
-        if (wres) atomicAdd(&sc->eos_resid, (unsigned long long)wres);
-        if (wsol) atomicAdd(&sc->eos_solve, (unsigned long long)wsol);
-        if (wg) atomicAdd(&sc->eos_g, (unsigned long long)wg);
-        if (sor) atomicOr(&sc->status_or, sor);
-    }
-}
 
 __global__ void __launch_bounds__(32 * kEosWarps, kEosBlocksPerSM)
     k_eos2_find(EvView v, int stage, const double *__restrict__ y, double *__restrict__ dens,

@@ -46,6 +46,21 @@ struct EosWork {
     unsigned resid, solve, g;
 };
 
+// a warp's work and status bits, to its event's counters
+__device__ __forceinline__ void add_eos_work(DevScalars *sc, const EosWork &w, unsigned st_or)
+{
+    const unsigned wres = __reduce_add_sync(0xFFFFFFFFu, w.resid);
+    const unsigned wsol = __reduce_add_sync(0xFFFFFFFFu, w.solve);
+    const unsigned wg = __reduce_add_sync(0xFFFFFFFFu, w.g);
+    const unsigned sor = __reduce_or_sync(0xFFFFFFFFu, st_or);
+    if ((threadIdx.x & 31) == 0) {
+        if (wres) atomicAdd(&sc->eos_resid, (unsigned long long)wres);
+        if (wsol) atomicAdd(&sc->eos_solve, (unsigned long long)wsol);
+        if (wg) atomicAdd(&sc->eos_g, (unsigned long long)wg);
+        if (sor) atomicOr(&sc->status_or, sor);
+    }
+}
+
 // g(T) = s(T, mu(T)) - s_target with mu_q(T) = n_q/(chi_q T^2)
 __device__ __forceinline__ void an_g(const EosDev &E, double T, double s, double c, double &g, double &gp)
 {

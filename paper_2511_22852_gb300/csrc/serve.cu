@@ -1070,8 +1070,8 @@ sph_status dmalloc(sph_server *S, void **p, size_t bytes)
     return SPH_OK;
 }
 
-// kernels a batch step launches: per stage 11 for the cell list and permutation, then the
-// density, EoS, gradient and equations-of-motion passes and the two of the work sum
+// kernels a batch step launches: per stage 11 for the cell list and permutation, then the density pass,
+// the two halves of the EoS pass, the gradient and equations-of-motion passes and the two of the work sum
 constexpr int kKernelsPerBatchStep = 2 * 18;
 
 // one batch step (both stages) on the server's stream; captured once into a graph.  marks (the

@@ -104,7 +104,7 @@ struct EvView {
     float supp2_hi;  // single-precision prefilter bound, >= (2h)^2 plus the worst rounding error
     float supp2_lo;  // below it the float r^2 proves r < 2h: the exact FP64 test is skipped
     int mixed;                 // 1: neighbour passes in FP32 with compensated sums (2D)
-    float cell_f;              // mixed: cell side 2h in single precision
+    float cell_f;              // cell side 2h in single precision
     float shell_lo, shell_hi;  // mixed: float r^2 below lo is inside, above hi outside, else FP64 test
     DevScalars *sc;
     EosDev eos;
@@ -267,48 +267,6 @@ __device__ __forceinline__ float rsqrt_apx(float x)
     return y;
 }
 
-// Exact bit-level helpers that keep work off the FP64 pipe (1/64 of the FP32 rate on GB300):
-// x != 0 for x >= 0 (true when any bit is set; +0 is all zero bits)
-__device__ __forceinline__ bool nonzero_nonneg(double x) { return __double_as_longlong(x) != 0LL; }
-// max(x, 0) for finite x, from the sign bit
-__device__ __forceinline__ double pos_part(double x)
-{
-    const long long b = __double_as_longlong(x);
-    return __longlong_as_double(b & ~(b >> 63));
-}
-// x / 4 for x = 0 or x >= 2^-1020, by lowering the exponent field by 2 (exact)
-__device__ __forceinline__ double quarter_nonneg(double x)
-{
-    return __hiloint2double(max(__double2hiint(x) - 0x00200000, 0), __double2loint(x));
-}
-
-// Warp sum of up to 8 per-lane values by recursive halving (a reduce-scatter): at each of the
-// first three levels a lane keeps half of its values and adds its partner's copy of them, then
-// two butterfly levels finish one value.  9 additions per lane instead of 5 per value for a full
-// butterfly -- on the 1:64 FP64 pipe a warp-wide addition costs as much as 32 lanes of pair
-// work.  Returns, in lanes 4k .. 4k+3, the warp total of v[k]; the order of the additions is
-// fixed, so results are reproducible.
-__device__ __forceinline__ double warp_reduce_scatter8(const double (&v)[8], int lane)
-{
-    const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4;
-    double h[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const double keep = b4 ? v[4 + i] : v[i], give = b4 ? v[i] : v[4 + i];
-        h[i] = keep + __shfl_xor_sync(0xFFFFFFFFu, give, 16);
-    }
-    double g[2];
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        const double keep = b3 ? h[2 + i] : h[i], give = b3 ? h[i] : h[2 + i];
-        g[i] = keep + __shfl_xor_sync(0xFFFFFFFFu, give, 8);
-    }
-    double f = (b2 ? g[1] : g[0]) + __shfl_xor_sync(0xFFFFFFFFu, b2 ? g[0] : g[1], 4);
-    f += __shfl_xor_sync(0xFFFFFFFFu, f, 2);
-    f += __shfl_xor_sync(0xFFFFFFFFu, f, 1);
-    return f;
-}
-
 // cubic spline kernel (Sec. "Kernel function") as functions of q = r/h:
 // W = sigma_d w(q), dW/dr = sigma_d/h w'(q)
 __device__ __forceinline__ double kernel_w(double q)
@@ -386,13 +344,6 @@ __device__ __forceinline__ Aff operator*(double s, Aff a) { return {s * a.c, s *
 __device__ __forceinline__ Aff operator*(Aff a, double s) { return {s * a.c, s * a.x, s * a.y}; }
 __device__ __forceinline__ Aff operator+(Aff a, double s) { return {a.c + s, a.x, a.y}; }
 __device__ __forceinline__ double at(Aff a, double ax, double ay) { return fma(a.x, ax, fma(a.y, ay, a.c)); }
-
-// warp-aggregated OR into a global word
-__device__ __forceinline__ void warp_or(unsigned int *dst, unsigned int v)
-{
-    unsigned int m = __reduce_or_sync(__activemask(), v);
-    if (m && (threadIdx.x & 31) == (__ffs(__activemask()) - 1)) atomicOr(dst, m);
-}
 
 // ---------------------------------------------------------------------------
 // launchers (implemented in cells.cu, density_eos.cu, gradient_eom.cu)
@@ -480,7 +431,7 @@ void launch_permute(const EvView &v, const CellBufs &cb, const double *const *sr
                     const int *nrows, int ngroups, const double *x, const double *u, const int *id_in, int *id_out,
                     double *dens, cudaStream_t st);
 // plain 2D neighbour passes over the half-pair lists (cb.pl.total > 0): row offsets from the
-// previous counts, then the forward and backward density passes
+// previous counts, then the forward pass, which lists every pair in both rows, and the density sums
 void launch_pairs_density(const EvView &v, const double *y, const double *Nq, CellBufs cb, double *dens, int *nnb,
                           cudaStream_t st);
 void launch_pairs_gradient(const EvView &v, int stage, const double *y, const double *gin, CellBufs cb,

@@ -255,20 +255,6 @@ struct Find3Ctx {
     __device__ void mark(int a, uint32_t st) { status[a] = st; }
 };
 
-__device__ __forceinline__ void add_eos_work3(DevScalars *sc, const EosWork &w, unsigned st_or)
-{
-    const unsigned wres = __reduce_add_sync(0xFFFFFFFFu, w.resid);
-    const unsigned wsol = __reduce_add_sync(0xFFFFFFFFu, w.solve);
-    const unsigned wg = __reduce_add_sync(0xFFFFFFFFu, w.g);
-    const unsigned sor = __reduce_or_sync(0xFFFFFFFFu, st_or);
-    if ((threadIdx.x & 31) == 0) {
-        if (wres) atomicAdd(&sc->eos_resid, (unsigned long long)wres);
-        if (wsol) atomicAdd(&sc->eos_solve, (unsigned long long)wsol);
-        if (wg) atomicAdd(&sc->eos_g, (unsigned long long)wg);
-        if (sor) atomicOr(&sc->status_or, sor);
-    }
-}
-
 __global__ void __launch_bounds__(32 * kEosWarps3, kEosBlocks3)
     k_eos3_find(EvView v, int stage, const double *__restrict__ y, double *__restrict__ dens,
                 uint32_t *__restrict__ status, const double *__restrict__ guess_in, double *__restrict__ guess_out)
@@ -277,7 +263,7 @@ __global__ void __launch_bounds__(32 * kEosWarps3, kEosBlocks3)
     Find3Ctx ctx{v, (size_t)v.n, G.g[3], G.sqrtg, y, dens, guess_out, status, guess_in};
     EosWork w = {0u, 0u, 0u};
     eos_find(v.eos, &v.sc->eos_claim, v.n, ctx, w);
-    add_eos_work3(v.sc, w, 0u);
+    add_eos_work(v.sc, w, 0u);
 }
 
 // a4, second half: the EoS there, stress inputs of the gradient pass, work rate
@@ -365,7 +351,7 @@ __global__ void __launch_bounds__(64, 5) k_eos3_finish(EvView v, int stage, cons
             wcontrib = (G.tau * G.tau * ((o.e + P) * u[3] * u[3] + pi[3][3]) + P) * isig;
         }
     }
-    add_eos_work3(v.sc, w, st_or);
+    add_eos_work(v.sc, w, st_or);
     wcontrib = warp_sum(wcontrib);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = wcontrib;
     __syncthreads();
