@@ -717,8 +717,9 @@ __device__ EosOut eos_invert(const EosDev &E, double cs2_cap, double s, const do
 // (polish), 1e-6 for the 1e-10 tolerance of the mixed and serving forms.
 // status bits between the halves: the point is taken as it is; the general inversion from the start
 constexpr uint32_t kNoVerify = 0x80000000u, kGeneral = 0x40000000u;
-// max |residual| / s of a polished point: the rounding of the interpolant, about 20 operations of 2^-53
-constexpr double kPolished = 4e-15;
+// max |residual| / s of a polished point: the rounding of the interpolant, about 20 operations of 2^-53 on node
+// values of a few s
+constexpr double kPolished = 8e-15;
 
 // magnitude-truncated single-precision value of a double, from its bits (|v| < 2^-126: zero)
 __device__ __forceinline__ float f32_bits(double v)
@@ -902,38 +903,35 @@ __device__ __forceinline__ bool rough_step(const float *d, float r, float target
 // Whether the FP32 step d from a point with residual r and FP32 Jacobian J is the exact one to 1/32 of its
 // length, so that a search along the one stalls as along the other: its error is J^-1 (E d) with |E_fk| <=
 // 2^-20 v_f, v_f the node values of field f, bounded by the target, the residual and the differences.
-__device__ __noinline__ bool exact_step(const float (&J)[4][4], const double *r, const double *tgt, const float *d)
+// Four lanes in a row (f = lane & 3) with the same arguments take a column of the inverse each.
+__device__ __forceinline__ bool exact_step(float (&J)[4][4], const double *r, const double *tgt, const float *d, int f)
 {
-    float err[4] = {0.f, 0.f, 0.f, 0.f}, rn = 0.f, sum = 0.f, top = 0.f;
+    float rn = 0.f, sum = 0.f, top = 0.f, v = 0.f, e[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         rn = fmaxf(rn, fabsf(f32_bits(r[k])));
         sum += fabsf(d[k]);
         top = fmaxf(top, fabsf(d[k]));
+        if (k == f) v = ((fabsf(J[k][0]) + fabsf(J[k][1])) + (fabsf(J[k][2]) + fabsf(J[k][3]))) + fabsf(f32_bits(tgt[k]));
+        e[k] = k == f ? 1.f : 0.f;
     }
-    bool ok = true;
-#pragma unroll
-    for (int f = 0; f < 4; ++f) {  // column f of the inverse
-        float A[4][4], e[4], v = rn + fabsf(f32_bits(tgt[f]));
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            e[i] = i == f ? 1.f : 0.f;
-            v += fabsf(J[f][i]);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) A[i][k] = J[i][k];
-        }
-        ok = solve4f(A, e) && ok;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) err[i] += fabsf(e[i]) * (0x1p-18f * v);
-    }
+    v = 0x1p-18f * (v + rn) * sum;
     // a step below the single-precision range is zero here
-    return ok && top > 0.f && fmaxf(fmaxf(err[0], err[1]), fmaxf(err[2], err[3])) * sum <= 0x1p-5f * top;
+    bool ok = solve4f(J, e) && top > 0.f;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        float err = fabsf(e[i]) * v;
+        err += __shfl_xor_sync(0xFFFFFFFFu, err, 1);
+        err += __shfl_xor_sync(0xFFFFFFFFu, err, 2);
+        ok = ok && err <= 0x1p-5f * top;
+    }
+    return ok;
 }
 
 // The line searches of a warp's lanes in todo after a full step without a decrease: the halvings
 // 1/2 .. 1/2^8 of one particle at a time, a lane for each, and the largest that decreases the
 // residual (the first that a search trial by trial would take).  xt: the point found; false: none, and
-// exact says whether the step is an exact_step (a ninth lane looks, at the point itself).
+// exact says whether the step is an exact_step (the other lanes look, at the point itself).
 // One trial a trip held the whole pass for particles beyond a table edge, whose searches fail
 // every stage: 40 k event with three such particles, EoS pass 341 us per step, now 270.
 __device__ __noinline__ bool line_searches(const EosDev &E, unsigned todo, const double *xi, const float *d,
@@ -955,23 +953,18 @@ __device__ __noinline__ bool line_searches(const EosDev &E, unsigned todo, const
             ds[k] = __shfl_sync(FULL, d[k], src);
         }
         const long long rs = __shfl_sync(FULL, rn, src);
-        bool less = false, ex = false;
         double r[4];
         float J[4][4];
-        if (lane < 9) {
-            if (lane < 8) trial_point(top, xs, ds, __int_as_float((126 - lane) << 23), xl);
+        if (lane < 8) trial_point(top, xs, ds, __int_as_float((126 - lane) << 23), xl);
 #pragma unroll
-            for (int k = 0; k < 4; ++k) xl[k] = lane < 8 ? xl[k] : xs[k];
-            tab_resid_steps(E, xl, ts, r, J);
-            less = lane < 8 && resid_norm(r) < rs;
-        }
-        const unsigned m = __ballot_sync(FULL, less);
-        if (m == 0u && lane == 8) ex = exact_step(J, r, ts, ds);
-        const unsigned mx = __ballot_sync(FULL, ex);
+        for (int k = 0; k < 4; ++k) xl[k] = lane < 8 ? xl[k] : xs[k];
+        tab_resid_steps(E, xl, ts, r, J);
+        const unsigned m = __ballot_sync(FULL, lane < 8 && resid_norm(r) < rs);
+        const unsigned mx = m ? 0u : __ballot_sync(FULL, exact_step(J, r, ts, ds, lane & 3) && (lane >> 2) == 2);
         if (lane == src) {
             trials = m ? (unsigned)__ffs(m) : 8u;
             found = m != 0u;
-            exact = mx != 0u;
+            exact = mx == 0xF00u;
             if (m) trial_point(top, xi, d, __int_as_float((127 - __ffs(m)) << 23), xt);  // evaluated and accepted next
         }
     }
