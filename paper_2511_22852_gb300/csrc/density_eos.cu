@@ -40,7 +40,7 @@ constexpr int kWarps = 4;  // warps (particles in flight) per block of the neigh
 // results are reproducible.
 // Runs for events without lists: read-outs of new states, and stages whose lists overflowed.
 // Bound: the FP64 pipe, 9 operations per pair (22 with distance and kernel in FP64) and 9 additions a
-// particle (25).  Read-out of a new 39,001-particle state (all passes and copies) 1,090 -> 691 us.
+// particle (25).  Read-out of a new 39,001-particle state (all passes and copies) 1,090 -> 680 us.
 __global__ void __launch_bounds__(32 * kWarps) k_density2(EvView v, const double *__restrict__ y,
                                                           const float2 *__restrict__ fpos,
                                                           const double *__restrict__ Nq,

@@ -161,8 +161,9 @@ __device__ __forceinline__ void diff_finish(const EvView &v, int stage, const do
 // pair-list form (plain 2D events): half a warp per particle over the entries of its row with the
 // kernel gradient stored there (grad_a W_ab h / sigma_d), in integers (pairs_fixed.cuh) but for
 // alpha_b - alpha_a, an FP64 subtraction; the fluxes are summed as the gradient pass sums the stresses.
-// Bound: the latency of the gathers; 40 k event, diffusion and EoS passes per step 1,561 -> 860 us
-// (17 FP64 operations per pair before).
+// Bound: issue and the latency of the gathers; 40 k event: 295 us a stage (652 with 17 FP64 operations
+// per pair; 223 with the differences and units taken from the values alone).  The values in planes of
+// 32 bytes took 320.
 __global__ void __launch_bounds__(32 * kDiffWarps, 4) k_diff_pairs(EvView v, int stage, const double *__restrict__ dens,
                                                                    PairBufs pl)
 {

@@ -709,9 +709,9 @@ __device__ EosOut eos_invert(const EosDev &E, double cs2_cap, double s, const do
 // and so do, from their starts, the particles that the search left to it.
 //
 // Bound: the FP64 pipe (64 cycles per warp instruction and quadrant).  Measured per stage on the
-// 40 k viscous BSQ event: 106 us (196 in one pass with the derivatives and the solve of every
-// evaluation in FP64), ideal Gubser lattice 31 (303), eight served events (437 k particles) 588 (772),
-// 3+1D Milne event of 258 k particles, mixed form, 502 (976).
+// 40 k viscous BSQ event: 111 us (196 in one pass with the derivatives and the solve of every
+// evaluation in FP64), ideal Gubser lattice 31 (303), eight served events (437 k particles) 593 (772),
+// 3+1D Milne event of 258 k particles, mixed form, 505 (976).
 //
 // Hand-over bounds on max |residual| / s: 1e-10 where the point has to be the root to rounding
 // (polish), 1e-6 for the 1e-10 tolerance of the mixed and serving forms.
@@ -933,7 +933,8 @@ __device__ __forceinline__ bool exact_step(float (&J)[4][4], const double *r, co
 // residual (the first that a search trial by trial would take).  xt: the point found; false: none, and
 // exact says whether the step is an exact_step (the other lanes look, at the point itself).
 // One trial a trip held the whole pass for particles beyond a table edge, whose searches fail
-// every stage: 40 k event with three such particles, EoS pass 341 us per step, now 270.
+// every stage: 40 k event with three such particles, EoS pass 341 us per step, 270 with the trials side
+// by side, 290 with the look at the step (after 1,200 steps, with 133 such particles, 346 and 359).
 __device__ __noinline__ bool line_searches(const EosDev &E, unsigned todo, const double *xi, const float *d,
                                            const double *tgt, long long rn, double *xt, unsigned &trials, bool &exact)
 {

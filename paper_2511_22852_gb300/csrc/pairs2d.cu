@@ -4,12 +4,12 @@
 // (Sec. "SPH formalism", the n = 0 and n = -1 derivative forms) use W(r_ab) and dW/dr(r_ab) / r_ab
 // of every accepted pair; both depend on r_ab only, so they are the same for (a, b) and (b, a).
 // Each stage's forward pass evaluates them once per unordered pair -- on the pairs b > a of particle
-// a (sorted index) -- and keeps them with the pair in fixed point; the sum and gradient passes then
-// add every pair's contribution to both of its particles in integers (pairs_fixed.cuh), which do not
-// depend on the order, so results are reproducible run to run.
+// a (sorted index) -- and keeps them with the pair; the sum and gradient passes then add every pair's
+// contribution to both of its particles in integers (pairs_fixed.cuh), which do not depend on the
+// order, so results are reproducible run to run.
 //
 // FP64 operations per unordered pair fall from 56 (26 for the kernel, 10 for the density and 20 for
-// the gradient sums of its two particles) to 4; the 40 k event's step 2,038 -> 1,262 us.
+// the gradient sums of its two particles) to 4; the 40 k event's step 2,038 -> 1,272 us.
 //
 // Rows: a particle's row holds its previous neighbour count plus a margin (a prefix scan per
 // stage); forward entries fill it from the start, backward entries from the end.
@@ -119,10 +119,11 @@ __global__ void __launch_bounds__(kScanThreads) k_rows_apply(int n, const uint32
 // integers (pair_kernel) run on full warps.  W and grad W go into a's row and, at a place taken
 // from b's counter, into b's row.  The particles' own values go into limbs.
 // (Listing b < a in a's own walk, and finding its W by a search in b's row, kept the sums waiting
-// for memory: 40 k event, sum pass 197 -> 92 us a stage, gradient pass 150 -> 137.)
+// for memory: 40 k event, sum pass 197 -> 92 us a stage, gradient pass 150 -> 137, with the sums' units
+// taken from the values alone.)
 // Bound: latency and the L2 sectors of the scattered writes (b's row: three sectors a pair).  4 FP64
 // operations per unordered pair (12 with the kernel's distance in FP64, 31 with spline and sums).
-// 40 k event: 192 us a stage (212 with the distance in FP64 and every cell walked, 325 with the
+// 40 k event: 195 us a stage (212 with the distance in FP64 and every cell walked, 325 with the
 // spline in FP64).
 __global__ void __launch_bounds__(32 * kWarps, 8) k_pairs_fwd(EvView v, const double *__restrict__ y,
                                                            const float2 *__restrict__ fpos,
@@ -265,7 +266,9 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_pairs_fwd(EvView v, const do
 
 // Density sums, half a warp per particle a, over the entries of its row, in integers, each in the unit
 // of its own largest term (pairs_fixed.cuh).
-// Bound: the latency of the gathers; 40 k event 92 us a stage, 3+1D event of 258 k particles 0.92 ms.
+// Bound: issue and the ALU pipe (67 and 66 % busy), then the latency of the gathers; 40 k event 95 us a
+// stage, 3+1D event of 258 k particles 0.95 ms (92 and 0.92 with the units taken from the values alone,
+// without the kernel value of the pair).
 __global__ void __launch_bounds__(32 * kWarps, 7) k_pairs_sum(EvView v, PairBufs pl, double *__restrict__ dens,
                                                            int *__restrict__ nnb)
 {
@@ -369,8 +372,9 @@ __global__ void __launch_bounds__(32 * kWarps, 7) k_pairs_sum(EvView v, PairBufs
 // Gradient pass, half a warp per particle a, over the entries of its row with G = grad_a W_ab h /
 // sigma_d, forming in integers the sums of the per-particle pass: sum grad W, sum X_b grad W, sum u_b grad W, each in
 // the unit of its own largest term (a first look over the exponents).
-// Bound: the latency of the gathers; 40 k event 137 us a stage (298 us with 10 FP64 operations per
-// pair).  Two entries at a time: 150 against 173 us; 5 blocks per SM: 6 gave 161, 8 150, 10 193.
+// Bound: issue, then the latency of the gathers; 40 k event 161 us a stage (298 us with 10 FP64
+// operations per pair; 137 with one unit for the stresses and one for u, from the values alone).  Two
+// entries at a time; 5 blocks per SM: 4 took 5 % longer, 3 28 %.
 __global__ void __launch_bounds__(32 * kWarps, 5) k_pairs_gradient(EvView v, int stage, const double *__restrict__ gin,
                                                                 PairBufs pl, double *__restrict__ gout)
 {

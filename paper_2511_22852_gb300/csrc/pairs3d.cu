@@ -1,7 +1,7 @@
 // pairs3d.cu -- plain 3D neighbour passes over half-pair lists: the 3D counterpart of the plain
 // 2D passes (the same rows and fallback), over the 27 cells of the generalized Morton table.  Per
 // accepted pair the forward pass evaluates W and grad W once (both depend on r_ab only; grad_b W_ba
-// = -grad_a W_ab) and keeps them in fixed point in both particles' rows; the sum and gradient passes
+// = -grad_a W_ab) and keeps them in both particles' rows; the sum and gradient passes
 // add them in integers (pairs_fixed.cuh), independent of the order: reproducible.
 #include "pairs_fixed.cuh"
 #include "sph_internal.cuh"
@@ -19,14 +19,16 @@ constexpr unsigned kFull = 0xFFFFFFFFu;
 // integers (pair_kernel) run on full warps.  W and grad W go into a's row and, at a place taken
 // from b's counter, into b's row.  The particles' own values go into limbs.
 // (Listing b < a in a's own walk, and finding its W by a search in b's row, kept the sums waiting
-// for memory: 40 k event, sum pass 197 -> 92 us a stage, gradient pass 150 -> 137; 258 k particles
-// in 3+1D 2.5 -> 0.9 and 3.4 -> 2.6 ms.)
+// for memory: 258 k particles, sum pass 2.5 -> 0.9, gradient pass 3.4 -> 2.6 ms a stage, with the sums'
+// units taken from the values alone.)
 // Bound: the L2 sectors of the scattered writes to b's row.  The three components of grad W lie in
 // one 32-byte sector and are written by one store (three 8-byte stores at a stride of 24 bytes
 // wrote 7.6 sectors a pair against 4.4); with that and 6 FP64 operations per unordered pair (15
-// with the kernel's distance in FP64), 258 k particles: density pass 4.36 -> 3.24 ms a stage, the
+// with the kernel's distance in FP64), 258 k particles: both density passes 4.36 -> 3.24 ms a stage, the
 // gradient pass, which reads 36 instead of 28 bytes an entry, 2.6 -> 2.9.  The integers alone gave
-// nothing here (the stores bound it), the layout alone was not measured.
+// nothing here (the stores bound it), the layout alone was not measured.  W in the record's fourth
+// word, read by the sum pass at a stride of 32 bytes: both passes 2 ms a stage more at 1.01 M particles.
+// Now 2.57 ms a stage at 258 k (3.5 with the sum pass).
 __global__ void __launch_bounds__(32 * kWarps, 8) k_pairs3_fwd(EvView v, const double *__restrict__ y,
                                                            const float4 *__restrict__ fpos,
                                                            const double *__restrict__ Nq,
@@ -179,9 +181,12 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_pairs3_fwd(EvView v, const d
 // Gradient pass, half a warp per particle a, over the entries of its row, in integers
 // (pairs_fixed.cuh): sum grad W (3), sum X_b^{j i} grad_j W (3), sum u_b^j grad_k W (9); the
 // epilogue as the per-particle pass.
-// Bound: the latency of the gathers; 258 k particles: 2.9 ms a stage (6.0 with 21 FP64 operations per
-// pair).  4 blocks per SM (of the 2.6 ms with 24-byte entries: 3 gave 3.7, 5 3.8, 6 4.8 ms).  Entries
-// kept out of L1, or the index taken from the padding of the 32-byte entry: no difference.
+// Each sum in the unit of its own largest term, from a first look over the exponents.
+// Bound: issue (59 %) and the gathers of four 32-byte words; 258 k particles: 3.7 ms a stage (2.9 with
+// one unit for the stresses and one for u, from the values alone; 6.0 with 21 FP64 operations per
+// pair).  4 blocks per SM (1.01 M particles: 3 took 1 % less, at 269 k 6 % more; 5 took 15 % more).  The
+// first look without the gradients (looser units) takes 3 % less, without any look 13 %, one unit
+// for all stresses and one for u 13 %; unrolling the look by 2 or 4, or prefetching it: none or worse.
 __global__ void __launch_bounds__(32 * kWarps, 4) k_pairs3_gradient(EvView v, int stage, const double *__restrict__ gin,
                                                                  PairBufs pl, double *__restrict__ gout)
 {
